@@ -366,11 +366,9 @@ int32_t gnntrk_stage_times(gnntrk_handle* h, int32_t max_stages, char* names, do
  *     by the shared memory, registers and tensor-memory columns each CTA needs;
  *     choice[0..3] = node encoder, edge encoder, node step, edge step;
  *   - FP32 SIMT kernels (FP32 handles, and the FP32 re-score of BF16/FP8 handles
- *     with a re-score band): variant 0 (4 warps per block), 1 (8 warps per
- *     block) or 2 (4 warps per block with the layer weights of the edge and
- *     node-step kernels at hidden 32 copied once per block into shared memory
- *     and the next tile's row indices loaded ahead; other kernels and widths
- *     run variant 0 then); choice[4..6] = encoders, node step, edge step;
+ *     with a re-score band): variant 0 (tile height by the number of rows of
+ *     the launch), 1 (tall tiles always) or 2 (short tiles always);
+ *     choice[4..6] = encoders, node step, edge step;
  *   - the BF16 edge step at hidden 32 (BF16 handles): form 0 (each thread
  *     copies its row's [e, h_src, h_dst] into the tile), 1 (the tile is
  *     loaded by TMA: one box of 128 e rows and row gathers of h_src, h_dst)

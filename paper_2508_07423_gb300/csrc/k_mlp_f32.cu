@@ -1,14 +1,10 @@
 // FP32 SIMT kernels of the embedding MLP and the interaction network.
 //
-// Work is cut into tiles of TM rows (hits or edges). A block of 256 threads
-// stages the tile's input rows TRANSPOSED in shared memory (As[k][row], so a
-// warp reading one k for 32 row groups touches consecutive words) and computes
-// each layer as a register-tiled product: thread (lane, warp) owns RM rows x CW
-// columns of the output, reads RM inputs per k with one vector shared-memory
-// load and CW weights with CW/4 warp-uniform float4 loads through the
-// read-only cache, and keeps RM x CW FP32 accumulators in registers (inputs are
-// added in increasing k order). A hidden layer is written back transposed; one
-// thread per row then applies LayerNorm + ReLU over it in place.
+// Row-tiled register products: a lane keeps rows x columns of a layer's output
+// in registers, the input rows of its tile are staged in shared memory, and the
+// inputs of an output element are added in increasing k order, two columns per
+// packed FMA. The interaction-network kernels work per warp (WarpTile), the
+// embedding per block of 256 threads.
 //
 //  k_embed_f32     embedding MLP (Sec. "Hit Embedding and Rough Graph
 //                  Construction") on (r/s0, phi/s1, z/s2), ReLU between layers
@@ -24,6 +20,7 @@
 #include <mutex>
 
 #include "internal.cuh"
+#include "tc_ptx.cuh"
 
 namespace gnntrk {
 
@@ -36,34 +33,27 @@ constexpr int kRowGroups = 32;                     // lanes of a warp
 constexpr int kColGroups = kThreads / kRowGroups;  // warps of the embedding block
 
 // Interaction network: every warp owns whole rows. Lane (rg = lane / 8,
-// cg = lane % 8) holds RM rows (rg + 4 i) x CW columns (32 j + 4 cg + u) of a
-// layer's output in registers (RM x CW = 32 accumulators); a warp covers
-// WR = 4 RM rows and all H columns, so a row's LayerNorm is a reduction over
-// the 8 lanes of its row group and no block-wide barrier is needed. Inputs are
+// cg = lane % 8) holds RM rows (rg + 4 i) x CW columns (32 c + 4 cg + u) of a
+// layer's output in registers; a warp covers WR = 4 RM rows and all H columns,
+// so a row's LayerNorm is a reduction over the 8 lanes of its row group and no
+// block-wide barrier is needed. A lane's part of a reduction is summed in
+// column order and the 8 parts pairwise (0+1, 2+3, ... first), so the result
+// does not depend on RM: every tile height gives the same bits. Inputs are
 // staged row-major in the warp's own shared-memory slice with a row stride of
 // H + 4 floats: the four rows a warp reads at one k fall in distinct bank
 // quads, and the eight lanes of a row group read the same address (broadcast).
-template <int H>
+template <int H_, int RM_>
 struct WarpTile {
-  static constexpr int CW = H / 8;    // columns per lane
-  static constexpr int RM = 256 / H;  // rows per lane
-  static constexpr int WR = 4 * RM;   // rows per warp
-  static constexpr int NJ = CW / 4;   // float4 column chunks per lane
-  static constexpr int LDH = H + 4;   // row stride of staged rows (floats)
-};
-
-// Warps per block, per variant (the autotuner picks one per kernel family).
-template <int V>
-struct Warps {
-  static constexpr int NW = V == 0 ? 4 : 8;
+  static constexpr int H = H_, RM = RM_;
+  static constexpr int CW = H / 8;   // columns per lane
+  static constexpr int RG = 4;       // row groups
+  static constexpr int WR = RG * RM; // rows per warp
+  static constexpr int NJ = H / 32;  // float4 column chunks per lane
+  static constexpr int LDH = H + 4;  // row stride of staged rows (floats)
 };
 
 // Variant chosen per (hidden index, kernel family: 0 encoders, 1 node step,
-// 2 edge step and classifier); set by the autotuner, process wide. Variants:
-// 0 = 4 warps per block, 1 = 8 warps per block, 2 = 4 warps per block with the
-// weight matrices of the edge kernels and the node step staged once per block
-// in shared memory at hidden 32 (the row gathers evict them from L1; the node
-// encoder, and every kernel at hidden 64 and 128, run variant 0 then).
+// 2 edge step and classifier); set by the autotuner, process wide.
 std::atomic<int> g_f32_variant[3][3] = {};
 
 enum GMode : int { G_NODE_ENC = 0, G_EDGE_ENC = 1, G_NODE_UPD = 2, G_EDGE_UPD = 3,
@@ -73,177 +63,295 @@ __device__ __forceinline__ bool input_bad(const Ws& w) {
   return (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) != 0;
 }
 
-// acc[i][4j+u] (+)= sum_{k < KV} A[rg + 4i][k] * WT[(k_off + k) * ldo + 32j + 4cg + u],
-// k ascending; A row-major with stride LDA (K a multiple of 4, KV <= K valid)
-// (SW: the weights WT are in shared memory, row stride ldo)
-template <int H, int K, int KV, int LDA, bool SW = false>
-__device__ __forceinline__ void warp_layer(const float* A, const LayerF32& L, int k_off, int rg,
-                                           int cg, float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
-  constexpr int RM = WarpTile<H>::RM, NJ = WarpTile<H>::NJ;
-  const float* wp = L.WT + size_t(k_off) * L.ldo + 4 * cg;
+// first column of a lane's chunk c
+__device__ __forceinline__ int col_of(int c, int cg) { return 32 * c + 4 * cg; }
+
+// acc[i][4c+u] (+)= sum_{k < KV} A[rg + RG i][k] * W[k * ldo + col_of(c) + u], k ascending;
+// A row-major with stride LDA (K a multiple of 4, KV <= K valid); the weights
+// in global memory, or (SW) in shared memory
+template <class T, int K, int KV, int LDA, bool SW>
+__device__ __forceinline__ void warp_product(const float* A, const float* W, int ldo, int rg, int cg,
+                                             float (&acc)[T::RM][T::CW]) {
+  constexpr int RM = T::RM, NC = T::NJ;
+  const float* wp = W + 4 * cg;
 #pragma unroll 2
-  for (int k4 = 0; k4 < K; k4 += 4) {
+  for (int k0 = 0; k0 < K; k0 += 4) {
     float4 a[RM];
 #pragma unroll
     for (int i = 0; i < RM; ++i)
-      a[i] = *reinterpret_cast<const float4*>(A + (rg + 4 * i) * LDA + k4);
+      a[i] = *reinterpret_cast<const float4*>(A + (rg + T::RG * i) * LDA + k0);
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-      if (KV < K && k4 + t >= KV) break;
-      float4 q[NJ];
+      if (KV < K && k0 + t >= KV) break;
+      float4 q[NC];
 #pragma unroll
-      for (int j = 0; j < NJ; ++j)
-        q[j] = SW ? *reinterpret_cast<const float4*>(wp + size_t(k4 + t) * L.ldo + 32 * j)
-                  : __ldg(reinterpret_cast<const float4*>(wp + size_t(k4 + t) * L.ldo + 32 * j));
+      for (int c = 0; c < NC; ++c) {
+        const float* wc = wp + (k0 + t) * ldo + 32 * c;
+        q[c] = SW ? *reinterpret_cast<const float4*>(wc) : __ldg(reinterpret_cast<const float4*>(wc));
+      }
 #pragma unroll
       for (int i = 0; i < RM; ++i) {
         const float av = t == 0 ? a[i].x : (t == 1 ? a[i].y : (t == 2 ? a[i].z : a[i].w));
         const float2 a2 = make_float2(av, av);
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) {
+        for (int c = 0; c < NC; ++c) {
           // two columns per packed FMA (each lane rounds like fmaf)
-          float2 c01 = __ffma2_rn(a2, make_float2(q[j].x, q[j].y),
-                                  make_float2(acc[i][4 * j], acc[i][4 * j + 1]));
-          float2 c23 = __ffma2_rn(a2, make_float2(q[j].z, q[j].w),
-                                  make_float2(acc[i][4 * j + 2], acc[i][4 * j + 3]));
-          acc[i][4 * j] = c01.x;
-          acc[i][4 * j + 1] = c01.y;
-          acc[i][4 * j + 2] = c23.x;
-          acc[i][4 * j + 3] = c23.y;
+          float2 c01 = __ffma2_rn(a2, make_float2(q[c].x, q[c].y),
+                                  make_float2(acc[i][4 * c], acc[i][4 * c + 1]));
+          float2 c23 = __ffma2_rn(a2, make_float2(q[c].z, q[c].w),
+                                  make_float2(acc[i][4 * c + 2], acc[i][4 * c + 3]));
+          acc[i][4 * c] = c01.x;
+          acc[i][4 * c + 1] = c01.y;
+          acc[i][4 * c + 2] = c23.x;
+          acc[i][4 * c + 3] = c23.y;
         }
       }
     }
   }
 }
 
-template <int H>
-__device__ __forceinline__ void acc_bias(const float* b, int cg,
-                                         float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
+template <class T>
+__device__ __forceinline__ void acc_bias(const float* b, int cg, float (&acc)[T::RM][T::CW]) {
 #pragma unroll
-  for (int j = 0; j < WarpTile<H>::NJ; ++j) {
-    const float4 v = __ldg(reinterpret_cast<const float4*>(b + 32 * j + 4 * cg));
+  for (int c = 0; c < T::NJ; ++c) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(b + col_of(c, cg)));
 #pragma unroll
-    for (int i = 0; i < WarpTile<H>::RM; ++i) {
-      acc[i][4 * j] = v.x;
-      acc[i][4 * j + 1] = v.y;
-      acc[i][4 * j + 2] = v.z;
-      acc[i][4 * j + 3] = v.w;
+    for (int i = 0; i < T::RM; ++i) {
+      acc[i][4 * c] = v.x;
+      acc[i][4 * c + 1] = v.y;
+      acc[i][4 * c + 2] = v.z;
+      acc[i][4 * c + 3] = v.w;
     }
   }
 }
 
-// acc += S[rg + 4i][32j + 4cg + u] (each lane reads only its own elements)
-template <int H>
+// acc += S[rg + RG i][col] (each lane reads only its own elements)
+template <class T>
 __device__ __forceinline__ void acc_add_smem(const float* S, int rg, int cg,
-                                             float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
-  constexpr int LD = WarpTile<H>::LDH;
+                                             float (&acc)[T::RM][T::CW]) {
 #pragma unroll
-  for (int i = 0; i < WarpTile<H>::RM; ++i)
+  for (int i = 0; i < T::RM; ++i)
 #pragma unroll
-    for (int j = 0; j < WarpTile<H>::NJ; ++j) {
-      const float4 v = *reinterpret_cast<const float4*>(S + (rg + 4 * i) * LD + 32 * j + 4 * cg);
-      acc[i][4 * j] += v.x;
-      acc[i][4 * j + 1] += v.y;
-      acc[i][4 * j + 2] += v.z;
-      acc[i][4 * j + 3] += v.w;
+    for (int c = 0; c < T::NJ; ++c) {
+      const float4 v =
+          *reinterpret_cast<const float4*>(S + (rg + T::RG * i) * T::LDH + col_of(c, cg));
+      acc[i][4 * c] += v.x;
+      acc[i][4 * c + 1] += v.y;
+      acc[i][4 * c + 2] += v.z;
+      acc[i][4 * c + 3] += v.w;
     }
 }
 
-template <int H>
+// acc += X[rows[r]][offx + col] (TWO: + Y[rows2[r]][offy + col], the two added
+// first), straight from global memory (missing rows read row 0; their result
+// is dropped)
+template <class T, bool TWO>
+__device__ __forceinline__ void acc_add_rows(const int* rows, const float* X, int64_t ldx,
+                                             const int* rows2, const float* Y, int64_t ldy,
+                                             int rg, int cg, float (&acc)[T::RM][T::CW]) {
+#pragma unroll
+  for (int i = 0; i < T::RM; ++i) {
+    const int r = rg + T::RG * i;
+    const float* x = X + size_t(max(rows[r], 0)) * ldx;
+    const float* y = TWO ? Y + size_t(max(rows2[r], 0)) * ldy : nullptr;
+#pragma unroll
+    for (int c = 0; c < T::NJ; ++c) {
+      float4 v = __ldcg(reinterpret_cast<const float4*>(x + col_of(c, cg)));
+      if constexpr (TWO) {
+        const float4 u = __ldcg(reinterpret_cast<const float4*>(y + col_of(c, cg)));
+        v.x += u.x;
+        v.y += u.y;
+        v.z += u.z;
+        v.w += u.w;
+      }
+      acc[i][4 * c] += v.x;
+      acc[i][4 * c + 1] += v.y;
+      acc[i][4 * c + 2] += v.z;
+      acc[i][4 * c + 3] += v.w;
+    }
+  }
+}
+
+template <class T>
 __device__ __forceinline__ void acc_store_smem(float* S, int rg, int cg,
-                                               const float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
-  constexpr int LD = WarpTile<H>::LDH;
+                                               const float (&acc)[T::RM][T::CW]) {
 #pragma unroll
-  for (int i = 0; i < WarpTile<H>::RM; ++i)
+  for (int i = 0; i < T::RM; ++i)
 #pragma unroll
-    for (int j = 0; j < WarpTile<H>::NJ; ++j)
-      *reinterpret_cast<float4*>(S + (rg + 4 * i) * LD + 32 * j + 4 * cg) =
-          make_float4(acc[i][4 * j], acc[i][4 * j + 1], acc[i][4 * j + 2], acc[i][4 * j + 3]);
+    for (int c = 0; c < T::NJ; ++c)
+      *reinterpret_cast<float4*>(S + (rg + T::RG * i) * T::LDH + col_of(c, cg)) =
+          make_float4(acc[i][4 * c], acc[i][4 * c + 1], acc[i][4 * c + 2], acc[i][4 * c + 3]);
 }
 
 // rows of the warp to global: dst[rows[r] * ld + off + col] (rows < 0 skipped)
-template <int H>
+template <class T>
 __device__ __forceinline__ void acc_store_rows(float* dst, int64_t ld, int off, const int* rows,
-                                               int rg, int cg,
-                                               const float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
+                                               int rg, int cg, const float (&acc)[T::RM][T::CW]) {
 #pragma unroll
-  for (int i = 0; i < WarpTile<H>::RM; ++i) {
-    const int row = rows[rg + 4 * i];
+  for (int i = 0; i < T::RM; ++i) {
+    const int row = rows[rg + T::RG * i];
     if (row < 0) continue;
-    float* d = dst + size_t(row) * ld + off + 4 * cg;
+    float* d = dst + size_t(row) * ld + off;
 #pragma unroll
-    for (int j = 0; j < WarpTile<H>::NJ; ++j)
-      *reinterpret_cast<float4*>(d + 32 * j) =
-          make_float4(acc[i][4 * j], acc[i][4 * j + 1], acc[i][4 * j + 2], acc[i][4 * j + 3]);
+    for (int c = 0; c < T::NJ; ++c)
+      *reinterpret_cast<float4*>(d + col_of(c, cg)) =
+          make_float4(acc[i][4 * c], acc[i][4 * c + 1], acc[i][4 * c + 2], acc[i][4 * c + 3]);
   }
 }
 
-// sum over the 8 lanes of a row group (lane bits 0..2)
-__device__ __forceinline__ float row_sum(float v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
+// Sums over the 8 lanes of a row group for every row: part[i] is this lane's
+// part of row i; pairwise, by a butterfly that hands half of the remaining rows
+// to the other lane of each pair, so that the work after the sum (a division, a
+// square root) runs once per row and not in all 8 lanes: with 8 rows per lane
+// LayerNorm takes 2.7 k cycles per tile instead of 6.2 k (hidden 64). tot[j] is
+// the sum of row row_of<T>(j, cg) (with fewer rows than lanes several lanes
+// hold the same row).
+template <class T>
+struct RowSums {
+  static constexpr int M = T::RM < 8 ? T::RM : 8;  // lanes that hold distinct rows
+  static constexpr int N = T::RM / M;              // rows per lane
+  static_assert(T::RM % M == 0 && (M & (M - 1)) == 0, "whole butterflies");
+};
+
+template <class T>
+__device__ __forceinline__ int row_of(int j, int cg) {
+  return j * RowSums<T>::M + (cg & (RowSums<T>::M - 1));
+}
+
+template <class T>
+__device__ __forceinline__ void row_sums(const float (&part)[T::RM], int cg,
+                                         float (&tot)[RowSums<T>::N]) {
+  float v[T::RM];
+#pragma unroll
+  for (int i = 0; i < T::RM; ++i) v[i] = part[i];
+  int n = T::RM;
+#pragma unroll
+  for (int o = 1; o < 8; o *= 2) {
+    if (n > RowSums<T>::N) {
+      const bool up = (cg & o) != 0;
+#pragma unroll
+      for (int j = 0; j < T::RM / 2; ++j) {
+        if (2 * j >= n) break;
+        const float keep = up ? v[2 * j + 1] : v[2 * j], send = up ? v[2 * j] : v[2 * j + 1];
+        v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+      n /= 2;
+    } else {
+#pragma unroll
+      for (int j = 0; j < RowSums<T>::N; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < RowSums<T>::N; ++j) tot[j] = v[j];
+}
+
+// the value that row_sums' owner of row i holds, in every lane of the row group
+template <class T>
+__device__ __forceinline__ float row_value(const float (&own)[RowSums<T>::N], int i, int lane) {
+  constexpr int M = RowSums<T>::M;
+  return __shfl_sync(0xffffffffu, own[i / M], (lane & ~(M - 1)) | (i % M));
 }
 
 // per row: ReLU((v - mean) / sqrt(var + eps)) over the H columns
-template <int H>
-__device__ __forceinline__ void acc_ln_relu(float (&acc)[WarpTile<H>::RM][WarpTile<H>::CW]) {
-  constexpr int CW = WarpTile<H>::CW;
+template <class T>
+__device__ __forceinline__ void acc_ln_relu(float (&acc)[T::RM][T::CW], int lane) {
+  constexpr int CW = T::CW, RM = T::RM, H = T::H, N = RowSums<T>::N;
+  const int cg = lane & 7;
+  float part[RM], mean[N], inv[N];
 #pragma unroll
-  for (int i = 0; i < WarpTile<H>::RM; ++i) {
-    float s = 0.f;
+  for (int i = 0; i < RM; ++i) {
+    part[i] = 0.f;
 #pragma unroll
-    for (int c = 0; c < CW; ++c) s += acc[i][c];
-    const float mean = row_sum(s) / float(H);
-    float q = 0.f;
+    for (int c = 0; c < CW; ++c) part[i] += acc[i][c];
+  }
+  row_sums<T>(part, cg, mean);
+#pragma unroll
+  for (int j = 0; j < N; ++j) mean[j] /= float(H);
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    const float m = row_value<T>(mean, i, lane);
+    part[i] = 0.f;
 #pragma unroll
     for (int c = 0; c < CW; ++c) {
-      const float t = acc[i][c] - mean;
-      q = fmaf(t, t, q);
+      acc[i][c] -= m;
+      part[i] = fmaf(acc[i][c], acc[i][c], part[i]);
     }
-    const float inv = 1.0f / sqrtf(row_sum(q) / float(H) + kLnEps);
+  }
+  row_sums<T>(part, cg, inv);
 #pragma unroll
-    for (int c = 0; c < CW; ++c) acc[i][c] = fmaxf((acc[i][c] - mean) * inv, 0.f);
+  for (int j = 0; j < N; ++j) inv[j] = 1.0f / sqrtf(inv[j] / float(H) + kLnEps);
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    const float r = row_value<T>(inv, i, lane);
+#pragma unroll
+    for (int c = 0; c < CW; ++c) acc[i][c] = fmaxf(acc[i][c] * r, 0.f);
   }
 }
 
-// S[r][col] = X[rows[r]][off + col] (+ Y[rows2[r]][off2 + col]), zero for rows < 0;
+// bias + dot product of every row (after LayerNorm and ReLU) with the 1-unit
+// layer L: out[j] is row row_of<T>(j, cg)'s
+template <class T>
+__device__ __forceinline__ void row_dots(const float (&acc)[T::RM][T::CW], const LayerF32& L, int cg,
+                                         float (&out)[RowSums<T>::N]) {
+  float part[T::RM];
+#pragma unroll
+  for (int i = 0; i < T::RM; ++i) part[i] = 0.f;
+#pragma unroll
+  for (int c = 0; c < T::NJ; ++c)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float wv = __ldg(L.WT + size_t(col_of(c, cg) + u) * L.ldo);
+#pragma unroll
+      for (int i = 0; i < T::RM; ++i) part[i] = fmaf(acc[i][4 * c + u], wv, part[i]);
+    }
+  row_sums<T>(part, cg, out);
+#pragma unroll
+  for (int j = 0; j < RowSums<T>::N; ++j) out[j] = L.b[0] + out[j];
+}
+
+// S[r][col] = X[rows[r]][offx + col] (+ Y[rows2[r]][offy + col]), zero for rows < 0;
 // 8 lanes per row, one float4 column chunk each, four rows per instruction.
 // Loads are unconditional (row 0 stands in for a missing row, its value is
-// then dropped) so that all of a lane's loads are in flight together.
-template <int H, bool TWO>
+// then dropped) so that a lane's loads (up to 16 at a time) are in flight
+// together.
+template <class T, bool TWO>
 __device__ __forceinline__ void stage_rows(float* S, const int* rows, const float* X, int64_t ldx,
                                            int offx, const int* rows2, const float* Y,
                                            int64_t ldy, int offy, int lane) {
-  constexpr int RM = WarpTile<H>::RM, NJ = WarpTile<H>::NJ, LD = WarpTile<H>::LDH;
+  constexpr int NR = T::WR / 4, NJ = T::NJ, LD = T::LDH;
+  constexpr int G = NR * NJ <= 16 ? NR : 16 / NJ;  // rows per lane and batch of loads
+  static_assert(NR % G == 0, "whole batches");
   const int gr = lane >> 3, q = lane & 7;
-  float4 v[RM][NJ];
+#pragma unroll 1
+  for (int i0 = 0; i0 < NR; i0 += G) {
+    float4 v[G][NJ];
 #pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const int row = rows[gr + 4 * i];
-    const int rx = max(row, 0);
-    const int ry = TWO ? (row >= 0 ? rows2[gr + 4 * i] : 0) : 0;
+    for (int i = 0; i < G; ++i) {
+      const int row = rows[gr + 4 * (i0 + i)];
+      const int rx = max(row, 0);
+      const int ry = TWO ? (row >= 0 ? rows2[gr + 4 * (i0 + i)] : 0) : 0;
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
-      v[i][j] = __ldcg(reinterpret_cast<const float4*>(X + size_t(rx) * ldx + offx + 32 * j + 4 * q));
-      if (TWO) {
-        const float4 y =
-            __ldcg(reinterpret_cast<const float4*>(Y + size_t(ry) * ldy + offy + 32 * j + 4 * q));
-        v[i][j].x += y.x;
-        v[i][j].y += y.y;
-        v[i][j].z += y.z;
-        v[i][j].w += y.w;
+      for (int j = 0; j < NJ; ++j) {
+        v[i][j] = __ldcg(reinterpret_cast<const float4*>(X + size_t(rx) * ldx + offx + 32 * j + 4 * q));
+        if (TWO) {
+          const float4 y =
+              __ldcg(reinterpret_cast<const float4*>(Y + size_t(ry) * ldy + offy + 32 * j + 4 * q));
+          v[i][j].x += y.x;
+          v[i][j].y += y.y;
+          v[i][j].z += y.z;
+          v[i][j].w += y.w;
+        }
       }
     }
-  }
 #pragma unroll
-  for (int i = 0; i < RM; ++i) {
-    const bool ok = rows[gr + 4 * i] >= 0;
+    for (int i = 0; i < G; ++i) {
+      const int r = gr + 4 * (i0 + i);
+      const bool ok = rows[r] >= 0;
 #pragma unroll
-    for (int j = 0; j < NJ; ++j)
-      *reinterpret_cast<float4*>(S + (gr + 4 * i) * LD + 32 * j + 4 * q) =
-          ok ? v[i][j] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int j = 0; j < NJ; ++j)
+        *reinterpret_cast<float4*>(S + r * LD + 32 * j + 4 * q) =
+            ok ? v[i][j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
   }
 }
 
@@ -267,163 +375,240 @@ struct GnnArgs {
   const int32_t* tn;
   float* tlogit;
   uint8_t* tkeep;
+  int short_rounds;  // see k_gnn_f32
 };
 
-template <int H, int MODE>
-__host__ __device__ constexpr int g_lda() {
-  return MODE == G_NODE_ENC ? 8 : WarpTile<H>::LDH;
+__host__ __device__ constexpr bool g_edge_rows(int mode) {
+  return mode != G_NODE_ENC && mode != G_NODE_UPD;
 }
 
-// shared memory of one warp (floats): staged input A, hidden Hs, row ids and,
-// for the node step, a third row buffer Bs
-template <int H, int MODE>
-__host__ __device__ constexpr int g_warp_floats() {
-  return WarpTile<H>::WR * (g_lda<H, MODE>() + WarpTile<H>::LDH) + 4 * WarpTile<H>::WR +
-         (MODE == G_NODE_UPD ? WarpTile<H>::WR * WarpTile<H>::LDH : 0);
-}
+// Where a kernel reads its layer weights: copies of the whole matrices in shared
+// memory (hidden 32 and 64), or a ring of chunks in shared memory that bulk
+// copies refill as the block's warps walk through the layers (hidden 128, whose
+// matrices do not fit).
+enum Weights : int { W_BLOCK = 1, W_RING = 2 };
 
-// Resident blocks per SM the register budget is sized for: at h = 32 the
-// 4-warp edge kernels fit 5 blocks of shared memory per SM, so their
-// registers are capped to let 5 blocks (20 warps) reside; elsewhere the
-// compiler's choice stands.
-template <int H, int MODE, int NW, bool SW>
-__host__ __device__ constexpr int g_min_blocks() {
-  return (H == 32 && NW == 4 && MODE != G_NODE_ENC && MODE != G_NODE_UPD) ? (SW ? 4 : 5) : 1;
-}
+// Shape of one kernel: a tall and a short warp tile, warps per block (one block
+// per SM: fewer, larger blocks measured faster at the same number of warps,
+// the layer weights being there once) and the source of the weights.
+//
+// A warp's row buffer holds one tall tile: its input segments pass through the
+// buffer in turn, the residual row is read again and the projected rows are
+// added straight from global memory, which leaves room for 12-20 warps of tall
+// tiles. Short tiles are for calls of few rows: more warps share the rows, and
+// every input segment has a buffer of its own, so that all gathers are in
+// flight at once. Every output element is the same sum in the same order in
+// both.
+template <int H_, int RM_, int RM_SHORT_, int MODE_, int NW_, int WEIGHTS_>
+struct GnnShape {
+  using Tall = WarpTile<H_, RM_>;
+  using Short = WarpTile<H_, RM_SHORT_>;
+  static constexpr int H = H_, MODE = MODE_, NW = NW_;
+  static constexpr bool COPIES = WEIGHTS_ == W_BLOCK, RING = WEIGHTS_ == W_RING;
+  // input segments with a buffer of their own in a short tile
+  static constexpr int SEGS = MODE == G_NODE_UPD ? 3 : MODE == G_NODE_ENC || MODE == G_CLS ? 1 : 2;
+  static constexpr int ROWS = Tall::WR > SEGS * Short::WR ? Tall::WR : SEGS * Short::WR;
+  // row buffers, features of the node encoder (8 floats per row), row ids
+  static constexpr int FEATS = MODE == G_NODE_ENC ? 8 * Tall::WR : 0;
+  static constexpr int IDS = Tall::WR * (g_edge_rows(MODE) ? 3 : 1);
+  static constexpr int WARP_FLOATS = ROWS * Tall::LDH + FEATS + IDS;
+  // H x H matrices a tile's layers use, in this order (layer_mat)
+  static constexpr int MATS = MODE == G_NODE_ENC ? 3
+                              : MODE == G_NODE_UPD ? 6
+                              : MODE == G_EDGE_UPD || MODE == G_TRIP ? 2
+                              : MODE == G_EDGE_UPD_CLS ? 3 : 1;
+  // ring of weight chunks (RING): KC rows of a matrix per chunk
+  static constexpr int KC = 16, NST = 4;
+  [[maybe_unused]] static constexpr int CPL = H / KC;  // chunks per matrix
+  static constexpr int WEIGHT_FLOATS = COPIES ? MATS * H * H
+                                       : RING ? NST * KC * H + 4 * NST : 0;  // chunks, barriers, counts
+  static constexpr size_t SMEM = (size_t(NW) * WARP_FLOATS + WEIGHT_FLOATS) * 4;
+};
 
-// Weight matrices a kernel keeps in shared memory (variant 2), in units of
-// H x H floats: edge steps the e block of the first layer, the second layer
-// and (last step) the classifier's first layer; the edge encoder its second
-// layer; the node step its first layer (3 blocks: h, m_out, m_in) and its
-// second layer, which leaves the node kernel at the 3 blocks per SM its
-// registers allow. (Staging only one matrix in the edge steps, so that a
-// fifth block fits an SM, measured slower: 2.14 against 2.06 ms per step of
-// the headline's re-score edge steps.)
+// matrix m (H rows, row stride ldo = H) of a tile's layer sequence
 template <int MODE>
-__host__ __device__ constexpr int g_sw_mats() {
-  return MODE == G_EDGE_ENC ? 1
-         : MODE == G_EDGE_UPD ? 2
-         : MODE == G_EDGE_UPD_CLS ? 3
-         : MODE == G_NODE_UPD ? 4 : 0;
+__device__ __forceinline__ const float* layer_mat(const GnnArgs& p, int m) {
+  if constexpr (MODE == G_NODE_ENC) return m == 0 ? p.m.l2.WT : m == 1 ? p.proj.src.WT : p.proj.dst.WT;
+  if constexpr (MODE == G_NODE_UPD)
+    return m < 3 ? p.m.l1.WT + size_t(m) * p.m.l2.in * p.m.l1.ldo
+                 : m == 3 ? p.m.l2.WT : m == 4 ? p.proj.src.WT : p.proj.dst.WT;
+  if constexpr (MODE == G_EDGE_ENC) return p.m.l2.WT;
+  if constexpr (MODE == G_CLS) return p.cls.l1.WT;
+  if constexpr (MODE == G_TRIP) return p.m.l1.WT + size_t(m) * p.m.l1.out * p.m.l1.ldo;
+  return m == 0 ? p.m.l1.WT : m == 1 ? p.m.l2.WT : p.cls.l1.WT;
 }
 
-// copy rows [0, R) of a transposed layer (row stride ldo) into S (row stride H)
-template <int H, int NT, int R = H>
-__device__ __forceinline__ void stage_weights(float* S, const LayerF32& L) {
-  for (int i = threadIdx.x; i < R * H / 4; i += NT) {
-    const int k = i / (H / 4), c = 4 * (i % (H / 4));
-    *reinterpret_cast<float4*>(S + k * H + c) =
-        __ldg(reinterpret_cast<const float4*>(L.WT + size_t(k) * L.ldo + c));
-  }
-}
+// The ring of weight chunks of one block: chunk g (g = 0, 1, ...) is rows
+// [(g % CPL) KC, + KC) of matrix (g / CPL) % RMATS and lies in stage g % NST;
+// a stage's barrier completes when its bytes have landed, and the last of the
+// block's NW warps to finish a chunk refills the stage with chunk g + NST. A
+// wait that runs out latches ST_TIMEOUT; the warp then waits no more.
+constexpr long long kRingWaitCycles = 4000000000LL;  // about 2 s
 
-template <int H, int MODE, int NW, bool SW = false>
-__global__ void __launch_bounds__(NW * 32, (g_min_blocks<H, MODE, NW, SW>())) k_gnn_f32(const GnnArgs p) {
-  using T = WarpTile<H>;
-  constexpr int RM = T::RM, CW = T::CW, WR = T::WR;
-  constexpr int LDA = g_lda<H, MODE>();
-  constexpr bool EDGE_ROWS = MODE != G_NODE_ENC && MODE != G_NODE_UPD;
-  static_assert(!SW || g_sw_mats<MODE>() > 0, "weights in shared memory: edge and node-step kernels");
-  extern __shared__ __align__(16) float sm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float* As = sm + warp * g_warp_floats<H, MODE>();  // [WR][LDA]
-  float* Hs = As + WR * LDA;                          // [WR][H + 4]
-  int* rows = reinterpret_cast<int*>(Hs + WR * T::LDH);
-  int* srcs = rows + WR;
-  int* dsts = srcs + WR;
-  const Ws& w = p.w;
-  if (input_bad(w)) return;
-  int lo, hi;
-  if constexpr (MODE == G_TRIP) {
-    if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_CAPACITY) return;
-    lo = 0;
-    hi = min(*p.tn, int(w.t_cap));
-    if (hi <= 0) return;
-  } else {
-    if (!sel_rows(p.b, w, p.sel, EDGE_ROWS, lo, hi)) return;
-  }
-  const int rg = lane >> 3, cg = lane & 7;
-  const int E = clamp_edges(w.counters, w.e_cap);
-  // the layers this kernel multiplies by: global memory, or (SW) copies in
-  // shared memory after the warps' slices (row stride H)
-  LayerF32 l1 = p.m.l1, l2 = p.m.l2, c1 = p.cls.l1;
-  if constexpr (SW && MODE == G_NODE_UPD) {
-    float* S = sm + NW * g_warp_floats<H, MODE>();
-    stage_weights<H, NW * 32, 3 * H>(S, p.m.l1);  // [h, m_out, m_in] -> H
-    l1 = LayerF32{S, p.m.l1.b, 3 * H, H, H};
-    S += 3 * H * H;
-    stage_weights<H, NW * 32>(S, p.m.l2);
-    l2 = LayerF32{S, p.m.l2.b, H, H, H};
-    __syncthreads();
-  } else if constexpr (SW) {
-    float* S = sm + NW * g_warp_floats<H, MODE>();
-    if constexpr (MODE != G_EDGE_ENC) {
-      stage_weights<H, NW * 32>(S, p.m.l1);  // rows [0, H): the e block
-      l1 = LayerF32{S, p.m.l1.b, H, H, H};
-      S += H * H;
-    }
-    stage_weights<H, NW * 32>(S, p.m.l2);
-    l2 = LayerF32{S, p.m.l2.b, H, H, H};
-    S += H * H;
-    if constexpr (MODE == G_EDGE_UPD_CLS) {
-      stage_weights<H, NW * 32>(S, p.cls.l1);
-      c1 = LayerF32{S, p.cls.l1.b, H, H, H};
-    }
-    __syncthreads();
-  }
-  (void)l1;
-  (void)l2;
-  (void)c1;
+template <class X>
+struct WeightRing {
+  float* buf;
+  uint64_t* full;
+  int* done;
+  int g = 0, total = 0;
+  bool dead = false;
 
-  // Edge rows: the index chain (row id from the list, then its source and
-  // target) is loaded ahead in registers, lane r holding row r of a tile: the
-  // row ids two tiles ahead and the source / target one tile ahead are loaded
-  // during a tile and first used in the next one, so a tile's row gathers
-  // start without waiting for its indices.
-  // (variant 2 only: the index registers push the 5-block register budget of
-  // the other variants into spills)
-  constexpr bool AHEAD = SW && EDGE_ROWS && MODE != G_TRIP;
-  const int tstride = gridDim.x * NW * WR;
-  const int base0 = lo + (blockIdx.x * NW + warp) * WR;
-  auto row_at = [&](int b) {
-    const int pos = b + lane;
-    return (lane < WR && pos < hi) ? sel_row(p.sel, pos) : -1;
-  };
-  int r_cur = -1, s_cur = 0, d_cur = 0, r_next = -1;
-  if constexpr (AHEAD) {
-    r_cur = row_at(base0);
-    s_cur = r_cur >= 0 ? w.src[r_cur] : 0;
-    d_cur = r_cur >= 0 ? w.col[r_cur] : 0;
-    r_next = row_at(base0 + tstride);
+  __device__ __forceinline__ void load(const GnnArgs& p, int c) {
+    const int m = (c / X::CPL) % X::MATS, k = (c % X::CPL) * X::KC;
+    uint64_t* f = full + c % X::NST;
+    constexpr uint32_t bytes = X::KC * X::H * 4;
+    tc::mbar_expect_tx(f, bytes);
+    tc::bulk_g2s(buf + (c % X::NST) * X::KC * X::H, layer_mat<X::MODE>(p, m) + size_t(k) * X::H, bytes, f);
   }
-  for (int base = base0; base < hi; base += tstride) {
-    // ---- rows of this warp -----------------------------------------------
-    if constexpr (AHEAD) {
-      if (lane < WR) {
-        rows[lane] = r_cur;
-        srcs[lane] = s_cur;
-        dsts[lane] = d_cur;
+  // block-wide; tiles: the block's tiles
+  __device__ __forceinline__ void start(const GnnArgs& p, float* smem, int tiles) {
+    buf = smem;
+    full = reinterpret_cast<uint64_t*>(smem + X::NST * X::KC * X::H);
+    done = reinterpret_cast<int*>(full + X::NST);
+    total = tiles * X::MATS * X::CPL;
+    if (threadIdx.x == 0) {
+      for (int s = 0; s < X::NST; ++s) {
+        tc::mbar_init(full + s, 1);
+        done[s] = 0;
       }
-      s_cur = r_next >= 0 ? w.src[r_next] : 0;
-      d_cur = r_next >= 0 ? w.col[r_next] : 0;
-      r_cur = r_next;
-      r_next = row_at(base + 2 * tstride);
-    } else if (lane < WR) {
-      const int pos = base + lane;
-      int row = -1, a = 0, c = 0;
-      if (pos < hi) {
-        row = MODE == G_TRIP ? pos : sel_row(p.sel, pos);
-        if (MODE == G_TRIP) {
-          a = p.t1[row];
-          c = p.t2[row];
-        } else if (EDGE_ROWS) {
-          a = w.src[row];
-          c = w.col[row];
+      tc::fence_mbar_init();
+      for (int c = 0; c < X::NST && c < total; ++c) load(p, c);
+    }
+    __syncthreads();
+  }
+  // the next matrix of the sequence times the staged rows A
+  template <class T>
+  __device__ __forceinline__ void product(const GnnArgs& p, const float* A, int rg, int cg,
+                                          float (&acc)[T::RM][T::CW]) {
+#pragma unroll 1
+    for (int c = 0; c < X::CPL; ++c) {
+      const int st = g % X::NST;
+      if (!dead && !tc::mbar_wait_bounded(full + st, (g / X::NST) & 1, kRingWaitCycles)) {
+        dead = true;
+        set_status(p.w.counters, ST_TIMEOUT);
+      }
+      warp_product<T, X::KC, X::KC, T::LDH, true>(A + c * X::KC, buf + st * X::KC * X::H, X::H, rg,
+                                                  cg, acc);
+      __syncwarp();  // every lane is done with the chunk
+      if ((threadIdx.x & 31) == 0 && g + X::NST < total) {
+        __threadfence_block();
+        if (atomicAdd(done + st, 1) == X::NW - 1) {
+          done[st] = 0;
+          __threadfence_block();
+          load(p, g + X::NST);
         }
       }
-      rows[lane] = row;
-      srcs[lane] = a;
-      dsts[lane] = c;
+      ++g;
+    }
+  }
+};
+
+// The weights a kernel multiplies by: matrix m of its layer sequence from the
+// copies in shared memory, or from the ring (which serves the matrices of every
+// tile in their order).
+template <class X>
+struct LayerWeights {
+  const GnnArgs& p;
+  WeightRing<X> ring;
+  const float* copies = nullptr;
+
+  // block-wide; smem: WEIGHT_FLOATS floats, tiles: the block's tiles
+  __device__ __forceinline__ LayerWeights(const GnnArgs& a, float* smem, int tiles) : p(a) {
+    if constexpr (X::RING) ring.start(p, smem, tiles);
+    if constexpr (X::COPIES) {
+      constexpr int N = X::H * X::H / 4;
+      for (int i = threadIdx.x; i < X::MATS * N; i += X::NW * 32)
+        reinterpret_cast<float4*>(smem)[i] =
+            __ldg(reinterpret_cast<const float4*>(layer_mat<X::MODE>(p, i / N)) + i % N);
+      __syncthreads();
+      copies = smem;
+    }
+  }
+  // acc += A (staged rows) x matrix m
+  template <class T>
+  __device__ __forceinline__ void product(const float* A, int m, int rg, int cg,
+                                          float (&acc)[T::RM][T::CW]) {
+    constexpr int H = X::H;
+    if constexpr (X::RING)
+      ring.template product<T>(p, A, rg, cg, acc);
+    else
+      warp_product<T, H, H, T::LDH, true>(A, copies + m * H * H, H, rg, cg, acc);
+  }
+};
+
+// The block's tiles of T::WR rows of positions [lo, hi): tile t goes to block
+// t % gridDim.x, warp (t / gridDim.x) % NW, so that few tiles spread over all
+// blocks.
+template <class X, class T>
+__device__ __forceinline__ void gnn_rows(const GnnArgs& p, float* sm, int lo, int hi) {
+  constexpr int MODE = X::MODE, NW = X::NW, H = X::H;
+  constexpr bool MULTI = T::RM == X::Short::RM;  // a row buffer per input segment
+  constexpr int RM = T::RM, CW = T::CW, WR = T::WR, LD = T::LDH;
+  constexpr bool EDGE_ROWS = g_edge_rows(MODE);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float* B0 = sm + warp * X::WARP_FLOATS;  // [WR][H + 4]
+  float* B1 = MULTI && X::SEGS > 1 ? B0 + WR * LD : B0;
+  float* B2 = MULTI && X::SEGS > 2 ? B0 + 2 * WR * LD : B0;
+  float* F = B0 + X::ROWS * LD;  // node encoder: [WR][8] features
+  int* rows = reinterpret_cast<int*>(F + X::FEATS);
+  int* srcs = EDGE_ROWS ? rows + WR : nullptr;
+  int* dsts = EDGE_ROWS ? srcs + WR : nullptr;
+  (void)B1;
+  (void)B2;
+  const Ws& w = p.w;
+  const int rg = lane >> 3, cg = lane & 7;
+  const int tstride = gridDim.x * NW * WR;
+  const int block0 = lo + blockIdx.x * WR;
+  if (block0 >= hi) return;  // no rows for this block
+  LayerWeights<X> weights(p, sm + NW * X::WARP_FLOATS, (hi - block0 + tstride - 1) / tstride);
+
+  // Edge rows: the index chain (row id from the list, then its source and
+  // target) is loaded ahead in registers, lane r holding row r (and r + 32) of
+  // a tile: the row ids two tiles ahead and the source / target one tile
+  // ahead are loaded during a tile and first used in the next one, so a tile's
+  // row gathers start without waiting for its indices.
+  constexpr bool AHEAD = EDGE_ROWS && MODE != G_TRIP;
+  constexpr int NI = (WR + 31) / 32;
+  const int base0 = block0 + warp * gridDim.x * WR;
+  auto row_at = [&](int b, int i) {
+    const int r = lane + 32 * i, pos = b + r;
+    return (r < WR && pos < hi) ? sel_row(p.sel, pos) : -1;
+  };
+  int r_cur[NI], s_cur[NI], d_cur[NI], r_next[NI];
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      r_cur[i] = row_at(base0, i);
+      s_cur[i] = r_cur[i] >= 0 ? w.src[r_cur[i]] : 0;
+      d_cur[i] = r_cur[i] >= 0 ? w.col[r_cur[i]] : 0;
+      r_next[i] = row_at(base0 + tstride, i);
+    }
+  }
+  // (with a weight ring every warp of the block walks every tile of the block)
+  for (int base = base0; (X::RING ? base - base0 + block0 : base) < hi; base += tstride) {
+    // ---- rows of this warp -----------------------------------------------
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int r = lane + 32 * i;
+      if constexpr (AHEAD) {
+        if (r < WR) {
+          rows[r] = r_cur[i];
+          srcs[r] = s_cur[i];
+          dsts[r] = d_cur[i];
+        }
+        s_cur[i] = r_next[i] >= 0 ? w.src[r_next[i]] : 0;
+        d_cur[i] = r_next[i] >= 0 ? w.col[r_next[i]] : 0;
+        r_cur[i] = r_next[i];
+        r_next[i] = row_at(base + 2 * tstride, i);
+      } else if (r < WR) {
+        const int pos = base + r;
+        const bool in = pos < hi;
+        rows[r] = in ? (MODE == G_TRIP ? pos : sel_row(p.sel, pos)) : -1;
+        if constexpr (MODE == G_TRIP) {
+          srcs[r] = in ? p.t1[pos] : 0;
+          dsts[r] = in ? p.t2[pos] : 0;
+        }
+      }
     }
     __syncwarp();
     float acc[RM][CW];
@@ -431,130 +616,155 @@ __global__ void __launch_bounds__(NW * 32, (g_min_blocks<H, MODE, NW, SW>())) k_
     if constexpr (MODE == G_NODE_ENC || MODE == G_NODE_UPD) {
       if constexpr (MODE == G_NODE_ENC) {
         // features (x/s3, y/s4, z/s5) of each hit, column 3 zero
-        if (lane < WR) {
-          const int row = rows[lane];
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          const int r = lane + 32 * i;
+          if (r >= WR) break;
+          const int row = rows[r];
           float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
           if (row >= 0) {
             const float4 q = w.pos[row];
             f = make_float4(q.x / p.fs[3], q.y / p.fs[4], q.z / p.fs[5], 0.f);
           }
-          *reinterpret_cast<float4*>(As + lane * LDA) = f;
+          *reinterpret_cast<float4*>(F + r * 8) = f;
         }
         __syncwarp();
-        acc_bias<H>(p.m.l1.b, cg, acc);
-        warp_layer<H, 4, 3, LDA>(As, p.m.l1, 0, rg, cg, acc);
-        acc_ln_relu<H>(acc);
-        acc_store_smem<H>(Hs, rg, cg, acc);
+        acc_bias<T>(p.m.l1.b, cg, acc);
+        warp_product<T, 4, 3, 8, false>(F, p.m.l1.WT, p.m.l1.ldo, rg, cg, acc);
+        acc_ln_relu<T>(acc, lane);
+        acc_store_smem<T>(B0, rg, cg, acc);
         __syncwarp();
-        acc_bias<H>(p.m.l2.b, cg, acc);
-        warp_layer<H, H, H, T::LDH>(Hs, p.m.l2, 0, rg, cg, acc);
-        __syncwarp();  // all lanes are done reading Hs
+        acc_bias<T>(p.m.l2.b, cg, acc);
+        weights.template product<T>(B0, 0, rg, cg, acc);
+        __syncwarp();  // all lanes are done reading B0
       } else {
-        // [h, sum_out e, sum_in e]: h in Hs, the two sums (written into the
-        // node's projection row by k_msg_f32) in As and Bs
-        float* Bs = Hs + WR * T::LDH + 4 * WR;
-        stage_rows<H, false>(Hs, rows, w.hstate, H, 0, nullptr, nullptr, 0, 0, lane);
-        stage_rows<H, false>(As, rows, w.pstate, 2 * H, 0, nullptr, nullptr, 0, 0, lane);
-        stage_rows<H, false>(Bs, rows, w.pstate, 2 * H, H, nullptr, nullptr, 0, 0, lane);
+        // [h, sum_out e, sum_in e] (the two sums written into the node's
+        // projection row by k_msg_f32)
+        stage_rows<T, false>(B0, rows, w.hstate, H, 0, nullptr, nullptr, 0, 0, lane);
+        if constexpr (MULTI) {
+          stage_rows<T, false>(B1, rows, w.pstate, 2 * H, 0, nullptr, nullptr, 0, 0, lane);
+          stage_rows<T, false>(B2, rows, w.pstate, 2 * H, H, nullptr, nullptr, 0, 0, lane);
+        }
         __syncwarp();
-        acc_bias<H>(p.m.l1.b, cg, acc);
-        warp_layer<H, H, H, T::LDH, SW>(Hs, l1, 0, rg, cg, acc);
-        warp_layer<H, H, H, LDA, SW>(As, l1, H, rg, cg, acc);
-        warp_layer<H, H, H, T::LDH, SW>(Bs, l1, 2 * H, rg, cg, acc);
-        acc_ln_relu<H>(acc);
-        __syncwarp();  // all lanes are done reading As
-        acc_store_smem<H>(As, rg, cg, acc);
+        acc_bias<T>(p.m.l1.b, cg, acc);
+        weights.template product<T>(B0, 0, rg, cg, acc);
+        if constexpr (!MULTI) {
+          __syncwarp();
+          stage_rows<T, false>(B0, rows, w.pstate, 2 * H, 0, nullptr, nullptr, 0, 0, lane);
+          __syncwarp();
+        }
+        weights.template product<T>(B1, 1, rg, cg, acc);
+        if constexpr (!MULTI) {
+          __syncwarp();
+          stage_rows<T, false>(B0, rows, w.pstate, 2 * H, H, nullptr, nullptr, 0, 0, lane);
+          __syncwarp();
+        }
+        weights.template product<T>(B2, 2, rg, cg, acc);
+        acc_ln_relu<T>(acc, lane);
+        __syncwarp();  // all lanes are done reading B1 (which is B0 without MULTI)
+        acc_store_smem<T>(B1, rg, cg, acc);
         __syncwarp();
-        acc_bias<H>(p.m.l2.b, cg, acc);
-        warp_layer<H, H, H, LDA, SW>(As, l2, 0, rg, cg, acc);
-        acc_add_smem<H>(Hs, rg, cg, acc);  // residual h
+        acc_bias<T>(p.m.l2.b, cg, acc);
+        weights.template product<T>(B1, 3, rg, cg, acc);
+        if constexpr (MULTI) {
+          acc_add_smem<T>(B0, rg, cg, acc);  // residual h
+        } else {
+          acc_add_rows<T, false>(rows, w.hstate, H, nullptr, nullptr, 0, rg, cg, acc);
+          __syncwarp();  // all lanes are done reading B0
+        }
       }
-      acc_store_rows<H>(w.hstate, H, 0, rows, rg, cg, acc);
+      acc_store_rows<T>(w.hstate, H, 0, rows, rg, cg, acc);
       // ---- projections of the new node state for the next edge layer -------
-      acc_store_smem<H>(Hs, rg, cg, acc);
+      acc_store_smem<T>(B0, rg, cg, acc);
       __syncwarp();
-      acc_bias<H>(p.proj.src.b, cg, acc);
-      warp_layer<H, H, H, T::LDH>(Hs, p.proj.src, 0, rg, cg, acc);
-      acc_store_rows<H>(w.pstate, 2 * H, 0, rows, rg, cg, acc);
-      acc_bias<H>(p.proj.dst.b, cg, acc);
-      warp_layer<H, H, H, T::LDH>(Hs, p.proj.dst, 0, rg, cg, acc);
-      acc_store_rows<H>(w.pstate, 2 * H, H, rows, rg, cg, acc);
+      acc_bias<T>(p.proj.src.b, cg, acc);
+      weights.template product<T>(B0, X::MATS - 2, rg, cg, acc);
+      acc_store_rows<T>(w.pstate, 2 * H, 0, rows, rg, cg, acc);
+      acc_bias<T>(p.proj.dst.b, cg, acc);
+      weights.template product<T>(B0, X::MATS - 1, rg, cg, acc);
+      acc_store_rows<T>(w.pstate, 2 * H, H, rows, rg, cg, acc);
     } else if constexpr (MODE == G_TRIP) {
       // ---- triplet classifier: [e^K(first), e^K(second)] -> Linear ->
       //      LayerNorm -> ReLU -> dot, then the triplet cut -----------------
-      stage_rows<H, false>(As, srcs, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
-      stage_rows<H, false>(Hs, dsts, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
+      stage_rows<T, false>(B0, srcs, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
+      if constexpr (MULTI)
+        stage_rows<T, false>(B1, dsts, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
       __syncwarp();
-      acc_bias<H>(p.m.l1.b, cg, acc);
-      warp_layer<H, H, H, LDA>(As, p.m.l1, 0, rg, cg, acc);
-      warp_layer<H, H, H, T::LDH>(Hs, p.m.l1, H, rg, cg, acc);
-      acc_ln_relu<H>(acc);
-      const LayerF32& tl2 = p.m.l2;
+      acc_bias<T>(p.m.l1.b, cg, acc);
+      weights.template product<T>(B0, 0, rg, cg, acc);
+      if constexpr (!MULTI) {
+        __syncwarp();
+        stage_rows<T, false>(B0, dsts, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
+        __syncwarp();
+      }
+      weights.template product<T>(B1, 1, rg, cg, acc);
+      acc_ln_relu<T>(acc, lane);
+      float lg[RowSums<T>::N];
+      row_dots<T>(acc, p.m.l2, cg, lg);
 #pragma unroll
-      for (int i = 0; i < RM; ++i) {
-        float part = 0.f;
-#pragma unroll
-        for (int j = 0; j < T::NJ; ++j)
-#pragma unroll
-          for (int u = 0; u < 4; ++u)
-            part = fmaf(acc[i][4 * j + u], __ldg(tl2.WT + size_t(32 * j + 4 * cg + u) * tl2.ldo), part);
-        const float lg = tl2.b[0] + row_sum(part);
-        const int row = rows[rg + 4 * i];
-        if (cg == 0 && row >= 0) {
-          p.tlogit[row] = lg;
-          p.tkeep[row] = lg >= p.cut ? 1 : 0;
+      for (int j = 0; j < RowSums<T>::N; ++j) {
+        const int row = rows[rg + T::RG * row_of<T>(j, cg)];
+        if (cg < RowSums<T>::M && row >= 0) {
+          p.tlogit[row] = lg[j];
+          p.tkeep[row] = lg[j] >= p.cut ? 1 : 0;
         }
       }
     } else {
       if constexpr (MODE != G_CLS) {
         // ---- layer 1: b + W_e e + (W_src h_src + W_dst h_dst, projected) ----
-        stage_rows<H, true>(Hs, srcs, w.pstate, 2 * H, 0, dsts, w.pstate, 2 * H, H, lane);
+        if constexpr (MULTI)
+          stage_rows<T, true>(B1, srcs, w.pstate, 2 * H, 0, dsts, w.pstate, 2 * H, H, lane);
         if constexpr (MODE != G_EDGE_ENC)
-          stage_rows<H, false>(As, rows, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
+          stage_rows<T, false>(B0, rows, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
         __syncwarp();
-        acc_bias<H>(p.m.l1.b, cg, acc);
-        if constexpr (MODE != G_EDGE_ENC) warp_layer<H, H, H, LDA, SW>(As, l1, 0, rg, cg, acc);
-        acc_add_smem<H>(Hs, rg, cg, acc);
-        acc_ln_relu<H>(acc);
-        acc_store_smem<H>(Hs, rg, cg, acc);  // own elements only
+        acc_bias<T>(p.m.l1.b, cg, acc);
+        if constexpr (MODE != G_EDGE_ENC) weights.template product<T>(B0, 0, rg, cg, acc);
+        if constexpr (MULTI) {
+          acc_add_smem<T>(B1, rg, cg, acc);
+        } else {
+          acc_add_rows<T, true>(srcs, w.pstate, 2 * H, dsts, w.pstate + H, 2 * H, rg, cg, acc);
+        }
+        acc_ln_relu<T>(acc, lane);
+        if constexpr (!MULTI) __syncwarp();  // all lanes are done reading B0 (= B1)
+        acc_store_smem<T>(B1, rg, cg, acc);
         __syncwarp();
         // ---- layer 2 (+ residual e) -----------------------------------------
-        acc_bias<H>(p.m.l2.b, cg, acc);
-        warp_layer<H, H, H, T::LDH, SW>(Hs, l2, 0, rg, cg, acc);
-        if constexpr (MODE != G_EDGE_ENC) acc_add_smem<H>(As, rg, cg, acc);
-        if constexpr (MODE != G_EDGE_UPD_CLS) acc_store_rows<H>(w.estate, H, 0, rows, rg, cg, acc);
+        acc_bias<T>(p.m.l2.b, cg, acc);
+        weights.template product<T>(B1, MODE == G_EDGE_ENC ? 0 : 1, rg, cg, acc);
+        if constexpr (MODE != G_EDGE_ENC) {
+          if constexpr (MULTI)
+            acc_add_smem<T>(B0, rg, cg, acc);
+          else
+            acc_add_rows<T, false>(rows, w.estate, H, nullptr, nullptr, 0, rg, cg, acc);
+        }
+        if constexpr (MODE != G_EDGE_UPD_CLS) acc_store_rows<T>(w.estate, H, 0, rows, rg, cg, acc);
         if constexpr (MODE == G_EDGE_UPD_CLS) {
-          acc_store_smem<H>(As, rg, cg, acc);  // own elements only
+          if constexpr (!MULTI) __syncwarp();  // all lanes are done reading B0
+          acc_store_smem<T>(B0, rg, cg, acc);
         }
       } else {
-        stage_rows<H, false>(As, rows, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
+        stage_rows<T, false>(B0, rows, w.estate, H, 0, nullptr, nullptr, 0, 0, lane);
       }
       if constexpr (MODE == G_EDGE_UPD_CLS || MODE == G_CLS) {
         // ---- classifier: Linear -> LayerNorm -> ReLU -> dot, then the cut ----
         __syncwarp();
-        acc_bias<H>(p.cls.l1.b, cg, acc);
-        warp_layer<H, H, H, LDA, SW && MODE == G_EDGE_UPD_CLS>(As, c1, 0, rg, cg, acc);
-        acc_ln_relu<H>(acc);
-        const LayerF32& cl2 = p.cls.l2;
+        acc_bias<T>(p.cls.l1.b, cg, acc);
+        weights.template product<T>(B0, X::MATS - 1, rg, cg, acc);
+        acc_ln_relu<T>(acc, lane);
+        float lg[RowSums<T>::N];
+        row_dots<T>(acc, p.cls.l2, cg, lg);
 #pragma unroll
-        for (int i = 0; i < RM; ++i) {
-          float part = 0.f;
-#pragma unroll
-          for (int j = 0; j < T::NJ; ++j)
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-              part = fmaf(acc[i][4 * j + u], __ldg(cl2.WT + size_t(32 * j + 4 * cg + u) * cl2.ldo), part);
-          const float lg = cl2.b[0] + row_sum(part);
-          const int row = rows[rg + 4 * i];
-          if (cg == 0 && row >= 0) {
+        for (int j = 0; j < RowSums<T>::N; ++j) {
+          const int row = rows[rg + T::RG * row_of<T>(j, cg)];
+          if (cg < RowSums<T>::M && row >= 0) {
             bool write = true;
             if (p.rescore_only) {
               const float old = w.logit[row];
               write = old > p.band_lo && old < p.band_hi;
             }
             if (write) {
-              w.logit[row] = lg;
-              w.keep[row] = lg >= p.cut ? 1 : 0;
+              w.logit[row] = lg[j];
+              w.keep[row] = lg[j] >= p.cut ? 1 : 0;
             }
           }
         }
@@ -562,6 +772,36 @@ __global__ void __launch_bounds__(NW * 32, (g_min_blocks<H, MODE, NW, SW>())) k_
     }
     __syncwarp();  // the next tile overwrites this warp's shared memory
   }
+  if constexpr (X::RING) {
+    // (after a timeout: no copy may land after the block is gone)
+    if (weights.ring.dead && lane == 0)
+      for (int st = 0; st < X::NST; ++st)
+        tc::mbar_wait_bounded(weights.ring.full + st, 0, kRingWaitCycles);
+  }
+}
+
+template <class X>
+__global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
+  extern __shared__ __align__(16) float sm[];
+  const Ws& w = p.w;
+  if (input_bad(w)) return;
+  int lo, hi;
+  if constexpr (X::MODE == G_TRIP) {
+    if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_CAPACITY) return;
+    lo = 0;
+    hi = min(*p.tn, int(w.t_cap));
+    if (hi <= 0) return;
+  } else {
+    if (!sel_rows(p.b, w, p.sel, g_edge_rows(X::MODE), lo, hi)) return;
+  }
+  // short tiles while they fill at most `short_rounds` rounds of the grid's
+  // warps (launch_shape; the number of rows of an edge kernel or of a row list
+  // is known only here)
+  const int64_t short_rows = int64_t(gridDim.x) * X::NW * X::Short::WR;
+  if (hi - lo <= p.short_rounds * short_rows)
+    gnn_rows<X, typename X::Short>(p, sm, lo, hi);
+  else
+    gnn_rows<X, typename X::Tall>(p, sm, lo, hi);
 }
 
 // ---------------------------------------------------------------------------
@@ -795,37 +1035,56 @@ int blocks_per_sm(const void* fn, int threads, size_t smem) {
   return n;
 }
 
-template <int H, int MODE, int V>
-void launch_gnn_v(const GnnArgs& a, int64_t rows_hint, cudaStream_t s) {
-  // (at hidden 64 and 128 the matrices would cost most of the shared memory
-  // the warps' slices need, so variant 2 is variant 0 there)
-  constexpr bool SW = V == 2 && H == 32 && g_sw_mats<MODE>() > 0;
-  constexpr int NW = Warps<V == 1 ? 1 : 0>::NW, WR = WarpTile<H>::WR;
-  const size_t smem =
-      (size_t(NW) * g_warp_floats<H, MODE>() + (SW ? size_t(g_sw_mats<MODE>()) * H * H : 0)) *
-      sizeof(float);
-  const void* fn = (const void*)k_gnn_f32<H, MODE, NW, SW>;
-  const int full = device_sms() * blocks_per_sm(fn, NW * 32, smem);
-  dim3 grid(full, 1);
-  if (a.sel.rows == nullptr && rows_hint >= 0)
-    grid.x = rows_hint == 0 ? 1 : unsigned(std::min<int64_t>(full, div_up(rows_hint, NW * WR)));
-  k_gnn_f32<H, MODE, NW, SW><<<grid, NW * 32, smem, s>>>(a);
-}
-
 constexpr int f32_family(int mode) {
   return (mode == G_NODE_ENC || mode == G_EDGE_ENC) ? 0 : (mode == G_NODE_UPD ? 1 : 2);
 }
 
+// Variant (0 the default; the autotuner may pick another, see
+// gnntrk_set_tuning): 0 = short tiles for calls whose rows fill at most one
+// round of short tiles over the grid's warps, tall tiles above; 1 = tall tiles
+// always; 2 = short tiles always. The line of variant 0: up to one round every
+// warp has one short tile, and a call's time is the time of one tile (one
+// event of 2146 hits at hidden 64: node step 17.9 us against 31.0 us with tall
+// tiles); with two rounds or more the short tiles' weight loads, one per row
+// group and k instead of one for 8 rows, cost more than the idle warps
+// (16 652 edges, 2.3 rounds: edge step 20.1 us against 17.1 us with tall
+// tiles).
+//
+// Shapes (GB300; edge steps and node steps of a call, against the kernels they
+// replaced, whose warps of 4-warp blocks had 32 accumulators per lane):
+//   hidden 32, 20 warps, 32-row tiles: 4.0 M edges x 4 steps 1.80 ms (2.42),
+//     0.67 M hits x 4 steps 0.71 ms (0.95). 16 warps: 1.85 ms; 8 warps x 2
+//     blocks: 1.99 ms; a 4-lane row group (half the LayerNorm work per row,
+//     8-column lanes): 2.05 ms and more, fewer warps for the registers.
+//   hidden 64, 12 warps, 32-row tiles (64 accumulators per lane): 1.76 M edges
+//     x 8 steps 4.74 ms (6.58), 0.22 M hits x 8 steps 1.73 ms (2.27). 4 warps
+//     x 3 blocks 5.42 ms; weights through L1 5.01 ms, through the ring 5.02 ms.
+//   hidden 128, 12 warps, 16-row tiles, weights through the ring: 1.83 M listed
+//     edges 2.35 ms (4.56), 0.74 M hits 2.83 ms (5.16). Before, one 16-byte
+//     weight load fed 8 products and the L1 pipe was the bound; the six
+//     matrices of the node step (384 KB) miss L1 (4.05 ms without the ring).
+// Now 55 % (hidden 32) to 68 % (hidden 64) of the FP32 rate that packed FMAs
+// reach alone (75 TFLOP/s); what is left is the row gathers and the LayerNorm
+// between the products.
+template <class X>
+void launch_shape(GnnArgs a, int64_t rows_hint, cudaStream_t s) {
+  const int v = g_f32_variant[X::H == 32 ? 0 : (X::H == 64 ? 1 : 2)][f32_family(X::MODE)].load(
+      std::memory_order_relaxed);
+  a.short_rounds = v == 0 ? 1 : v == 1 ? 0 : 1 << 20;
+  const void* fn = (const void*)k_gnn_f32<X>;
+  int grid = device_sms() * blocks_per_sm(fn, X::NW * 32, X::SMEM);
+  if (rows_hint >= 0) grid = std::max(1, std::min(grid, div_up(rows_hint, X::Short::WR)));
+  k_gnn_f32<X><<<grid, X::NW * 32, X::SMEM, s>>>(a);
+}
+
 template <int H, int MODE>
 void launch_gnn(const GnnArgs& a, int64_t rows_hint, cudaStream_t s) {
-  const int v =
-      g_f32_variant[H == 32 ? 0 : (H == 64 ? 1 : 2)][f32_family(MODE)].load(std::memory_order_relaxed);
-  if (v == 2)
-    launch_gnn_v<H, MODE, 2>(a, rows_hint, s);
-  else if (v == 1)
-    launch_gnn_v<H, MODE, 1>(a, rows_hint, s);
+  if constexpr (H == 32)
+    launch_shape<GnnShape<32, 8, 1, MODE, 20, W_BLOCK>>(a, rows_hint, s);
+  else if constexpr (H == 64)
+    launch_shape<GnnShape<64, 8, 1, MODE, 12, W_BLOCK>>(a, rows_hint, s);
   else
-    launch_gnn_v<H, MODE, 0>(a, rows_hint, s);
+    launch_shape<GnnShape<128, 4, 1, MODE, 12, W_RING>>(a, rows_hint, s);
 }
 
 void launch_gnn_any(int h, int mode, const GnnArgs& a, int64_t rows_hint, cudaStream_t s) {

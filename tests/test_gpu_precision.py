@@ -422,3 +422,34 @@ def test_tensor_core_throughput_probe():
     rates = [pkg.tc_throughput(n, iters=4000) for n in (32, 128)]
     assert 0 < rates[0] <= rates[1] * 1.05
     assert rates[1] < 2600.0
+
+
+@pytest.mark.parametrize("name,tracks", [("cfg1_plain_fp32", 1), ("cfg1_plain_fp32", 3),
+                                         ("cfg2_run3_single", 2), ("cfg2_run3_single", 400),
+                                         ("cfg4_batched_fp8", 1), ("cfg4_batched_fp8", 60)])
+def test_fp32_tile_heights_at_ragged_sizes(name, tracks):
+    """Tall, short and size-chosen FP32 tiles at hidden 32, 64 and 128 on one
+    event whose rows fill less than one tile, a ragged last tile, or many
+    rounds: logits, edges and labels are the same bits, and those of the event
+    inside a batch of four."""
+    wl = synth.workload(name)
+    parts = [synth.gen_batch(1, 91 + i, {"kind": "fixed", "n": n}, wl["noise"])
+             for i, n in enumerate((tracks, 5, 37, 12))]
+    one, four = parts[0], synth.concat(parts)
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=four.n_hits, max_events=4,
+                                  edges_per_hit=48)
+    ref = None
+    try:
+        for v in (0, 1, 2):
+            tr.set_tuning({"f32_encoders": v, "f32_node_update": v, "f32_edge_update": v})
+            for b in (one, four):
+                labels = pkg.run_batch(tr, b)[:one.n_hits]
+                g = tr.get_graph(0)
+                if ref is None:
+                    ref = (labels, g)
+                assert np.array_equal(labels, ref[0]), v
+                for k in g:
+                    assert np.array_equal(g[k], ref[1][k]), (v, k)
+    finally:
+        tr.set_tuning({})
+        tr.close()
