@@ -453,3 +453,37 @@ def test_fp32_tile_heights_at_ragged_sizes(name, tracks):
     finally:
         tr.set_tuning({})
         tr.close()
+
+
+@pytest.mark.parametrize("embed", [[3, 64, 64, 4], [3, 64, 64, 64, 6], [3, 128, 128, 1],
+                                   [3, 128, 128, 128, 16], [3, 64, 32, 4], [3, 48, 48, 2]])
+@pytest.mark.parametrize("tracks", [1, 7, 380])
+def test_embedding_shapes_against_float64(embed, tracks):
+    """The FP32 embedding (warp tiles for widths 64 and 128, short and tall, and
+    the block kernel for other shapes), seen through the squared distances of
+    the graph's edges: within the FP32 rounding of the MLP of the float64 ones.
+    Bound: an output's error is below (fan-in + layers) 2^-23 times the sum of
+    the |products|, here below 2e-5 max|e|; d^2 moves by at most 2 sqrt(D) d
+    times that (and its own rounding)."""
+    wl = dict(synth.workload("cfg1_plain_fp32"))
+    wl["model"] = {"embed": embed, "hidden": 32, "iters": 0}
+    ev = synth.gen_batch(1, 17, {"kind": "fixed", "n": tracks}, 0.05)
+    ws = synth.weight_arrays(synth.workload_weights(wl))
+    a = np.stack([np.hypot(ev.x, ev.y, dtype=np.float64) / 45,
+                  np.arctan2(ev.y.astype(np.float64), ev.x.astype(np.float64)) / np.pi,
+                  ev.z.astype(np.float64) / 750], axis=1)
+    for i, (W, b) in enumerate(ws[:len(embed) - 1]):
+        a = a @ W.astype(np.float64).T + b
+        if i + 2 < len(embed):
+            a = np.maximum(a, 0.0)
+    wl["radius2"] = float(np.float32(0.02 * np.mean(np.sum((a - a.mean(0)) ** 2, axis=1)) + 1e-6))
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=ev.n_hits, max_events=1,
+                                  edges_per_hit=64)
+    pkg.run_batch(tr, ev)
+    g = tr.get_graph(0)
+    tr.close()
+    if tracks > 1:
+        assert g["src"].size > 0
+    want = np.sum((a[g["src"]] - a[g["dst"]]) ** 2, axis=1)
+    err = 2e-5 * np.abs(a).max()
+    assert np.all(np.abs(g["d2"] - want) <= 2 * np.sqrt(embed[-1] * wl["radius2"]) * err + 1e-6 * want)
