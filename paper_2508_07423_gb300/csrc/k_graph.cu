@@ -11,11 +11,15 @@
 //  k_scan_*       exclusive scan in two kernels (block sums, with the last
 //                 block scanning them; then block scans plus the block offset),
 //                 used by the triplet stage.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "internal.cuh"
 
 namespace gnntrk {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -160,8 +164,8 @@ __device__ __forceinline__ void load_row(const float* r, float (&q)[D]) {
 // sum_d (q_d - c_d)^2 accumulated by fmaf in increasing d, bit for bit:
 //  CandRows  rows of D floats (global memory, events too large to stage);
 //  CandNegT  the event staged in shared memory transposed and negated,
-//            t[d * ns + c] = -e_c[d], so that two candidates c, c + 1 of one
-//            dimension are one 8-byte load and q_d + (-c_d) (exactly q_d - c_d)
+//            t[d * ns + c] = -e_c[d], so that four candidates c .. c + 3 of one
+//            dimension are one 16-byte load and q_d + (-c_d) (exactly q_d - c_d)
 //            runs as a packed FP32 add, two candidates per instruction.
 template <int D>
 struct CandRows {
@@ -185,16 +189,18 @@ struct CandNegT {
     }
     return s;
   }
-  // d^2 of the candidates c and c + 1 (c even), in one lane each
-  __device__ __forceinline__ float2 d2_pair(const float (&q)[D], int c) const {
-    float2 s = make_float2(0.0f, 0.0f);
+  // d^2 of the candidates c .. c + 3 (c a multiple of 4)
+  __device__ __forceinline__ float4 d2_quad(const float (&q)[D], int c) const {
+    float2 s = make_float2(0.0f, 0.0f), z = s;
 #pragma unroll
     for (int d = 0; d < D; ++d) {
-      const float2 nc = *reinterpret_cast<const float2*>(t + d * ns + c);
-      const float2 u = __fadd2_rn(make_float2(q[d], q[d]), nc);
+      const float4 nc = *reinterpret_cast<const float4*>(t + d * ns + c);
+      const float2 u = __fadd2_rn(make_float2(q[d], q[d]), make_float2(nc.x, nc.y));
+      const float2 v = __fadd2_rn(make_float2(q[d], q[d]), make_float2(nc.z, nc.w));
       s = __ffma2_rn(u, u, s);
+      z = __ffma2_rn(v, v, z);
     }
-    return s;
+    return make_float4(s.x, s.y, z.x, z.y);
   }
   __device__ __forceinline__ void row(int c, float (&q)[D]) const {
 #pragma unroll
@@ -325,24 +331,41 @@ __device__ void select_capped(const Cand& cd, const float (&qe)[D], int c0, int 
 // events) from a look-back over the totals its predecessors publish: an event
 // publishes its own edge count as soon as its degrees are known and its
 // inclusive prefix after its look-back, so a block only waits for blocks that
-// took their tickets before it and are therefore running. Per event:
-//   1. degrees: one thread per query hit, the 32 lanes of a warp on 32 hits
-//      of one plane, so that they read the same candidate rows (broadcast);
-//      the event's embeddings are staged in shared memory when they fit, and
-//      then each hit's in-radius candidates are kept as a bit mask (a hit
-//      over k_max keeps its k_max selected ones);
-//   2. CSR offsets: block scan of min(deg, k_max), look-back, row pointers;
-//   3. fill: one thread per query hit walking its mask bits in ascending
-//      order (or, without masks, its candidates; a hit over k_max is then
-//      filled by its warp, fill_capped);
-//   4. in-edge index: in-degrees by shared-memory atomics, a block scan,
-//      placement by cursors, then each target's list put in ascending edge
-//      id.
-constexpr int kGraphThreads = 512;
+// took their tickets before it and are therefore running. Per event, all in
+// shared memory when it fits (GraphPlan):
+//   1. masks: an item is 32 query hits of one plane (a lane each, so that the
+//      lanes read the same candidate rows, broadcast) x 32 candidates, one
+//      mask word per hit; degrees are the popcounts; a hit over k_max keeps its
+//      k_max selected candidates;
+//   2. CSR offsets: block scan, the event's count published;
+//   3. targets: a thread per hit lists its mask's bits as 16-bit targets and
+//      counts the in-edges of each;
+//   4. in-edge lists: a scan of the counts, placement by cursors, a thread per
+//      edge; an entry's place is the number of smaller entries in its list;
+//   5. after the look-back: the edges (a thread per edge, d^2 again from the
+//      staged rows), the lists and the row pointers, all in coalesced stores.
+// An event too large for that falls back step by step: without the lists the
+// hits write their mask's edges one by one and the in-edge index is built over
+// global memory (csc_general); without the masks the candidates are tested
+// again in the fill; without the staged rows they are read from global memory.
+//
+// What bounds it: the distance tests (an event of 1689 hits in 4 dimensions and
+// 10.1 k edges: 44 of about 102 thousand cycles, 117 of 228 at 2195 hits in 8
+// dimensions), then the latency of the short steps. Before, each lane stored
+// its hit's edges to scattered places (68 of 275 thousand cycles; 326 of 655),
+// and the in-edge lists of an event over 14 k list words were sorted in global
+// memory (155 thousand cycles).
+
+// One block of 1024 threads per SM with all of its shared memory: every event
+// of up to about 2.5 k hits then stays in shared memory, and the threads of one
+// event finish its short steps sooner than those of two events side by side.
+// Per call (two blocks of 512 threads with half the memory each; before the
+// lists were built in shared memory): 1000 events of 1685 hits 433 us (568;
+// 626), 400 events of 2185 hits and 13 k edges 248 us (648; 622), one event of
+// 2146 hits in 8 dimensions 116 us (299; 287).
+constexpr int kGraphThreads = 1024;
 constexpr int kGraphWarps = kGraphThreads / 32;
-constexpr int kGraphBlocksPerSm = 2;            // 16 warps each: 54-62 registers per thread
-constexpr int kGraphSmemBytes = 110 * 1024;  // an event of up to about 4600 hits staged
-constexpr int kGraphSmemInts = kGraphSmemBytes / 4;
+constexpr int kGraphInts = 224 * 1024 / 4;
 constexpr unsigned long long kDescAgg = 1ull << 62;  // the event's own edge count
 constexpr unsigned long long kDescInc = 2ull << 62;  // edges up to and including the event
 constexpr unsigned long long kDescVal = (1ull << 62) - 1;
@@ -390,14 +413,6 @@ __device__ long long graph_wait(unsigned long long* desc, int ev, long long agg,
   return excl;
 }
 
-// warp 0: publish, then wait
-__device__ __forceinline__ long long graph_lookback(unsigned long long* desc, int ev, long long agg,
-                                                    int32_t* counters) {
-  if ((threadIdx.x & 31) == 0) graph_publish(desc, ev, agg);
-  __syncwarp();
-  return graph_wait(desc, ev, agg, counters);
-}
-
 // exclusive scan of min(in[i], clamp) over i < n into out (both may be
 // shared or global memory); every thread gets the total
 __device__ int block_scan(const int32_t* in, int32_t* out, int n, int clamp, int* wsum) {
@@ -435,52 +450,114 @@ __device__ __forceinline__ int clamp31(long long v) {
   return int(v > 0x7fffffffLL ? 0x7fffffffLL : v);
 }
 
-// The query hits of an event are processed in items of up to 32 hits of one
-// plane (a lane per hit), so that the lanes of a warp read the same
-// candidate rows; item t is on plane p with chunk_s[p] <= t < chunk_s[p + 1].
+// Per-plane layout of an event, computed by warp 0: plane p's query hits are cut
+// into chunks of up to 32 (chunk[p] chunks before plane p), each of its hits
+// owns nw[p] mask words from words[p] on, and its mask items (chunk x word)
+// start at items[p]. All arrays end with the total at [P - 1] (the last plane
+// holds no query hits).
+struct GraphPlanes {
+  int po[kMaxPlanes + 1];  // event-local plane offsets
+  int chunk[kMaxPlanes + 1], items[kMaxPlanes + 1], words[kMaxPlanes + 1], nw[kMaxPlanes + 1];
+};
+
+// first candidate of a mask: the first hit of plane p + 1, rounded down to a quad
+__device__ __forceinline__ int mask_first(int c0) { return c0 & ~3; }
+
+__device__ __forceinline__ void graph_planes(GraphPlanes& g, int P) {  // warp 0
+  const int lane = threadIdx.x & 31;
+  int carry[3] = {0, 0, 0};
+  for (int p0 = 0; p0 < P; p0 += 32) {
+    const int p = p0 + lane;
+    int v[3] = {0, 0, 0}, nw = 0;
+    if (p + 1 < P) {
+      const int np = g.po[p + 1] - g.po[p], c0 = g.po[p + 1], c1 = g.po[min(p + 3, P)];
+      nw = np > 0 && c1 > c0 ? (c1 - mask_first(c0) + 31) / 32 : 0;
+      v[0] = (np + 31) / 32;
+      v[1] = v[0] * nw;
+      v[2] = np * nw;
+    }
+    int x[3] = {v[0], v[1], v[2]};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const int y = __shfl_up_sync(kFull, x[i], o);
+        if (lane >= o) x[i] += y;
+      }
+    if (p < P) {
+      g.chunk[p] = carry[0] + x[0] - v[0];
+      g.items[p] = carry[1] + x[1] - v[1];
+      g.words[p] = carry[2] + x[2] - v[2];
+      g.nw[p] = nw;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) carry[i] += __shfl_sync(kFull, x[i], 31);
+  }
+}
+
+// the plane p with first[p] <= t < first[p + 1] (warp-uniform t below the total)
+__device__ __forceinline__ int plane_of(const int* first, int P, int t) {
+  const int lane = threadIdx.x & 31;
+  int p = 0;
+  for (int p0 = 1; p0 < P; p0 += 32)
+    p += __popc(__ballot_sync(kFull, p0 + lane < P && first[p0 + lane] <= t));
+  return p;
+}
+
 struct GraphItem {
   int q0, q1, c0, c1;  // its hits [q0, q1) and their candidates [c0, c1), event-local
 };
 
-__device__ __forceinline__ GraphItem graph_item(const int* po_s, const int* chunk_s, int P, int t) {
-  int p = 0;
-  while (chunk_s[p + 1] <= t) ++p;
-  return GraphItem{po_s[p] + (t - chunk_s[p]) * 32, po_s[p + 1], po_s[p + 1], po_s[min(p + 3, P)]};
+__device__ __forceinline__ GraphItem graph_item(const GraphPlanes& g, int P, int t) {
+  const int p = plane_of(g.chunk, P, t);
+  return GraphItem{g.po[p] + (t - g.chunk[p]) * 32, g.po[p + 1], g.po[p + 1], g.po[min(p + 3, P)]};
 }
 
-// 1. degrees (uncapped) of the event's query hits. With PAIR (the staged,
-// transposed rows) two candidates per step from an even start cA = c0 & ~1,
-// and, when mw > 0, the in-radius candidates of hit q as bit masks:
-// mask[q * mw + k] bit b is candidate cA + 32 k + b.
-template <int D, bool PAIR, class Cand>
-__device__ void graph_degrees(const Cand& cd, const int* po_s, const int* chunk_s, int P,
-                              int n_items, float r2, int32_t* deg, uint32_t* mask, int mw) {
+// mask words of query hit q on plane p
+__device__ __forceinline__ int mask_word(const GraphPlanes& g, int p, int q) {
+  return g.words[p] + (q - g.po[p]) * g.nw[p];
+}
+
+// 1. mask words: bit b of word k of a hit is candidate mask_first + 32 k + b; this
+// block's share of the items, rank of `ranks` blocks
+template <int D>
+__device__ void graph_masks(const CandNegT<D>& cd, const GraphPlanes& g, int P, float r2,
+                            uint32_t* mask, int rank, int ranks) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < n_items; t += kGraphWarps) {
-    const GraphItem it = graph_item(po_s, chunk_s, P, t);
+  const int n_items = g.items[P - 1];
+  for (int t = warp * ranks + rank; t < n_items; t += kGraphWarps * ranks) {
+    const int p = plane_of(g.items, P, t);
+    const int nw = g.nw[p], chunk = (t - g.items[p]) / nw, k = t - g.items[p] - chunk * nw;
+    const int q = g.po[p] + 32 * chunk + lane, c0 = g.po[p + 1], c1 = g.po[min(p + 3, P)];
+    const bool valid = q < c0;
+    float qe[D];
+    cd.row(valid ? q : g.po[p], qe);
+    const int wb = mask_first(c0) + 32 * k;
+    unsigned m = 0;
+#pragma unroll
+    for (int c = 0; c < 32; c += 4) {  // (past c1: staged pad or other rows, masked off)
+      const float4 s = cd.d2_quad(qe, wb + c);
+      m |= (s.x < r2 ? 1u << c : 0u) | (s.y < r2 ? 2u << c : 0u) | (s.z < r2 ? 4u << c : 0u) |
+           (s.w < r2 ? 8u << c : 0u);
+    }
+    if (wb < c0) m &= ~0u << (c0 - wb);
+    if (c1 - wb < 32) m &= (1u << (c1 - wb)) - 1u;
+    if (valid) mask[mask_word(g, p, q) + k] = m;
+  }
+}
+
+// 1. degrees (uncapped) of the event's query hits, without masks
+template <int D, class Cand>
+__device__ void graph_degrees(const Cand& cd, const GraphPlanes& g, int P, float r2, int32_t* deg) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+    const GraphItem it = graph_item(g, P, t);
     const int q = it.q0 + lane;
     const bool valid = q < it.q1;
     float qe[D];
     cd.row(valid ? q : it.q0, qe);
     int cnt = 0;
-    if constexpr (PAIR) {
-      const int cA = it.c0 & ~1;
-      for (int wb = cA; wb < it.c1; wb += 32) {
-        const int we = min(it.c1, wb + 32);
-        unsigned m = 0;
-#pragma unroll 4
-        for (int c = wb; c < we; c += 2) {
-          const float2 s = cd.d2_pair(qe, c);
-          m |= ((s.x < r2 ? 1u : 0u) | (s.y < r2 ? 2u : 0u)) << (c - wb);
-        }
-        if (wb == cA && it.c0 != cA) m &= ~1u;       // c0 - 1 is not a candidate
-        if (we - wb < 32) m &= (1u << (we - wb)) - 1u;  // nor c1 (odd end)
-        cnt += __popc(m);
-        if (mw > 0 && valid) mask[q * mw + (wb - cA) / 32] = m;
-      }
-    } else {
-      for (int c = it.c0; c < it.c1; ++c) cnt += cd.d2(qe, c) < r2;
-    }
+    for (int c = it.c0; c < it.c1; ++c) cnt += cd.d2(qe, c) < r2;
     if (valid) deg[q] = cnt;
   }
 }
@@ -490,21 +567,19 @@ __device__ void graph_degrees(const Cand& cd, const int* po_s, const int* chunk_
 // set bits of its mask in ascending order, recomputes d^2 there from the
 // staged rows and writes its edges at base + off[q].
 template <int D>
-__device__ void graph_fill_masks(const Ws& w, const CandNegT<D>& cd, const int* po_s,
-                                 const int* chunk_s, int P, int n_items, const int32_t* off,
-                                 const uint32_t* mask, int mw, long long base, int v0) {
+__device__ void graph_fill_masks(const Ws& w, const CandNegT<D>& cd, const GraphPlanes& g, int P,
+                                 const int32_t* off, const uint32_t* mask, long long base, int v0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < n_items; t += kGraphWarps) {
-    const GraphItem it = graph_item(po_s, chunk_s, P, t);
-    const int q = it.q0 + lane;
-    if (q >= it.q1) continue;
+  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+    const int p = plane_of(g.chunk, P, t);
+    const int q = g.po[p] + (t - g.chunk[p]) * 32 + lane;
+    if (q >= g.po[p + 1]) continue;
     float qe[D];
     cd.row(q, qe);
     int64_t e = base + off[q];
-    const int cA = it.c0 & ~1;
-    const int nw = (it.c1 - cA + 31) / 32;
-    for (int k = 0; k < nw; ++k) {
-      unsigned m = mask[q * mw + k];
+    const int cA = mask_first(g.po[p + 1]);
+    for (int k = 0; k < g.nw[p]; ++k) {
+      unsigned m = mask[mask_word(g, p, q) + k];
       while (m) {
         const int c = cA + 32 * k + __ffs(m) - 1;
         m &= m - 1;
@@ -523,12 +598,12 @@ __device__ void graph_fill_masks(const Ws& w, const CandNegT<D>& cd, const int* 
 // ascending order and writes its edges at base + off[q]; a hit over k_max is
 // filled by its warp (fill_capped).
 template <int D, class Cand>
-__device__ void graph_fill(const Ws& w, const Cand& cd, const int* po_s, const int* chunk_s, int P,
-                           int n_items, float r2, int k_max, const int32_t* deg,
-                           const int32_t* off, long long base, int v0) {
+__device__ void graph_fill(const Ws& w, const Cand& cd, const GraphPlanes& g, int P, float r2,
+                           int k_max, const int32_t* deg, const int32_t* off, long long base,
+                           int v0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < n_items; t += kGraphWarps) {
-    const GraphItem it = graph_item(po_s, chunk_s, P, t);
+  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+    const GraphItem it = graph_item(g, P, t);
     const int q = it.q0 + lane;
     const bool valid = q < it.q1;
     const int cnt = valid ? deg[q] : 0;
@@ -570,8 +645,8 @@ __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, 
                             int* wsum) {
   const int tid = threadIdx.x;
   const int ne = e1 - e0;
-  const bool full = 2 * int64_t(n) + 2 * int64_t(ne) <= kGraphSmemInts;
-  const bool c_smem = n <= kGraphSmemInts;
+  const bool full = 2 * int64_t(n) + 2 * int64_t(ne) <= kGraphInts;
+  const bool c_smem = n <= kGraphInts;
   int32_t* C = c_smem ? sm_i : w.in_cnt + v0;
   int32_t* St = sm_i + n;               // (full only) list starts, event-local
   int32_t* L = full ? sm_i + 2 * n : w.in_edge + e0;
@@ -645,139 +720,297 @@ __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, 
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kGraphThreads, kGraphBlocksPerSm) k_graph_event(Batch b, Ws w, GraphParams g) {
+// Shared-memory layout of an event (in ints): [off n + 1][cnt n][start n][mask
+// words][rows D x ns + pad][targets, 16 bit][sources, 16 bit]. cnt: degrees, then
+// in-degrees, then cursors; start: starts of the in-edge lists; the lists (16
+// bit) take the mask words' place once the targets are listed. ns: a multiple
+// of 4 (quads). Without room for the sources an edge's source is found by
+// bisection of the offsets.
+struct GraphPlan {
+  int n, ns, words, ne;
+  int cnt, start, mask, rows, targets;  // offsets; off at 0
+  int lists, sources;                   // the in-edge lists, the edges' sources (16 bit)
+  int64_t ints_rows, ints_masks, ints_all;
+  bool with_sources;                    // the sources fit too
+
+  template <int D>
+  __device__ __forceinline__ void rows_and_masks(int n_, int words_) {
+    n = n_;
+    ns = (n + 3) & ~3;
+    words = words_;
+    cnt = n + 1;
+    start = cnt + n;
+    mask = start + n;
+    ints_rows = 3 * int64_t(n) + 1 + int64_t(D) * ns + 40;  // without masks
+    ints_masks = ints_rows + words;
+  }
+  // (after ints_masks was found to fit)
+  template <int D>
+  __device__ __forceinline__ void place_rows(bool masks) {
+    rows = (mask + (masks ? words : 0) + 3) & ~3;
+  }
+  template <int D>
+  __device__ __forceinline__ void edges(int ne_) {
+    ne = ne_;
+    const int half = (ne + 1) / 2;
+    targets = rows + D * ns + 36;  // (36: a mask word reads up to 35 past the last row)
+    lists = half <= words ? mask : targets + half;
+    sources = half <= words ? targets + half : lists + half;
+    ints_all = sources;
+    with_sources = int64_t(sources) + half <= kGraphInts;
+  }
+};
+
+// CLUSTER: the blocks of a cluster share an event's mask items (the bulk of its
+// arithmetic) and write their words into the first block's shared memory, which
+// alone does the rest.
+template <int D, bool CLUSTER>
+__global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w, GraphParams g) {
   extern __shared__ __align__(16) float sm_graph[];
-  __shared__ int po_s[kMaxPlanes + 1];     // event-local plane offsets
-  __shared__ int chunk_s[kMaxPlanes + 1];  // 32-hit chunks of the query planes before p
+  __shared__ GraphPlanes pl;
   __shared__ int wsum[kGraphWarps];
-  __shared__ int ticket_s, mw_s;
+  __shared__ int ticket_s;
   __shared__ long long base_s;
-  if (input_bad(w)) return;
+  if (input_bad(w)) return;  // (written by an earlier kernel: uniform over the grid)
+  constexpr int NT = kGraphThreads;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int rank = CLUSTER ? int(cluster.block_rank()) : 0;
+  const int ranks = CLUSTER ? int(cluster.num_blocks()) : 1;
   const int P = g.n_planes;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float r2 = g.radius2;
   const int k_max = g.k_max;
   int32_t* sm_i = reinterpret_cast<int32_t*>(sm_graph);
   for (;;) {
-    if (tid == 0) ticket_s = atomicAdd(&w.counters[C_GRAPH_TICKET], 1);
-    __syncthreads();
+    if (tid == 0 && rank == 0) {
+      const int t = atomicAdd(&w.counters[C_GRAPH_TICKET], 1);
+      for (int r = 0; r < ranks; ++r) *(CLUSTER ? cluster.map_shared_rank(&ticket_s, r) : &ticket_s) = t;
+    }
+    if constexpr (CLUSTER)
+      cluster.sync();
+    else
+      __syncthreads();
     const int ev = ticket_s;
     if (ev >= b.n_events) return;
     const int v0 = int(w.ev_off[ev]), v1 = int(w.ev_off[ev + 1]);
     const int n = v1 - v0;
     const int32_t* po = w.plane_off + size_t(ev) * (P + 1);
-    for (int i = tid; i <= P; i += kGraphThreads) po_s[i] = po[i] - v0;
-    __syncthreads();
-    if (tid == 0) {
-      int run = 0, words = 0;
-      for (int p = 0; p + 1 < P; ++p) {
-        chunk_s[p] = run;
-        run += (po_s[p + 1] - po_s[p] + 31) / 32;
-        if (po_s[p + 1] > po_s[p])
-          words = max(words, (po_s[min(p + 3, P)] - (po_s[p + 1] & ~1) + 31) / 32);
-      }
-      chunk_s[P > 1 ? P - 1 : 0] = run;
-      mw_s = words;
+    if (warp == 0) {
+      for (int i = lane; i <= P; i += 32) pl.po[i] = po[i] - v0;
+      __syncwarp();
+      graph_planes(pl, P);
     }
-    __syncthreads();  // chunk_s and mw_s (which sets the layout below) visible
-    // rows of this event, event-local index, in shared memory when they fit:
-    //   [off n][mask n*mw][deg n][t D*ns]
-    // off: CSR offsets; mask: in-radius candidates per hit (when they fit too);
-    // t: the embeddings transposed and negated, t[d * ns + i] = -e_i[d]
-    // (8-byte aligned, for the candidate pairs). Else global scratch.
-    const int ns = (n + 2) & ~1;  // even, with a pad column read by the last pair
-    const int64_t rows_ints = int64_t(D) * ns + 3;
-    const bool staged = rows_ints + 2 * int64_t(n) <= kGraphSmemInts;
-    const int mw = staged && rows_ints + int64_t(n) * (2 + mw_s) <= kGraphSmemInts ? mw_s : 0;
+    __syncthreads();  // the layout below depends on the planes
+    GraphPlan L{};
+    L.rows_and_masks<D>(n, pl.words[P - 1]);
+    const bool staged = L.ints_rows <= kGraphInts;
+    const bool masks = staged && L.ints_masks <= kGraphInts && n <= 65535;
+    L.place_rows<D>(masks);
     int32_t* off = staged ? sm_i : w.in_cnt + v0;
-    uint32_t* mask = reinterpret_cast<uint32_t*>(sm_i + n);
-    int32_t* deg = staged ? sm_i + n * (1 + mw) : w.deg + v0;
-    float* tT = sm_graph + ((n * (2 + mw) + 3) & ~3);
+    int32_t* deg = staged ? sm_i + L.cnt : w.deg + v0;
+    uint32_t* mask = reinterpret_cast<uint32_t*>(sm_i + L.mask);
+    float* tT = sm_graph + L.rows;
     if (staged) {
-      for (int k = tid; k < n * D; k += kGraphThreads) {
+      for (int k = tid; k < n * D; k += NT) {
         const int i = k / D, d = k - i * D;
-        tT[d * ns + i] = -w.emb[size_t(v0) * D + k];
-      }
-      for (int k = tid; k < D * (ns - n); k += kGraphThreads) {
-        const int d = k / (ns - n);
-        tT[d * ns + n + (k - d * (ns - n))] = 0.0f;
+        tT[d * L.ns + i] = -w.emb[size_t(v0) * D + k];
       }
     }
     __syncthreads();
-    const int n_items = chunk_s[P > 1 ? P - 1 : 0];
-    const CandNegT<D> cst{tT, ns};
+    const CandNegT<D> cst{tT, L.ns};
     const CandRows<D> cgl{w.emb + size_t(v0) * D};
 
     // 1. degrees (uncapped); with masks, a hit over k_max keeps only its
     //    k_max selected candidates in its mask (the masks then hold exactly
     //    the edges)
-    if (staged)
-      graph_degrees<D, true>(cst, po_s, chunk_s, P, n_items, r2, deg, mask, mw);
-    else
-      graph_degrees<D, false>(cgl, po_s, chunk_s, P, n_items, r2, deg, nullptr, 0);
-    if (P >= 1)
-      for (int q = po_s[P - 1] + tid; q < n; q += kGraphThreads) deg[q] = 0;  // no candidates
-    __syncthreads();
-    if (mw > 0) {
-      for (int t = warp; t < n_items; t += kGraphWarps) {
-        const GraphItem it = graph_item(po_s, chunk_s, P, t);
-        unsigned capped = __ballot_sync(kFull, it.q0 + lane < it.q1 && deg[it.q0 + lane] > k_max);
+    if (masks) {
+      if constexpr (CLUSTER) {
+        graph_masks<D>(cst, pl, P, r2, cluster.map_shared_rank(mask, 0), rank, ranks);
+        cluster.sync();
+      } else {
+        graph_masks<D>(cst, pl, P, r2, mask, 0, 1);
+        __syncthreads();
+      }
+    }
+    if (rank > 0) continue;  // (the next ticket comes when the first block is done)
+    if (masks) {
+      for (int t = warp; t < pl.chunk[P - 1]; t += kGraphWarps) {
+        const int p = plane_of(pl.chunk, P, t);
+        const int q0 = pl.po[p] + (t - pl.chunk[p]) * 32, q = q0 + lane;
+        const int c0 = pl.po[p + 1], c1 = pl.po[min(p + 3, P)];
+        int cnt = 0;
+        if (q < c0) {
+          for (int k = 0; k < pl.nw[p]; ++k) cnt += __popc(mask[mask_word(pl, p, q) + k]);
+          deg[q] = cnt;
+        }
+        unsigned capped = __ballot_sync(kFull, cnt > k_max);
         while (capped) {
-          const int qq = it.q0 + __ffs(capped) - 1;
+          const int qq = q0 + __ffs(capped) - 1;
           capped &= capped - 1;
           float qe[D];
           cst.row(qq, qe);
-          select_capped<D>(cst, qe, it.c0, it.c1, it.c0 & ~1, r2, k_max, mask + qq * mw);
+          select_capped<D>(cst, qe, c0, c1, mask_first(c0), r2, k_max, mask + mask_word(pl, p, qq));
+        }
+      }
+    } else if (staged) {
+      graph_degrees<D>(cst, pl, P, r2, deg);
+    } else {
+      graph_degrees<D>(cgl, pl, P, r2, deg);
+    }
+    for (int q = pl.po[P - 1] + tid; q < n; q += NT) deg[q] = 0;  // no candidates
+    __syncthreads();
+
+    // 2. offsets: event-local exclusive scan of min(deg, k_max), the event's
+    //    count published
+    const int total = block_scan(deg, off, n, k_max, wsum);
+    if (tid == 0) graph_publish(w.graph_desc, ev, total);
+    L.edges<D>(total);
+    const bool lists = masks && L.ints_all <= kGraphInts && total <= 65535;
+    uint16_t* tgt = reinterpret_cast<uint16_t*>(sm_i + L.targets);
+    uint16_t* list = reinterpret_cast<uint16_t*>(sm_i + L.lists);
+    uint16_t* srcs = reinterpret_cast<uint16_t*>(sm_i + L.sources);
+    int32_t* start = sm_i + L.start;
+    if (lists) {
+      // 3. targets and in-degrees
+      if (tid == 0) off[n] = total;
+      for (int i = tid; i < n; i += NT) deg[i] = 0;
+      __syncthreads();
+      for (int t = warp; t < pl.chunk[P - 1]; t += kGraphWarps) {
+        const int p = plane_of(pl.chunk, P, t);
+        const int q = pl.po[p] + (t - pl.chunk[p]) * 32 + lane;
+        if (q >= pl.po[p + 1]) continue;
+        int e = off[q];
+        const int cA = mask_first(pl.po[p + 1]), w0 = mask_word(pl, p, q);
+        for (int k = 0; k < pl.nw[p]; ++k) {
+          unsigned m = mask[w0 + k];
+          while (m) {
+            const int c = cA + 32 * k + __ffs(m) - 1;
+            m &= m - 1;
+            tgt[e] = uint16_t(c);
+            if (L.with_sources) srcs[e] = uint16_t(q);
+            ++e;
+            atomicAdd(&deg[c], 1);
+          }
         }
       }
       __syncthreads();
+      // 4. in-edge lists
+      block_scan(deg, start, n, 0x7fffffff, wsum);
+      for (int i = tid; i < n; i += NT) deg[i] = start[i];
+      __syncthreads();
+      for (int k = tid; k < total; k += NT) list[atomicAdd(&deg[tgt[k]], 1)] = uint16_t(k);
+      __syncthreads();  // deg[i]: the end of target i's list
     }
 
-    // 2. offsets: event-local exclusive scan of min(deg, k_max), then the
-    //    event's base by the look-back
-    const int total = block_scan(deg, off, n, k_max, wsum);
+    // 5. the event's base, then the stores
     if (warp == 0) {
-      const long long ex = graph_lookback(w.graph_desc, ev, total, w.counters);
+      const long long ex = graph_wait(w.graph_desc, ev, total, w.counters);
       if (lane == 0) base_s = ex;
     }
     __syncthreads();
     const long long base = base_s;
-    for (int i = tid; i < n; i += kGraphThreads) w.row_ptr[v0 + i] = clamp31(base + off[i]);
+    for (int i = tid; i < n; i += NT) w.row_ptr[v0 + i] = clamp31(base + off[i]);
     if (ev == b.n_events - 1 && tid == 0) {
       const long long all = base + total;
       w.row_ptr[v1] = clamp31(all);
       w.counters[C_EDGES] = clamp31(all);
       if (all > w.e_cap || all > 0x7fffffffLL) set_status(w.counters, ST_CAPACITY);
     }
-
-    // 3. fill
-    if (mw > 0)
-      graph_fill_masks<D>(w, cst, po_s, chunk_s, P, n_items, off, mask, mw, base, v0);
-    else if (staged)
-      graph_fill<D>(w, cst, po_s, chunk_s, P, n_items, r2, k_max, deg, off, base, v0);
-    else
-      graph_fill<D>(w, cgl, po_s, chunk_s, P, n_items, r2, k_max, deg, off, base, v0);
-    __syncthreads();  // edges written; shared memory free
-
-    // 4. in-edge index of the event's edges [e0, e1)
     const int e0 = int(base < w.e_cap ? base : w.e_cap);
     const int e1 = int(base + total < w.e_cap ? base + total : w.e_cap);
-    csc_general(w, n, v0, v1, e0, e1, sm_i, wsum);
+    const bool fits = base + total <= w.e_cap;
+    if (lists) {
+      for (int k = tid; k < total; k += NT) {
+        if (!fits && base + k >= w.e_cap) break;
+        int lo = 0;
+        if (L.with_sources) {
+          lo = srcs[k];
+        } else {
+          int hi = n;  // off[lo] <= k < off[hi]
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (off[mid] <= k)
+              lo = mid;
+            else
+              hi = mid;
+          }
+        }
+        const int c = tgt[k];
+        float qe[D];
+        cst.row(lo, qe);
+        w.col[base + k] = v0 + c;
+        w.src[base + k] = v0 + lo;
+        w.d2[base + k] = cst.d2(qe, c);
+      }
+    } else if (masks) {
+      graph_fill_masks<D>(w, cst, pl, P, off, mask, base, v0);
+    } else if (staged) {
+      graph_fill<D>(w, cst, pl, P, r2, k_max, deg, off, base, v0);
+    } else {
+      graph_fill<D>(w, cgl, pl, P, r2, k_max, deg, off, base, v0);
+    }
+    if (lists && fits) {
+      for (int i = tid; i < total; i += NT) {
+        const int k = list[i], t = tgt[k];
+        const int lo = start[t], hi = deg[t];
+        int rank = 0;
+        for (int m = lo; m < hi; ++m) rank += list[m] < k;
+        w.in_edge[e0 + lo + rank] = e0 + k;
+      }
+      for (int i = tid; i < n; i += NT) w.in_ptr[v0 + i] = e0 + start[i];
+      if (tid == 0) w.in_ptr[v1] = e1;  // the next event writes the same value
+    } else {  // (an event that overflows the workspace: its lists end there)
+      __syncthreads();  // edges written; shared memory free
+      csc_general(w, n, v0, v1, e0, e1, sm_i, wsum);
+    }
     __syncthreads();  // shared memory and ticket_s are reused by the next event
   }
 }
 
+int num_sms() {
+  // queried once per process (thread-safe initialisation of a local static)
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 1;
+  }();
+  return n;
+}
+
+// Blocks per event: while the events leave SMs idle, clusters of 2, 4 or 8 blocks
+// share an event's mask items (one event of 2146 hits in 8 dimensions: 112 of
+// 215 thousand cycles in one block; 75 events of 1671 hits: 44 of 83 thousand).
+// A block takes a whole SM, and clusters are placed within groups of SMs, so
+// the lines leave room: 8 blocks up to 12 events, 4 up to 30, 2 up to 76.
 template <int D>
-void graph_d(const Batch& b, const Ws& w, const GraphParams& g, int grid, cudaStream_t s) {
+void graph_d(const Batch& b, const Ws& w, const GraphParams& g, cudaStream_t s) {
   // set once per instantiation (thread-safe initialisation of a local static)
   static const bool attr = [] {
-    cudaFuncSetAttribute(k_graph_event<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kGraphSmemBytes);
+    cudaFuncSetAttribute(k_graph_event<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kGraphInts * 4);
+    cudaFuncSetAttribute(k_graph_event<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         kGraphInts * 4);
     return true;
   }();
   (void)attr;
-  k_graph_event<D><<<grid, kGraphThreads, kGraphSmemBytes, s>>>(b, w, g);
+  const int sms = num_sms(), n = b.n_events;
+  const int ranks = 12 * n <= sms ? 8 : 5 * n <= sms ? 4 : 2 * n <= sms ? 2 : 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(std::min(n, sms) * ranks);
+  cfg.blockDim = dim3(kGraphThreads);
+  cfg.dynamicSmemBytes = kGraphInts * 4;
+  cfg.stream = s;
+  cudaLaunchAttribute a[1];
+  a[0].id = cudaLaunchAttributeClusterDimension;
+  a[0].val.clusterDim.x = ranks;
+  a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+  cfg.attrs = a;
+  cfg.numAttrs = ranks > 1 ? 1 : 0;
+  if (ranks > 1)
+    cudaLaunchKernelEx(&cfg, k_graph_event<D, true>, b, w, g);
+  else
+    cudaLaunchKernelEx(&cfg, k_graph_event<D, false>, b, w, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -878,16 +1111,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int32_t* in, 
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = counters[total_slot];
 }
 
-int num_sms() {
-  // queried once per process (thread-safe initialisation of a local static)
-  static const int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 1;
-  }();
-  return n;
-}
 
 }  // namespace
 
@@ -906,17 +1129,16 @@ void launch_scan(const int32_t* in, int32_t* out, int n, int clamp_max, int32_t*
 void launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s) {
   if (b.n_events <= 0) return;
   cudaMemsetAsync(w.graph_desc, 0, sizeof(unsigned long long) * b.n_events, s);
-  const int grid = std::min(b.n_events, num_sms() * kGraphBlocksPerSm);
   switch (D) {
-    case 1: graph_d<1>(b, w, g, grid, s); break;
-    case 2: graph_d<2>(b, w, g, grid, s); break;
-    case 3: graph_d<3>(b, w, g, grid, s); break;
-    case 4: graph_d<4>(b, w, g, grid, s); break;
-    case 5: graph_d<5>(b, w, g, grid, s); break;
-    case 6: graph_d<6>(b, w, g, grid, s); break;
-    case 7: graph_d<7>(b, w, g, grid, s); break;
-    case 8: graph_d<8>(b, w, g, grid, s); break;
-    case 16: graph_d<16>(b, w, g, grid, s); break;
+    case 1: graph_d<1>(b, w, g, s); break;
+    case 2: graph_d<2>(b, w, g, s); break;
+    case 3: graph_d<3>(b, w, g, s); break;
+    case 4: graph_d<4>(b, w, g, s); break;
+    case 5: graph_d<5>(b, w, g, s); break;
+    case 6: graph_d<6>(b, w, g, s); break;
+    case 7: graph_d<7>(b, w, g, s); break;
+    case 8: graph_d<8>(b, w, g, s); break;
+    case 16: graph_d<16>(b, w, g, s); break;
     default: break;
   }
 }

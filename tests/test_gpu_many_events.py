@@ -116,3 +116,38 @@ def test_many_events_rescore_rows_and_logits(batch):
     # node and edge encoders, K x 3 FP32 steps, components
     K = synth.shape_of(wl).iters
     assert st["launches"] == 1 + 2 + 1 + 1 + 3 * K + 1 + 2 + 3 * K + 1, st["launches"]
+
+
+@pytest.mark.parametrize("n_events", [1, 12, 13, 30, 31, 76, 77])
+@pytest.mark.parametrize("dim", [4, 7])
+def test_graph_kernel_branches_match_float64(n_events, dim):
+    """The graph kernel's ways through an event at the sizes where they switch:
+    clusters of 8, 4, 2 blocks or one block per event (by the number of events),
+    everything in shared memory, without the edges' sources, without the in-edge
+    lists, without the masks, without the staged rows (by the event's size and
+    the number of edges), capped and uncapped hits. Edges against the oracle's
+    brute force (pairs within the radius tolerance excepted, as everywhere), the
+    in-edge index through the scores of a network with one message step."""
+    wl = dict(synth.workload("cfg1_plain_fp32"))
+    wl["model"] = {"embed": [3, 8, dim], "hidden": 32, "iters": 1}
+    sh = synth.shape_of(wl)
+    model = oracle.Model(synth.workload_weights(wl), sh.embed, sh.hidden, sh.iters)
+    sizes = [(150, 8, 0.02), (4, 64, 0.1), (235, 64, 0.02), (285, 64, 0.01), (520, 64, 0.002),
+             (900, 5, 0.004)]
+    for tracks, k_max, r2 in sizes if n_events in (1, 77) else sizes[:1]:
+        big = synth.gen_batch(1, 23 + tracks, {"kind": "fixed", "n": tracks}, 0.02)
+        parts = [big] + [synth.gen_batch(1, 5000 + i, {"kind": "fixed", "n": 3}, 0.1)
+                         for i in range(n_events - 1)]
+        b = synth.concat(parts)
+        w = dict(wl, k_max=k_max, radius2=r2)
+        tr = pkg.tracker_for_workload(w, precision="fp32", max_hits=b.n_hits, max_events=n_events,
+                                      edges_per_hit=64)
+        labels = pkg.run_batch(tr, b)
+        fs = pkg.feat_scale_of(tr.cfg)
+        for e in {0, n_events // 2, n_events - 1}:
+            ev, a = b.event(e), int(b.offsets[e])
+            rep = compare_event(ev, tr.get_graph(e), labels[a:a + ev.n_hits], model, r2, k_max,
+                                sh.iters, wl["cut"], fs)
+            assert not rep.bad_pairs, (tracks, e, rep.bad_pairs[:3])
+            assert rep.max_score_err <= 1e-4, (tracks, e, rep.max_score_err)
+        tr.close()
