@@ -377,8 +377,7 @@ void enqueue_pipeline(gnntrk_handle* h, const Batch& b, const int64_t* offsets, 
   if (h->profiling) collect_stages(h);
   h->last_launches = 0;
   cudaMemsetAsync(w.counters, 0, C_COUNT * sizeof(int32_t), s);
-  cudaMemcpyAsync(w.ev_off, offsets, sizeof(int64_t) * (b.n_events + 1), cudaMemcpyDeviceToDevice, s);
-  stage(h, "sort", s, 1, [&] { launch_sort(b, w, c.n_planes, s); });
+  stage(h, "sort", s, 1, [&] { launch_sort(b, w, offsets, c.n_planes, s); });
   const Sel all{nullptr, nullptr};
   const bool tc = c.precision != GNNTRK_FP32;
   const bool i8 = c.embed_int8 != 0;

@@ -183,7 +183,9 @@ int launch_rescore_sets(const Batch& b, const Ws& w, float band_lo, float band_h
 // ---------------------------------------------------------------------------
 // launchers (host functions), one per kernel family
 // ---------------------------------------------------------------------------
-void launch_sort(const Batch& b, const Ws& w, int n_planes, cudaStream_t s);
+// plane sort; also copies the caller's event offsets to w.ev_off and clears the
+// look-back words of the graph and re-score kernels
+void launch_sort(const Batch& b, const Ws& w, const int64_t* offsets, int n_planes, cudaStream_t s);
 // Column blocks of an edge layer's first Linear for the inputs h_src and
 // h_dst (views into its transposed weights, zero bias): the node kernels
 // project each node once, P[v] = [W_src h_v, W_dst h_v], and the edge kernels
@@ -286,6 +288,53 @@ __device__ __forceinline__ void set_status(int32_t* counters, int bits) {
 __device__ __forceinline__ int clamp_edges(const int32_t* counters, int64_t cap) {
   int e = counters[C_EDGES];
   return e < cap ? e : int(cap);
+}
+
+// Programmatic dependent launch: every kernel of a call is launched so that its
+// blocks may take their places while the kernel before it drains; it waits for
+// that kernel's completion (pdl_wait, before any access to memory that the call
+// writes) and then lets the next one's blocks in (pdl_trigger, after the wait, so
+// that at most one kernel waits behind a running one). What a kernel does
+// before pdl_wait (barriers, tensor memory, copies of the weights) overlaps the
+// kernel before it. One FP32 event (17 kernels): 154 -> 123 us per call, 75
+// trained events (33 kernels) 516 -> 473 us.
+//
+// `early` (launch_pdl) says whether a kernel's blocks may come in before the
+// kernel ahead of it is done. Not the message kernels: their blocks, which need
+// no shared memory, then share SMs with a kernel that holds most of it, and
+// with what L1 is left the sums run slower (400 events in FP32 4.04 -> 4.46 ms per
+// call). Not the triplet kernels (500 events 2.96 -> 3.10 ms), and the
+// tensor-core kernels only up to kEarlyTcHits hits, where the launches count
+// (one event of 2146 hits in BF16 1.11 -> 1.07 ms; 1000 events 9.67 -> 9.78 ms).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_begin() {
+  pdl_wait();
+  pdl_trigger();
+}
+
+constexpr int kEarlyTcHits = 1 << 18;
+
+// cluster: blocks per cluster (1: none)
+template <class... P, class... A>
+inline void launch_pdl(bool early, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s,
+                       int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(unsigned(grid));
+  cfg.blockDim = dim3(unsigned(block));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute a[2];
+  a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  a[1].id = cudaLaunchAttributeClusterDimension;
+  a[1].val.clusterDim.x = unsigned(cluster);
+  a[1].val.clusterDim.y = a[1].val.clusterDim.z = 1;
+  cfg.attrs = a;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 inline int div_up(int64_t a, int64_t b) { return int((a + b - 1) / b); }

@@ -54,6 +54,7 @@ __device__ __forceinline__ void uf_union(volatile int32_t* P, int a, int b, int3
 }
 
 __global__ void k_cc_union(Ws w) {
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
   const int E = clamp_edges(w.counters, w.e_cap);
   for (int base = blockIdx.x * blockDim.x; base < E; base += gridDim.x * blockDim.x) {
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(kCcThreads) k_cc_event(Batch b, Ws w) {
   extern __shared__ int32_t sm_cc[];
   int32_t* sP = sm_cc;                // [kCcSmemHits] parents (event-local input index)
   int32_t* sL = sm_cc + kCcSmemHits;  // [kCcSmemHits] local input index of sorted position
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
   const int E = clamp_edges(w.counters, w.e_cap);
   int kept = 0;
@@ -198,7 +200,7 @@ static cudaError_t noalloc_scratch(cudaStream_t s, int32_t** out) {
 
 void launch_cc(const Batch& b, const Ws& w, cudaStream_t s) {
   if (b.n_events <= 0 || b.n_hits <= 0) {
-    k_cc_union<<<device_sms() * 8, 256, 0, s>>>(w);
+    launch_pdl(true, k_cc_union, device_sms() * 8, 256, 0, s, 1, w);
     return;
   }
   // set once per process (thread-safe initialisation of a local static)
@@ -208,8 +210,8 @@ void launch_cc(const Batch& b, const Ws& w, cudaStream_t s) {
     return true;
   }();
   (void)attr_set;
-  k_cc_event<<<std::min(b.n_events, device_sms() * 16), kCcThreads,
-               2 * kCcSmemHits * sizeof(int32_t), s>>>(b, w);
+  launch_pdl(true, k_cc_event, std::min(b.n_events, device_sms() * 16), kCcThreads,
+             2 * kCcSmemHits * sizeof(int32_t), s, 1, b, w);
 }
 
 }  // namespace gnntrk

@@ -91,7 +91,6 @@ __device__ __forceinline__ void i8_layer_from(const uint32_t* act_in, const int4
 __global__ void __launch_bounds__(kI8Threads) k_embed_int8(Batch b, Ws w, Int8Embed m, int D,
                                                            GraphParams g) {
   extern __shared__ __align__(16) uint8_t smem_i8[];
-  if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
   const int tid = threadIdx.x;
   // stage weights (int4 rows), scales, biases and activation buffers
   int4* sW[kMaxEmbedLayers];
@@ -116,6 +115,8 @@ __global__ void __launch_bounds__(kI8Threads) k_embed_int8(Batch b, Ws w, Int8Em
   uint32_t* act1 = act0 + m.max_in4 * kI8Threads;
   float* inv = reinterpret_cast<float*>(act1 + m.max_in4 * kI8Threads);
   for (int i = tid; i < m.n; i += kI8Threads) inv[i] = m.inv[i];
+  pdl_begin();
+  if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
   __syncthreads();
   for (int base = blockIdx.x * kI8Threads; base < b.n_hits; base += gridDim.x * kI8Threads) {
     const int v = base + tid;
@@ -212,7 +213,7 @@ void launch_embed_int8(const Batch& b, const Ws& w, const Int8Embed& m, int D,
     }
   }
   const int grid = std::max(1, std::min(div_up(b.n_hits, kI8Threads), device_sms() * 8));
-  k_embed_int8<<<grid, kI8Threads, smem, s>>>(b, w, m, D, g);
+  launch_pdl(true, k_embed_int8, grid, kI8Threads, smem, s, 1, b, w, m, D, g);
 }
 
 void launch_embed_amax(const float* xyz, int n_hits, const EmbedAmax& m, const GraphParams& g,

@@ -36,15 +36,22 @@ __device__ __forceinline__ bool input_bad(const Ws& w) {
 // ---------------------------------------------------------------------------
 // stable plane sort, one block per event
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads) k_sort(Batch b, Ws w, int P) {
+__global__ void __launch_bounds__(kSortThreads) k_sort(Batch b, Ws w, const int64_t* offsets, int P) {
   __shared__ int cnt[kMaxPlanes];
   __shared__ int base[kMaxPlanes];
   __shared__ int wcnt[kSortThreads / 32][kMaxPlanes];
   __shared__ int ctot[kMaxPlanes];
   __shared__ int bad;
   const int ev = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t o0 = b.offsets[ev], o1 = b.offsets[ev + 1];
+  pdl_begin();
+  const int64_t o0 = offsets[ev], o1 = offsets[ev + 1];
+  if (w.rs_counts != nullptr && ev == 0)
+    for (int i = tid; i < 6 * (kMaxIters + 2); i += kSortThreads) w.rs_counts[i] = 0;
   if (tid == 0) {
+    w.ev_off[ev] = o0;
+    if (ev == b.n_events - 1) w.ev_off[ev + 1] = o1;
+    w.graph_desc[ev] = 0;
+    if (w.rs_desc != nullptr) w.rs_desc[ev] = 0;
     int f = 0;
     if (o0 < 0 || o1 < o0 || o1 > b.n_hits) f = 1;
     if (ev == 0 && o0 != 0) f = 1;
@@ -771,6 +778,7 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
   __shared__ int wsum[kGraphWarps];
   __shared__ int ticket_s;
   __shared__ long long base_s;
+  pdl_begin();
   if (input_bad(w)) return;  // (written by an earlier kernel: uniform over the grid)
   constexpr int NT = kGraphThreads;
   const cg::cluster_group cluster = cg::this_cluster();
@@ -996,21 +1004,8 @@ void graph_d(const Batch& b, const Ws& w, const GraphParams& g, cudaStream_t s) 
   (void)attr;
   const int sms = num_sms(), n = b.n_events;
   const int ranks = 12 * n <= sms ? 8 : 5 * n <= sms ? 4 : 2 * n <= sms ? 2 : 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(std::min(n, sms) * ranks);
-  cfg.blockDim = dim3(kGraphThreads);
-  cfg.dynamicSmemBytes = kGraphInts * 4;
-  cfg.stream = s;
-  cudaLaunchAttribute a[1];
-  a[0].id = cudaLaunchAttributeClusterDimension;
-  a[0].val.clusterDim.x = ranks;
-  a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
-  cfg.attrs = a;
-  cfg.numAttrs = ranks > 1 ? 1 : 0;
-  if (ranks > 1)
-    cudaLaunchKernelEx(&cfg, k_graph_event<D, true>, b, w, g);
-  else
-    cudaLaunchKernelEx(&cfg, k_graph_event<D, false>, b, w, g);
+  launch_pdl(true, ranks > 1 ? k_graph_event<D, true> : k_graph_event<D, false>,
+             std::min(n, sms) * ranks, kGraphThreads, kGraphInts * 4, s, ranks, b, w, g);
 }
 
 // ---------------------------------------------------------------------------
@@ -1049,6 +1044,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int32_t* in,
                                                               int64_t cap) {
   __shared__ int warp_s[32];
   __shared__ int is_last;
+  pdl_begin();
   if ((*(volatile int32_t*)&counters[C_STATUS]) & ST_INPUT) return;
   const int base = blockIdx.x * kScanChunk;
   int v = 0;
@@ -1090,6 +1086,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int32_t* in, 
                                                              const int32_t* counters,
                                                              int total_slot) {
   __shared__ int warp_s[32];
+  pdl_begin();
   if ((*(volatile const int32_t*)&counters[C_STATUS]) & ST_INPUT) return;
   const int base = blockIdx.x * kScanChunk + threadIdx.x * kScanPer;
   int v[kScanPer];
@@ -1114,21 +1111,22 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const int32_t* in, 
 
 }  // namespace
 
-void launch_sort(const Batch& b, const Ws& w, int n_planes, cudaStream_t s) {
+void launch_sort(const Batch& b, const Ws& w, const int64_t* offsets, int n_planes, cudaStream_t s) {
   if (b.n_events <= 0) return;
-  k_sort<<<b.n_events, kSortThreads, 0, s>>>(b, w, n_planes);
+  launch_pdl(true, k_sort, b.n_events, kSortThreads, 0, s, 1, b, w, offsets, n_planes);
 }
 
 void launch_scan(const int32_t* in, int32_t* out, int n, int clamp_max, int32_t* counters,
                  int total_slot, int64_t cap, int32_t* blocks, cudaStream_t s) {
   const int nb = div_up(n > 0 ? n : 1, kScanChunk);
-  k_scan_reduce<<<nb, kScanThreads, 0, s>>>(in, n, clamp_max, blocks, counters, total_slot, cap);
-  k_scan_apply<<<nb, kScanThreads, 0, s>>>(in, out, n, clamp_max, blocks, counters, total_slot);
+  launch_pdl(false, k_scan_reduce, nb, kScanThreads, 0, s, 1, in, n, clamp_max, blocks, counters,
+             total_slot, cap);
+  launch_pdl(false, k_scan_apply, nb, kScanThreads, 0, s, 1, in, out, n, clamp_max, blocks, counters,
+             total_slot);
 }
 
 void launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s) {
   if (b.n_events <= 0) return;
-  cudaMemsetAsync(w.graph_desc, 0, sizeof(unsigned long long) * b.n_events, s);
   switch (D) {
     case 1: graph_d<1>(b, w, g, s); break;
     case 2: graph_d<2>(b, w, g, s); break;

@@ -452,8 +452,8 @@ struct GnnShape {
 // The ring of weight chunks of one block: chunk g (g = 0, 1, ...) is rows
 // [(g % CPL) KC, + KC) of matrix (g / CPL) % RMATS and lies in stage g % NST;
 // a stage's barrier completes when its bytes have landed, and the last of the
-// block's NW warps to finish a chunk refills the stage with chunk g + NST. A
-// wait that runs out latches ST_TIMEOUT; the warp then waits no more.
+// `users` warps that have a tile to finish a chunk refills the stage with chunk
+// g + NST. A wait that runs out latches ST_TIMEOUT; the warp then waits no more.
 constexpr long long kRingWaitCycles = 4000000000LL;  // about 2 s
 
 template <class X>
@@ -464,7 +464,7 @@ struct WeightRing {
   float* buf;
   uint64_t* full;
   int* done;
-  int g = 0, total = 0;
+  int g = 0, total = 0, users = 0;
   bool dead = false;
 
   __device__ __forceinline__ void load(const typename X::Args& p, int c) {
@@ -473,21 +473,23 @@ struct WeightRing {
     tc::mbar_expect_tx(f, STAGE * 4);
     tc::bulk_g2s(buf + (c % W::NST) * STAGE, X::mat(p, m) + size_t(k) * X::H, STAGE * 4, f);
   }
-  // block-wide; tiles: the block's tiles
-  __device__ __forceinline__ void start(const typename X::Args& p, float* smem, int tiles) {
+  __device__ __forceinline__ void init(float* smem) {  // (a block barrier follows)
     buf = smem;
     full = reinterpret_cast<uint64_t*>(smem + W::NST * STAGE);
     done = reinterpret_cast<int*>(full + W::NST);
-    total = tiles * W::MATS * CPL;
     if (threadIdx.x == 0) {
       for (int s = 0; s < W::NST; ++s) {
         tc::mbar_init(full + s, 1);
         done[s] = 0;
       }
       tc::fence_mbar_init();
-      for (int c = 0; c < W::NST && c < total; ++c) load(p, c);
     }
-    __syncthreads();
+  }
+  // the block walks `tiles` tiles
+  __device__ __forceinline__ void start(const typename X::Args& p, int tiles) {
+    total = tiles * W::MATS * CPL;
+    if (threadIdx.x == 0)
+      for (int c = 0; c < W::NST && c < total; ++c) load(p, c);
   }
   // the next matrix of the sequence times the staged rows A
   template <class T>
@@ -505,7 +507,7 @@ struct WeightRing {
       __syncwarp();  // every lane is done with the chunk
       if ((threadIdx.x & 31) == 0 && g + W::NST < total) {
         __threadfence_block();
-        if (atomicAdd(done + st, 1) == X::NW - 1) {
+        if (atomicAdd(done + st, 1) == users - 1) {
           done[st] = 0;
           __threadfence_block();
           load(p, g + W::NST);
@@ -526,17 +528,26 @@ struct LayerWeights {
   WeightRing<X> ring;
   const float* copies = nullptr;
 
-  // block-wide; smem: W::FLOATS floats, tiles: the block's tiles
-  __device__ __forceinline__ LayerWeights(const typename X::Args& a, float* smem, int tiles) : p(a) {
-    if constexpr (W::RING) ring.start(p, smem, tiles);
+  // block-wide, before pdl_wait (the weights are constant); smem: W::FLOATS floats
+  __device__ __forceinline__ LayerWeights(const typename X::Args& a, float* smem) : p(a) {
+    if constexpr (W::RING) ring.init(smem);
     if constexpr (W::COPIES) {
       constexpr int N = X::H * X::H / 4;
       for (int i = threadIdx.x; i < W::MATS * N; i += X::NW * 32)
         reinterpret_cast<float4*>(smem)[i] =
             __ldg(reinterpret_cast<const float4*>(X::mat(p, i / N)) + i % N);
-      __syncthreads();
       copies = smem;
     }
+    __syncthreads();
+  }
+  // the block walks tiles of `step` rows (per block) from block0 on
+  __device__ __forceinline__ void start(int block0, int step, int hi) {
+    if constexpr (W::RING) ring.start(p, (hi - block0 + step - 1) / step);
+  }
+  // the block's round of tiles that begins at `first` (its warp 0's tile; the
+  // warps' tiles are `stride` rows apart)
+  __device__ __forceinline__ void round(int first, int stride, int hi) {
+    if constexpr (W::RING) ring.users = min(X::NW, (hi - first + stride - 1) / stride);
   }
   // acc += A (staged rows) x matrix m
   template <class T>
@@ -561,7 +572,8 @@ struct LayerWeights {
 // t % gridDim.x, warp (t / gridDim.x) % NW, so that few tiles spread over all
 // blocks.
 template <class X, class T>
-__device__ __forceinline__ void gnn_rows(const GnnArgs& p, float* sm, int lo, int hi) {
+__device__ __forceinline__ void gnn_rows(const GnnArgs& p, LayerWeights<X>& weights, float* sm,
+                                         int lo, int hi) {
   constexpr int MODE = X::MODE, NW = X::NW, H = X::H;
   constexpr bool MULTI = T::RM == X::Short::RM;  // a row buffer per input segment
   constexpr int RM = T::RM, CW = T::CW, WR = T::WR, LD = T::LDH;
@@ -581,7 +593,7 @@ __device__ __forceinline__ void gnn_rows(const GnnArgs& p, float* sm, int lo, in
   const int tstride = gridDim.x * NW * WR;
   const int block0 = lo + blockIdx.x * WR;
   if (block0 >= hi) return;  // no rows for this block
-  LayerWeights<X> weights(p, sm + NW * X::WARP_FLOATS, (hi - block0 + tstride - 1) / tstride);
+  weights.start(block0, tstride, hi);
 
   // Edge rows: the index chain (row id from the list, then its source and
   // target) is loaded ahead in registers, lane r holding row r (and r + 32) of
@@ -605,8 +617,8 @@ __device__ __forceinline__ void gnn_rows(const GnnArgs& p, float* sm, int lo, in
       r_next[i] = row_at(base0 + tstride, i);
     }
   }
-  // (with a weight ring every warp of the block walks every tile of the block)
-  for (int base = base0; (X::W::RING ? base - base0 + block0 : base) < hi; base += tstride) {
+  for (int base = base0; base < hi; base += tstride) {
+    weights.round(base - base0 + block0, int(gridDim.x) * WR, hi);
     // ---- rows of this warp -----------------------------------------------
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
@@ -800,6 +812,8 @@ template <class X>
 __global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
   extern __shared__ __align__(16) float sm[];
   const Ws& w = p.w;
+  LayerWeights<X> weights(p, sm + X::NW * X::WARP_FLOATS);
+  pdl_begin();
   if (input_bad(w)) return;
   int lo, hi;
   if constexpr (X::MODE == G_TRIP) {
@@ -815,9 +829,9 @@ __global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
   // is known only here)
   const int64_t short_rows = int64_t(gridDim.x) * X::NW * X::Short::WR;
   if (hi - lo <= p.short_rounds * short_rows)
-    gnn_rows<X, typename X::Short>(p, sm, lo, hi);
+    gnn_rows<X, typename X::Short>(p, weights, sm, lo, hi);
   else
-    gnn_rows<X, typename X::Tall>(p, sm, lo, hi);
+    gnn_rows<X, typename X::Tall>(p, weights, sm, lo, hi);
 }
 
 // ---------------------------------------------------------------------------
@@ -832,6 +846,7 @@ __global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
 template <int H>
 __global__ void __launch_bounds__(256) k_msg_f32(Batch b, Ws w, Sel sel) {
   constexpr int NJ = H / 32, U = 8 / NJ;
+  pdl_begin();
   if (input_bad(w)) return;
   int lo, hi;
   if (!sel_rows(b, w, sel, false, lo, hi)) return;
@@ -972,6 +987,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_embed_f32(Batch b, Ws w, EmbedL
                                                         int n_embed, int D, GraphParams g,
                                                         int maxw) {
   extern __shared__ __align__(16) float sm[];
+  pdl_begin();
   if (input_bad(w)) return;
   const int tid = threadIdx.x;
   for (int base = blockIdx.x * kEmbedTM; base < b.n_hits; base += gridDim.x * kEmbedTM) {
@@ -1042,7 +1058,7 @@ template <int W_, int RM_, int NH_, int NW_, int WEIGHTS_>
 struct EmbedShape {
   using Args = EmbedArgs;
   using Tall = WarpTile<W_, RM_>;
-  using Short = WarpTile<W_, 1>;
+  using Short = WarpTile<W_, W_ == 128 ? 2 : 1>;
   static constexpr int H = W_, NH = NH_, NW = NW_;
   static constexpr int WARP_FLOATS = Tall::WR * (Tall::LDH + 8);  // rows, features
   using W = WeightSource<W_, NH_, WEIGHTS_>;
@@ -1060,23 +1076,22 @@ __device__ __forceinline__ void acc_relu(float (&acc)[T::RM][T::CW]) {
 }
 
 template <class X, class T>
-__device__ __forceinline__ void embed_rows(const EmbedArgs& p, float* sm) {
+__device__ __forceinline__ void embed_rows(const EmbedArgs& p, LayerWeights<X>& weights, float* sm) {
   constexpr int NW = X::NW, H = X::H, WR = T::WR, LD = T::LDH;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int rg = lane >> 3, cg = lane & 7;
   const int n = p.b.n_hits;
   float* A = sm + warp * X::WARP_FLOATS;  // [WR][H + 4]
   float* F = A + WR * LD;                 // [WR][8] features
-  float* last = sm + NW * X::WARP_FLOATS + X::W::FLOATS;
+  const float* last = sm + NW * X::WARP_FLOATS + X::W::FLOATS;
   const int tstride = gridDim.x * NW * WR;
   const int block0 = blockIdx.x * WR;
   if (block0 >= n) return;  // no rows for this block
   const LayerF32& lo = p.em.l[X::NH + 1];  // W -> D
-  for (int i = threadIdx.x; i < H * lo.ldo; i += NW * 32) last[i] = lo.WT[i];
-  __syncthreads();
-  LayerWeights<X> weights(p, sm + NW * X::WARP_FLOATS, (n - block0 + tstride - 1) / tstride);
+  weights.start(block0, tstride, n);
   const int base0 = block0 + warp * gridDim.x * WR;
-  for (int base = base0; (X::W::RING ? base - base0 + block0 : base) < n; base += tstride) {
+  for (int base = base0; base < n; base += tstride) {
+    weights.round(base - base0 + block0, int(gridDim.x) * WR, n);
     if (lane < WR) {
       const int v = base + lane;
       float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1140,13 +1155,18 @@ __device__ __forceinline__ void embed_rows(const EmbedArgs& p, float* sm) {
 template <class X>
 __global__ void __launch_bounds__(X::NW * 32, 1) k_embed_tiles(const EmbedArgs p) {
   extern __shared__ __align__(16) float sm[];
+  const LayerF32& lo = p.em.l[X::NH + 1];
+  for (int i = threadIdx.x; i < X::H * lo.ldo; i += X::NW * 32)
+    sm[X::NW * X::WARP_FLOATS + X::W::FLOATS + i] = lo.WT[i];
+  LayerWeights<X> weights(p, sm + X::NW * X::WARP_FLOATS);  // (ends with a block barrier)
+  pdl_begin();
   if (input_bad(p.w)) return;
   // short tiles while they fill at most one round of the grid's warps, as the
   // interaction-network kernels
   if (p.b.n_hits <= int64_t(gridDim.x) * X::NW * X::Short::WR)
-    embed_rows<X, typename X::Short>(p, sm);
+    embed_rows<X, typename X::Short>(p, weights, sm);
   else
-    embed_rows<X, typename X::Tall>(p, sm);
+    embed_rows<X, typename X::Tall>(p, weights, sm);
 }
 
 // occupancy of (kernel, block size, shared memory), queried once and cached
@@ -1203,6 +1223,9 @@ constexpr int f32_family(int mode) {
 //     edges 2.35 ms (4.56), 0.74 M hits 2.83 ms (5.16). Before, one 16-byte
 //     weight load fed 8 products and the L1 pipe was the bound; the six
 //     matrices of the node step (384 KB) miss L1 (4.05 ms without the ring).
+//     Short tiles of 8 rows: a warp reads a whole matrix from shared memory per
+//     tile whatever its height (a 16-byte load takes 4 cycles of the pipe), so
+//     half the rows per warp would read twice as much.
 // Now 55 % (hidden 32) to 68 % (hidden 64) of the FP32 rate that packed FMAs
 // reach alone (75 TFLOP/s); what is left is the row gathers and the LayerNorm
 // between the products.
@@ -1214,7 +1237,7 @@ void launch_shape(GnnArgs a, int64_t rows_hint, cudaStream_t s) {
   const void* fn = (const void*)k_gnn_f32<X>;
   int grid = device_sms() * blocks_per_sm(fn, X::NW * 32, X::SMEM);
   if (rows_hint >= 0) grid = std::max(1, std::min(grid, div_up(rows_hint, X::Short::WR)));
-  k_gnn_f32<X><<<grid, X::NW * 32, X::SMEM, s>>>(a);
+  launch_pdl(true, k_gnn_f32<X>, grid, X::NW * 32, X::SMEM, s, 1, a);
 }
 
 template <int H, int MODE>
@@ -1224,7 +1247,7 @@ void launch_gnn(const GnnArgs& a, int64_t rows_hint, cudaStream_t s) {
   else if constexpr (H == 64)
     launch_shape<GnnShape<64, 8, 1, MODE, 12, W_BLOCK>>(a, rows_hint, s);
   else
-    launch_shape<GnnShape<128, 4, 1, MODE, 12, W_RING>>(a, rows_hint, s);
+    launch_shape<GnnShape<128, 4, 2, MODE, 12, W_RING>>(a, rows_hint, s);
 }
 
 void launch_gnn_any(int h, int mode, const GnnArgs& a, int64_t rows_hint, cudaStream_t s) {
@@ -1292,7 +1315,7 @@ template <class X>
 void launch_embed_tiles(const EmbedArgs& a, cudaStream_t s) {
   const int full = device_sms() * blocks_per_sm((const void*)k_embed_tiles<X>, X::NW * 32, X::SMEM);
   const int grid = std::max(1, std::min(full, div_up(a.b.n_hits, X::Short::WR)));
-  k_embed_tiles<X><<<grid, X::NW * 32, X::SMEM, s>>>(a);
+  launch_pdl(true, k_embed_tiles<X>, grid, X::NW * 32, X::SMEM, s, 1, a);
 }
 
 // The warp-tile kernel for one or two hidden layers W -> W of the usual widths
@@ -1326,7 +1349,7 @@ void launch_embed_f32(const Batch& b, const Ws& w, const LayerF32* embed, int n_
   const size_t smem = size_t(2) * maxw * kEmbedTM * sizeof(float);
   const int full = device_sms() * blocks_per_sm((const void*)k_embed_f32, kThreads, smem);
   const int grid = std::max(1, std::min(full, div_up(b.n_hits, kEmbedTM)));
-  k_embed_f32<<<grid, kThreads, smem, s>>>(b, w, a.em, n_embed, D, g, maxw);
+  launch_pdl(true, k_embed_f32, grid, kThreads, smem, s, 1, b, w, a.em, n_embed, D, g, maxw);
 }
 }  // namespace
 
@@ -1357,11 +1380,11 @@ void launch_messages_f32(const Batch& b, const Ws& w, int h, Sel sel, cudaStream
   const int full = device_sms() * 8;
   const int grid = sel.rows ? full : std::max(1, std::min(full, div_up(b.n_hits, 32)));
   if (h == 32)
-    k_msg_f32<32><<<grid, 256, 0, s>>>(b, w, sel);
+    launch_pdl(false, k_msg_f32<32>, grid, 256, 0, s, 1, b, w, sel);
   else if (h == 64)
-    k_msg_f32<64><<<grid, 256, 0, s>>>(b, w, sel);
+    launch_pdl(false, k_msg_f32<64>, grid, 256, 0, s, 1, b, w, sel);
   else
-    k_msg_f32<128><<<grid, 256, 0, s>>>(b, w, sel);
+    launch_pdl(false, k_msg_f32<128>, grid, 256, 0, s, 1, b, w, sel);
 }
 
 void launch_node_update_f32(const Batch& b, const Ws& w, const Mlp2F32& m, const EdgeProj& proj,

@@ -197,6 +197,7 @@ __device__ void rs_lookback(const RsDesc& d, int ev, int nv, const int* cnt, int
 __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc d, float lo,
                                                           float hi, int K) {
   extern __shared__ __align__(16) int8_t sm_lev[];  // endpoints and levels of the event
+  pdl_begin();
   if (input_bad(w.counters)) return;
   __shared__ int wsum[kRsEvWarps];
   __shared__ int wcnt[kRsLists][kRsEvWarps];  // per list and warp: rows, then offsets
@@ -302,10 +303,7 @@ __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc
 
 int launch_rescore_sets(const Batch& b, const Ws& w, float band_lo, float band_hi, int K,
                         cudaStream_t s) {
-  const int NL = kMaxIters + 2;
-  cudaMemsetAsync(w.rs_counts, 0, sizeof(int32_t) * 6 * NL, s);
-  if (b.n_events <= 0) return 0;
-  cudaMemsetAsync(w.rs_desc, 0, sizeof(int32_t) * b.n_events, s);
+  if (b.n_events <= 0) return 0;  // (k_sort clears the counts and the look-back flags)
   const int nv = 2 * (K + 1);
   const RsDesc d{w.rs_desc, w.rs_desc + b.n_events, w.rs_desc + b.n_events + size_t(b.n_events) * nv};
   // set once per process (thread-safe initialisation of a local static)
@@ -314,8 +312,8 @@ int launch_rescore_sets(const Batch& b, const Ws& w, float band_lo, float band_h
     return true;
   }();
   (void)attr;
-  k_rs_event<<<std::min(b.n_events, device_sms() * 2), kRsEvThreads, kRsSmemBytes, s>>>(
-      b, w, d, band_lo, band_hi, K);
+  launch_pdl(true, k_rs_event, std::min(b.n_events, device_sms() * 2), kRsEvThreads, kRsSmemBytes, s, 1, b,
+             w, d, band_lo, band_hi, K);
   return 1;
 }
 

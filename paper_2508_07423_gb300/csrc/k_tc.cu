@@ -462,10 +462,6 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
 
   const int tid = threadIdx.x, warp = tid >> 5;
   const Ws& w = p.w;
-  // (the triplet lists are only valid when the triplet workspace held them)
-  if (*(volatile int32_t*)&w.counters[C_STATUS] & (MODE == M_TRIP ? (ST_INPUT | ST_CAPACITY) : ST_INPUT))
-    return;
-
   // ---- set-up: barriers, TMEM, weights --------------------------------------
   if (tid == 0) {
     mbar_init(&bar[0], 1);
@@ -511,9 +507,13 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
   const bool weights_late = __syncthreads_or(!ok);
   bool aborted = weights_late;
 
+  pdl_begin();
   const bool edge_rows = MODE != M_NODE_ENC && MODE != M_NODE_UPD;
   int lo = 0, hi = 0;
-  {
+  // no tiles after an input error (the triplet lists are only valid when the
+  // triplet workspace held them)
+  const int stop = MODE == M_TRIP ? (ST_INPUT | ST_CAPACITY) : ST_INPUT;
+  if (!(*(volatile int32_t*)&w.counters[C_STATUS] & stop)) {
     const Batch& b = p.b;
     hi = edge_rows ? clamp_edges(w.counters, w.e_cap) : b.n_hits;
     if constexpr (MODE == M_TRIP) hi = min(*p.tn, int(w.t_cap));
@@ -1091,6 +1091,7 @@ __global__ void __launch_bounds__(kRows, 5)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Ws& w = p.w;
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
 
   if (tid == 0) {
@@ -1439,6 +1440,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Ws& w = p.w;
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
 
   if (tid == 0) {
@@ -1697,6 +1699,7 @@ __global__ void __launch_bounds__(256) k_msg_bf16(Batch b, Ws w) {
   constexpr int LPN = H / 8;    // lanes per hit: 8 columns (16 bytes) each
   constexpr int NPW = 32 / LPN; // hits per warp
   constexpr int U = 8;
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
   const int E = clamp_edges(w.counters, w.e_cap);
   const int q = threadIdx.x % LPN;
@@ -1835,7 +1838,7 @@ template <bool CLS>
 void launch_edge_tma(const TcArgs& a, const TcModel& m, cudaStream_t s) {
   using L = TmaLayout<32, CLS>;
   const int grid = device_sms() * tma_blocks_per_sm<CLS>();
-  k_tc_edge_tma<32, CLS><<<grid, kRows, L::ALLOC, s>>>(a, m.map_e, m.map_h);
+  launch_pdl(a.b.n_hits <= kEarlyTcHits, k_tc_edge_tma<32, CLS>, grid, kRows, L::ALLOC, s, 1, a, m.map_e, m.map_h);
 }
 
 // CTAs per SM of the warp-specialised edge step (shared memory bound)
@@ -1861,7 +1864,7 @@ template <bool CLS>
 void launch_edge_ws(const TcArgs& a, const TcModel& m, cudaStream_t s) {
   using L = WsLayout<CLS>;
   const int grid = device_sms() * ws_blocks_per_sm<CLS>();
-  k_tc_edge_ws<CLS><<<grid, kWsThreads, L::ALLOC, s>>>(a, m.map_e, m.map_h);
+  launch_pdl(a.b.n_hits <= kEarlyTcHits, k_tc_edge_ws<CLS>, grid, kWsThreads, L::ALLOC, s, 1, a, m.map_e, m.map_h);
 }
 
 template <int H, bool FP8, int MODE>
@@ -1872,7 +1875,7 @@ void launch_mode(const TcArgs& a, cudaStream_t s, int rows_hint) {
   if (tuned > 0 && tuned < per_sm) per_sm = tuned;
   int grid = device_sms() * per_sm;
   if (rows_hint >= 0) grid = rows_hint == 0 ? 1 : min(grid, div_up(rows_hint, kRows));
-  k_tc<H, FP8, MODE><<<grid, kRows, L::TOTAL, s>>>(a);
+  launch_pdl(a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows, L::TOTAL, s, 1, a);
 }
 
 template <int H, bool FP8>
@@ -2170,11 +2173,11 @@ void tc_node_prep(const Batch& b, const Ws& w, const TcModel& m, const LayerF32*
 void tc_messages(const Batch& b, const Ws& w, int h, bool fp8, cudaStream_t s) {
   const int grid = std::max(1, std::min(device_sms() * 8, div_up(b.n_hits, 256 / (h / 8))));
   if (h == 32)
-    fp8 ? k_msg_bf16<32, false><<<grid, 256, 0, s>>>(b, w) : k_msg_bf16<32, true><<<grid, 256, 0, s>>>(b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<32, false> : k_msg_bf16<32, true>, grid, 256, 0, s, 1, b, w);
   else if (h == 64)
-    fp8 ? k_msg_bf16<64, false><<<grid, 256, 0, s>>>(b, w) : k_msg_bf16<64, true><<<grid, 256, 0, s>>>(b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<64, false> : k_msg_bf16<64, true>, grid, 256, 0, s, 1, b, w);
   else
-    fp8 ? k_msg_bf16<128, false><<<grid, 256, 0, s>>>(b, w) : k_msg_bf16<128, true><<<grid, 256, 0, s>>>(b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<128, false> : k_msg_bf16<128, true>, grid, 256, 0, s, 1, b, w);
 }
 
 void tc_gnn(const Batch& b, const Ws& w, const TcModel& m, int h, int K, const GraphParams& g,

@@ -99,6 +99,7 @@ __device__ __forceinline__ int block_scan(int v, int* sw, int& total) {
 
 // ---- 1. triplet counts per hit ----------------------------------------------
 __global__ void k_trip_count(Batch b, Ws w) {
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.n_hits; c += gridDim.x * blockDim.x) {
     int kout = 0, kin = 0;
@@ -111,6 +112,7 @@ __global__ void k_trip_count(Batch b, Ws w) {
 
 // ---- 2. triplet lists ----------------------------------------------------------
 __global__ void k_trip_fill(Batch b, Ws w) {
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < b.n_hits; c += gridDim.x * blockDim.x) {
     const int o0 = w.row_ptr[c], o1 = w.row_ptr[c + 1];
@@ -193,6 +195,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
   __shared__ unsigned long long s_last;
   __shared__ unsigned long long s_pairs[kPairSort];
   __shared__ int s_w[kTbThreads / 32];
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   const int tid = threadIdx.x;
   for (int ev = blockIdx.x; ev < b.n_events; ev += gridDim.x) {
@@ -412,6 +415,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
                                                           int64_t max_tracks, int64_t max_hits) {
   __shared__ int s_w[kTbThreads / 32];
   __shared__ int s_t, s_h;
+  pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   const int tid = threadIdx.x;
   const int64_t total_tracks = ev_tracks[b.n_events];
@@ -504,6 +508,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
 // totals: kept triplets
 __global__ void k_trip_kept(const uint8_t* ka, const int32_t* na, const uint8_t* ke,
                             const int32_t* ne, int32_t* counters) {
+  pdl_begin();
   if (*(volatile int32_t*)&counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   const int a = *na, e = *ne;
   int k = 0;
@@ -517,30 +522,30 @@ __global__ void k_trip_kept(const uint8_t* ka, const int32_t* na, const uint8_t*
 
 void launch_triplets(const Batch& b, const Ws& w, int h, cudaStream_t s) {
   const int grid = std::max(1, std::min(div_up(b.n_hits, 256), device_sms() * 8));
-  k_trip_count<<<grid, 256, 0, s>>>(b, w);
+  launch_pdl(false, k_trip_count, grid, 256, 0, s, 1, b, w);
   launch_scan(w.trip_cnt_a, w.trip_off_a, b.n_hits, 1 << 30, w.counters, C_TRIP_A, w.t_cap,
               w.scan_blocks, s);
   launch_scan(w.trip_cnt_e, w.trip_off_e, b.n_hits, 1 << 30, w.counters, C_TRIP_E, w.t_cap,
               w.scan_blocks, s);
-  k_trip_fill<<<grid, 256, 0, s>>>(b, w);
+  launch_pdl(false, k_trip_fill, grid, 256, 0, s, 1, b, w);
   (void)h;
 }
 
 void launch_triplet_kept(const Ws& w, cudaStream_t s) {
-  k_trip_kept<<<device_sms() * 4, 256, 0, s>>>(w.trip_akeep, w.counters + C_TRIP_A, w.trip_ekeep,
-                                               w.counters + C_TRIP_E, w.counters);
+  launch_pdl(false, k_trip_kept, device_sms() * 4, 256, 0, s, 1, w.trip_akeep, w.counters + C_TRIP_A,
+             w.trip_ekeep, w.counters + C_TRIP_E, w.counters);
 }
 
 void launch_track_build(const Batch& b, const Ws& w, const TrackOut& out, cudaStream_t s) {
   if (b.n_events <= 0) return;
   const int grid = std::min(b.n_events, device_sms() * 8);
-  k_tb_event<<<grid, kTbThreads, 0, s>>>(b, w);
+  launch_pdl(false, k_tb_event, grid, kTbThreads, 0, s, 1, b, w);
   launch_scan(w.tb_ev_tracks, out.ev_tracks, b.n_events, 1 << 30, w.counters, C_TRACKS,
               int64_t(1) << 40, w.scan_blocks, s);
   launch_scan(w.tb_ev_hits, w.tb_ev_hit_off, b.n_events, 1 << 30, w.counters, C_TRACK_HITS,
               int64_t(1) << 40, w.scan_blocks, s);
-  k_tb_write<<<grid, kTbThreads, 0, s>>>(b, w, out.ev_tracks, out.track_off, out.track_hits,
-                                         out.max_tracks, out.max_hits);
+  launch_pdl(false, k_tb_write, grid, kTbThreads, 0, s, 1, b, w, out.ev_tracks, out.track_off,
+             out.track_hits, out.max_tracks, out.max_hits);
 }
 
 }  // namespace gnntrk
