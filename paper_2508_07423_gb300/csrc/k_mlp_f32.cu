@@ -20,6 +20,7 @@
 #include <mutex>
 
 #include "internal.cuh"
+#include "msg.cuh"
 #include "tc_ptx.cuh"
 
 namespace gnntrk {
@@ -835,66 +836,38 @@ __global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
 }
 
 // ---------------------------------------------------------------------------
-// messages of the node step: m_v = [sum of e over v's out edges, sum over its
-// in edges], each sum in increasing list order starting from zero, written to
-// the node's projection row P[v] = [m_out | m_in] (the node step reads it
-// there and then overwrites the row with the new projections). One group of
-// 8 lanes per node, one float4 column chunk per lane; U list entries per
-// round are loaded together (entries past the end reload a valid row and are
-// dropped), so each lane keeps U loads in flight.
+// messages of the node step (msg.cuh) from the FP32 edge rows, written to the
+// node's projection row P[v] = [m_out | m_in] (the node step reads it there and
+// then overwrites the row with the new projections)
 // ---------------------------------------------------------------------------
 template <int H>
-__global__ void __launch_bounds__(256) k_msg_f32(Batch b, Ws w, Sel sel) {
-  constexpr int NJ = H / 32, U = 8 / NJ;
+struct MsgF32 {
+  static constexpr int LANES = H / 4;
+  using Chunk = float4;
+  struct Acc {
+    float2 a = make_float2(0.f, 0.f), b = a;
+    __device__ __forceinline__ void add(const float4& v) {
+      a = __fadd2_rn(a, make_float2(v.x, v.y));
+      b = __fadd2_rn(b, make_float2(v.z, v.w));
+    }
+  };
+  static __device__ __forceinline__ float4 load(const Ws& w, int e, int q) {
+    return __ldg(reinterpret_cast<const float4*>(w.estate + size_t(e) * H) + q);
+  }
+  static __device__ __forceinline__ void store(const Ws& w, int row, int side, int q, const Acc& s) {
+    *(reinterpret_cast<float4*>(w.pstate + size_t(row) * 2 * H + side * H) + q) =
+        make_float4(s.a.x, s.a.y, s.b.x, s.b.y);
+  }
+};
+
+// (5 blocks per SM: row lists of the re-score, random in the batch, want warps)
+template <int H>
+__global__ void __launch_bounds__(256, 5) k_msg_f32(Batch b, Ws w, Sel sel) {
   pdl_begin();
   if (input_bad(w)) return;
   int lo, hi;
   if (!sel_rows(b, w, sel, false, lo, hi)) return;
-  const int E = clamp_edges(w.counters, w.e_cap);
-  const int q = threadIdx.x & 7;
-  const int groups = gridDim.x * (blockDim.x >> 3);
-  for (int pos = lo + blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3); pos < hi; pos += groups) {
-    const int row = sel_row(sel, pos);
-    float* out = w.pstate + size_t(row) * 2 * H + 4 * q;
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-      int a, n;
-      if (side == 0) {
-        a = min(w.row_ptr[row], E);
-        n = min(w.row_ptr[row + 1], E) - a;
-      } else {
-        a = w.in_ptr[row];
-        n = w.in_ptr[row + 1] - a;
-      }
-      float4 s[NJ];
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) s[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      for (int t0 = 0; t0 < n; t0 += U) {
-        float4 v[U][NJ];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int at = a + min(t0 + u, n - 1);
-          const int e = side == 0 ? at : __ldg(w.in_edge + at);
-#pragma unroll
-          for (int j = 0; j < NJ; ++j)
-            v[u][j] = __ldg(reinterpret_cast<const float4*>(w.estate + size_t(e) * H + 32 * j + 4 * q));
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (t0 + u < n) {
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-              const float2 lo = __fadd2_rn(make_float2(s[j].x, s[j].y), make_float2(v[u][j].x, v[u][j].y));
-              const float2 hi = __fadd2_rn(make_float2(s[j].z, s[j].w), make_float2(v[u][j].z, v[u][j].w));
-              s[j] = make_float4(lo.x, lo.y, hi.x, hi.y);
-            }
-          }
-      }
-#pragma unroll
-      for (int j = 0; j < NJ; ++j)
-        *reinterpret_cast<float4*>(out + side * H + 32 * j) = s[j];
-    }
-  }
+  message_sums<MsgF32<H>>(w, sel, lo, hi);
 }
 
 // ---- transposed register tiles of the embedding MLP -------------------------
@@ -1378,13 +1351,9 @@ void launch_edge_enc_f32(const Batch& b, const Ws& w, const Mlp2F32& m, int h, S
 void launch_messages_f32(const Batch& b, const Ws& w, int h, Sel sel, cudaStream_t s) {
   if (b.n_hits <= 0) return;
   const int full = device_sms() * 8;
-  const int grid = sel.rows ? full : std::max(1, std::min(full, div_up(b.n_hits, 32)));
-  if (h == 32)
-    launch_pdl(false, k_msg_f32<32>, grid, 256, 0, s, 1, b, w, sel);
-  else if (h == 64)
-    launch_pdl(false, k_msg_f32<64>, grid, 256, 0, s, 1, b, w, sel);
-  else
-    launch_pdl(false, k_msg_f32<128>, grid, 256, 0, s, 1, b, w, sel);
+  const int grid = sel.rows ? full : std::max(1, std::min(full, div_up(b.n_hits, 256 / (h / 4))));
+  launch_pdl(false, h == 32 ? k_msg_f32<32> : h == 64 ? k_msg_f32<64> : k_msg_f32<128>, grid, 256, 0,
+             s, 1, b, w, sel);
 }
 
 void launch_node_update_f32(const Batch& b, const Ws& w, const Mlp2F32& m, const EdgeProj& proj,

@@ -34,6 +34,7 @@
 #include <cstring>
 
 #include "../../include/gnntrk.h"
+#include "msg.cuh"
 #include "tc.cuh"
 #include "tc_ptx.cuh"
 
@@ -1686,68 +1687,47 @@ __global__ void __launch_bounds__(kWsThreads, 2)
 }
 
 // ---------------------------------------------------------------------------
-// messages of the node step from the BF16 edge states: P[v] = [sum of e over
-// v's out edges | sum over its in edges], FP32 sums in increasing list order
-// starting from zero, stored as FP32 (FP8 path: the node step quantises them
-// with a per-row scale) or rounded to BF16 (BF16 path: the layer-1 operand
-// as the node step would round it). One group of 8 lanes per node, H/8
-// columns per lane; U list entries per round are loaded together (entries
-// past the end reload a valid row and are dropped).
+// messages of the node step (msg.cuh) from the BF16 edge states, P[v] = [m_out |
+// m_in], stored as FP32 (FP8 path: the node step quantises them with a per-row
+// scale) or rounded to BF16 (BF16 path: the layer-1 operand as the node step
+// would round it)
 // ---------------------------------------------------------------------------
 template <int H, bool OUT16>
-__global__ void __launch_bounds__(256) k_msg_bf16(Batch b, Ws w) {
-  constexpr int LPN = H / 8;    // lanes per hit: 8 columns (16 bytes) each
-  constexpr int NPW = 32 / LPN; // hits per warp
-  constexpr int U = 8;
-  pdl_begin();
-  if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
-  const int E = clamp_edges(w.counters, w.e_cap);
-  const int q = threadIdx.x % LPN;
-  const int groups = gridDim.x * (blockDim.x / LPN);
-  (void)NPW;
-  for (int row = blockIdx.x * (blockDim.x / LPN) + threadIdx.x / LPN; row < b.n_hits; row += groups) {
-#pragma unroll 1
-    for (int side = 0; side < 2; ++side) {
-      int a, n;
-      if (side == 0) {
-        a = min(w.row_ptr[row], E);
-        n = min(w.row_ptr[row + 1], E) - a;
-      } else {
-        a = w.in_ptr[row];
-        n = w.in_ptr[row + 1] - a;
-      }
-      float2 s[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) s[c] = make_float2(0.f, 0.f);
-      for (int t0 = 0; t0 < n; t0 += U) {
-        uint4 v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int at = a + min(t0 + u, n - 1);
-          const int e = side == 0 ? at : __ldg(w.in_edge + at);
-          v[u] = __ldg(reinterpret_cast<const uint4*>(w.estate16 + size_t(e) * H) + q);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (t0 + u < n) {
-            s[0] = __fadd2_rn(s[0], make_float2(bf16_lo(v[u].x), bf16_hi(v[u].x)));
-            s[1] = __fadd2_rn(s[1], make_float2(bf16_lo(v[u].y), bf16_hi(v[u].y)));
-            s[2] = __fadd2_rn(s[2], make_float2(bf16_lo(v[u].z), bf16_hi(v[u].z)));
-            s[3] = __fadd2_rn(s[3], make_float2(bf16_lo(v[u].w), bf16_hi(v[u].w)));
-          }
-      }
-      if constexpr (OUT16) {
-        uint4* o16 = reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(w.pstate) +
-                                              size_t(row) * 2 * H + side * H) + q;
-        *o16 = make_uint4(pack_bf16(s[0].x, s[0].y), pack_bf16(s[1].x, s[1].y),
-                          pack_bf16(s[2].x, s[2].y), pack_bf16(s[3].x, s[3].y));
-      } else {
-        float4* o = reinterpret_cast<float4*>(w.pstate + size_t(row) * 2 * H + side * H + 8 * q);
-        o[0] = make_float4(s[0].x, s[0].y, s[1].x, s[1].y);
-        o[1] = make_float4(s[2].x, s[2].y, s[3].x, s[3].y);
-      }
+struct MsgBf16 {
+  static constexpr int LANES = H / 8;
+  using Chunk = uint4;
+  struct Acc {
+    float2 s[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
+                   make_float2(0.f, 0.f)};
+    __device__ __forceinline__ void add(const uint4& v) {
+      s[0] = __fadd2_rn(s[0], make_float2(bf16_lo(v.x), bf16_hi(v.x)));
+      s[1] = __fadd2_rn(s[1], make_float2(bf16_lo(v.y), bf16_hi(v.y)));
+      s[2] = __fadd2_rn(s[2], make_float2(bf16_lo(v.z), bf16_hi(v.z)));
+      s[3] = __fadd2_rn(s[3], make_float2(bf16_lo(v.w), bf16_hi(v.w)));
+    }
+  };
+  static __device__ __forceinline__ uint4 load(const Ws& w, int e, int q) {
+    return __ldg(reinterpret_cast<const uint4*>(w.estate16 + size_t(e) * H) + q);
+  }
+  static __device__ __forceinline__ void store(const Ws& w, int row, int side, int q, const Acc& a) {
+    if constexpr (OUT16) {
+      *(reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(w.pstate) + size_t(row) * 2 * H +
+                                 side * H) + q) =
+          make_uint4(pack_bf16(a.s[0].x, a.s[0].y), pack_bf16(a.s[1].x, a.s[1].y),
+                     pack_bf16(a.s[2].x, a.s[2].y), pack_bf16(a.s[3].x, a.s[3].y));
+    } else {
+      float4* o = reinterpret_cast<float4*>(w.pstate + size_t(row) * 2 * H + side * H + 8 * q);
+      o[0] = make_float4(a.s[0].x, a.s[0].y, a.s[1].x, a.s[1].y);
+      o[1] = make_float4(a.s[2].x, a.s[2].y, a.s[3].x, a.s[3].y);
     }
   }
+};
+
+template <int H, bool OUT16>
+__global__ void __launch_bounds__(256, 4) k_msg_bf16(Batch b, Ws w) {
+  pdl_begin();
+  if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
+  message_sums<MsgBf16<H, OUT16>>(w, Sel{nullptr, nullptr}, 0, b.n_hits);
 }
 
 // ---------------------------------------------------------------------------
