@@ -1209,7 +1209,9 @@ void launch_shape(GnnArgs a, int64_t rows_hint, cudaStream_t s) {
   a.short_rounds = v == 0 ? 1 : v == 1 ? 0 : 1 << 20;
   const void* fn = (const void*)k_gnn_f32<X>;
   int grid = device_sms() * blocks_per_sm(fn, X::NW * 32, X::SMEM);
-  if (rows_hint >= 0) grid = std::max(1, std::min(grid, div_up(rows_hint, X::Short::WR)));
+  // four short tiles per block before another block is used
+  constexpr int kRowsPerBlock = 4 * X::Short::WR;
+  grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRowsPerBlock - 1) / kRowsPerBlock)));
   launch_pdl(true, k_gnn_f32<X>, grid, X::NW * 32, X::SMEM, s, 1, a);
 }
 
@@ -1267,14 +1269,14 @@ void launch_triplet_scores_f32(const Batch& b, const Ws& w, const TripletHeads& 
   a.tn = w.counters + C_TRIP_A;
   a.tlogit = w.trip_alogit;
   a.tkeep = w.trip_akeep;
-  launch_gnn_any(h, G_TRIP, a, -1, s);
+  launch_gnn_any(h, G_TRIP, a, triplet_rows_hint(b.n_hits), s);
   a.m = t.elb;
   a.t1 = w.trip_e1;
   a.t2 = w.trip_e2;
   a.tn = w.counters + C_TRIP_E;
   a.tlogit = w.trip_elogit;
   a.tkeep = w.trip_ekeep;
-  launch_gnn_any(h, G_TRIP, a, -1, s);
+  launch_gnn_any(h, G_TRIP, a, triplet_rows_hint(b.n_hits), s);
 }
 
 void f32_set_variant(int h, int family, int v) {
@@ -1287,7 +1289,7 @@ namespace {
 template <class X>
 void launch_embed_tiles(const EmbedArgs& a, cudaStream_t s) {
   const int full = device_sms() * blocks_per_sm((const void*)k_embed_tiles<X>, X::NW * 32, X::SMEM);
-  const int grid = std::max(1, std::min(full, div_up(a.b.n_hits, X::Short::WR)));
+  const int grid = std::max(1, std::min(full, div_up(a.b.n_hits, 4 * X::Short::WR)));
   launch_pdl(true, k_embed_tiles<X>, grid, X::NW * 32, X::SMEM, s, 1, a);
 }
 
@@ -1345,7 +1347,7 @@ void launch_edge_enc_f32(const Batch& b, const Ws& w, const Mlp2F32& m, int h, S
                          cudaStream_t s) {
   GnnArgs a = gnn_args(b, w, sel);
   a.m = m;
-  launch_gnn_any(h, G_EDGE_ENC, a, -1, s);
+  launch_gnn_any(h, G_EDGE_ENC, a, edge_rows_hint(b.n_hits), s);
 }
 
 void launch_messages_f32(const Batch& b, const Ws& w, int h, Sel sel, cudaStream_t s) {
@@ -1376,7 +1378,7 @@ void launch_edge_update_f32(const Batch& b, const Ws& w, const Mlp2F32& m, const
   a.band_lo = band_lo;
   a.band_hi = band_hi;
   const int mode = cls == nullptr ? G_EDGE_UPD : (m.l1.WT == nullptr ? G_CLS : G_EDGE_UPD_CLS);
-  launch_gnn_any(h, mode, a, -1, s);
+  launch_gnn_any(h, mode, a, edge_rows_hint(b.n_hits), s);
 }
 
 }  // namespace gnntrk

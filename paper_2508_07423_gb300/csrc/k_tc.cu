@@ -1848,18 +1848,18 @@ void launch_edge_ws(const TcArgs& a, const TcModel& m, cudaStream_t s) {
 }
 
 template <int H, bool FP8, int MODE>
-void launch_mode(const TcArgs& a, cudaStream_t s, int rows_hint) {
+void launch_mode(const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   using L = Layout<H, FP8, MODE>;
   int per_sm = tc_blocks_per_sm<H, FP8, MODE>();
   const int tuned = g_tuned[FP8 ? 1 : 0][hidx(H)][family_of(MODE)].load(std::memory_order_relaxed);
   if (tuned > 0 && tuned < per_sm) per_sm = tuned;
   int grid = device_sms() * per_sm;
-  if (rows_hint >= 0) grid = rows_hint == 0 ? 1 : min(grid, div_up(rows_hint, kRows));
-  launch_pdl(a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows, L::TOTAL, s, 1, a);
+  grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRows - 1) / kRows)));
+  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows, L::TOTAL, s, 1, a);
 }
 
 template <int H, bool FP8>
-void launch_h(int mode, const TcArgs& a, cudaStream_t s, int rows_hint) {
+void launch_h(int mode, const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   switch (mode) {
     case M_NODE_ENC: launch_mode<H, FP8, M_NODE_ENC>(a, s, rows_hint); break;
     case M_EDGE_ENC: launch_mode<H, FP8, M_EDGE_ENC>(a, s, rows_hint); break;
@@ -1887,7 +1887,7 @@ constexpr int smem_total(int H, int mode) {
 #undef GNNTRK_LT
 }
 
-void launch_any(int H, bool fp8, int mode, const TcArgs& a, cudaStream_t s, int rows_hint) {
+void launch_any(int H, bool fp8, int mode, const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   if (fp8) {
     if (H == 32) launch_h<32, true>(mode, a, s, rows_hint);
     else if (H == 64) launch_h<64, true>(mode, a, s, rows_hint);
@@ -2183,10 +2183,10 @@ void tc_gnn(const Batch& b, const Ws& w, const TcModel& m, int h, int K, const G
   if (stage < 0 || stage == 0) {
     if (m.enc16) {
       set(m.edge_enc16);
-      launch_any(h, false, M_EDGE_ENC, a, s, -1);
+      launch_any(h, false, M_EDGE_ENC, a, s, edge_rows_hint(b.n_hits));
     } else {
       set(m.edge_enc);
-      launch_any(h, fp8, M_EDGE_ENC, a, s, -1);
+      launch_any(h, fp8, M_EDGE_ENC, a, s, edge_rows_hint(b.n_hits));
     }
   }
   for (int k = 0; k < K; ++k) {
@@ -2208,11 +2208,11 @@ void tc_gnn(const Batch& b, const Ws& w, const TcModel& m, int h, int K, const G
       else if (form == 2)
         launch_edge_ws<false>(a, m, s);
       else
-        launch_any(h, fp8, last && fuse ? M_EDGE_UPD_CLS : M_EDGE_UPD, a, s, -1);
-      if (last && !fuse) launch_any(h, fp8, M_CLS, a, s, -1);
+        launch_any(h, fp8, last && fuse ? M_EDGE_UPD_CLS : M_EDGE_UPD, a, s, edge_rows_hint(b.n_hits));
+      if (last && !fuse) launch_any(h, fp8, M_CLS, a, s, edge_rows_hint(b.n_hits));
     }
   }
-  if (K == 0 && (stage < 0 || stage == 1)) launch_any(h, fp8, M_CLS, a, s, -1);
+  if (K == 0 && (stage < 0 || stage == 1)) launch_any(h, fp8, M_CLS, a, s, edge_rows_hint(b.n_hits));
 }
 
 void tc_set_edge_form(int form) {
@@ -2283,7 +2283,7 @@ void tc_triplet_scores(const Batch& b, const Ws& w, const TcModel& m, int h, con
   a.tn = w.counters + C_TRIP_A;
   a.tlogit = w.trip_alogit;
   a.tkeep = w.trip_akeep;
-  launch_any(h, false, M_TRIP, a, s, -1);
+  launch_any(h, false, M_TRIP, a, s, triplet_rows_hint(b.n_hits));
   // elbows
   a.W1 = static_cast<const uint8_t*>(m.elb1.B);
   a.b1 = elb_b1;
@@ -2293,7 +2293,7 @@ void tc_triplet_scores(const Batch& b, const Ws& w, const TcModel& m, int h, con
   a.tn = w.counters + C_TRIP_E;
   a.tlogit = w.trip_elogit;
   a.tkeep = w.trip_ekeep;
-  launch_any(h, false, M_TRIP, a, s, -1);
+  launch_any(h, false, M_TRIP, a, s, triplet_rows_hint(b.n_hits));
 }
 
 bool tc_cls_fused(int h, int precision) {
