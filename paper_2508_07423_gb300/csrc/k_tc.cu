@@ -98,9 +98,10 @@ struct Layout {
   // The encoders see hit coordinates, whose useful precision (a 12 um
   // resolution over a 45 mm radius) is finer than BF16's 8-bit mantissa.
   static constexpr bool SPLIT = !FP8 && (MODE == M_NODE_ENC || MODE == M_EDGE_ENC);
-  // at hidden 128 the split edge encoder runs layer 1 in two passes over one
-  // [h_src, h_dst] tile (hi parts, then lo parts accumulated into the same
-  // tensor memory) against the plain weight image, so it fits shared memory
+  // at hidden 128 the split edge encoder runs layer 1 in four passes of K = H
+  // over a one-segment tile (hi h_src, hi h_dst, lo h_src, lo h_dst, accumulated
+  // into the same tensor memory) against the K halves of the plain weight image,
+  // so that two tiles fit beside the weights
   static constexpr bool SPLIT2 = SPLIT && MODE == M_EDGE_ENC && H > 64;
   // FP8 edge steps at hidden 128 run layer 1 in three passes of K = H over a
   // one-segment tile (e, then h_src, then h_dst) against the K chunks of the
@@ -127,21 +128,34 @@ struct Layout {
   // copies through registers (2.27 ms against 2.59-3.12 ms per 4 launches).
   static constexpr bool PIPE = !FP8 && MODE == M_NODE_UPD;
   static constexpr bool PREFETCH = false;
+  // tiles in flight per CTA, each worked on by a warpgroup of its own with its
+  // own buffers and accumulators; they share the weights. Two in the edge encoder
+  // at hidden 128, whose weights leave room for one CTA per SM (the node step's
+  // three accumulators of 128 columns fill the tensor memory with one tile, the
+  // edge steps' two CTAs with two).
+  static constexpr int G = SPLIT2 ? 2 : 1;
   static constexpr int A = align1k(WC + WC_BYTES);
-  static constexpr int A_BYTES = MODE == M_NODE_ENC ? 0 : kRows * (P3 ? H : K1) * ESZ;
+  static constexpr int A_BYTES = MODE == M_NODE_ENC ? 0 : kRows * (P3 || SPLIT2 ? H : K1) * ESZ;
   static constexpr int NBUF = PIPE && PREFETCH ? 2 : 1;
   // hidden / classifier input: its own tile with two input buffers, else it
   // overwrites the layer-1 input once the layer-1 MMAs are done
   static constexpr int HA = NBUF == 2 || MODE == M_NODE_ENC ? align1k(A + NBUF * A_BYTES) : A;
   static constexpr int HA_BYTES = NBUF == 2 || MODE == M_NODE_ENC ? kRows * K2 * ESZ : 0;
-  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + HA_BYTES : A + NBUF * A_BYTES);
+  static_assert(G == 1 || (NBUF == 1 && HA_BYTES == 0 && A_BYTES % 1024 == 0), "one buffer per warpgroup");
+  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + HA_BYTES : A + G * NBUF * A_BYTES);
   // fp32 parameters: b1, b2, bc1, s1, s2, sc, c2 weights, ne1 (3 x H + H)
   static constexpr int PAR_FLOATS = 7 * H + 4 * H + 8;
   static constexpr int BAR = PAR + PAR_FLOATS * 4;
-  static constexpr int TOTAL = BAR + 64;
+  // hidden 128: each warp's state rows pass through a staging block of 32 rows x
+  // 64 bytes (80-byte stride) on their way in (residual) and out
+  static constexpr bool COOP = H == 128 && MODE != M_CLS && MODE != M_TRIP;
+  static constexpr int STAGE = BAR + 64;
+  static constexpr int STAGE_ROW = 80;
+  static constexpr int TOTAL = STAGE + (COOP ? G * kRows * STAGE_ROW : 0);
   // FP8: one accumulator block per layer-1 segment scale
   static constexpr int TSEG = P3 ? 2 : (FP8 ? NSEG : 1);
   static constexpr int TMEM_COLS = pow2_cols(TSEG * H);
+  static_assert(G * TMEM_COLS <= 512, "tensor memory of one SM");
 };
 
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
@@ -233,24 +247,6 @@ __device__ __forceinline__ float put_row_bf16(uint8_t* tile, int row, int kchunk
   }
 }
 
-// One BF16 row of H values from global memory into an E4M3 tile at element
-// k0, each value multiplied by `inv` (the caller's per-row scale).
-template <int H>
-__device__ __forceinline__ void put_row_bf16_e4m3(uint8_t* tile, int row, int kchunks, int k0,
-                                                  const __nv_bfloat16* src, float inv) {
-  const uint4* s4 = reinterpret_cast<const uint4*>(src);
-#pragma unroll
-  for (int c = 0; c < H / 16; ++c) {
-    const uint4 a = s4[2 * c], b = s4[2 * c + 1];
-    uint4 u;
-    u.x = pack_e4m3x4(bf16_lo(a.x) * inv, bf16_hi(a.x) * inv, bf16_lo(a.y) * inv, bf16_hi(a.y) * inv);
-    u.y = pack_e4m3x4(bf16_lo(a.z) * inv, bf16_hi(a.z) * inv, bf16_lo(a.w) * inv, bf16_hi(a.w) * inv);
-    u.z = pack_e4m3x4(bf16_lo(b.x) * inv, bf16_hi(b.x) * inv, bf16_lo(b.y) * inv, bf16_hi(b.y) * inv);
-    u.w = pack_e4m3x4(bf16_lo(b.z) * inv, bf16_hi(b.z) * inv, bf16_lo(b.w) * inv, bf16_hi(b.w) * inv);
-    *reinterpret_cast<uint4*>(tile + tile_off(row, (k0 >> 4) + c, kchunks)) = u;
-  }
-}
-
 // Write n FP32 values (a multiple of 8) into a BF16 tile as two parts, hi =
 // bf16(v) at element k_hi and lo = bf16(v - hi) at element k_lo.
 __device__ __forceinline__ void put_row_split(uint8_t* tile, int row, int kchunks, int k_hi,
@@ -269,54 +265,174 @@ __device__ __forceinline__ void put_row_split(uint8_t* tile, int row, int kchunk
   }
 }
 
-// One FP32 row of H values from global memory into a BF16 tile, split as above.
-template <int H>
-__device__ __forceinline__ void put_row_f32_split(uint8_t* tile, int row, int kchunks, int k_hi,
-                                                  int k_lo, const float* src) {
-  const float4* s4 = reinterpret_cast<const float4*>(src);
+// ---- cooperative row copies (hidden 128) -----------------------------------
+// A warp copies its 32 rows of a tile eight at a time: lane (r = lane & 7,
+// q = lane >> 3) takes chunk q, q + 4, ... of row r, so that the four lanes of a row
+// read 128 consecutive bytes (a thread copying a row of its own makes every
+// load instruction touch 32 lines, which bound these kernels on the L1 pipe)
+// and the eight lanes of a chunk store 128 consecutive bytes of the tile.
+// `id`: each lane's own row (lane l: row l of the warp), negative: zeros.
+
+// 32 consecutive bytes of global memory
+struct B32 {
+  uint4 a, b;
+};
+__device__ __forceinline__ B32 ld32(const void* p) {
+  const uint4* q = reinterpret_cast<const uint4*>(p);
+  return B32{q[0], q[1]};
+}
+__device__ __forceinline__ uint4 e4m3_of_bf16(const B32& v, float inv) {
+  uint4 u;
+  u.x = pack_e4m3x4(bf16_lo(v.a.x) * inv, bf16_hi(v.a.x) * inv, bf16_lo(v.a.y) * inv, bf16_hi(v.a.y) * inv);
+  u.y = pack_e4m3x4(bf16_lo(v.a.z) * inv, bf16_hi(v.a.z) * inv, bf16_lo(v.a.w) * inv, bf16_hi(v.a.w) * inv);
+  u.z = pack_e4m3x4(bf16_lo(v.b.x) * inv, bf16_hi(v.b.x) * inv, bf16_lo(v.b.y) * inv, bf16_hi(v.b.y) * inv);
+  u.w = pack_e4m3x4(bf16_lo(v.b.z) * inv, bf16_hi(v.b.z) * inv, bf16_lo(v.b.w) * inv, bf16_hi(v.b.w) * inv);
+  return u;
+}
+__device__ __forceinline__ float amax_bf16(const uint4& v) {
+  float m = 0.f;
+  const uint32_t q[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-  for (int c = 0; c < H / 8; ++c) {
-    const float4 a = s4[2 * c], b = s4[2 * c + 1];
-    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    put_row_split(tile, row, kchunks, k_hi + 8 * c, k_lo + 8 * c, v, 8);
-  }
+  for (int j = 0; j < 4; ++j) m = fmaxf(m, fmaxf(fabsf(bf16_lo(q[j])), fabsf(bf16_hi(q[j]))));
+  return m;
 }
 
-// One FP32 row of H values into a BF16 tile at element k0: its hi parts
-// bf16(v) (lo = false) or its lo parts bf16(v - bf16(v)) (lo = true).
+// The chunks of a warp's 32 BF16 rows, in registers between their load and
+// their way into the tile (so that a load can be in flight during an MMA or
+// the epilogue).
 template <int H>
-__device__ __forceinline__ void put_row_f32_part(uint8_t* tile, int row, int kchunks, int k0,
-                                                 const float* src, bool lo) {
-  const float4* s4 = reinterpret_cast<const float4*>(src);
+struct CoopRows {
+  static constexpr int PER = H / 64;
+  B32 v[4][PER];
+  // (missing rows read row 0)
+  __device__ __forceinline__ void load(const __nv_bfloat16* src, int id) {
+    const int lane = threadIdx.x & 31, r = lane & 7, q = lane >> 3;
 #pragma unroll
-  for (int c = 0; c < H / 8; ++c) {
-    const float4 a = s4[2 * c], b = s4[2 * c + 1];
-    float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    if (lo) {
+    for (int g = 0; g < 4; ++g) {
+      const int row = __shfl_sync(0xffffffffu, id, 8 * g + r);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] -= __bfloat162float(__float2bfloat16_rn(v[j]));
+      for (int j = 0; j < PER; ++j)
+        v[g][j] = ld32(src + size_t(max(row, 0)) * H + 16 * (q + 4 * j));
     }
-    *reinterpret_cast<uint4*>(tile + tile_off(row, (k0 >> 3) + c, kchunks)) =
-        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]),
-                   pack_bf16(v[6], v[7]));
   }
-}
-
-template <int H>
-__device__ __forceinline__ void add_bf16_row(float* acc, const __nv_bfloat16* src) {
-  const uint4* s4 = reinterpret_cast<const uint4*>(src);
+  // into a BF16 tile as they are
+  __device__ __forceinline__ void put(uint8_t* tile, int kchunks, int id) {
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (kRows - 1)) >> 5;
+    const int r = lane & 7, q = lane >> 3;
 #pragma unroll
-  for (int c = 0; c < H / 8; ++c) {
-    const uint4 u = s4[c];
-    acc[8 * c + 0] += bf16_lo(u.x);
-    acc[8 * c + 1] += bf16_hi(u.x);
-    acc[8 * c + 2] += bf16_lo(u.y);
-    acc[8 * c + 3] += bf16_hi(u.y);
-    acc[8 * c + 4] += bf16_lo(u.z);
-    acc[8 * c + 5] += bf16_hi(u.z);
-    acc[8 * c + 6] += bf16_lo(u.w);
-    acc[8 * c + 7] += bf16_hi(u.w);
+    for (int g = 0; g < 4; ++g) {
+      const bool in = __shfl_sync(0xffffffffu, id, 8 * g + r) >= 0;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const uint32_t at = tile_off(32 * warp + 8 * g + r, 2 * (q + 4 * j), kchunks);
+        *reinterpret_cast<uint4*>(tile + at) = in ? v[g][j].a : make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(tile + at + 128) = in ? v[g][j].b : make_uint4(0, 0, 0, 0);
+      }
+    }
   }
+  // into an E4M3 tile at element k0 under one scale per row: the row's own
+  // maximum (OWN; the owner lane gets the scale) or each lane's `inv`
+  template <bool OWN>
+  __device__ __forceinline__ float put_e4m3(uint8_t* tile, int kchunks, int k0, int id, float inv) {
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (kRows - 1)) >> 5;
+    const int r = lane & 7, q = lane >> 3;
+    float own = 1.f;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int row = __shfl_sync(0xffffffffu, id, 8 * g + r);
+      float iv;
+      if constexpr (OWN) {
+        float m = 0.f;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) m = fmaxf(m, fmaxf(amax_bf16(v[g][j].a), amax_bf16(v[g][j].b)));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        iv = m > 0.f ? 448.f / m : 1.f;
+        const float mine = __shfl_sync(0xffffffffu, m, lane & 7);
+        if (q == g) own = mine > 0.f ? mine / 448.f : 1.f;
+      } else {
+        iv = __shfl_sync(0xffffffffu, inv, 8 * g + r);
+      }
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        *reinterpret_cast<uint4*>(tile + tile_off(32 * warp + 8 * g + r, (k0 >> 4) + q + 4 * j, kchunks)) =
+            row >= 0 ? e4m3_of_bf16(v[g][j], iv) : make_uint4(0, 0, 0, 0);
+    }
+    return own;
+  }
+};
+
+// A warp's 32 state rows of H BF16 values, 32 columns (64 bytes) at a time,
+// through its staging block: lane (row lane / 4 + 8 i, part lane % 4) moves 16
+// bytes between global memory and the block, lane l reads and writes row l.
+template <int H, int STRIDE>
+struct RowStage {
+  uint8_t* blk;                // the warp's block
+  const __nv_bfloat16* first;  // the warp's first row
+  int n;                       // rows of the warp that exist
+  uint4 v[4];
+
+  __device__ __forceinline__ uint4* slot(int row, int part) const {
+    return reinterpret_cast<uint4*>(blk + row * STRIDE + 16 * part);
+  }
+  // columns 32 c .. 32 c + 31 of every row into registers (missing rows: row 0)
+  __device__ __forceinline__ void fetch(int c) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int row = (lane >> 2) + 8 * i;
+      v[i] = n > 0 ? *(reinterpret_cast<const uint4*>(first + size_t(row < n ? row : 0) * H + 32 * c) + (lane & 3))
+                   : make_uint4(0, 0, 0, 0);
+    }
+  }
+  // the fetched columns of this lane's row
+  __device__ __forceinline__ void rows(uint4 (&out)[4]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *slot((lane >> 2) + 8 * i, lane & 3) = v[i];
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) out[j] = *slot(lane, j);
+    __syncwarp();
+  }
+  // columns 32 c .. of this lane's row to global memory
+  __device__ __forceinline__ void put(int c, const uint4 (&in)[4]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *slot(lane, j) = in[j];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int row = (lane >> 2) + 8 * i;
+      if (row < n)
+        *(reinterpret_cast<uint4*>(const_cast<__nv_bfloat16*>(first) + size_t(row) * H + 32 * c) + (lane & 3)) =
+            *slot(row, lane & 3);
+    }
+    __syncwarp();
+  }
+};
+
+// the lo parts of 32 columns, bf16(z - bf16(z))
+__device__ __forceinline__ void store_lo(__nv_bfloat16* dst, const float (&z)[32]) {
+  float l[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j) l[j] = z[j] - __bfloat162float(__float2bfloat16_rn(z[j]));
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    reinterpret_cast<uint4*>(dst)[q] =
+        make_uint4(pack_bf16(l[8 * q], l[8 * q + 1]), pack_bf16(l[8 * q + 2], l[8 * q + 3]),
+                   pack_bf16(l[8 * q + 4], l[8 * q + 5]), pack_bf16(l[8 * q + 6], l[8 * q + 7]));
+}
+// acc[0..7] += the 8 BF16 values of u
+__device__ __forceinline__ void add_bf16x8(float* acc, const uint4& u) {
+  acc[0] += bf16_lo(u.x);
+  acc[1] += bf16_hi(u.x);
+  acc[2] += bf16_lo(u.y);
+  acc[3] += bf16_hi(u.y);
+  acc[4] += bf16_lo(u.z);
+  acc[5] += bf16_hi(u.z);
+  acc[6] += bf16_lo(u.w);
+  acc[7] += bf16_hi(u.w);
 }
 
 // x[j] = v[j] + b[j] (BF16) or fma(v[j], sc[j], b[j]) (FP8) for 32 columns,
@@ -390,6 +506,24 @@ __device__ __forceinline__ void issue_pass_e4m3(uint32_t tmem, const uint8_t* A,
   }
 }
 
+// One pass of the split edge encoder's layer 1 at hidden 128 (K = 2H): the
+// one-segment BF16 A tile times K half pass % 2 of the weight image; pass 0
+// starts the accumulator, the others add to it.
+template <int H>
+__device__ __forceinline__ void issue_pass_bf16(uint32_t tmem, const uint8_t* A, const uint8_t* W,
+                                                int pass) {
+  constexpr uint32_t IDESC = idesc_bf16(kRows, H);
+  constexpr uint32_t SBO_A = uint32_t(H * 2 / 16) * 128;
+  constexpr uint32_t SBO_W = uint32_t(2 * H * 2 / 16) * 128;
+  const uint32_t a0 = smem_u32(A), w0 = smem_u32(W) + uint32_t((pass & 1) * (H * 2 / 16)) * 128;
+#pragma unroll
+  for (int k = 0; k < H; k += 16) {
+    const uint32_t byte_k = uint32_t(k * 2 / 16) * 128;
+    mma_bf16(tmem, smem_desc(a0 + byte_k, 128, SBO_A), smem_desc(w0 + byte_k, 128, SBO_W), IDESC,
+             (pass > 0 || k > 0) ? 1u : 0u);
+  }
+}
+
 // Copy slot l (0 .. H/8 - 1) of thread tid in a tile copy: warp w covers rows
 // 32w .. 32w+31; a quarter-warp (8 lanes) takes one 16-byte chunk of 8
 // consecutive rows, a contiguous 128-byte run of the canonical tile, so the
@@ -442,8 +576,32 @@ __device__ __forceinline__ void gather_async(uint8_t* dst, const TcArgs& p, int 
   }
 }
 
+// barrier of a tile's 128 threads: the CTA's, or with two warpgroups their own
+template <int G>
+__device__ __forceinline__ void group_sync(int wg) {
+  if constexpr (G == 1)
+    __syncthreads();
+  else
+    asm volatile("barrier.cta.sync.aligned %0, %1;" ::"r"(1 + wg), "n"(kRows) : "memory");
+}
+template <int G>
+__device__ __forceinline__ bool group_sync_or(int wg, bool v) {
+  if constexpr (G == 1) {
+    return __syncthreads_or(v);
+  } else {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred.aligned q, %2, %3, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
+        : "=r"(r)
+        : "r"(uint32_t(v)), "r"(1 + wg), "n"(kRows)
+        : "memory");
+    return r != 0;
+  }
+}
+
 template <int H, bool FP8, int MODE>
-__global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
+__global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(const TcArgs p) {
   using L = Layout<H, FP8, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sW1 = smem + L::W1;
@@ -458,19 +616,22 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
   float* psc = par + 5 * H;
   float* pc2 = par + 6 * H;      // classifier layer 2 weights [H] + bias
   float* pne = par + 7 * H + 4;  // node encoder layer 1: W[3][H], b[H]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::BAR);  // [0] weights, [1] mma
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + L::BAR + 16);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::BAR);  // [0] weights, [1 + wg] mma
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + L::BAR + 48);
 
-  const int tid = threadIdx.x, warp = tid >> 5;
+  constexpr int G = L::G;
+  // warpgroup, row of its tile, warp of the warpgroup
+  const int wg = G == 1 ? 0 : int(threadIdx.x) / kRows;
+  const int tid = G == 1 ? int(threadIdx.x) : int(threadIdx.x) % kRows, warp = tid >> 5;
+  uint64_t* mma_bar = bar + 1 + wg;
   const Ws& w = p.w;
   // ---- set-up: barriers, TMEM, weights --------------------------------------
-  if (tid == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 1 + G; ++i) mbar_init(&bar[i], 1);
     fence_mbar_init();
   }
-  if (warp == 0) {
-    tmem_alloc(tslot, L::TMEM_COLS);
+  if (threadIdx.x < 32) {
+    tmem_alloc(tslot, G * L::TMEM_COLS);
     tmem_relinquish();
   }
   for (int i = tid; i < H; i += kRows) {
@@ -492,10 +653,10 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tslot;
+  const uint32_t tmem_base = *tslot + uint32_t(wg * L::TMEM_COLS);
   const uint32_t tmem_lane = tmem_base + (uint32_t(warp * 32) << 16);
 
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     uint32_t bytes = uint32_t(L::W1_BYTES + L::W2_BYTES + L::WC_BYTES);
     mbar_expect_tx(&bar[0], bytes);
     if (L::HAS_W1) bulk_g2s(sW1, MODE == M_CLS ? p.Wc : p.W1, L::W1_BYTES, &bar[0]);
@@ -522,16 +683,21 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
   const int n_tiles = (hi - lo + kRows - 1) / kRows;
   constexpr int K1 = L::K1;
   constexpr int KCH1 = K1 * L::ESZ / 16;  // 16-byte chunks per A row, layer 1
-  constexpr int KCHA = L::P3 ? H * L::ESZ / 16 : KCH1;  // per row of the A tile
+  constexpr int KCHA = L::P3 || L::SPLIT2 ? H * L::ESZ / 16 : KCH1;  // per row of the A tile
   constexpr int KCHH = H * L::ESZ / 16;   // 16-byte chunks per A row, K = H
   constexpr int KCH2 = L::K2 * L::ESZ / 16;  // 16-byte chunks per A row, layer 2
 
+  // The node encoder leaves its encoding h in two parts, hi = bf16(h) in hstate16
+  // and lo = bf16(h - hi) in the place of the FP32 states (which the re-score
+  // computes anew); the edge encoder copies both into its tile.
+  __nv_bfloat16* hlo = reinterpret_cast<__nv_bfloat16*>(w.hstate);
+  (void)hlo;
   // wait for the MMAs committed so far; false on timeout (uniform across CTA)
   auto wait_mma = [&]() -> bool {
     mma_pending = true;
-    bool good = mbar_wait_bounded(&bar[1], mma_phase, kWaitCycles);
+    bool good = mbar_wait_bounded(mma_bar, mma_phase, kWaitCycles);
     tc_fence_after();
-    if (__syncthreads_or(!good)) return false;
+    if (group_sync_or<G>(wg, !good)) return false;
     mma_phase ^= 1;
     mma_pending = false;
     return true;
@@ -542,13 +708,44 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
       gather_async<H, MODE>(smem + L::A, p, lo + int(blockIdx.x) * kRows, hi, tid);
     cp_async_commit();
   }
+  // FP8 edge steps at hidden 128: the next tile's e rows, hits and h maxima are
+  // loaded during a tile (its indices when the tile begins, the rows before its
+  // epilogue), and the h rows of a pass during the MMAs of the pass before
+  const int t_first = int(blockIdx.x) * G + wg;
+  CoopRows<L::P3 || L::SPLIT2 ? H : 64> pre;
+  int nid_s = -1, nid_d = -1;
+  float n_amax = 0.f;
+  auto p3_ids = [&](int t) {
+    const int r = lo + t * kRows + tid;
+    const bool in = t < n_tiles && r < hi;
+    nid_s = in ? w.src[r] : -1;
+    nid_d = in ? w.col[r] : -1;
+  };
+  auto p3_amax = [&] { n_amax = nid_s >= 0 ? fmaxf(w.hamax[nid_s], w.hamax[nid_d]) : 0.f; };
+  auto p3_rows = [&](int t) {
+    const int r = lo + t * kRows + tid;
+    pre.load(w.estate16, t < n_tiles && r < hi ? r : -1);
+  };
+  // (the split edge encoder: the rows of a pass during the MMAs of the pass before)
+  if constexpr (L::SPLIT2) {
+    p3_ids(t_first);
+    pre.load(w.hstate16, nid_s);
+  }
+  if constexpr (L::P3) {
+    p3_ids(t_first);
+    p3_rows(t_first);
+    p3_amax();
+  }
   int it = 0;
-  for (int t = blockIdx.x; t < n_tiles && !aborted; t += gridDim.x, ++it) {
+  for (int t = t_first; t < n_tiles && !aborted; t += int(gridDim.x) * G, ++it) {
     const int r = lo + t * kRows + tid;
     const bool valid = r < hi;
-    uint8_t* sA = smem + L::A + (L::NBUF == 2 ? (it & 1) * L::A_BYTES : 0);
+    uint8_t* sA = smem + L::A + wg * L::A_BYTES + (L::NBUF == 2 ? (it & 1) * L::A_BYTES : 0);
     uint8_t* sHA = L::HA == L::A ? sA : smem + L::HA;  // layer-2 input and classifier input
     float sa[3] = {1.f, 1.f, 1.f};  // FP8 per-row scales of the layer-1 segments
+    int id_s = -1, id_d = -1;       // this row's source and target hit (hidden 128)
+    (void)id_s;
+    (void)id_d;
     uint4 keep_row[(H <= 64) ? H / 8 : 1];
     (void)keep_row;
 
@@ -556,14 +753,14 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
     if constexpr (L::PIPE && L::PREFETCH) {
       // every thread is done with the other buffer (tile it - 1): fill it with
       // the next tile, then wait for this tile's copies
-      __syncthreads();
-      const int tn = t + int(gridDim.x);
+      group_sync<G>(wg);
+      const int tn = t + int(gridDim.x) * G;
       if (tn < n_tiles)
         gather_async<H, MODE>(smem + L::A + ((it + 1) & 1) * L::A_BYTES, p, lo + tn * kRows, hi, tid);
       cp_async_commit();
       cp_async_wait<1>();
     } else if constexpr (L::PIPE) {
-      __syncthreads();  // every thread is done with the buffer (tile it - 1)
+      group_sync<G>(wg);  // every thread is done with the buffer (tile it - 1)
       gather_async<H, MODE>(sA, p, lo + t * kRows, hi, tid);
       cp_async_commit();
       cp_async_wait<0>();
@@ -639,6 +836,21 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
         float z[16] = {};
         for (int k = 0; k < K1; k += 16) put_row_f32<FP8>(sA, tid, KCH1, k, z, 16, 1.f);
       }
+    } else if constexpr (L::P3) {
+      // pass 0 holds e alone; h_src and h_dst follow in passes 1 and 2 with one
+      // scale, the larger of their two row maxima (the node kernels store each
+      // row's maximum as they write it)
+      id_s = nid_s;
+      id_d = nid_d;
+      sa[1] = n_amax > 0.f ? n_amax / 448.f : 1.f;
+      p3_ids(t + int(gridDim.x) * G);
+      sa[0] = pre.template put_e4m3<true>(sA, KCHA, 0, valid ? r : -1, 1.f);
+    } else if constexpr (L::SPLIT2) {
+      // pass 0: hi(h_src)
+      id_s = nid_s;
+      id_d = nid_d;
+      p3_ids(t + int(gridDim.x) * G);
+      pre.put(sA, KCHA, id_s);
     } else {
       // edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
       if (valid) {
@@ -649,24 +861,17 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
           sa[1] = put_row_bf16<H, FP8>(sA, tid, KCH1, H, w.estate16 + size_t(p.t2[r]) * H, nullptr);
           seg = 2;
         } else if constexpr (MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS || MODE == M_CLS) {
-          sa[0] = put_row_bf16<H, FP8>(sA, tid, KCHA, 0, w.estate16 + size_t(r) * H,
+          sa[0] = put_row_bf16<H, FP8>(sA, tid, KCH1, 0, w.estate16 + size_t(r) * H,
                                        (H <= 64 && MODE != M_CLS) ? keep_row : nullptr);
           seg = 1;
         }
-        if constexpr (L::P3) {
-          // pass 0 holds e alone; h_src and h_dst follow in passes 1 and 2
-          // with one scale, the larger of their two row maxima
-          // (the node kernels store each row's maximum as they write it)
-          const float amax = fmaxf(w.hamax[w.src[r]], w.hamax[w.col[r]]);
-          sa[1] = amax > 0.f ? amax / 448.f : 1.f;
-        } else if constexpr (L::SPLIT2) {
-          // pass 1: [hi(h_src), hi(h_dst)] (the lo parts follow after the MMA)
-          put_row_f32_part<H>(sA, tid, KCH1, 0, w.hstate + size_t(w.src[r]) * H, false);
-          put_row_f32_part<H>(sA, tid, KCH1, H, w.hstate + size_t(w.col[r]) * H, false);
-        } else if constexpr (L::SPLIT) {
-          // [hi(h_src), hi(h_dst), lo(h_src), lo(h_dst)] from the FP32 encodings
-          put_row_f32_split<H>(sA, tid, KCH1, 0, 2 * H, w.hstate + size_t(w.src[r]) * H);
-          put_row_f32_split<H>(sA, tid, KCH1, H, 3 * H, w.hstate + size_t(w.col[r]) * H);
+        if constexpr (L::SPLIT) {
+          // [hi(h_src), hi(h_dst), lo(h_src), lo(h_dst)]
+          const size_t src = size_t(w.src[r]) * H, dst = size_t(w.col[r]) * H;
+          put_row_bf16<H, false>(sA, tid, KCH1, 0, w.hstate16 + src, nullptr);
+          put_row_bf16<H, false>(sA, tid, KCH1, H, w.hstate16 + dst, nullptr);
+          put_row_bf16<H, false>(sA, tid, KCH1, 2 * H, hlo + src, nullptr);
+          put_row_bf16<H, false>(sA, tid, KCH1, 3 * H, hlo + dst, nullptr);
         } else if constexpr (MODE != M_CLS && MODE != M_TRIP) {
           sa[seg] = put_row_bf16<H, FP8>(sA, tid, KCH1, seg * H, w.hstate16 + size_t(w.src[r]) * H,
                                          nullptr);
@@ -675,12 +880,12 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
         }
       } else {
         float z[16] = {};
-        for (int k = 0; k < (L::P3 ? H : K1); k += 16) put_row_f32<FP8>(sA, tid, KCHA, k, z, 16, 1.f);
+        for (int k = 0; k < K1; k += 16) put_row_f32<FP8>(sA, tid, KCH1, k, z, 16, 1.f);
       }
     }
     fence_proxy_async();
     tc_fence_before();
-    __syncthreads();
+    group_sync<G>(wg);
 
     float hid_scale = 1.f;  // FP8 per-row scale of the layer-2 input
     if constexpr (MODE != M_NODE_ENC) {
@@ -689,10 +894,14 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
         tc_fence_after();
         if constexpr (L::P3)
           issue_pass_e4m3<H>(tmem_base, sA, sW1, 0);
+        else if constexpr (L::SPLIT2)
+          issue_pass_bf16<H>(tmem_base, sA, sW1, 0);
         else
           issue_layer<H, FP8>(tmem_base, sA, sW1, K1, FP8 ? L::NSEG : 1);
-        mma_commit(&bar[1]);
+        mma_commit(mma_bar);
       }
+      if constexpr (L::P3) pre.load(w.hstate16, id_s);
+      if constexpr (L::SPLIT2) pre.load(w.hstate16, id_d);
       if (!wait_mma()) {
         aborted = true;
         break;
@@ -702,39 +911,39 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
         // the pass before have read it); invalid rows keep pass 0's zeros
         const float hinv = 1.f / sa[1];
         for (int pass = 1; pass <= 2 && !aborted; ++pass) {
-          if (valid)
-            put_row_bf16_e4m3<H>(sA, tid, KCHA, 0,
-                                 w.hstate16 + size_t(pass == 1 ? w.src[r] : w.col[r]) * H, hinv);
+          pre.template put_e4m3<false>(sA, KCHA, 0, id_s, hinv);  // (id_s: whether the row exists)
           fence_proxy_async();
           tc_fence_before();
-          __syncthreads();
+          group_sync<G>(wg);
           if (tid == 0) {
             tc_fence_after();
             issue_pass_e4m3<H>(tmem_base + uint32_t(H), sA, sW1, pass);
-            mma_commit(&bar[1]);
+            mma_commit(mma_bar);
           }
+          if (pass == 1)
+            pre.load(w.hstate16, id_d);
+          else
+            p3_amax();
           if (!wait_mma()) aborted = true;
         }
         if (aborted) break;
       }
       if constexpr (L::SPLIT2) {
-        // pass 2: [lo(h_src), lo(h_dst)] into the same tile, accumulated
-        if (valid) {
-          put_row_f32_part<H>(sA, tid, KCH1, 0, w.hstate + size_t(w.src[r]) * H, true);
-          put_row_f32_part<H>(sA, tid, KCH1, H, w.hstate + size_t(w.col[r]) * H, true);
+        // hi(h_dst), lo(h_src), lo(h_dst) into the same tile, accumulated
+        for (int pass = 1; pass <= 3 && !aborted; ++pass) {
+          pre.put(sA, KCHA, id_s);  // (id_s: whether the row exists)
+          fence_proxy_async();
+          tc_fence_before();
+          group_sync<G>(wg);
+          if (tid == 0) {
+            tc_fence_after();
+            issue_pass_bf16<H>(tmem_base, sA, sW1, pass);
+            mma_commit(mma_bar);
+          }
+          if (pass < 3) pre.load(hlo, pass == 1 ? id_s : id_d);
+          if (!wait_mma()) aborted = true;
         }
-        fence_proxy_async();
-        tc_fence_before();
-        __syncthreads();
-        if (tid == 0) {
-          tc_fence_after();
-          issue_layer<H, FP8>(tmem_base, sA, sW1, K1, 1, true);
-          mma_commit(&bar[1]);
-        }
-        if (!wait_mma()) {
-          aborted = true;
-          break;
-        }
+        if (aborted) break;
       }
       if constexpr (L::PIPE && L::HA == L::A) {
         // the hidden tile overwrites the layer-1 input: keep this row's
@@ -744,7 +953,7 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
           for (int c = 0; c < H / 8; ++c)
             keep_row[c] = *reinterpret_cast<const uint4*>(sA + tile_off(tid, c, KCH1));
         }
-        __syncthreads();
+        group_sync<G>(wg);
       }
       // ---- 3. bias + LayerNorm + ReLU (-> A as the next operand, or the
       //         classifier output for M_CLS) -------------------------------
@@ -836,7 +1045,7 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      group_sync<G>(wg);
     } else {
       hid_scale = sa[0];
     }
@@ -845,8 +1054,10 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
     if (tid == 0) {
       tc_fence_after();
       issue_layer<H, FP8>(tmem_base, sHA, sW2, L::K2, 1);
-      mma_commit(&bar[1]);
+      mma_commit(mma_bar);
     }
+    if constexpr (L::P3) p3_rows(t + int(gridDim.x) * G);
+    if constexpr (L::SPLIT2) pre.load(w.hstate16, nid_s);
     if (!wait_mma()) {
       aborted = true;
       break;
@@ -862,9 +1073,22 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
       }
       add_params<FP8>(v, pb2 + c * 32, ps2 + c * 32, z);
     };
+    // hidden 128: the warp's state rows through its staging block
+    constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
+    const int row0 = r - (tid & 31);
+    RowStage<H, L::STAGE_ROW> st{smem + L::STAGE + (wg * kRows + warp * 32) * L::STAGE_ROW,
+                                 (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(row0) * H,
+                                 min(max(hi - row0, 0), 32), {}};
+    (void)st;
     // residual input row (BF16) for the update modes
     auto resid = [&](int c, float (&z)[32]) {
-      if constexpr (MODE == M_NODE_UPD || MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS) {
+      if constexpr (L::COOP && MODE == M_EDGE_UPD_CLS) {
+        uint4 e[4];
+        st.fetch(c);
+        st.rows(e);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) add_bf16x8(z + 8 * q, e[q]);
+      } else if constexpr (MODE == M_NODE_UPD || MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS) {
         const __nv_bfloat16* rowp = (MODE == M_NODE_UPD ? w.hstate16 : w.estate16) + size_t(r) * H;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -872,23 +1096,42 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
                               ? *reinterpret_cast<const uint4*>(sA + tile_off(tid, c * 4 + q, KCH1))
                           : (H <= 64) ? keep_row[c * 4 + q]
                                       : reinterpret_cast<const uint4*>(rowp)[c * 4 + q];
-          z[8 * q + 0] += bf16_lo(u.x);
-          z[8 * q + 1] += bf16_hi(u.x);
-          z[8 * q + 2] += bf16_lo(u.y);
-          z[8 * q + 3] += bf16_hi(u.y);
-          z[8 * q + 4] += bf16_lo(u.z);
-          z[8 * q + 5] += bf16_hi(u.z);
-          z[8 * q + 6] += bf16_lo(u.w);
-          z[8 * q + 7] += bf16_hi(u.w);
+          add_bf16x8(z + 8 * q, u);
         }
       }
     };
 
     if constexpr (MODE != M_EDGE_UPD_CLS) {
       // ---- 5. store the new state (BF16) -----------------------------------
-      constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
       __nv_bfloat16* dst = (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(r) * H;
       float row_max = 0.f;  // largest |stored value| of a node row
+      if constexpr (L::COOP) {
+        constexpr bool RESID = MODE == M_NODE_UPD || MODE == M_EDGE_UPD;
+        if constexpr (RESID) st.fetch(0);
+#pragma unroll
+        for (int c = 0; c < H / 32; ++c) {
+          float z[32];
+          zval(c, z);
+          if constexpr (RESID) {
+            uint4 e[4];
+            st.rows(e);
+            if (c + 1 < H / 32) st.fetch(c + 1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) add_bf16x8(z + 8 * q, e[q]);
+          }
+          if constexpr (L::SPLIT && MODE == M_NODE_ENC) {
+            if (valid) store_lo(hlo + size_t(r) * H + 32 * c, z);
+          }
+          uint4 o[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            o[q] = make_uint4(pack_bf16(z[8 * q], z[8 * q + 1]), pack_bf16(z[8 * q + 2], z[8 * q + 3]),
+                              pack_bf16(z[8 * q + 4], z[8 * q + 5]), pack_bf16(z[8 * q + 6], z[8 * q + 7]));
+            if constexpr (NODE_ROWS) row_max = fmaxf(row_max, amax_bf16(o[q]));
+          }
+          st.put(c, o);
+        }
+      } else {
 #pragma unroll
       for (int c = 0; c < H / 32; ++c) {
         float z[32];
@@ -896,10 +1139,7 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
         if (valid) {
           resid(c, z);
           if constexpr (L::SPLIT && MODE == M_NODE_ENC) {
-            // the FP32 encoding, read by the edge encoder
-            float4* f4 = reinterpret_cast<float4*>(w.hstate + size_t(r) * H) + c * 8;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) f4[q] = make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
+            store_lo(hlo + size_t(r) * H + 32 * c, z);
           }
           uint4* d4 = reinterpret_cast<uint4*>(dst) + c * 4;
 #pragma unroll
@@ -907,14 +1147,9 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
             const uint4 u = make_uint4(pack_bf16(z[8 * q], z[8 * q + 1]), pack_bf16(z[8 * q + 2], z[8 * q + 3]),
                                        pack_bf16(z[8 * q + 4], z[8 * q + 5]), pack_bf16(z[8 * q + 6], z[8 * q + 7]));
             d4[q] = u;
-            if constexpr (NODE_ROWS && H == 128) {
-              const uint32_t pk[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                row_max = fmaxf(row_max, fmaxf(fabsf(bf16_lo(pk[j])), fabsf(bf16_hi(pk[j]))));
-            }
           }
         }
+      }
       }
       // (read by the FP8 edge steps at hidden 128 for their shared h scale)
       if constexpr (NODE_ROWS && H == 128)
@@ -947,11 +1182,11 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      group_sync<G>(wg);
       if (tid == 0) {
         tc_fence_after();
         issue_layer<H, FP8>(tmem_base, sHA, sWC, H, 1);
-        mma_commit(&bar[1]);
+        mma_commit(mma_bar);
       }
       if (!wait_mma()) {
         aborted = true;
@@ -1020,13 +1255,13 @@ __global__ void __launch_bounds__(kRows, 1) k_tc(const TcArgs p) {
   if (aborted) {
     if (tid == 0) set_status(w.counters, ST_TIMEOUT);
     if (weights_late) mbar_wait_bounded(&bar[0], 0, kWaitCycles);
-    if (mma_pending) mbar_wait_bounded(&bar[1], mma_phase, kWaitCycles);
+    if (mma_pending) mbar_wait_bounded(mma_bar, mma_phase, kWaitCycles);
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (threadIdx.x < 32) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, L::TMEM_COLS);
+    tmem_dealloc(tmem_base, G * L::TMEM_COLS);
   }
 }
 
@@ -1747,7 +1982,7 @@ int tc_blocks_per_sm() {
                                cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int n = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tc<H, FP8, MODE>, kRows, L::TOTAL);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tc<H, FP8, MODE>, kRows * L::G, L::TOTAL);
     // the same bound from the kernel's resources: registers (allocated per warp
     // in units of 256), shared memory (228 KB per SM, 1 KB reserved per CTA),
     // 2048 threads per SM. CTAs never wait on one another, so a bound above
@@ -1756,7 +1991,7 @@ int tc_blocks_per_sm() {
     int est = 16;
     if (cudaFuncGetAttributes(&fa, k_tc<H, FP8, MODE>) == cudaSuccess && fa.numRegs > 0) {
       const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-      est = std::min(est, 65536 / (regs_warp * (kRows / 32)));
+      est = std::min(est, 65536 / (regs_warp * (L::G * kRows / 32)));
     }
     est = std::min(est, 233472 / (L::TOTAL + 1024));
     if (e != cudaSuccess) cudaGetLastError();
@@ -1765,7 +2000,7 @@ int tc_blocks_per_sm() {
               int(FP8), MODE, n, cudaGetErrorString(e), est);
     n = std::max(n, est);
     n = n < 1 ? 1 : n;
-    while (n > 1 && n * L::TMEM_COLS > 512) --n;
+    while (n > 1 && n * L::G * L::TMEM_COLS > 512) --n;
     if (getenv("GNNTRK_VERBOSE"))
       fprintf(stderr, "gnntrk: k_tc<%d,%d,%d> smem %d B, %d CTAs/SM\n", H, int(FP8), MODE,
               L::TOTAL, n);
@@ -1854,8 +2089,8 @@ void launch_mode(const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   const int tuned = g_tuned[FP8 ? 1 : 0][hidx(H)][family_of(MODE)].load(std::memory_order_relaxed);
   if (tuned > 0 && tuned < per_sm) per_sm = tuned;
   int grid = device_sms() * per_sm;
-  grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRows - 1) / kRows)));
-  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows, L::TOTAL, s, 1, a);
+  grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRows * L::G - 1) / (kRows * L::G))));
+  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows * L::G, L::TOTAL, s, 1, a);
 }
 
 template <int H, bool FP8>
