@@ -850,6 +850,7 @@ struct MsgF32 {
       a = __fadd2_rn(a, make_float2(v.x, v.y));
       b = __fadd2_rn(b, make_float2(v.z, v.w));
     }
+    __device__ __forceinline__ void finish() {}
   };
   static __device__ __forceinline__ float4 load(const Ws& w, int e, int q) {
     return __ldg(reinterpret_cast<const float4*>(w.estate + size_t(e) * H) + q);

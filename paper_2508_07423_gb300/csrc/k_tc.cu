@@ -109,6 +109,8 @@ struct Layout {
   // one tensor-memory block (e into the other), so that the tiles (86 KB)
   // and the accumulators (256 columns) of two CTAs fit an SM
   static constexpr bool P3 = FP8 && H == 128 && (MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS);
+  // FP8 node step at hidden 128: the next tile's rows are loaded during a tile
+  static constexpr bool NODE8 = FP8 && H == 128 && MODE == M_NODE_UPD;
   static constexpr int K1 = (MODE == M_NODE_ENC) ? H : (SPLIT && !SPLIT2 ? 2 : 1) * NSEG * H;
   static constexpr int K2 = (SPLIT && MODE == M_NODE_ENC) ? 2 * H : H;
   static constexpr bool HAS_W1 = MODE != M_NODE_ENC;
@@ -315,8 +317,8 @@ struct CoopRows {
         v[g][j] = ld32(src + size_t(max(row, 0)) * H + 16 * (q + 4 * j));
     }
   }
-  // into a BF16 tile as they are
-  __device__ __forceinline__ void put(uint8_t* tile, int kchunks, int id) {
+  // into a tile as they are, from chunk c0 on
+  __device__ __forceinline__ void put(uint8_t* tile, int kchunks, int c0, int id) {
     const int lane = threadIdx.x & 31, warp = (threadIdx.x & (kRows - 1)) >> 5;
     const int r = lane & 7, q = lane >> 3;
 #pragma unroll
@@ -324,7 +326,7 @@ struct CoopRows {
       const bool in = __shfl_sync(0xffffffffu, id, 8 * g + r) >= 0;
 #pragma unroll
       for (int j = 0; j < PER; ++j) {
-        const uint32_t at = tile_off(32 * warp + 8 * g + r, 2 * (q + 4 * j), kchunks);
+        const uint32_t at = tile_off(32 * warp + 8 * g + r, c0 + 2 * (q + 4 * j), kchunks);
         *reinterpret_cast<uint4*>(tile + at) = in ? v[g][j].a : make_uint4(0, 0, 0, 0);
         *reinterpret_cast<uint4*>(tile + at + 128) = in ? v[g][j].b : make_uint4(0, 0, 0, 0);
       }
@@ -458,6 +460,17 @@ __device__ __forceinline__ void add_params(const float (&v)[32], const float* b,
       x[4 * q + 3] = v[4 * q + 3] + bb.w;
     }
   }
+}
+
+// FP8 messages of a hit in the projection rows' memory ([h_cap][2H] floats): 2H
+// codes [m_out | m_in] per hit from the start, then two scales per hit
+template <int H>
+__device__ __forceinline__ uint8_t* msg_codes(const Ws& w, int row) {
+  return reinterpret_cast<uint8_t*>(w.pstate) + size_t(row) * 2 * H;
+}
+template <int H>
+__device__ __forceinline__ float* msg_scales(const Ws& w, int row) {
+  return w.pstate + size_t(w.h_cap) * (2 * H / 4) + size_t(row) * 2;
 }
 
 // Issue the MMAs of one layer: A tile (kchunks 16-byte chunks per row) times
@@ -712,7 +725,11 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
   // loaded during a tile (its indices when the tile begins, the rows before its
   // epilogue), and the h rows of a pass during the MMAs of the pass before
   const int t_first = int(blockIdx.x) * G + wg;
-  CoopRows<L::P3 || L::SPLIT2 ? H : 64> pre;
+  CoopRows<L::P3 || L::SPLIT2 || L::NODE8 ? H : 64> pre;
+  CoopRows<L::NODE8 ? H : 64> pre_m;  // NODE8: the 2H message codes of a hit
+  float n_scale[2] = {1.f, 1.f};
+  (void)pre_m;
+  (void)n_scale;
   int nid_s = -1, nid_d = -1;
   float n_amax = 0.f;
   auto p3_ids = [&](int t) {
@@ -726,6 +743,16 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
     const int r = lo + t * kRows + tid;
     pre.load(w.estate16, t < n_tiles && r < hi ? r : -1);
   };
+  auto node8_rows = [&](int t) {
+    const int r = lo + t * kRows + tid;
+    const bool in = t < n_tiles && r < hi;
+    pre.load(w.hstate16, in ? r : -1);
+    pre_m.load(reinterpret_cast<const __nv_bfloat16*>(msg_codes<H>(w, 0)), in ? r : -1);
+    const float2 sc = *reinterpret_cast<const float2*>(msg_scales<H>(w, in ? r : 0));
+    n_scale[0] = in ? sc.x : 1.f;
+    n_scale[1] = in ? sc.y : 1.f;
+  };
+  if constexpr (L::NODE8) node8_rows(t_first);
   // (the split edge encoder: the rows of a pass during the MMAs of the pass before)
   if constexpr (L::SPLIT2) {
     p3_ids(t_first);
@@ -805,33 +832,23 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
         for (int i = 0; i < H; ++i) hid[i] = 0.f;
         for (int k = 0; k < L::K2; k += H) put_row_f32<FP8>(sHA, tid, KCH2, k, hid, H, 1.f);
       }
+    } else if constexpr (L::NODE8) {
+      // h under its own scale, the messages as the message kernel left them
+      sa[1] = n_scale[0];
+      sa[2] = n_scale[1];
+      sa[0] = pre.template put_e4m3<true>(sA, KCH1, 0, valid ? r : -1, 1.f);
+      pre_m.put(sA, KCH1, H / 16, valid ? r : -1);
     } else if constexpr (MODE == M_NODE_UPD) {
+      // (FP8, hidden 32 and 64; the BF16 node step is gathered above)
       if (valid) {
         sa[0] = put_row_bf16<H, FP8>(sA, tid, KCH1, 0, w.hstate16 + size_t(r) * H,
                                      H <= 64 ? keep_row : nullptr);
-        // the message sums [sum_out e, sum_in e] (FP32, written by k_msg_bf16
-        // into the node's projection row)
-        const float4* m4 = reinterpret_cast<const float4*>(w.pstate + size_t(r) * 2 * H);
-#pragma unroll 1
-        for (int side = 0; side < 2; ++side) {
-          float acc[H];
+        const uint4* m4 = reinterpret_cast<const uint4*>(msg_codes<H>(w, r));
 #pragma unroll
-          for (int i = 0; i < H / 4; ++i) {
-            const float4 v = m4[side * (H / 4) + i];
-            acc[4 * i] = v.x;
-            acc[4 * i + 1] = v.y;
-            acc[4 * i + 2] = v.z;
-            acc[4 * i + 3] = v.w;
-          }
-          float amax = 0.f;
-          if constexpr (FP8) {
-#pragma unroll
-            for (int i = 0; i < H; ++i) amax = fmaxf(amax, fabsf(acc[i]));
-          }
-          sa[1 + side] = FP8 ? (amax > 0.f ? amax / 448.f : 1.f) : 1.f;
-          put_row_f32<FP8>(sA, tid, KCH1, (1 + side) * H, acc, H,
-                           FP8 ? (amax > 0.f ? 448.f / amax : 1.f) : 1.f);
-        }
+        for (int c = 0; c < 2 * H / 16; ++c)
+          *reinterpret_cast<uint4*>(sA + tile_off(tid, H / 16 + c, KCH1)) = m4[c];
+        sa[1] = msg_scales<H>(w, r)[0];
+        sa[2] = msg_scales<H>(w, r)[1];
       } else {
         float z[16] = {};
         for (int k = 0; k < K1; k += 16) put_row_f32<FP8>(sA, tid, KCH1, k, z, 16, 1.f);
@@ -850,7 +867,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       id_s = nid_s;
       id_d = nid_d;
       p3_ids(t + int(gridDim.x) * G);
-      pre.put(sA, KCHA, id_s);
+      pre.put(sA, KCHA, 0, id_s);
     } else {
       // edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
       if (valid) {
@@ -931,7 +948,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       if constexpr (L::SPLIT2) {
         // hi(h_dst), lo(h_src), lo(h_dst) into the same tile, accumulated
         for (int pass = 1; pass <= 3 && !aborted; ++pass) {
-          pre.put(sA, KCHA, id_s);  // (id_s: whether the row exists)
+          pre.put(sA, KCHA, 0, id_s);  // (id_s: whether the row exists)
           fence_proxy_async();
           tc_fence_before();
           group_sync<G>(wg);
@@ -1057,6 +1074,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       mma_commit(mma_bar);
     }
     if constexpr (L::P3) p3_rows(t + int(gridDim.x) * G);
+    if constexpr (L::NODE8) node8_rows(t + int(gridDim.x) * G);
     if constexpr (L::SPLIT2) pre.load(w.hstate16, nid_s);
     if (!wait_mma()) {
       aborted = true;
@@ -1923,46 +1941,59 @@ __global__ void __launch_bounds__(kWsThreads, 2)
 
 // ---------------------------------------------------------------------------
 // messages of the node step (msg.cuh) from the BF16 edge states, P[v] = [m_out |
-// m_in], stored as FP32 (FP8 path: the node step quantises them with a per-row
-// scale) or rounded to BF16 (BF16 path: the layer-1 operand as the node step
-// would round it)
+// m_in], as the node step's operand: rounded to BF16 (BF16 path), or E4M3 codes
+// under one scale amax / 448 per sum (FP8 path: a quarter of the FP32 sums' bytes
+// to write and to read), rows of 2H codes and two scales (msg_codes, msg_scales)
 // ---------------------------------------------------------------------------
-template <int H, bool OUT16>
+template <int H, bool FP8>
 struct MsgBf16 {
   static constexpr int LANES = H / 8;
   using Chunk = uint4;
   struct Acc {
     float2 s[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                    make_float2(0.f, 0.f)};
+    float amax = 0.f;
     __device__ __forceinline__ void add(const uint4& v) {
       s[0] = __fadd2_rn(s[0], make_float2(bf16_lo(v.x), bf16_hi(v.x)));
       s[1] = __fadd2_rn(s[1], make_float2(bf16_lo(v.y), bf16_hi(v.y)));
       s[2] = __fadd2_rn(s[2], make_float2(bf16_lo(v.z), bf16_hi(v.z)));
       s[3] = __fadd2_rn(s[3], make_float2(bf16_lo(v.w), bf16_hi(v.w)));
     }
+    // FP8: the largest |sum| of the row, over the lanes of its group
+    __device__ __forceinline__ void finish() {
+      if constexpr (FP8) {
+        amax = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) amax = fmaxf(amax, fmaxf(fabsf(s[c].x), fabsf(s[c].y)));
+#pragma unroll
+        for (int o = 1; o < LANES; o *= 2) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+      }
+    }
   };
   static __device__ __forceinline__ uint4 load(const Ws& w, int e, int q) {
     return __ldg(reinterpret_cast<const uint4*>(w.estate16 + size_t(e) * H) + q);
   }
   static __device__ __forceinline__ void store(const Ws& w, int row, int side, int q, const Acc& a) {
-    if constexpr (OUT16) {
+    if constexpr (FP8) {
+      const float inv = a.amax > 0.f ? 448.f / a.amax : 1.f;
+      *(reinterpret_cast<uint2*>(msg_codes<H>(w, row) + side * H) + q) =
+          make_uint2(pack_e4m3x4(a.s[0].x * inv, a.s[0].y * inv, a.s[1].x * inv, a.s[1].y * inv),
+                     pack_e4m3x4(a.s[2].x * inv, a.s[2].y * inv, a.s[3].x * inv, a.s[3].y * inv));
+      if (q == 0) msg_scales<H>(w, row)[side] = a.amax > 0.f ? a.amax / 448.f : 1.f;
+    } else {
       *(reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(w.pstate) + size_t(row) * 2 * H +
                                  side * H) + q) =
           make_uint4(pack_bf16(a.s[0].x, a.s[0].y), pack_bf16(a.s[1].x, a.s[1].y),
                      pack_bf16(a.s[2].x, a.s[2].y), pack_bf16(a.s[3].x, a.s[3].y));
-    } else {
-      float4* o = reinterpret_cast<float4*>(w.pstate + size_t(row) * 2 * H + side * H + 8 * q);
-      o[0] = make_float4(a.s[0].x, a.s[0].y, a.s[1].x, a.s[1].y);
-      o[1] = make_float4(a.s[2].x, a.s[2].y, a.s[3].x, a.s[3].y);
     }
   }
 };
 
-template <int H, bool OUT16>
+template <int H, bool FP8>
 __global__ void __launch_bounds__(256, 4) k_msg_bf16(Batch b, Ws w) {
   pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
-  message_sums<MsgBf16<H, OUT16>>(w, Sel{nullptr, nullptr}, 0, b.n_hits);
+  message_sums<MsgBf16<H, FP8>>(w, Sel{nullptr, nullptr}, 0, b.n_hits);
 }
 
 // ---------------------------------------------------------------------------
@@ -2388,11 +2419,11 @@ void tc_node_prep(const Batch& b, const Ws& w, const TcModel& m, const LayerF32*
 void tc_messages(const Batch& b, const Ws& w, int h, bool fp8, cudaStream_t s) {
   const int grid = std::max(1, std::min(device_sms() * 8, div_up(b.n_hits, 256 / (h / 8))));
   if (h == 32)
-    launch_pdl(false, fp8 ? k_msg_bf16<32, false> : k_msg_bf16<32, true>, grid, 256, 0, s, 1, b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<32, true> : k_msg_bf16<32, false>, grid, 256, 0, s, 1, b, w);
   else if (h == 64)
-    launch_pdl(false, fp8 ? k_msg_bf16<64, false> : k_msg_bf16<64, true>, grid, 256, 0, s, 1, b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<64, true> : k_msg_bf16<64, false>, grid, 256, 0, s, 1, b, w);
   else
-    launch_pdl(false, fp8 ? k_msg_bf16<128, false> : k_msg_bf16<128, true>, grid, 256, 0, s, 1, b, w);
+    launch_pdl(false, fp8 ? k_msg_bf16<128, true> : k_msg_bf16<128, false>, grid, 256, 0, s, 1, b, w);
 }
 
 void tc_gnn(const Batch& b, const Ws& w, const TcModel& m, int h, int K, const GraphParams& g,

@@ -23,7 +23,7 @@
 
 namespace gnntrk {
 
-// R: LANES, Chunk (16 bytes), Acc (add(chunk)); load(w, edge, q), store(w, row,
+// R: LANES, Chunk (16 bytes), Acc (add(chunk), finish() by the whole warp); load(w, edge, q), store(w, row,
 // side, q, acc)
 template <class R>
 __device__ __forceinline__ void message_sums(const Ws& w, Sel sel, int lo, int hi) {
@@ -75,6 +75,7 @@ __device__ __forceinline__ void message_sums(const Ws& w, Sel sel, int lo, int h
       for (int u = 0; u < U; ++u)
         if (t + u < on) s.add(v[u]);
     }
+    s.finish();
     if (row >= 0) R::store(w, row, 0, q, s);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -93,6 +94,7 @@ __device__ __forceinline__ void message_sums(const Ws& w, Sel sel, int lo, int h
       for (int u = 0; u < U; ++u)
         if (t + u < in) s.add(v[u]);
     }
+    s.finish();
     if (row >= 0) R::store(w, row, 1, q, s);
     row = row1;
     row1 = row2;
