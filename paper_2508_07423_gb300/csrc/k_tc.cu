@@ -4,17 +4,20 @@
 // One CTA of 128 threads works on tiles of 128 rows (edges or hits); thread t
 // owns row t of the tile and TMEM lane t (warp w reads lanes 32w..32w+31). Per
 // tile:
-//   1. gather: each thread copies the pieces of its input row ([e, h_src,
-//      h_dst], [h, sum_out e, sum_in e], ...) from global memory into the A
-//      tile in shared memory, laid out as 8-row x 16-byte core matrices
-//      (K-major, no swizzle: row r, 16-byte chunk c at
+//   1. gather: the pieces of the input rows ([e, h_src, h_dst], [h, sum_out e,
+//      sum_in e], ...) come from global memory into the A tile in shared memory.
+//      BF16: by cp.async, four lanes per 64 bytes of a row, into blocks of 32
+//      columns in the 64-byte swizzle layout, during the tile before (see
+//      Layout::SWZ). FP8 and the three-pass forms: through registers into 8-row x
+//      16-byte core matrices (K-major, no swizzle: row r, 16-byte chunk c at
 //      ((r/8) * (K/epc) + c) * 128 + (r%8) * 16);
 //   2. one thread issues the layer-1 MMAs (weights resident in shared memory,
 //      loaded once per CTA by cp.async.bulk) and commits them to an mbarrier;
 //   3. every thread reads its row of the accumulator back with tcgen05.ld,
 //      adds the bias, applies LayerNorm and ReLU and writes the hidden row as
 //      the next A tile; layer 2 follows the same way;
-//   4. the epilogue adds the residual and stores the new state (BF16); at the
+//   4. the epilogue adds the residual and stores the new state (BF16, the rows of
+//      a warp through shared memory so that the stores are whole lines); at the
 //      last step the edge classifier (a third MMA, LayerNorm, ReLU and a dot
 //      product) and the cut run instead of the store.
 // FP8: each input segment of layer 1 (e.g. e, h_src, h_dst) is quantised with
@@ -122,14 +125,20 @@ struct Layout {
   static constexpr int W2_BYTES = HAS_W2 ? H * K2 * ESZ : 0;
   static constexpr int WC = align1k(W2 + W2_BYTES);
   static constexpr int WC_BYTES = HAS_WC ? H * H * ESZ : 0;
-  // BF16 node-step tiles ([h, m_out, m_in], contiguous rows) are gathered by
-  // coalesced cp.async copies; with PREFETCH into two alternating layer-1
-  // input buffers (tile t + 1 loads while tile t computes). Edge tiles keep
-  // the per-row copies: on the 1000-event batch they measured faster than
-  // cp.async (single or double buffered) and than conflict-free coalesced
-  // copies through registers (2.27 ms against 2.59-3.12 ms per 4 launches).
-  static constexpr bool PIPE = !FP8 && MODE == M_NODE_UPD;
-  static constexpr bool PREFETCH = false;
+  // BF16 layer-1 inputs (but the three-pass forms' and the node encoder's) are
+  // kept as blocks of 128 rows x 64 bytes in the 64-byte swizzle layout and filled
+  // by cp.async with four lanes per row: one copy instruction then touches 8 lines
+  // of global memory and 4 x 128 bytes of shared memory without bank conflicts.
+  // With the canonical layout (8 rows x 16 bytes) either the loads touch 32 lines
+  // or the stores conflict four ways, and the kernels were bound by the shared
+  // memory pipe (82-87 % of its cycles). Hidden 32, 1024 events, us per launch
+  // before and after: edge encoder (10.1 M rows) 638 -> 338, edge step 499 -> 340,
+  // node step (1.7 M rows) 130 -> 68.
+  static constexpr bool SWZ = !FP8 && MODE != M_NODE_ENC && !SPLIT2;
+  // the next tile's rows load while this tile's layer 2 and epilogue run; the
+  // hidden row then needs a tile of its own (in the edge encoder at hidden 64 that
+  // would leave room for one CTA per SM instead of two)
+  static constexpr bool PREF = SWZ && (H == 32 || !SPLIT);
   // tiles in flight per CTA, each worked on by a warpgroup of its own with its
   // own buffers and accumulators; they share the weights. Two in the edge encoder
   // at hidden 128, whose weights leave room for one CTA per SM (the node step's
@@ -138,19 +147,21 @@ struct Layout {
   static constexpr int G = SPLIT2 ? 2 : 1;
   static constexpr int A = align1k(WC + WC_BYTES);
   static constexpr int A_BYTES = MODE == M_NODE_ENC ? 0 : kRows * (P3 || SPLIT2 ? H : K1) * ESZ;
-  static constexpr int NBUF = PIPE && PREFETCH ? 2 : 1;
-  // hidden / classifier input: its own tile with two input buffers, else it
-  // overwrites the layer-1 input once the layer-1 MMAs are done
-  static constexpr int HA = NBUF == 2 || MODE == M_NODE_ENC ? align1k(A + NBUF * A_BYTES) : A;
-  static constexpr int HA_BYTES = NBUF == 2 || MODE == M_NODE_ENC ? kRows * K2 * ESZ : 0;
-  static_assert(G == 1 || (NBUF == 1 && HA_BYTES == 0 && A_BYTES % 1024 == 0), "one buffer per warpgroup");
-  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + HA_BYTES : A + G * NBUF * A_BYTES);
+  // hidden / classifier input: its own tile or over the layer-1 input
+  static constexpr bool OWN_HA = MODE == M_NODE_ENC || (PREF && HAS_W2);
+  static constexpr int HA = OWN_HA ? align1k(A + A_BYTES) : A;
+  static constexpr int HA_BYTES = OWN_HA ? kRows * K2 * ESZ : 0;
+  static_assert(G == 1 || (HA_BYTES == 0 && A_BYTES % 1024 == 0), "one buffer per warpgroup");
+  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + HA_BYTES : A + G * A_BYTES);
   // fp32 parameters: b1, b2, bc1, s1, s2, sc, c2 weights, ne1 (3 x H + H)
   static constexpr int PAR_FLOATS = 7 * H + 4 * H + 8;
   static constexpr int BAR = PAR + PAR_FLOATS * 4;
   // hidden 128: each warp's state rows pass through a staging block of 32 rows x
   // 64 bytes (80-byte stride) on their way in (residual) and out
   static constexpr bool COOP = H == 128 && MODE != M_CLS && MODE != M_TRIP;
+  // BF16 at hidden 32 and 64: out through the hidden tile, which is free by then
+  static constexpr bool OUT_STAGE = !FP8 && H <= 64 && MODE != M_CLS && MODE != M_TRIP && MODE != M_EDGE_UPD_CLS;
+  static_assert(!(SWZ && (NODE8 || P3)) && !(OUT_STAGE && COOP), "one way in, one way out");
   static constexpr int STAGE = BAR + 64;
   static constexpr int STAGE_ROW = 80;
   static constexpr int TOTAL = STAGE + (COOP ? G * kRows * STAGE_ROW : 0);
@@ -206,47 +217,36 @@ __device__ __forceinline__ void put_row_f32(uint8_t* tile, int row, int kchunks,
   }
 }
 
-// Copy one BF16 row of H values from global memory into the A tile (BF16) or
-// quantise it (FP8, per-row scale returned). `keep` receives the raw row when
-// not null.
-template <int H, bool FP8>
-__device__ __forceinline__ float put_row_bf16(uint8_t* tile, int row, int kchunks, int k0,
+// Quantise one BF16 row of H values from global memory into an E4M3 A tile (the
+// per-row scale is returned). `keep` receives the raw row when not null.
+template <int H>
+__device__ __forceinline__ float put_row_e4m3(uint8_t* tile, int row, int kchunks, int k0,
                                               const __nv_bfloat16* src, uint4* keep) {
   const uint4* s4 = reinterpret_cast<const uint4*>(src);
-  if constexpr (!FP8) {
+  uint4 r[H / 8];
+  float amax = 0.f;
 #pragma unroll
-    for (int c = 0; c < H / 8; ++c) {
-      const uint4 u = s4[c];
-      if (keep) keep[c] = u;
-      *reinterpret_cast<uint4*>(tile + tile_off(row, (k0 >> 3) + c, kchunks)) = u;
-    }
-    return 1.0f;
-  } else {
-    uint4 r[H / 8];
-    float amax = 0.f;
+  for (int c = 0; c < H / 8; ++c) {
+    r[c] = s4[c];
+    if (keep) keep[c] = r[c];
+    const uint32_t q[4] = {r[c].x, r[c].y, r[c].z, r[c].w};
 #pragma unroll
-    for (int c = 0; c < H / 8; ++c) {
-      r[c] = s4[c];
-      if (keep) keep[c] = r[c];
-      const uint32_t q[4] = {r[c].x, r[c].y, r[c].z, r[c].w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        amax = fmaxf(amax, fmaxf(fabsf(bf16_lo(q[j])), fabsf(bf16_hi(q[j]))));
-    }
-    const float scale = amax > 0.f ? amax / 448.f : 1.f;
-    const float inv = amax > 0.f ? 448.f / amax : 1.f;
-#pragma unroll
-    for (int c = 0; c < H / 16; ++c) {
-      const uint4 a = r[2 * c], b = r[2 * c + 1];
-      uint4 u;
-      u.x = pack_e4m3x4(bf16_lo(a.x) * inv, bf16_hi(a.x) * inv, bf16_lo(a.y) * inv, bf16_hi(a.y) * inv);
-      u.y = pack_e4m3x4(bf16_lo(a.z) * inv, bf16_hi(a.z) * inv, bf16_lo(a.w) * inv, bf16_hi(a.w) * inv);
-      u.z = pack_e4m3x4(bf16_lo(b.x) * inv, bf16_hi(b.x) * inv, bf16_lo(b.y) * inv, bf16_hi(b.y) * inv);
-      u.w = pack_e4m3x4(bf16_lo(b.z) * inv, bf16_hi(b.z) * inv, bf16_lo(b.w) * inv, bf16_hi(b.w) * inv);
-      *reinterpret_cast<uint4*>(tile + tile_off(row, (k0 >> 4) + c, kchunks)) = u;
-    }
-    return scale;
+    for (int j = 0; j < 4; ++j)
+      amax = fmaxf(amax, fmaxf(fabsf(bf16_lo(q[j])), fabsf(bf16_hi(q[j]))));
   }
+  const float scale = amax > 0.f ? amax / 448.f : 1.f;
+  const float inv = amax > 0.f ? 448.f / amax : 1.f;
+#pragma unroll
+  for (int c = 0; c < H / 16; ++c) {
+    const uint4 a = r[2 * c], b = r[2 * c + 1];
+    uint4 u;
+    u.x = pack_e4m3x4(bf16_lo(a.x) * inv, bf16_hi(a.x) * inv, bf16_lo(a.y) * inv, bf16_hi(a.y) * inv);
+    u.y = pack_e4m3x4(bf16_lo(a.z) * inv, bf16_hi(a.z) * inv, bf16_lo(a.w) * inv, bf16_hi(a.w) * inv);
+    u.z = pack_e4m3x4(bf16_lo(b.x) * inv, bf16_hi(b.x) * inv, bf16_lo(b.y) * inv, bf16_hi(b.y) * inv);
+    u.w = pack_e4m3x4(bf16_lo(b.z) * inv, bf16_hi(b.z) * inv, bf16_lo(b.w) * inv, bf16_hi(b.w) * inv);
+    *reinterpret_cast<uint4*>(tile + tile_off(row, (k0 >> 4) + c, kchunks)) = u;
+  }
+  return scale;
 }
 
 // Write n FP32 values (a multiple of 8) into a BF16 tile as two parts, hi =
@@ -366,7 +366,8 @@ struct CoopRows {
 
 // A warp's 32 state rows of H BF16 values, 32 columns (64 bytes) at a time,
 // through its staging block: lane (row lane / 4 + 8 i, part lane % 4) moves 16
-// bytes between global memory and the block, lane l reads and writes row l.
+// bytes between global memory and the block, lane l reads and writes row l (rows
+// STRIDE bytes apart: 80, or 64 with the parts swizzled).
 template <int H, int STRIDE>
 struct RowStage {
   uint8_t* blk;                // the warp's block
@@ -375,7 +376,7 @@ struct RowStage {
   uint4 v[4];
 
   __device__ __forceinline__ uint4* slot(int row, int part) const {
-    return reinterpret_cast<uint4*>(blk + row * STRIDE + 16 * part);
+    return reinterpret_cast<uint4*>(blk + row * STRIDE + 16 * (STRIDE == 64 ? part ^ ((row >> 1) & 3) : part));
   }
   // columns 32 c .. 32 c + 31 of every row into registers (missing rows: row 0)
   __device__ __forceinline__ void fetch(int c) {
@@ -414,16 +415,15 @@ struct RowStage {
   }
 };
 
-// the lo parts of 32 columns, bf16(z - bf16(z))
-__device__ __forceinline__ void store_lo(__nv_bfloat16* dst, const float (&z)[32]) {
+// the lo parts of 32 columns, bf16(z - bf16(z)), packed
+__device__ __forceinline__ void lo_parts(const float (&z)[32], uint4 (&o)[4]) {
   float l[32];
 #pragma unroll
   for (int j = 0; j < 32; ++j) l[j] = z[j] - __bfloat162float(__float2bfloat16_rn(z[j]));
 #pragma unroll
   for (int q = 0; q < 4; ++q)
-    reinterpret_cast<uint4*>(dst)[q] =
-        make_uint4(pack_bf16(l[8 * q], l[8 * q + 1]), pack_bf16(l[8 * q + 2], l[8 * q + 3]),
-                   pack_bf16(l[8 * q + 4], l[8 * q + 5]), pack_bf16(l[8 * q + 6], l[8 * q + 7]));
+    o[q] = make_uint4(pack_bf16(l[8 * q], l[8 * q + 1]), pack_bf16(l[8 * q + 2], l[8 * q + 3]),
+                      pack_bf16(l[8 * q + 4], l[8 * q + 5]), pack_bf16(l[8 * q + 6], l[8 * q + 7]));
 }
 // acc[0..7] += the 8 BF16 values of u
 __device__ __forceinline__ void add_bf16x8(float* acc, const uint4& u) {
@@ -500,6 +500,18 @@ __device__ __forceinline__ void issue_layer(uint32_t tmem, const uint8_t* A, con
   }
 }
 
+// Layer 1 of a BF16 tile kept as swizzled blocks of 32 columns (K of them in all).
+template <int H, int K>
+__device__ __forceinline__ void issue_blocks_bf16(uint32_t tmem, const uint8_t* A, const uint8_t* W) {
+  constexpr uint32_t IDESC = idesc_bf16(kRows, H);
+  constexpr uint32_t SBO_W = uint32_t(K * 2 / 16) * 128;
+  const uint32_t a0 = smem_u32(A), w0 = smem_u32(W);
+#pragma unroll
+  for (int k = 0; k < K; k += 16)
+    mma_bf16(tmem, smem_desc_sw64(a0 + uint32_t((k / 32) * (kRows * 64) + (k % 32) * 2)),
+             smem_desc(w0 + uint32_t(k * 2 / 16) * 128, 128, SBO_W), IDESC, k > 0 ? 1u : 0u);
+}
+
 // One pass of a three-pass FP8 layer 1 (K = 3H): the one-segment A tile
 // (E4M3, H per row) times K chunk `pass` of the weight image (E4M3, 3H per
 // row); pass 0 starts its accumulator, pass 1 starts the other, pass 2 adds
@@ -537,55 +549,52 @@ __device__ __forceinline__ void issue_pass_bf16(uint32_t tmem, const uint8_t* A,
   }
 }
 
-// Copy slot l (0 .. H/8 - 1) of thread tid in a tile copy: warp w covers rows
-// 32w .. 32w+31; a quarter-warp (8 lanes) takes one 16-byte chunk of 8
-// consecutive rows, a contiguous 128-byte run of the canonical tile, so the
-// shared-memory stores are conflict-free, and a warp instruction reads 8 rows
-// x 4 chunks.
-template <int CH>
-__device__ __forceinline__ void copy_slot(int tid, int l, int& rr, int& c) {
-  const int warp = tid >> 5, lane = tid & 31;
-  const int g = l % 4, cq = l / 4;  // row group of 8, chunk quad
-  rr = warp * 32 + g * 8 + (lane & 7);
-  c = cq * 4 + (lane >> 3);
-}
-
-// Issue the cp.async copies of one BF16 tile's layer-1 input (rows row0 ..
-// row0 + 127; rows at or past `hi` are zero-filled): segment s of row r, chunk
-// c (16 bytes) lands at tile_off(r, s * H/8 + c). Consecutive threads take the
-// chunks of one row, so a warp reads 8 rows x H*2 bytes per segment.
+// Issue the cp.async copies of a warp's 32 rows of a BF16 tile's layer-1 input
+// into the swizzled blocks of `A` (16-byte chunk c of row r at chunk
+// c ^ ((r >> 1) & 3)): lane (row lane / 4 + 8 i, part lane % 4). Rows at or past
+// `hi` are zero-filled. id_a, id_b: each lane's own row's two gathered rows.
 template <int H, int MODE>
-__device__ __forceinline__ void gather_async(uint8_t* dst, const TcArgs& p, int row0, int hi,
-                                             int tid) {
-  constexpr int CH = H / 8;
-  constexpr int NSEG = n_seg(MODE);
-  constexpr int KCH = NSEG * CH;
+__device__ __forceinline__ void gather_blocks(uint8_t* A, const TcArgs& p, int row0, int hi, int warp,
+                                              int id_a, int id_b) {
+  using bf = __nv_bfloat16;
+  constexpr int NS = MODE == M_EDGE_ENC ? 4 : n_seg(MODE);
   const Ws& w = p.w;
-  const __nv_bfloat16* msg16 = reinterpret_cast<const __nv_bfloat16*>(w.pstate);
+  const int lane = threadIdx.x & 31, part = lane & 3;
 #pragma unroll
-  for (int l = 0; l < CH; ++l) {
-    int rr, c;
-    copy_slot<CH>(tid, l, rr, c);
-    const int r = row0 + rr;
-    const uint32_t n = r < hi ? 16u : 0u;
-    const int rs = r < hi ? r : 0;
-    const __nv_bfloat16* src[3];
+  for (int i = 0; i < 4; ++i) {
+    const int wr = (lane >> 2) + 8 * i, rr = 32 * warp + wr, r = row0 + rr;
+    const bool in = r < hi;
+    const size_t row = size_t(in ? r : 0) * H;
+    size_t ga = 0, gb = 0;
+    if constexpr (MODE != M_NODE_UPD && MODE != M_CLS) {
+      ga = size_t(max(__shfl_sync(0xffffffffu, id_a, wr), 0)) * H;
+      gb = size_t(max(__shfl_sync(0xffffffffu, id_b, wr), 0)) * H;
+    }
+    const bf* src[4] = {};
     if constexpr (MODE == M_NODE_UPD) {
-      src[0] = w.hstate16 + size_t(rs) * H;
-      src[1] = msg16 + size_t(rs) * 2 * H;
+      src[0] = w.hstate16 + row;
+      src[1] = reinterpret_cast<const bf*>(w.pstate) + 2 * row;
       src[2] = src[1] + H;
     } else if constexpr (MODE == M_EDGE_ENC) {
-      src[0] = w.hstate16 + size_t(w.src[rs]) * H;
-      src[1] = w.hstate16 + size_t(w.col[rs]) * H;
-    } else if constexpr (MODE == M_CLS) {
-      src[0] = w.estate16 + size_t(rs) * H;
+      const bf* hlo = reinterpret_cast<const bf*>(w.hstate);
+      src[0] = w.hstate16 + ga;
+      src[1] = w.hstate16 + gb;
+      src[2] = hlo + ga;
+      src[3] = hlo + gb;
+    } else if constexpr (MODE == M_TRIP) {
+      src[0] = w.estate16 + ga;
+      src[1] = w.estate16 + gb;
     } else {
-      src[0] = w.estate16 + size_t(rs) * H;
-      src[1] = w.hstate16 + size_t(w.src[rs]) * H;
-      src[2] = w.hstate16 + size_t(w.col[rs]) * H;
+      src[0] = w.estate16 + row;
+      src[1] = w.hstate16 + ga;
+      src[2] = w.hstate16 + gb;
     }
+    uint8_t* d = A + rr * 64 + ((part ^ ((rr >> 1) & 3)) << 4);
 #pragma unroll
-    for (int sg = 0; sg < NSEG; ++sg) cp_async16(dst + tile_off(rr, sg * CH + c, KCH), src[sg] + 8 * c, n);
+    for (int sg = 0; sg < NS; ++sg)
+#pragma unroll
+      for (int c = 0; c < H / 32; ++c)
+        cp_async16(d + (sg * (H / 32) + c) * (kRows * 64), src[sg] + 32 * c + 8 * part, in ? 16u : 0u);
   }
 }
 
@@ -613,8 +622,13 @@ __device__ __forceinline__ bool group_sync_or(int wg, bool v) {
   }
 }
 
+// Tiles per SM that the registers must allow: BF16 at hidden 32 as many as the
+// shared memory holds (edge step on 10.1 M rows 356 us with four, 340 us with five;
+// the node encoder would spill).
+constexpr int min_ctas(int H, bool FP8, int MODE) { return !FP8 && H == 32 && MODE != M_NODE_ENC ? 5 : 1; }
+
 template <int H, bool FP8, int MODE>
-__global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(const TcArgs p) {
+__global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H, FP8, MODE)) k_tc(const TcArgs p) {
   using L = Layout<H, FP8, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sW1 = smem + L::W1;
@@ -716,11 +730,6 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
     return true;
   };
 
-  if constexpr (L::PIPE && L::PREFETCH) {
-    if (int(blockIdx.x) < n_tiles && !aborted)
-      gather_async<H, MODE>(smem + L::A, p, lo + int(blockIdx.x) * kRows, hi, tid);
-    cp_async_commit();
-  }
   // FP8 edge steps at hidden 128: the next tile's e rows, hits and h maxima are
   // loaded during a tile (its indices when the tile begins, the rows before its
   // epilogue), and the h rows of a pass during the MMAs of the pass before
@@ -735,8 +744,9 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
   auto p3_ids = [&](int t) {
     const int r = lo + t * kRows + tid;
     const bool in = t < n_tiles && r < hi;
-    nid_s = in ? w.src[r] : -1;
-    nid_d = in ? w.col[r] : -1;
+    if constexpr (MODE == M_NODE_UPD || MODE == M_CLS) return;
+    nid_s = in ? (MODE == M_TRIP ? p.t1 : w.src)[r] : -1;
+    nid_d = in ? (MODE == M_TRIP ? p.t2 : w.col)[r] : -1;
   };
   auto p3_amax = [&] { n_amax = nid_s >= 0 ? fmaxf(w.hamax[nid_s], w.hamax[nid_d]) : 0.f; };
   auto p3_rows = [&](int t) {
@@ -763,11 +773,20 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
     p3_rows(t_first);
     p3_amax();
   }
-  int it = 0;
-  for (int t = t_first; t < n_tiles && !aborted; t += int(gridDim.x) * G, ++it) {
+  // BF16: rows of tile t into the blocks (its ids loaded a tile ahead)
+  auto gather = [&](int t) {
+    if (t < n_tiles) gather_blocks<H, MODE>(smem + L::A, p, lo + t * kRows, hi, warp, nid_s, nid_d);
+    cp_async_commit();
+  };
+  (void)gather;
+  if constexpr (L::SWZ) {
+    p3_ids(t_first);
+    if constexpr (L::PREF) gather(t_first);
+  }
+  for (int t = t_first; t < n_tiles && !aborted; t += int(gridDim.x) * G) {
     const int r = lo + t * kRows + tid;
     const bool valid = r < hi;
-    uint8_t* sA = smem + L::A + wg * L::A_BYTES + (L::NBUF == 2 ? (it & 1) * L::A_BYTES : 0);
+    uint8_t* sA = smem + L::A + wg * L::A_BYTES;
     uint8_t* sHA = L::HA == L::A ? sA : smem + L::HA;  // layer-2 input and classifier input
     float sa[3] = {1.f, 1.f, 1.f};  // FP8 per-row scales of the layer-1 segments
     int id_s = -1, id_d = -1;       // this row's source and target hit (hidden 128)
@@ -777,19 +796,12 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
     (void)keep_row;
 
     // ---- 1. gather ---------------------------------------------------------
-    if constexpr (L::PIPE && L::PREFETCH) {
-      // every thread is done with the other buffer (tile it - 1): fill it with
-      // the next tile, then wait for this tile's copies
-      group_sync<G>(wg);
-      const int tn = t + int(gridDim.x) * G;
-      if (tn < n_tiles)
-        gather_async<H, MODE>(smem + L::A + ((it + 1) & 1) * L::A_BYTES, p, lo + tn * kRows, hi, tid);
-      cp_async_commit();
-      cp_async_wait<1>();
-    } else if constexpr (L::PIPE) {
-      group_sync<G>(wg);  // every thread is done with the buffer (tile it - 1)
-      gather_async<H, MODE>(sA, p, lo + t * kRows, hi, tid);
-      cp_async_commit();
+    if constexpr (L::SWZ) {
+      if constexpr (!L::PREF) {
+        group_sync<G>(wg);  // every thread is done with the buffer
+        gather(t);
+      }
+      p3_ids(t + int(gridDim.x));
       cp_async_wait<0>();
     } else if constexpr (MODE == M_NODE_ENC) {
       // FP32 first layer (K = 3) in registers, then LayerNorm + ReLU into A
@@ -839,10 +851,10 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       sa[0] = pre.template put_e4m3<true>(sA, KCH1, 0, valid ? r : -1, 1.f);
       pre_m.put(sA, KCH1, H / 16, valid ? r : -1);
     } else if constexpr (MODE == M_NODE_UPD) {
-      // (FP8, hidden 32 and 64; the BF16 node step is gathered above)
+      // (FP8, hidden 32 and 64)
       if (valid) {
-        sa[0] = put_row_bf16<H, FP8>(sA, tid, KCH1, 0, w.hstate16 + size_t(r) * H,
-                                     H <= 64 ? keep_row : nullptr);
+        sa[0] = put_row_e4m3<H>(sA, tid, KCH1, 0, w.hstate16 + size_t(r) * H,
+                                H <= 64 ? keep_row : nullptr);
         const uint4* m4 = reinterpret_cast<const uint4*>(msg_codes<H>(w, r));
 #pragma unroll
         for (int c = 0; c < 2 * H / 16; ++c)
@@ -869,31 +881,18 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       p3_ids(t + int(gridDim.x) * G);
       pre.put(sA, KCHA, 0, id_s);
     } else {
-      // edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
+      // (FP8) edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
       if (valid) {
         int seg = 0;
-        if constexpr (MODE == M_TRIP) {
-          // [e^K(first edge), e^K(second edge)]
-          sa[0] = put_row_bf16<H, FP8>(sA, tid, KCH1, 0, w.estate16 + size_t(p.t1[r]) * H, nullptr);
-          sa[1] = put_row_bf16<H, FP8>(sA, tid, KCH1, H, w.estate16 + size_t(p.t2[r]) * H, nullptr);
-          seg = 2;
-        } else if constexpr (MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS || MODE == M_CLS) {
-          sa[0] = put_row_bf16<H, FP8>(sA, tid, KCH1, 0, w.estate16 + size_t(r) * H,
-                                       (H <= 64 && MODE != M_CLS) ? keep_row : nullptr);
+        if constexpr (MODE != M_EDGE_ENC) {
+          sa[0] = put_row_e4m3<H>(sA, tid, KCH1, 0, w.estate16 + size_t(r) * H,
+                                  (H <= 64 && MODE != M_CLS) ? keep_row : nullptr);
           seg = 1;
         }
-        if constexpr (L::SPLIT) {
-          // [hi(h_src), hi(h_dst), lo(h_src), lo(h_dst)]
-          const size_t src = size_t(w.src[r]) * H, dst = size_t(w.col[r]) * H;
-          put_row_bf16<H, false>(sA, tid, KCH1, 0, w.hstate16 + src, nullptr);
-          put_row_bf16<H, false>(sA, tid, KCH1, H, w.hstate16 + dst, nullptr);
-          put_row_bf16<H, false>(sA, tid, KCH1, 2 * H, hlo + src, nullptr);
-          put_row_bf16<H, false>(sA, tid, KCH1, 3 * H, hlo + dst, nullptr);
-        } else if constexpr (MODE != M_CLS && MODE != M_TRIP) {
-          sa[seg] = put_row_bf16<H, FP8>(sA, tid, KCH1, seg * H, w.hstate16 + size_t(w.src[r]) * H,
-                                         nullptr);
-          sa[seg + 1] = put_row_bf16<H, FP8>(sA, tid, KCH1, (seg + 1) * H,
-                                             w.hstate16 + size_t(w.col[r]) * H, nullptr);
+        if constexpr (MODE != M_CLS) {
+          sa[seg] = put_row_e4m3<H>(sA, tid, KCH1, seg * H, w.hstate16 + size_t(w.src[r]) * H, nullptr);
+          sa[seg + 1] = put_row_e4m3<H>(sA, tid, KCH1, (seg + 1) * H, w.hstate16 + size_t(w.col[r]) * H,
+                                        nullptr);
         }
       } else {
         float z[16] = {};
@@ -913,6 +912,8 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
           issue_pass_e4m3<H>(tmem_base, sA, sW1, 0);
         else if constexpr (L::SPLIT2)
           issue_pass_bf16<H>(tmem_base, sA, sW1, 0);
+        else if constexpr (L::SWZ)
+          issue_blocks_bf16<H, K1>(tmem_base, sA, sW1);
         else
           issue_layer<H, FP8>(tmem_base, sA, sW1, K1, FP8 ? L::NSEG : 1);
         mma_commit(mma_bar);
@@ -962,16 +963,15 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
         }
         if (aborted) break;
       }
-      if constexpr (L::PIPE && L::HA == L::A) {
-        // the hidden tile overwrites the layer-1 input: keep this row's
-        // residual segment in registers first
-        if constexpr (MODE == M_NODE_UPD || MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS) {
+      if constexpr (L::SWZ && L::HAS_W2 && MODE != M_EDGE_ENC) {
+        // the residual: this row's first segment, before the buffer is refilled
+        constexpr int NK = H <= 64 ? H / 8 : 1;
 #pragma unroll
-          for (int c = 0; c < H / 8; ++c)
-            keep_row[c] = *reinterpret_cast<const uint4*>(sA + tile_off(tid, c, KCH1));
-        }
-        group_sync<G>(wg);
+        for (int c = 0; c < NK; ++c)
+          keep_row[c] = *reinterpret_cast<const uint4*>(sA + (c / 4) * (kRows * 64) + tid * 64 +
+                                                        (((c & 3) ^ ((tid >> 1) & 3)) << 4));
       }
+      if constexpr (L::PREF && !L::HAS_W2) gather(t + int(gridDim.x));
       // ---- 3. bias + LayerNorm + ReLU (-> A as the next operand, or the
       //         classifier output for M_CLS) -------------------------------
       // x[n] = s_w[n] * sum_seg s_a[seg] * acc_seg[n] + b[n]  (FP8)
@@ -1072,6 +1072,8 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       issue_layer<H, FP8>(tmem_base, sHA, sW2, L::K2, 1);
       mma_commit(mma_bar);
     }
+    // (every thread has its residual and is past the barrier above)
+    if constexpr (L::PREF) gather(t + int(gridDim.x));
     if constexpr (L::P3) p3_rows(t + int(gridDim.x) * G);
     if constexpr (L::NODE8) node8_rows(t + int(gridDim.x) * G);
     if constexpr (L::SPLIT2) pre.load(w.hstate16, nid_s);
@@ -1090,12 +1092,12 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       }
       add_params<FP8>(v, pb2 + c * 32, ps2 + c * 32, z);
     };
-    // hidden 128: the warp's state rows through its staging block
+    // hidden 128, BF16: the warp's state rows through its staging block
     constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
     const int row0 = r - (tid & 31);
-    RowStage<H, L::STAGE_ROW> st{smem + L::STAGE + (wg * kRows + warp * 32) * L::STAGE_ROW,
-                                 (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(row0) * H,
-                                 min(max(hi - row0, 0), 32), {}};
+    RowStage<H, L::OUT_STAGE ? 64 : L::STAGE_ROW> st{
+        L::OUT_STAGE ? sHA + warp * 32 * L::K2 * 2 : smem + L::STAGE + (wg * kRows + warp * 32) * L::STAGE_ROW,
+        (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(row0) * H, min(max(hi - row0, 0), 32), {}};
     (void)st;
     // residual input row (BF16) for the update modes
     auto resid = [&](int c, float (&z)[32]) {
@@ -1109,10 +1111,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
         const __nv_bfloat16* rowp = (MODE == M_NODE_UPD ? w.hstate16 : w.estate16) + size_t(r) * H;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const uint4 u = (L::PIPE && L::HA != L::A)
-                              ? *reinterpret_cast<const uint4*>(sA + tile_off(tid, c * 4 + q, KCH1))
-                          : (H <= 64) ? keep_row[c * 4 + q]
-                                      : reinterpret_cast<const uint4*>(rowp)[c * 4 + q];
+          const uint4 u = (H <= 64) ? keep_row[c * 4 + q] : reinterpret_cast<const uint4*>(rowp)[c * 4 + q];
           add_bf16x8(z + 8 * q, u);
         }
       }
@@ -1122,7 +1121,27 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
       // ---- 5. store the new state (BF16) -----------------------------------
       __nv_bfloat16* dst = (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(r) * H;
       float row_max = 0.f;  // largest |stored value| of a node row
-      if constexpr (L::COOP) {
+      auto st_lo = st;  // (node encoder: the lo parts)
+      if constexpr (MODE == M_NODE_ENC) st_lo.first = hlo + size_t(row0) * H;
+      (void)st_lo;
+      if constexpr (L::OUT_STAGE) {
+#pragma unroll
+        for (int c = 0; c < H / 32; ++c) {
+          float z[32];
+          zval(c, z);
+          if constexpr (MODE == M_NODE_UPD || MODE == M_EDGE_UPD) resid(c, z);
+          uint4 o[4];
+          if constexpr (MODE == M_NODE_ENC) {
+            lo_parts(z, o);
+            st_lo.put(c, o);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            o[q] = make_uint4(pack_bf16(z[8 * q], z[8 * q + 1]), pack_bf16(z[8 * q + 2], z[8 * q + 3]),
+                              pack_bf16(z[8 * q + 4], z[8 * q + 5]), pack_bf16(z[8 * q + 6], z[8 * q + 7]));
+          st.put(c, o);
+        }
+      } else if constexpr (L::COOP) {
         constexpr bool RESID = MODE == M_NODE_UPD || MODE == M_EDGE_UPD;
         if constexpr (RESID) st.fetch(0);
 #pragma unroll
@@ -1136,10 +1155,11 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
 #pragma unroll
             for (int q = 0; q < 4; ++q) add_bf16x8(z + 8 * q, e[q]);
           }
-          if constexpr (L::SPLIT && MODE == M_NODE_ENC) {
-            if (valid) store_lo(hlo + size_t(r) * H + 32 * c, z);
-          }
           uint4 o[4];
+          if constexpr (L::SPLIT && MODE == M_NODE_ENC) {
+            lo_parts(z, o);
+            st_lo.put(c, o);
+          }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             o[q] = make_uint4(pack_bf16(z[8 * q], z[8 * q + 1]), pack_bf16(z[8 * q + 2], z[8 * q + 3]),
@@ -1155,9 +1175,6 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
         zval(c, z);
         if (valid) {
           resid(c, z);
-          if constexpr (L::SPLIT && MODE == M_NODE_ENC) {
-            store_lo(hlo + size_t(r) * H + 32 * c, z);
-          }
           uint4* d4 = reinterpret_cast<uint4*>(dst) + c * 4;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
@@ -1263,7 +1280,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), 1) k_tc(con
 
   // ---- clean-up: on a timeout, give the outstanding MMAs one more bounded
   //      wait, then free the tensor memory -----------------------------------
-  if constexpr (L::PIPE) cp_async_wait<0>();  // no copy may land after the exit
+  if constexpr (L::SWZ) cp_async_wait<0>();  // no copy may land after the exit
   if (aborted) {
     if (tid == 0) set_status(w.counters, ST_TIMEOUT);
     if (weights_late) mbar_wait_bounded(&bar[0], 0, kWaitCycles);
@@ -2123,13 +2140,19 @@ void launch_h(int mode, const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   switch (mode) {
     case M_NODE_ENC: launch_mode<H, FP8, M_NODE_ENC>(a, s, rows_hint); break;
     case M_EDGE_ENC: launch_mode<H, FP8, M_EDGE_ENC>(a, s, rows_hint); break;
+    case M_TRIP:
+      if constexpr (!FP8) launch_mode<H, false, M_TRIP>(a, s, rows_hint);
+      break;
+    default: break;
+  }
+  // (hidden 128 has BF16 encoders and triplets only: its steps' tiles and weights
+  // exceed the shared memory)
+  if constexpr (FP8 || H <= 64) switch (mode) {
     case M_NODE_UPD: launch_mode<H, FP8, M_NODE_UPD>(a, s, rows_hint); break;
     case M_EDGE_UPD: launch_mode<H, FP8, M_EDGE_UPD>(a, s, rows_hint); break;
     case M_EDGE_UPD_CLS: launch_mode<H, FP8, M_EDGE_UPD_CLS>(a, s, rows_hint); break;
     case M_CLS: launch_mode<H, FP8, M_CLS>(a, s, rows_hint); break;
-    case M_TRIP:
-      if constexpr (!FP8) launch_mode<H, false, M_TRIP>(a, s, rows_hint);
-      break;
+    default: break;
   }
 }
 

@@ -487,3 +487,54 @@ def test_embedding_shapes_against_float64(embed, tracks):
     want = np.sum((a[g["src"]] - a[g["dst"]]) ** 2, axis=1)
     err = 2e-5 * np.abs(a).max()
     assert np.all(np.abs(g["d2"] - want) <= 2 * np.sqrt(embed[-1] * wl["radius2"]) * err + 1e-6 * want)
+
+
+@pytest.mark.parametrize("name,prec,tol", [
+    ("cfg3_batched_bf16", "bf16", 0.04), ("cfg2_run3_single", "bf16", 0.04),
+    ("cfg3_batched_bf16", "fp8", 0.4), ("cfg2_run3_single", "fp8", 0.4),
+    ("cfg4_batched_fp8", "fp8", 0.4)])
+@pytest.mark.parametrize("tracks", [1, 13, 300])
+def test_tensor_core_tiles_at_ragged_sizes(name, prec, tol, tracks):
+    """The tensor-core node, edge and triplet kernels at hidden 32, 64 and 128 on
+    an event of less than a tile of rows, of a ragged last tile and of more tiles
+    than fit the chip at once, alone and behind others (its rows then lie elsewhere
+    in their tiles): edge and triplet logits are the same bits, and close to FP32.
+    Bound: twice the mean logit error that the formats are held to on large events
+    (few rows scatter more); a wrong or misplaced row gives errors of order 1."""
+    wl = synth.workload(name)
+    sh = synth.shape_of(wl)
+    h = sh.hidden
+    rng = np.random.default_rng(5)
+    heads = []
+    for _ in range(2):
+        heads.append((rng.uniform(-0.2, 0.2, (h, 2 * h)).astype(np.float32),
+                      rng.uniform(-0.1, 0.1, h).astype(np.float32)))
+        heads.append((rng.uniform(-0.3, 0.3, (1, h)).astype(np.float32), np.zeros(1, np.float32)))
+    blob = synth.pack_weights(synth.weight_arrays(synth.workload_weights(wl)) + heads)
+    ev = [synth.gen_batch(1, 300 + i, {"kind": "fixed", "n": n}, wl["noise"])
+          for i, n in enumerate((tracks, 37, 5))]
+    alone, last = ev[0], synth.concat([ev[1], ev[2], ev[0]])
+
+    def one(b, precision):
+        cfg = pkg.make_cfg(wl["model"], wl["radius2"], k_max=wl["k_max"], max_hits=b.n_hits,
+                           max_events=b.n_events, precision=precision, edges_per_hit=32,
+                           triplets=True, triplets_per_hit=384)
+        tr = pkg.Tracker(blob, cfg)
+        pkg.run_batch_triplets(tr, b, tracks_per_hit=64, hits_per_hit=512)
+        e = b.n_events - 1
+        g, t = tr.get_graph(e), tr.get_triplets(e)
+        tr.close()
+        key = [(int(a), *map(int, hh)) for a, hh in zip(t["type"], t["hits"])]
+        return g, dict(zip(key, t["logit"].tolist()))
+
+    (g, t), (gb, tb), (g32, t32) = one(alone, prec), one(last, prec), one(alone, "fp32")
+    for k in g:
+        assert np.array_equal(g[k], gb[k]), k
+    assert t == tb
+    assert np.array_equal(g["src"], g32["src"]) and np.array_equal(g["dst"], g32["dst"])
+    if len(g["src"]):  # (a single track may leave no pair within the radius)
+        assert np.abs(g["logit"].astype(np.float64) - g32["logit"]).mean() < tol
+    both = sorted(set(t) & set(t32))
+    if both:
+        assert np.mean([abs(t[k] - t32[k]) for k in both]) < tol
+    assert tracks < 13 or (len(g["src"]) > 20 and len(both) > 20)
