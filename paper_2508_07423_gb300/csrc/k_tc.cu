@@ -8,7 +8,8 @@
 //      sum_in e], ...) come from global memory into the A tile in shared memory.
 //      BF16: by cp.async, four lanes per 64 bytes of a row, into blocks of 32
 //      columns in the 64-byte swizzle layout, during the tile before (see
-//      Layout::SWZ). FP8 and the three-pass forms: through registers into 8-row x
+//      Layout::SWZ). FP8 edge steps at hidden 128: by warpgroups of their own, see
+//      p3_loader. The others: through registers into 8-row x
 //      16-byte core matrices (K-major, no swizzle: row r, 16-byte chunk c at
 //      ((r/8) * (K/epc) + c) * 128 + (r%8) * 16);
 //   2. one thread issues the layer-1 MMAs (weights resident in shared memory,
@@ -106,14 +107,19 @@ struct Layout {
   // into the same tensor memory) against the K halves of the plain weight image,
   // so that two tiles fit beside the weights
   static constexpr bool SPLIT2 = SPLIT && MODE == M_EDGE_ENC && H > 64;
-  // FP8 edge steps at hidden 128 run layer 1 in three passes of K = H over a
-  // one-segment tile (e, then h_src, then h_dst) against the K chunks of the
+  // FP8 edge steps at hidden 128 run layer 1 in three passes of K = H over
+  // one-segment tiles (e, then h_src, then h_dst) against the K chunks of the
   // weight image; h_src and h_dst share one per-row scale and accumulate into
-  // one tensor-memory block (e into the other), so that the tiles (86 KB)
-  // and the accumulators (256 columns) of two CTAs fit an SM
+  // one tensor-memory block (e into the other), so that two tiles' accumulators
+  // (256 columns each) fill an SM. Two warpgroups work on a tile each; two more,
+  // the loaders, each load and quantise the rows of the next tile of one of them
+  // into a ring of P3_SLOTS one-segment tiles meanwhile. (One warpgroup doing both
+  // waited for its loads in each pass: 1.95 ms per launch on 5.2 M rows, 1.82 with
+  // loaders that copied four lanes to a row, 1.57 with half a warp to a row.)
   static constexpr bool P3 = FP8 && H == 128 && (MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS);
   // FP8 node step at hidden 128: the next tile's rows are loaded during a tile
   static constexpr bool NODE8 = FP8 && H == 128 && MODE == M_NODE_UPD;
+  static constexpr int P3_SLOTS = MODE == M_EDGE_UPD_CLS ? 2 : 3;
   static constexpr int K1 = (MODE == M_NODE_ENC) ? H : (SPLIT && !SPLIT2 ? 2 : 1) * NSEG * H;
   static constexpr int K2 = (SPLIT && MODE == M_NODE_ENC) ? 2 * H : H;
   static constexpr bool HAS_W1 = MODE != M_NODE_ENC;
@@ -140,19 +146,20 @@ struct Layout {
   // would leave room for one CTA per SM instead of two)
   static constexpr bool PREF = SWZ && (H == 32 || !SPLIT);
   // tiles in flight per CTA, each worked on by a warpgroup of its own with its
-  // own buffers and accumulators; they share the weights. Two in the edge encoder
+  // own buffers and accumulators; they share the weights. Two in the edge kernels
   // at hidden 128, whose weights leave room for one CTA per SM (the node step's
-  // three accumulators of 128 columns fill the tensor memory with one tile, the
-  // edge steps' two CTAs with two).
-  static constexpr int G = SPLIT2 ? 2 : 1;
+  // three accumulators of 128 columns fill the tensor memory with one tile).
+  static constexpr int G = SPLIT2 || P3 ? 2 : 1;
+  static constexpr int THREADS = kRows * (P3 ? 2 * G : G);
   static constexpr int A = align1k(WC + WC_BYTES);
-  static constexpr int A_BYTES = MODE == M_NODE_ENC ? 0 : kRows * (P3 || SPLIT2 ? H : K1) * ESZ;
+  static constexpr int A_BYTES =
+      MODE == M_NODE_ENC ? 0 : kRows * (P3 ? P3_SLOTS * H : (SPLIT2 ? H : K1)) * ESZ;
   // hidden / classifier input: its own tile or over the layer-1 input
-  static constexpr bool OWN_HA = MODE == M_NODE_ENC || (PREF && HAS_W2);
-  static constexpr int HA = OWN_HA ? align1k(A + A_BYTES) : A;
-  static constexpr int HA_BYTES = OWN_HA ? kRows * K2 * ESZ : 0;
-  static_assert(G == 1 || (HA_BYTES == 0 && A_BYTES % 1024 == 0), "one buffer per warpgroup");
-  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + HA_BYTES : A + G * A_BYTES);
+  static constexpr bool OWN_HA = MODE == M_NODE_ENC || (PREF && HAS_W2) || P3;
+  static constexpr int HA = OWN_HA ? align1k(A + G * A_BYTES) : A;
+  static constexpr int HA_BYTES = OWN_HA ? kRows * K2 * ESZ : 0;  // (per warpgroup)
+  static_assert(G == 1 || (HA_BYTES % 1024 == 0 && A_BYTES % 1024 == 0), "a buffer per warpgroup");
+  static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + G * HA_BYTES : A + G * A_BYTES);
   // fp32 parameters: b1, b2, bc1, s1, s2, sc, c2 weights, ne1 (3 x H + H)
   static constexpr int PAR_FLOATS = 7 * H + 4 * H + 8;
   static constexpr int BAR = PAR + PAR_FLOATS * 4;
@@ -161,8 +168,12 @@ struct Layout {
   static constexpr bool COOP = H == 128 && MODE != M_CLS && MODE != M_TRIP;
   // BF16 at hidden 32 and 64: out through the hidden tile, which is free by then
   static constexpr bool OUT_STAGE = !FP8 && H <= 64 && MODE != M_CLS && MODE != M_TRIP && MODE != M_EDGE_UPD_CLS;
-  static_assert(!(SWZ && (NODE8 || P3)) && !(OUT_STAGE && COOP), "one way in, one way out");
-  static constexpr int STAGE = BAR + 64;
+  static_assert(THREADS <= 512 && !(SWZ && (NODE8 || P3)) && !(OUT_STAGE && COOP), "one way in, one way out");
+  // P3: full and empty barriers of the rings, and the rows' two scales (of two
+  // tiles, by turns)
+  static constexpr int RING = BAR + 64;
+  static constexpr int SCALES = RING + (P3 ? 128 : 0);
+  static constexpr int STAGE = SCALES + (P3 ? G * 2 * kRows * 8 : 0);
   static constexpr int STAGE_ROW = 80;
   static constexpr int TOTAL = STAGE + (COOP ? G * kRows * STAGE_ROW : 0);
   // FP8: one accumulator block per layer-1 segment scale
@@ -297,6 +308,21 @@ __device__ __forceinline__ float amax_bf16(const uint4& v) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) m = fmaxf(m, fmaxf(fabsf(bf16_lo(q[j])), fabsf(bf16_hi(q[j]))));
   return m;
+}
+
+// the larger magnitudes of two pairs (a NaN gives way to the other, as in fmaxf)
+__device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  a &= 0x7fff7fffu;
+  b &= 0x7fff7fffu;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+// four BF16 values times f as E4M3 codes
+__device__ __forceinline__ uint32_t e4m3x4_of_bf16(uint32_t a, uint32_t b, float f) {
+  const float2 p = __fmul2_rn(make_float2(bf16_lo(a), bf16_hi(a)), make_float2(f, f));
+  const float2 q = __fmul2_rn(make_float2(bf16_lo(b), bf16_hi(b)), make_float2(f, f));
+  return pack_e4m3x4(p.x, p.y, q.x, q.y);
 }
 
 // The chunks of a warp's 32 BF16 rows, in registers between their load and
@@ -512,23 +538,21 @@ __device__ __forceinline__ void issue_blocks_bf16(uint32_t tmem, const uint8_t* 
              smem_desc(w0 + uint32_t(k * 2 / 16) * 128, 128, SBO_W), IDESC, k > 0 ? 1u : 0u);
 }
 
-// One pass of a three-pass FP8 layer 1 (K = 3H): the one-segment A tile
-// (E4M3, H per row) times K chunk `pass` of the weight image (E4M3, 3H per
-// row); pass 0 starts its accumulator, pass 1 starts the other, pass 2 adds
-// to it.
+// One pass of a three-pass FP8 layer 1 (K = 3H, H = 128): the one-segment A tile
+// (E4M3, 128 bytes per row, 128-byte swizzle) times K chunk `pass` of the weight
+// image (E4M3, 3H per row); pass 0 starts its accumulator, pass 1 starts the
+// other, pass 2 adds to it.
 template <int H>
 __device__ __forceinline__ void issue_pass_e4m3(uint32_t tmem, const uint8_t* A, const uint8_t* W,
                                                 int pass) {
+  static_assert(H == 128, "a row of one segment is one 128-byte swizzle row");
   constexpr uint32_t IDESC = idesc_e4m3(kRows, H);
-  constexpr uint32_t SBO_A = uint32_t(H / 16) * 128;
   constexpr uint32_t SBO_W = uint32_t(3 * H / 16) * 128;
   const uint32_t a0 = smem_u32(A), w0 = smem_u32(W) + uint32_t(pass * (H / 16)) * 128;
 #pragma unroll
-  for (int k = 0; k < H; k += 32) {
-    const uint32_t byte_k = uint32_t(k / 16) * 128;
-    mma_e4m3(tmem, smem_desc(a0 + byte_k, 128, SBO_A), smem_desc(w0 + byte_k, 128, SBO_W), IDESC,
+  for (int k = 0; k < H; k += 32)
+    mma_e4m3(tmem, smem_desc_sw128(a0 + uint32_t(k)), smem_desc(w0 + uint32_t(k / 16) * 128, 128, SBO_W), IDESC,
              (pass == 2 || k > 0) ? 1u : 0u);
-  }
 }
 
 // One pass of the split edge encoder's layer 1 at hidden 128 (K = 2H): the
@@ -622,13 +646,116 @@ __device__ __forceinline__ bool group_sync_or(int wg, bool v) {
   }
 }
 
+// The loaders of the FP8 edge steps at hidden 128: warpgroup `wg`'s tiles' rows,
+// quantised into its ring of one-segment tiles (128-byte swizzle). A warp fills its
+// own 32 rows of each in four steps of eight: half a warp copies a row, so that a
+// load reads whole lines and a store fills whole rows; the loads run a step ahead
+// (across segments and tiles: step 12 is the next tile's first). Rows that do not
+// exist repeat another (their results are not stored).
+// A wait that runs out ends the loader; the warpgroup's own wait then does too.
+template <int H, bool FP8, int MODE>
+__device__ __forceinline__ void p3_loader(const TcArgs& p, uint8_t* smem, int wg, int tid, int hi, int n_tiles) {
+  using L = Layout<H, FP8, MODE>;
+  const Ws& w = p.w;
+  const int lane = tid & 31, half = lane >> 4, piece = lane & 15, row0 = tid & ~31;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + L::RING) + wg * 2 * L::P3_SLOTS;
+  uint64_t* empty = full + L::P3_SLOTS;
+  float2* scales = reinterpret_cast<float2*>(smem + L::SCALES) + wg * 2 * kRows;
+  uint8_t* ring = smem + L::A + wg * L::A_BYTES;
+  const int step = int(gridDim.x) * L::G;
+  int slot = 0, uses = 0, turn = 0;
+  int t = int(blockIdx.x) * L::G + wg;
+  // the two hits of this lane's row of tile t
+  auto row_of = [&](int t) { return min(t * kRows + tid, hi - 1); };
+  if (t >= n_tiles) return;
+  int id_s = w.src[row_of(t)], id_d = w.col[row_of(t)];
+  float amax = fmaxf(w.hamax[id_s], w.hamax[id_d]);
+  uint4 v[2][4];
+  auto load_e = [&](uint4 (&v)[4], int t, int g) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      v[i] = reinterpret_cast<const uint4*>(
+          w.estate16 + size_t(min(t * kRows + row0 + 8 * g + 2 * i + half, hi - 1)) * H)[piece];
+  };
+  auto load_h = [&](uint4 (&v)[4], int id, int g) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      v[i] = reinterpret_cast<const uint4*>(
+          w.hstate16 + size_t(__shfl_sync(0xffffffffu, id, 8 * g + 2 * i + half)) * H)[piece];
+  };
+  // this lane's 8 bytes of rows 2 i + half of a step's eight
+  uint32_t at[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    at[i] = uint32_t((row0 + 2 * i + half) * H + (((piece >> 1) ^ (2 * i + half)) << 4) + (piece & 1) * 8);
+  load_e(v[0], t, 0);
+  for (; t < n_tiles; t += step) {
+    const int tn = min(t + step, n_tiles - 1);
+    const int nid_s = w.src[row_of(tn)], nid_d = w.col[row_of(tn)];
+    const float h_scale = amax > 0.f ? amax / 448.f : 1.f;
+    const float hinv = 1.f / h_scale;
+    scales[turn * kRows + tid].y = h_scale;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const int seg = k / 4, g = k % 4, n = k + 1;
+      if (n < 4)
+        load_e(v[n % 2], t, n);
+      else if (n < 12)
+        load_h(v[n % 2], n < 8 ? id_s : id_d, n % 4);
+      else
+        load_e(v[n % 2], tn, 0);
+      if (k == 6) amax = fmaxf(w.hamax[nid_s], w.hamax[nid_d]);  // (the next tile's)
+      if (g == 0) {  // (the slot's last MMA has read it)
+        const bool free = uses == 0 || mbar_wait_bounded(&empty[slot], uint32_t(uses - 1) & 1u, kWaitCycles);
+        if (!__all_sync(0xffffffffu, free)) return;
+      }
+      uint4 (&u)[4] = v[k % 2];
+      float iv = hinv;
+      if (seg == 0) {
+        // the rows' own scales: lane `piece` i of a half takes row i's maximum
+        float m = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          uint32_t q = max_abs_bf16x2(max_abs_bf16x2(u[i].x, u[i].y), max_abs_bf16x2(u[i].z, u[i].w));
+#pragma unroll
+          for (int d = 8; d > 0; d >>= 1) q = max_abs_bf16x2(q, __shfl_xor_sync(0xffffffffu, q, d));
+          if (piece == i) m = fmaxf(bf16_lo(q), bf16_hi(q));
+        }
+        iv = m > 0.f ? 448.f / m : 1.f;
+        if (piece < 4) scales[turn * kRows + row0 + 8 * g + 2 * piece + half].x = m > 0.f ? m / 448.f : 1.f;
+      }
+      uint8_t* rows = ring + slot * (kRows * H) + 8 * g * H;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float f = __shfl_sync(0xffffffffu, iv, seg == 0 ? 16 * half + i : 8 * g + 2 * i + half);
+        uint2 o;
+        o.x = e4m3x4_of_bf16(u[i].x, u[i].y, f);
+        o.y = e4m3x4_of_bf16(u[i].z, u[i].w, f);
+        *reinterpret_cast<uint2*>(rows + at[i]) = o;
+      }
+      if (g == 3) {
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full[slot]);
+        if (++slot == L::P3_SLOTS) {
+          slot = 0;
+          ++uses;
+        }
+      }
+    }
+    id_s = nid_s;
+    id_d = nid_d;
+    turn ^= 1;
+  }
+}
+
 // Tiles per SM that the registers must allow: BF16 at hidden 32 as many as the
 // shared memory holds (edge step on 10.1 M rows 356 us with four, 340 us with five;
 // the node encoder would spill).
 constexpr int min_ctas(int H, bool FP8, int MODE) { return !FP8 && H == 32 && MODE != M_NODE_ENC ? 5 : 1; }
 
 template <int H, bool FP8, int MODE>
-__global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H, FP8, MODE)) k_tc(const TcArgs p) {
+__global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, FP8, MODE)) k_tc(const TcArgs p) {
   using L = Layout<H, FP8, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sW1 = smem + L::W1;
@@ -647,6 +774,8 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + L::BAR + 48);
 
   constexpr int G = L::G;
+  uint64_t* ring_bar = reinterpret_cast<uint64_t*>(smem + L::RING);
+  (void)ring_bar;
   // warpgroup, row of its tile, warp of the warpgroup
   const int wg = G == 1 ? 0 : int(threadIdx.x) / kRows;
   const int tid = G == 1 ? int(threadIdx.x) : int(threadIdx.x) % kRows, warp = tid >> 5;
@@ -655,6 +784,8 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
   // ---- set-up: barriers, TMEM, weights --------------------------------------
   if (threadIdx.x == 0) {
     for (int i = 0; i < 1 + G; ++i) mbar_init(&bar[i], 1);
+    if constexpr (L::P3)  // full: a loader's four warps; empty: a commit
+      for (int i = 0; i < 2 * G * L::P3_SLOTS; ++i) mbar_init(&ring_bar[i], (i / L::P3_SLOTS) % 2 == 0 ? 4 : 1);
     fence_mbar_init();
   }
   if (threadIdx.x < 32) {
@@ -730,28 +861,19 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
     return true;
   };
 
-  // FP8 edge steps at hidden 128: the next tile's e rows, hits and h maxima are
-  // loaded during a tile (its indices when the tile begins, the rows before its
-  // epilogue), and the h rows of a pass during the MMAs of the pass before
   const int t_first = int(blockIdx.x) * G + wg;
-  CoopRows<L::P3 || L::SPLIT2 || L::NODE8 ? H : 64> pre;
+  CoopRows<L::SPLIT2 || L::NODE8 ? H : 64> pre;
   CoopRows<L::NODE8 ? H : 64> pre_m;  // NODE8: the 2H message codes of a hit
   float n_scale[2] = {1.f, 1.f};
   (void)pre_m;
   (void)n_scale;
   int nid_s = -1, nid_d = -1;
-  float n_amax = 0.f;
-  auto p3_ids = [&](int t) {
+  auto next_ids = [&](int t) {
     const int r = lo + t * kRows + tid;
     const bool in = t < n_tiles && r < hi;
     if constexpr (MODE == M_NODE_UPD || MODE == M_CLS) return;
     nid_s = in ? (MODE == M_TRIP ? p.t1 : w.src)[r] : -1;
     nid_d = in ? (MODE == M_TRIP ? p.t2 : w.col)[r] : -1;
-  };
-  auto p3_amax = [&] { n_amax = nid_s >= 0 ? fmaxf(w.hamax[nid_s], w.hamax[nid_d]) : 0.f; };
-  auto p3_rows = [&](int t) {
-    const int r = lo + t * kRows + tid;
-    pre.load(w.estate16, t < n_tiles && r < hi ? r : -1);
   };
   auto node8_rows = [&](int t) {
     const int r = lo + t * kRows + tid;
@@ -765,14 +887,23 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
   if constexpr (L::NODE8) node8_rows(t_first);
   // (the split edge encoder: the rows of a pass during the MMAs of the pass before)
   if constexpr (L::SPLIT2) {
-    p3_ids(t_first);
+    next_ids(t_first);
     pre.load(w.hstate16, nid_s);
   }
   if constexpr (L::P3) {
-    p3_ids(t_first);
-    p3_rows(t_first);
-    p3_amax();
+    // registers for the rows' passes, taken from the loaders
+    if (wg >= G) {
+      regs_lower<80>();
+      if (!aborted) p3_loader<H, FP8, MODE>(p, smem, wg - G, tid, hi, n_tiles);
+      __syncthreads();  // (the one before the clean-up)
+      return;
+    }
+    regs_raise<176>();
   }
+  int p3_slot = 0, p3_uses = 0, p3_turn = 0;
+  (void)p3_slot;
+  (void)p3_uses;
+  (void)p3_turn;
   // BF16: rows of tile t into the blocks (its ids loaded a tile ahead)
   auto gather = [&](int t) {
     if (t < n_tiles) gather_blocks<H, MODE>(smem + L::A, p, lo + t * kRows, hi, warp, nid_s, nid_d);
@@ -780,14 +911,14 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
   };
   (void)gather;
   if constexpr (L::SWZ) {
-    p3_ids(t_first);
+    next_ids(t_first);
     if constexpr (L::PREF) gather(t_first);
   }
   for (int t = t_first; t < n_tiles && !aborted; t += int(gridDim.x) * G) {
     const int r = lo + t * kRows + tid;
     const bool valid = r < hi;
     uint8_t* sA = smem + L::A + wg * L::A_BYTES;
-    uint8_t* sHA = L::HA == L::A ? sA : smem + L::HA;  // layer-2 input and classifier input
+    uint8_t* sHA = L::HA == L::A ? sA : smem + L::HA + wg * L::HA_BYTES;  // layer-2 input and classifier input
     float sa[3] = {1.f, 1.f, 1.f};  // FP8 per-row scales of the layer-1 segments
     int id_s = -1, id_d = -1;       // this row's source and target hit (hidden 128)
     (void)id_s;
@@ -801,7 +932,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
         group_sync<G>(wg);  // every thread is done with the buffer
         gather(t);
       }
-      p3_ids(t + int(gridDim.x));
+      next_ids(t + int(gridDim.x));
       cp_async_wait<0>();
     } else if constexpr (MODE == M_NODE_ENC) {
       // FP32 first layer (K = 3) in registers, then LayerNorm + ReLU into A
@@ -866,19 +997,12 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
         for (int k = 0; k < K1; k += 16) put_row_f32<FP8>(sA, tid, KCH1, k, z, 16, 1.f);
       }
     } else if constexpr (L::P3) {
-      // pass 0 holds e alone; h_src and h_dst follow in passes 1 and 2 with one
-      // scale, the larger of their two row maxima (the node kernels store each
-      // row's maximum as they write it)
-      id_s = nid_s;
-      id_d = nid_d;
-      sa[1] = n_amax > 0.f ? n_amax / 448.f : 1.f;
-      p3_ids(t + int(gridDim.x) * G);
-      sa[0] = pre.template put_e4m3<true>(sA, KCHA, 0, valid ? r : -1, 1.f);
+      // (the loaders)
     } else if constexpr (L::SPLIT2) {
       // pass 0: hi(h_src)
       id_s = nid_s;
       id_d = nid_d;
-      p3_ids(t + int(gridDim.x) * G);
+      next_ids(t + int(gridDim.x) * G);
       pre.put(sA, KCHA, 0, id_s);
     } else {
       // (FP8) edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
@@ -906,45 +1030,44 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
     float hid_scale = 1.f;  // FP8 per-row scale of the layer-2 input
     if constexpr (MODE != M_NODE_ENC) {
       // ---- 2. layer 1 ------------------------------------------------------
+      bool late = false;
       if (tid == 0) {
         tc_fence_after();
-        if constexpr (L::P3)
-          issue_pass_e4m3<H>(tmem_base, sA, sW1, 0);
-        else if constexpr (L::SPLIT2)
+        if constexpr (L::P3) {
+          // e, h_src, h_dst as the loaders fill their slots (after a wait that ran
+          // out: no commit, and wait_mma runs out too)
+          uint64_t* full = ring_bar + wg * 2 * L::P3_SLOTS;
+          bool filled = true;
+          for (int pass = 0; pass < 3 && filled; ++pass) {
+            const int sl = (p3_slot + pass) % L::P3_SLOTS;
+            const int use = p3_uses + (p3_slot + pass) / L::P3_SLOTS;
+            filled = mbar_wait_bounded(&full[sl], uint32_t(use) & 1u, kWaitCycles);
+            if (!filled) break;
+            issue_pass_e4m3<H>(tmem_base + uint32_t(pass > 0 ? H : 0), sA + sl * (kRows * H), sW1, pass);
+            mma_commit(&full[L::P3_SLOTS + sl]);
+          }
+          late = !filled;
+        } else if constexpr (L::SPLIT2)
           issue_pass_bf16<H>(tmem_base, sA, sW1, 0);
         else if constexpr (L::SWZ)
           issue_blocks_bf16<H, K1>(tmem_base, sA, sW1);
         else
           issue_layer<H, FP8>(tmem_base, sA, sW1, K1, FP8 ? L::NSEG : 1);
-        mma_commit(mma_bar);
+        if (!late) mma_commit(mma_bar);
       }
-      if constexpr (L::P3) pre.load(w.hstate16, id_s);
       if constexpr (L::SPLIT2) pre.load(w.hstate16, id_d);
       if (!wait_mma()) {
         aborted = true;
         break;
       }
       if constexpr (L::P3) {
-        // passes 1 and 2: h_src, then h_dst, into the same tile (the MMAs of
-        // the pass before have read it); invalid rows keep pass 0's zeros
-        const float hinv = 1.f / sa[1];
-        for (int pass = 1; pass <= 2 && !aborted; ++pass) {
-          pre.template put_e4m3<false>(sA, KCHA, 0, id_s, hinv);  // (id_s: whether the row exists)
-          fence_proxy_async();
-          tc_fence_before();
-          group_sync<G>(wg);
-          if (tid == 0) {
-            tc_fence_after();
-            issue_pass_e4m3<H>(tmem_base + uint32_t(H), sA, sW1, pass);
-            mma_commit(mma_bar);
-          }
-          if (pass == 1)
-            pre.load(w.hstate16, id_d);
-          else
-            p3_amax();
-          if (!wait_mma()) aborted = true;
-        }
-        if (aborted) break;
+        // (the barrier in wait_mma orders the loader's scales before these reads)
+        const float2 sc = reinterpret_cast<const float2*>(smem + L::SCALES)[(wg * 2 + p3_turn) * kRows + tid];
+        sa[0] = sc.x;
+        sa[1] = sc.y;
+        p3_turn ^= 1;
+        p3_uses += (p3_slot + 3) / L::P3_SLOTS;
+        p3_slot = (p3_slot + 3) % L::P3_SLOTS;
       }
       if constexpr (L::SPLIT2) {
         // hi(h_dst), lo(h_src), lo(h_dst) into the same tile, accumulated
@@ -1066,6 +1189,13 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
       hid_scale = sa[0];
     }
 
+    // hidden 128, BF16: the warp's state rows through its staging block
+    constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
+    const int row0 = r - (tid & 31);
+    RowStage<H, L::OUT_STAGE ? 64 : L::STAGE_ROW> st{
+        L::OUT_STAGE ? sHA + warp * 32 * L::K2 * 2 : smem + L::STAGE + (wg * kRows + warp * 32) * L::STAGE_ROW,
+        (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(row0) * H, min(max(hi - row0, 0), 32), {}};
+    (void)st;
     // ---- 4. layer 2 ----------------------------------------------------------
     if (tid == 0) {
       tc_fence_after();
@@ -1074,7 +1204,7 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
     }
     // (every thread has its residual and is past the barrier above)
     if constexpr (L::PREF) gather(t + int(gridDim.x));
-    if constexpr (L::P3) p3_rows(t + int(gridDim.x) * G);
+    if constexpr (L::P3) st.fetch(0);
     if constexpr (L::NODE8) node8_rows(t + int(gridDim.x) * G);
     if constexpr (L::SPLIT2) pre.load(w.hstate16, nid_s);
     if (!wait_mma()) {
@@ -1092,19 +1222,28 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
       }
       add_params<FP8>(v, pb2 + c * 32, ps2 + c * 32, z);
     };
-    // hidden 128, BF16: the warp's state rows through its staging block
-    constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
-    const int row0 = r - (tid & 31);
-    RowStage<H, L::OUT_STAGE ? 64 : L::STAGE_ROW> st{
-        L::OUT_STAGE ? sHA + warp * 32 * L::K2 * 2 : smem + L::STAGE + (wg * kRows + warp * 32) * L::STAGE_ROW,
-        (NODE_ROWS ? w.hstate16 : w.estate16) + size_t(row0) * H, min(max(hi - row0, 0), 32), {}};
-    (void)st;
+    // ZB chunks of 32 columns from chunk c on, their loads in flight together
+    constexpr int ZB = L::P3 ? 2 : 1;
+    auto zvals = [&](int c, float (*z)[32]) {
+#pragma unroll
+      for (int i = 0; i < ZB; ++i) tmem_ld32(tmem_lane + uint32_t((c + i) * 32), z[i]);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < ZB; ++i) {
+        if constexpr (FP8) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) z[i][j] *= hid_scale;
+        }
+        add_params<FP8>(z[i], pb2 + (c + i) * 32, ps2 + (c + i) * 32, z[i]);
+      }
+    };
+    (void)zvals;
     // residual input row (BF16) for the update modes
     auto resid = [&](int c, float (&z)[32]) {
       if constexpr (L::COOP && MODE == M_EDGE_UPD_CLS) {
         uint4 e[4];
-        st.fetch(c);
         st.rows(e);
+        if (c + 1 < H / 32) st.fetch(c + 1);
 #pragma unroll
         for (int q = 0; q < 4; ++q) add_bf16x8(z + 8 * q, e[q]);
       } else if constexpr (MODE == M_NODE_UPD || MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS) {
@@ -1143,11 +1282,12 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
         }
       } else if constexpr (L::COOP) {
         constexpr bool RESID = MODE == M_NODE_UPD || MODE == M_EDGE_UPD;
-        if constexpr (RESID) st.fetch(0);
+        if constexpr (RESID && !L::P3) st.fetch(0);
+        float zb[ZB][32];
 #pragma unroll
         for (int c = 0; c < H / 32; ++c) {
-          float z[32];
-          zval(c, z);
+          if (c % ZB == 0) zvals(c, zb);
+          float (&z)[32] = zb[c % ZB];
           if constexpr (RESID) {
             uint4 e[4];
             st.rows(e);
@@ -1192,10 +1332,11 @@ __global__ void __launch_bounds__((kRows * Layout<H, FP8, MODE>::G), min_ctas(H,
     } else {
       // ---- 5'. classifier on the new edge state, then the cut ---------------
       float zc[H / 32][32];  // the new state
+#pragma unroll
+      for (int c = 0; c < H / 32; c += ZB) zvals(c, zc + c);
       float emax = 0.f;
 #pragma unroll
       for (int c = 0; c < H / 32; ++c) {
-        zval(c, zc[c]);
         resid(c, zc[c]);
         if constexpr (FP8) {
 #pragma unroll
@@ -1669,9 +1810,6 @@ __device__ __forceinline__ bool ws_wait(uint64_t* m, uint32_t parity, volatile i
   }
   return true;
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* m) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(m)) : "memory");
-}
 
 template <bool CLS>
 __global__ void __launch_bounds__(kWsThreads, 2)
@@ -2024,7 +2162,7 @@ int tc_blocks_per_sm() {
                                cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     int n = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tc<H, FP8, MODE>, kRows * L::G, L::TOTAL);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tc<H, FP8, MODE>, L::THREADS, L::TOTAL);
     // the same bound from the kernel's resources: registers (allocated per warp
     // in units of 256), shared memory (228 KB per SM, 1 KB reserved per CTA),
     // 2048 threads per SM. CTAs never wait on one another, so a bound above
@@ -2033,7 +2171,7 @@ int tc_blocks_per_sm() {
     int est = 16;
     if (cudaFuncGetAttributes(&fa, k_tc<H, FP8, MODE>) == cudaSuccess && fa.numRegs > 0) {
       const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-      est = std::min(est, 65536 / (regs_warp * (L::G * kRows / 32)));
+      est = std::min(est, 65536 / (regs_warp * (L::THREADS / 32)));
     }
     est = std::min(est, 233472 / (L::TOTAL + 1024));
     if (e != cudaSuccess) cudaGetLastError();
@@ -2132,7 +2270,7 @@ void launch_mode(const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
   if (tuned > 0 && tuned < per_sm) per_sm = tuned;
   int grid = device_sms() * per_sm;
   grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRows * L::G - 1) / (kRows * L::G))));
-  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, kRows * L::G, L::TOTAL, s, 1, a);
+  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, L::THREADS, L::TOTAL, s, 1, a);
 }
 
 template <int H, bool FP8>
