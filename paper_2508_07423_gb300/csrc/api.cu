@@ -478,8 +478,7 @@ void enqueue_pipeline(gnntrk_handle* h, const Batch& b, const int64_t* offsets, 
     stage(h, "triplet_scores", s, 3, [&] {
       if (h->tc.has_trip) {
         // tensor cores: BF16 final edge encodings times BF16 first layers
-        tc_triplet_scores(b, w, h->tc, h->h, h->trip.art.l2, h->trip.elb.l2, h->trip.art.l1.b,
-                          h->trip.elb.l1.b, tcut, s);
+        tc_triplet_scores(b, w, h->tc, h->h, h->trip.art.l2, h->trip.elb.l2, tcut, s);
         launch_triplet_kept(w, s);
       } else {
         launch_triplet_scores_f32(b, w, h->trip, h->h, tcut, s);

@@ -70,6 +70,7 @@ struct LayerTC {
   const float* b;      // [out]
   const float* scale;  // [out], FP8 only (else nullptr)
   int in, out;
+  float hb[128], hs[128];  // b and scale on the host (kernel arguments)
 };
 
 struct Mlp2TC {

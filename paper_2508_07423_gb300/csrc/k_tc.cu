@@ -65,9 +65,6 @@ struct TcArgs {
   const float* b1;
   const float* b2;
   const float* bc1;
-  const float* s1;    // FP8 per-output-channel weight scales
-  const float* s2;
-  const float* sc;
   LayerF32 ne1;       // node encoder layer 1 (FP32, M_NODE_ENC)
   LayerF32 c2;        // classifier layer 2 (FP32, h -> 1)
   // M_TRIP: one triplet list (edge pairs, count on the device) and its outputs
@@ -78,6 +75,21 @@ struct TcArgs {
   uint8_t* tkeep;
   float fs[6];
   float cut;
+};
+
+// A launch's arguments, and the host copies of its layers' biases and scales
+struct TcCall : TcArgs {
+  const LayerTC *l1 = nullptr, *l2 = nullptr, *lc = nullptr;
+};
+
+// Biases and FP8 weight scales of a launch as kernel arguments: the epilogues read
+// them from the constant bank. (In shared memory each warp's 16-byte broadcast
+// loads of them took a third of the shared memory pipe's cycles: BF16 edge step at
+// hidden 32 on 10.1 M rows 340 -> 313 us, FP8 at 128 on 5.2 M 1.57 -> 1.48 ms.)
+template <int H, bool FP8>
+struct TcPar {
+  float b1[H], b2[H], bc[H];
+  float s1[FP8 ? H : 1], s2[FP8 ? H : 1], sc[FP8 ? H : 1];
 };
 
 __host__ __device__ constexpr int n_seg(int mode) {
@@ -160,8 +172,8 @@ struct Layout {
   static constexpr int HA_BYTES = OWN_HA ? kRows * K2 * ESZ : 0;  // (per warpgroup)
   static_assert(G == 1 || (HA_BYTES % 1024 == 0 && A_BYTES % 1024 == 0), "a buffer per warpgroup");
   static constexpr int PAR = align1k(HA_BYTES > 0 ? HA + G * HA_BYTES : A + G * A_BYTES);
-  // fp32 parameters: b1, b2, bc1, s1, s2, sc, c2 weights, ne1 (3 x H + H)
-  static constexpr int PAR_FLOATS = 7 * H + 4 * H + 8;
+  // fp32 parameters: c2 weights and bias, ne1 (3 x H + H)
+  static constexpr int PAR_FLOATS = 5 * H + 8;
   static constexpr int BAR = PAR + PAR_FLOATS * 4;
   // hidden 128: each warp's state rows pass through a staging block of 32 rows x
   // 64 bytes (80-byte stride) on their way in (residual) and out
@@ -465,26 +477,15 @@ __device__ __forceinline__ void add_bf16x8(float* acc, const uint4& u) {
 
 // x[j] = v[j] + b[j] (BF16) or fma(v[j], sc[j], b[j]) (FP8) for 32 columns,
 // the parameters read as 16-byte broadcasts from shared memory
-template <bool FP8>
-__device__ __forceinline__ void add_params(const float (&v)[32], const float* b, const float* sc,
-                                           float (&x)[32]) {
+__device__ __forceinline__ void add_params(const float (&v)[32], const float* b, float (&x)[32]) {
   const float4* b4 = reinterpret_cast<const float4*>(b);
-  const float4* s4 = reinterpret_cast<const float4*>(sc);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const float4 bb = b4[q];
-    if constexpr (FP8) {
-      const float4 ss = s4[q];
-      x[4 * q] = fmaf(v[4 * q], ss.x, bb.x);
-      x[4 * q + 1] = fmaf(v[4 * q + 1], ss.y, bb.y);
-      x[4 * q + 2] = fmaf(v[4 * q + 2], ss.z, bb.z);
-      x[4 * q + 3] = fmaf(v[4 * q + 3], ss.w, bb.w);
-    } else {
-      x[4 * q] = v[4 * q] + bb.x;
-      x[4 * q + 1] = v[4 * q + 1] + bb.y;
-      x[4 * q + 2] = v[4 * q + 2] + bb.z;
-      x[4 * q + 3] = v[4 * q + 3] + bb.w;
-    }
+    x[4 * q] = v[4 * q] + bb.x;
+    x[4 * q + 1] = v[4 * q + 1] + bb.y;
+    x[4 * q + 2] = v[4 * q + 2] + bb.z;
+    x[4 * q + 3] = v[4 * q + 3] + bb.w;
   }
 }
 
@@ -749,27 +750,33 @@ __device__ __forceinline__ void p3_loader(const TcArgs& p, uint8_t* smem, int wg
   }
 }
 
+// v (times the FP8 weight scale) plus the bias, columns 32 c .. 32 c + 31
+template <bool FP8, int N, int M>
+__device__ __forceinline__ void add_par(float (&v)[32], const float (&b)[N], const float (&sc)[M], int c) {
+#pragma unroll
+  for (int j = 0; j < 32; ++j) {
+    if constexpr (FP8)
+      v[j] = fmaf(v[j], sc[c * 32 + j], b[c * 32 + j]);
+    else
+      v[j] += b[c * 32 + j];
+  }
+}
+
 // Tiles per SM that the registers must allow: BF16 at hidden 32 as many as the
 // shared memory holds (edge step on 10.1 M rows 356 us with four, 340 us with five;
 // the node encoder would spill).
 constexpr int min_ctas(int H, bool FP8, int MODE) { return !FP8 && H == 32 && MODE != M_NODE_ENC ? 5 : 1; }
 
 template <int H, bool FP8, int MODE>
-__global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, FP8, MODE)) k_tc(const TcArgs p) {
+__global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, FP8, MODE)) k_tc(const TcArgs p, const __grid_constant__ TcPar<H, FP8> q) {
   using L = Layout<H, FP8, MODE>;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* sW1 = smem + L::W1;
   uint8_t* sW2 = smem + L::W2;
   uint8_t* sWC = smem + L::WC;
   float* par = reinterpret_cast<float*>(smem + L::PAR);
-  float* pb1 = par;
-  float* pb2 = par + H;
-  float* pbc = par + 2 * H;
-  float* ps1 = par + 3 * H;
-  float* ps2 = par + 4 * H;
-  float* psc = par + 5 * H;
-  float* pc2 = par + 6 * H;      // classifier layer 2 weights [H] + bias
-  float* pne = par + 7 * H + 4;  // node encoder layer 1: W[3][H], b[H]
+  float* pc2 = par;          // classifier layer 2 weights [H] + bias
+  float* pne = par + H + 4;  // node encoder layer 1: W[3][H], b[H]
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::BAR);  // [0] weights, [1 + wg] mma
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + L::BAR + 48);
 
@@ -793,14 +800,6 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
     tmem_relinquish();
   }
   for (int i = tid; i < H; i += kRows) {
-    pb1[i] = MODE == M_NODE_ENC ? p.ne1.b[i] : (MODE == M_CLS ? p.bc1[i] : p.b1[i]);
-    pb2[i] = (MODE == M_CLS || MODE == M_TRIP) ? 0.f : p.b2[i];
-    pbc[i] = (MODE == M_EDGE_UPD_CLS) ? p.bc1[i] : 0.f;
-    if constexpr (FP8) {
-      ps1[i] = MODE == M_NODE_ENC ? 1.f : (MODE == M_CLS ? p.sc[i] : p.s1[i]);
-      ps2[i] = (MODE == M_CLS || MODE == M_TRIP) ? 1.f : p.s2[i];
-      psc[i] = (MODE == M_EDGE_UPD_CLS) ? p.sc[i] : 1.f;
-    }
     if (MODE == M_EDGE_UPD_CLS || MODE == M_CLS || MODE == M_TRIP) pc2[i] = p.c2.WT[i * p.c2.ldo];
     if (MODE == M_NODE_ENC) {
       for (int j = 0; j < 3; ++j) pne[j * H + i] = p.ne1.WT[j * p.ne1.ldo + i];
@@ -1099,8 +1098,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       //         classifier output for M_CLS) -------------------------------
       // x[n] = s_w[n] * sum_seg s_a[seg] * acc_seg[n] + b[n]  (FP8)
       //      = acc[n] + b[n]                                   (BF16)
-      auto xval_ld = [&](int c, float (&x)[32]) {
-        float v[32];
+      auto xval_ld = [&](int c, float (&v)[32]) {
         tmem_ld32(tmem_lane + uint32_t(c * 32), v);
         if constexpr (FP8) {
 #pragma unroll
@@ -1114,7 +1112,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
           }
         }
         tmem_wait_ld();
-        add_params<FP8>(v, pb1 + c * 32, ps1 + c * 32, x);
+        add_par<FP8>(v, q.b1, q.s1, c);
       };
       // the row is read from tensor memory once and kept in registers (at h = 128
       // the three passes over it waited on tcgen05.ld each time: FP8 edge step on
@@ -1212,15 +1210,14 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       break;
     }
     // z[n] = s_w2[n] * s_h * acc[n] + b2[n] (FP8) or acc[n] + b2[n]
-    auto zval = [&](int c, float (&z)[32]) {
-      float v[32];
+    auto zval = [&](int c, float (&v)[32]) {
       tmem_ld32(tmem_lane + uint32_t(c * 32), v);
       tmem_wait_ld();
       if constexpr (FP8) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] *= hid_scale;
       }
-      add_params<FP8>(v, pb2 + c * 32, ps2 + c * 32, z);
+      add_par<FP8>(v, q.b2, q.s2, c);
     };
     // ZB chunks of 32 columns from chunk c on, their loads in flight together
     constexpr int ZB = L::P3 ? 2 : 1;
@@ -1234,7 +1231,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
 #pragma unroll
           for (int j = 0; j < 32; ++j) z[i][j] *= hid_scale;
         }
-        add_params<FP8>(z[i], pb2 + (c + i) * 32, ps2 + (c + i) * 32, z[i]);
+        add_par<FP8>(z[i], q.b2, q.s2, c + i);
       }
     };
     (void)zvals;
@@ -1365,15 +1362,14 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
         aborted = true;
         break;
       }
-      auto cval_ld = [&](int c, float (&x)[32]) {
-        float v[32];
+      auto cval_ld = [&](int c, float (&v)[32]) {
         tmem_ld32(tmem_lane + uint32_t(c * 32), v);
         tmem_wait_ld();
         if constexpr (FP8) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) v[j] *= es;
         }
-        add_params<FP8>(v, pbc + c * 32, psc + c * 32, x);
+        add_par<FP8>(v, q.bc, q.sc, c);
       };
       float cc[H / 32][32];
 #pragma unroll
@@ -1622,7 +1618,7 @@ __global__ void __launch_bounds__(kRows, 5)
       float v[32];
       tmem_ld32(tmem_lane, v);
       tmem_wait_ld();
-      add_params<false>(v, pb1, pb1, x);
+      add_params(v, pb1, x);
     }
     float sum = 0.f;
 #pragma unroll
@@ -1662,7 +1658,7 @@ __global__ void __launch_bounds__(kRows, 5)
       float v[32];
       tmem_ld32(tmem_lane, v);
       tmem_wait_ld();
-      add_params<false>(v, pb2, pb2, z);
+      add_params(v, pb2, z);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -1708,7 +1704,7 @@ __global__ void __launch_bounds__(kRows, 5)
         float v[32];
         tmem_ld32(tmem_lane, v);
         tmem_wait_ld();
-        add_params<false>(v, pbc, pbc, c);
+        add_params(v, pbc, c);
       }
       float cs = 0.f;
 #pragma unroll
@@ -1979,7 +1975,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
         float v[32];
         tmem_ld32(tmem_row, v);
         tmem_wait_ld();
-        add_params<false>(v, pb1, pb1, x);
+        add_params(v, pb1, x);
       }
       float sum = 0.f;
 #pragma unroll
@@ -2009,7 +2005,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
         float v[32];
         tmem_ld32(tmem_row, v);
         tmem_wait_ld();
-        add_params<false>(v, pb2, pb2, z);
+        add_params(v, pb2, z);
       }
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -2045,7 +2041,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
           float v[32];
           tmem_ld32(tmem_row, v);
           tmem_wait_ld();
-          add_params<false>(v, pbc, pbc, c);
+          add_params(v, pbc, c);
         }
         float cs = 0.f;
 #pragma unroll
@@ -2263,18 +2259,30 @@ void launch_edge_ws(const TcArgs& a, const TcModel& m, cudaStream_t s) {
 }
 
 template <int H, bool FP8, int MODE>
-void launch_mode(const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
+void launch_mode(const TcCall& a, cudaStream_t s, int64_t rows_hint) {
   using L = Layout<H, FP8, MODE>;
+  TcPar<H, FP8> q{};
+  const LayerTC* l1 = MODE == M_CLS ? a.lc : a.l1;
+  for (int i = 0; i < H; ++i) {
+    if (MODE != M_NODE_ENC) q.b1[i] = l1->hb[i];
+    if (L::HAS_W2) q.b2[i] = a.l2->hb[i];
+    if (L::HAS_WC) q.bc[i] = a.lc->hb[i];
+    if constexpr (FP8) {
+      if (MODE != M_NODE_ENC) q.s1[i] = l1->hs[i];
+      if (L::HAS_W2) q.s2[i] = a.l2->hs[i];
+      if (L::HAS_WC) q.sc[i] = a.lc->hs[i];
+    }
+  }
   int per_sm = tc_blocks_per_sm<H, FP8, MODE>();
   const int tuned = g_tuned[FP8 ? 1 : 0][hidx(H)][family_of(MODE)].load(std::memory_order_relaxed);
   if (tuned > 0 && tuned < per_sm) per_sm = tuned;
   int grid = device_sms() * per_sm;
   grid = int(std::max<int64_t>(1, std::min<int64_t>(grid, (rows_hint + kRows * L::G - 1) / (kRows * L::G))));
-  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, L::THREADS, L::TOTAL, s, 1, a);
+  launch_pdl(!FP8 && a.b.n_hits <= kEarlyTcHits, k_tc<H, FP8, MODE>, grid, L::THREADS, L::TOTAL, s, 1, static_cast<const TcArgs&>(a), q);
 }
 
 template <int H, bool FP8>
-void launch_h(int mode, const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
+void launch_h(int mode, const TcCall& a, cudaStream_t s, int64_t rows_hint) {
   switch (mode) {
     case M_NODE_ENC: launch_mode<H, FP8, M_NODE_ENC>(a, s, rows_hint); break;
     case M_EDGE_ENC: launch_mode<H, FP8, M_EDGE_ENC>(a, s, rows_hint); break;
@@ -2308,7 +2316,7 @@ constexpr int smem_total(int H, int mode) {
 #undef GNNTRK_LT
 }
 
-void launch_any(int H, bool fp8, int mode, const TcArgs& a, cudaStream_t s, int64_t rows_hint) {
+void launch_any(int H, bool fp8, int mode, const TcCall& a, cudaStream_t s, int64_t rows_hint) {
   if (fp8) {
     if (H == 32) launch_h<32, true>(mode, a, s, rows_hint);
     else if (H == 64) launch_h<64, true>(mode, a, s, rows_hint);
@@ -2457,7 +2465,7 @@ int tc_upload(TcModel& m, const HostLayer* L, int n_layers, int n_embed, int h, 
     }
   }
   std::vector<uint8_t> blob;
-  std::vector<size_t> off_img(items.size()), off_b(items.size()), off_s(items.size());
+  std::vector<size_t> off_img(items.size()), off_b(items.size()), off_s(items.size()), n_scales(items.size());
   auto align = [&](size_t a) { blob.resize((blob.size() + a - 1) / a * a, 0); };
   for (size_t i = 0; i < items.size(); ++i) {
     std::vector<uint8_t> img;
@@ -2485,6 +2493,7 @@ int tc_upload(TcModel& m, const HostLayer* L, int n_layers, int n_embed, int h, 
     std::memcpy(blob.data() + off_b[i], bb.data(), 4 * bb.size());
     align(16);
     off_s[i] = blob.size();
+    n_scales[i] = sc.size();
     blob.resize(blob.size() + 4 * sc.size());
     std::memcpy(blob.data() + off_s[i], sc.data(), 4 * sc.size());
   }
@@ -2505,7 +2514,9 @@ int tc_upload(TcModel& m, const HostLayer* L, int n_layers, int n_embed, int h, 
     const HostLayer& l = L[items[i].layer];
     *items[i].dst = LayerTC{base + off_img[i], reinterpret_cast<const float*>(base + off_b[i]),
                             reinterpret_cast<const float*>(base + off_s[i]),
-                            items[i].repeat_k ? 2 * l.in : l.in, l.out};
+                            items[i].repeat_k ? 2 * l.in : l.in, l.out, {}, {}};
+    std::memcpy(items[i].dst->hb, l.b.data(), 4 * l.b.size());
+    std::memcpy(items[i].dst->hs, blob.data() + off_s[i], 4 * n_scales[i]);
   }
   m.precision = precision;
   m.h = h;
@@ -2537,15 +2548,17 @@ int tc_upload_triplets(TcModel& m, const HostLayer& art1, const HostLayer& elb1,
   }
   *dmem = d;
   const uint8_t* base = static_cast<const uint8_t*>(d);
-  m.art1 = LayerTC{base, nullptr, nullptr, art1.in, art1.out};
-  m.elb1 = LayerTC{base + off_e, nullptr, nullptr, elb1.in, elb1.out};
+  m.art1 = LayerTC{base, nullptr, nullptr, art1.in, art1.out, {}, {}};
+  m.elb1 = LayerTC{base + off_e, nullptr, nullptr, elb1.in, elb1.out, {}, {}};
+  std::memcpy(m.art1.hb, art1.b.data(), 4 * art1.b.size());
+  std::memcpy(m.elb1.hb, elb1.b.data(), 4 * elb1.b.size());
   m.has_trip = true;
   return GNNTRK_OK;
 }
 
 namespace {
-TcArgs base_args(const Batch& b, const Ws& w, const GraphParams& g) {
-  TcArgs a{};
+TcCall base_args(const Batch& b, const Ws& w, const GraphParams& g) {
+  TcCall a{};
   a.b = b;
   a.w = w;
   for (int i = 0; i < 6; ++i) a.fs[i] = g.fs[i];
@@ -2562,12 +2575,12 @@ void tc_node_prep(const Batch& b, const Ws& w, const TcModel& m, const LayerF32*
   if (do_embed)
     launch_node_prep_f32(b, w, embed_f32, n_embed, Mlp2F32{}, EdgeProj{}, D, h, g, true, false,
                          all, s);
-  TcArgs a = base_args(b, w, g);
+  TcCall a = base_args(b, w, g);
   a.ne1 = ne1_f32;
   const Mlp2TC& ne = m.enc16 ? m.node_enc16 : m.node_enc;
   a.W2 = static_cast<const uint8_t*>(ne.l2.B);
   a.b2 = ne.l2.b;
-  a.s2 = ne.l2.scale;
+  a.l2 = &ne.l2;
   launch_any(h, m.precision == GNNTRK_FP8_E4M3 && !m.enc16, M_NODE_ENC, a, s, b.n_hits);
 }
 
@@ -2590,20 +2603,20 @@ int64_t tc_rows(int64_t n_hits) { return 2 * edge_rows_hint(n_hits); }
 void tc_gnn(const Batch& b, const Ws& w, const TcModel& m, int h, int K, const GraphParams& g,
             const LayerF32& cls2_f32, cudaStream_t s, int stage, bool store_final) {
   const bool fp8 = m.precision == GNNTRK_FP8_E4M3;
-  TcArgs a = base_args(b, w, g);
+  TcCall a = base_args(b, w, g);
   a.c2 = cls2_f32;
   a.Wc = static_cast<const uint8_t*>(m.cls.l1.B);
   a.bc1 = m.cls.l1.b;
-  a.sc = m.cls.l1.scale;
+  a.lc = &m.cls.l1;
   const bool fuse = !store_final &&
                     (fp8 ? smem_total<true>(h, M_EDGE_UPD_CLS) : smem_total<false>(h, M_EDGE_UPD_CLS)) <= kMaxSmem;
   auto set = [&](const Mlp2TC& mm) {
     a.W1 = static_cast<const uint8_t*>(mm.l1.B);
     a.b1 = mm.l1.b;
-    a.s1 = mm.l1.scale;
     a.W2 = static_cast<const uint8_t*>(mm.l2.B);
     a.b2 = mm.l2.b;
-    a.s2 = mm.l2.scale;
+    a.l1 = &mm.l1;
+    a.l2 = &mm.l2;
   };
   // stage < 0: everything; otherwise 0 = edge encoder, 1 + 2k = node step k,
   // 2 + 2k = edge step k (with the classifier at the last step)
@@ -2696,14 +2709,13 @@ int tc_get_ctas(int precision, int h, int family) {
 }
 
 void tc_triplet_scores(const Batch& b, const Ws& w, const TcModel& m, int h, const LayerF32& art2,
-                       const LayerF32& elb2, const float* art_b1, const float* elb_b1,
-                       float cut_logit, cudaStream_t s) {
+                       const LayerF32& elb2, float cut_logit, cudaStream_t s) {
   GraphParams g{};
   g.cut_logit = cut_logit;
-  TcArgs a = base_args(b, w, g);
+  TcCall a = base_args(b, w, g);
   // articulations
   a.W1 = static_cast<const uint8_t*>(m.art1.B);
-  a.b1 = art_b1;
+  a.l1 = &m.art1;
   a.c2 = art2;
   a.t1 = w.trip_a1;
   a.t2 = w.trip_a2;
@@ -2713,7 +2725,7 @@ void tc_triplet_scores(const Batch& b, const Ws& w, const TcModel& m, int h, con
   launch_any(h, false, M_TRIP, a, s, triplet_rows_hint(b.n_hits));
   // elbows
   a.W1 = static_cast<const uint8_t*>(m.elb1.B);
-  a.b1 = elb_b1;
+  a.l1 = &m.elb1;
   a.c2 = elb2;
   a.t1 = w.trip_e1;
   a.t2 = w.trip_e2;

@@ -54,8 +54,7 @@ int tc_upload_triplets(TcModel& m, const HostLayer& art1, const HostLayer& elb1,
 // layer (FP32) as a dot product; writes the logits and keep flags of both
 // triplet lists.
 void tc_triplet_scores(const Batch& b, const Ws& w, const TcModel& m, int h, const LayerF32& art2,
-                       const LayerF32& elb2, const float* art_b1, const float* elb_b1,
-                       float cut_logit, cudaStream_t s);
+                       const LayerF32& elb2, float cut_logit, cudaStream_t s);
 
 // FP32 embedding (its output feeds the radius test) and the node encoder
 // (FP32 K = 3 first layer, tensor-core second layer); writes w.emb and
