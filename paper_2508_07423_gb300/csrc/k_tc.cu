@@ -129,7 +129,9 @@ struct Layout {
   // waited for its loads in each pass: 1.95 ms per launch on 5.2 M rows, 1.82 with
   // loaders that copied four lanes to a row, 1.57 with half a warp to a row.)
   static constexpr bool P3 = FP8 && H == 128 && (MODE == M_EDGE_UPD || MODE == M_EDGE_UPD_CLS);
-  // FP8 node step at hidden 128: the next tile's rows are loaded during a tile
+  // FP8 node step at hidden 128: the next tile's rows are loaded during a tile, and
+  // the three segments' accumulators take turns in two blocks of tensor memory (the
+  // third starts once the first has been read), so that an SM works on two tiles
   static constexpr bool NODE8 = FP8 && H == 128 && MODE == M_NODE_UPD;
   static constexpr int P3_SLOTS = MODE == M_EDGE_UPD_CLS ? 2 : 3;
   static constexpr int K1 = (MODE == M_NODE_ENC) ? H : (SPLIT && !SPLIT2 ? 2 : 1) * NSEG * H;
@@ -158,10 +160,9 @@ struct Layout {
   // would leave room for one CTA per SM instead of two)
   static constexpr bool PREF = SWZ && (H == 32 || !SPLIT);
   // tiles in flight per CTA, each worked on by a warpgroup of its own with its
-  // own buffers and accumulators; they share the weights. Two in the edge kernels
-  // at hidden 128, whose weights leave room for one CTA per SM (the node step's
-  // three accumulators of 128 columns fill the tensor memory with one tile).
-  static constexpr int G = SPLIT2 || P3 ? 2 : 1;
+  // own buffers and accumulators; they share the weights. Two at hidden 128, where
+  // the weights leave room for one CTA per SM.
+  static constexpr int G = SPLIT2 || P3 || NODE8 ? 2 : 1;
   static constexpr int THREADS = kRows * (P3 ? 2 * G : G);
   static constexpr int A = align1k(WC + WC_BYTES);
   static constexpr int A_BYTES =
@@ -189,7 +190,7 @@ struct Layout {
   static constexpr int STAGE_ROW = 80;
   static constexpr int TOTAL = STAGE + (COOP ? G * kRows * STAGE_ROW : 0);
   // FP8: one accumulator block per layer-1 segment scale
-  static constexpr int TSEG = P3 ? 2 : (FP8 ? NSEG : 1);
+  static constexpr int TSEG = P3 || NODE8 ? 2 : (FP8 ? NSEG : 1);
   static constexpr int TMEM_COLS = pow2_cols(TSEG * H);
   static_assert(G * TMEM_COLS <= 512, "tensor memory of one SM");
 };
@@ -290,30 +291,6 @@ __device__ __forceinline__ void put_row_split(uint8_t* tile, int row, int kchunk
   }
 }
 
-// ---- cooperative row copies (hidden 128) -----------------------------------
-// A warp copies its 32 rows of a tile eight at a time: lane (r = lane & 7,
-// q = lane >> 3) takes chunk q, q + 4, ... of row r, so that the four lanes of a row
-// read 128 consecutive bytes (a thread copying a row of its own makes every
-// load instruction touch 32 lines, which bound these kernels on the L1 pipe)
-// and the eight lanes of a chunk store 128 consecutive bytes of the tile.
-// `id`: each lane's own row (lane l: row l of the warp), negative: zeros.
-
-// 32 consecutive bytes of global memory
-struct B32 {
-  uint4 a, b;
-};
-__device__ __forceinline__ B32 ld32(const void* p) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-  return B32{q[0], q[1]};
-}
-__device__ __forceinline__ uint4 e4m3_of_bf16(const B32& v, float inv) {
-  uint4 u;
-  u.x = pack_e4m3x4(bf16_lo(v.a.x) * inv, bf16_hi(v.a.x) * inv, bf16_lo(v.a.y) * inv, bf16_hi(v.a.y) * inv);
-  u.y = pack_e4m3x4(bf16_lo(v.a.z) * inv, bf16_hi(v.a.z) * inv, bf16_lo(v.a.w) * inv, bf16_hi(v.a.w) * inv);
-  u.z = pack_e4m3x4(bf16_lo(v.b.x) * inv, bf16_hi(v.b.x) * inv, bf16_lo(v.b.y) * inv, bf16_hi(v.b.y) * inv);
-  u.w = pack_e4m3x4(bf16_lo(v.b.z) * inv, bf16_hi(v.b.z) * inv, bf16_lo(v.b.w) * inv, bf16_hi(v.b.w) * inv);
-  return u;
-}
 __device__ __forceinline__ float amax_bf16(const uint4& v) {
   float m = 0.f;
   const uint32_t q[4] = {v.x, v.y, v.z, v.w};
@@ -337,68 +314,60 @@ __device__ __forceinline__ uint32_t e4m3x4_of_bf16(uint32_t a, uint32_t b, float
   return pack_e4m3x4(p.x, p.y, q.x, q.y);
 }
 
-// The chunks of a warp's 32 BF16 rows, in registers between their load and
-// their way into the tile (so that a load can be in flight during an MMA or
-// the epilogue).
-template <int H>
-struct CoopRows {
-  static constexpr int PER = H / 64;
-  B32 v[4][PER];
-  // (missing rows read row 0)
-  __device__ __forceinline__ void load(const __nv_bfloat16* src, int id) {
-    const int lane = threadIdx.x & 31, r = lane & 7, q = lane >> 3;
+// ---- row copies at hidden 128 -------------------------------------------------
+// A warp's 32 rows of 256 bytes (128 BF16 values, or two rows of 128 E4M3 codes),
+// in registers between their load and their way into a tile, so that a load can be
+// in flight during an MMA or the epilogue. Half a warp copies a row: a load reads
+// whole lines, and a store into 128-byte rows of the 128-byte swizzle fills whole
+// rows. (With a row per thread, or four lanes per row, every load touched 32 lines
+// and the kernels were bound by the shared memory pipe: edge encoder on 5.2 M rows
+// 1.52 -> 1.14 ms, node step on 0.87 M rows 0.41 -> 0.29 ms, the latter with the two
+// tiles per SM of Layout::NODE8.)
+// `id`: each lane's own row (lane l: row l of the warp); rows that do not exist read
+// another (their results are not stored).
+struct HalfRows {
+  static constexpr int kBlock = kRows * 128;  // bytes of a tile's block of 128-byte rows
+  uint4 v[16];
+  __device__ __forceinline__ void load(const void* src, int id) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const int row = __shfl_sync(0xffffffffu, id, 8 * g + r);
-#pragma unroll
-      for (int j = 0; j < PER; ++j)
-        v[g][j] = ld32(src + size_t(max(row, 0)) * H + 16 * (q + 4 * j));
+    for (int i = 0; i < 16; ++i) {
+      const int row = __shfl_sync(0xffffffffu, id, 2 * i + (lane >> 4));
+      v[i] = reinterpret_cast<const uint4*>(src)[size_t(max(row, 0)) * 16 + (lane & 15)];
     }
   }
-  // into a tile as they are, from chunk c0 on
-  __device__ __forceinline__ void put(uint8_t* tile, int kchunks, int c0, int id) {
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (kRows - 1)) >> 5;
-    const int r = lane & 7, q = lane >> 3;
+  // as they are: the rows' two halves of 128 bytes into two blocks
+  __device__ __forceinline__ void put(uint8_t* tile) const {
+    const int lane = threadIdx.x & 31, piece = lane & 15, warp = (threadIdx.x & (kRows - 1)) >> 5;
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const bool in = __shfl_sync(0xffffffffu, id, 8 * g + r) >= 0;
-#pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        const uint32_t at = tile_off(32 * warp + 8 * g + r, c0 + 2 * (q + 4 * j), kchunks);
-        *reinterpret_cast<uint4*>(tile + at) = in ? v[g][j].a : make_uint4(0, 0, 0, 0);
-        *reinterpret_cast<uint4*>(tile + at + 128) = in ? v[g][j].b : make_uint4(0, 0, 0, 0);
-      }
+    for (int i = 0; i < 16; ++i) {
+      const int row = 32 * warp + 2 * i + (lane >> 4);
+      *reinterpret_cast<uint4*>(tile + (piece >> 3) * kBlock + row * 128 + (((piece & 7) ^ (row & 7)) << 4)) = v[i];
     }
   }
-  // into an E4M3 tile at element k0 under one scale per row: the row's own
-  // maximum (OWN; the owner lane gets the scale) or each lane's `inv`
-  template <bool OWN>
-  __device__ __forceinline__ float put_e4m3(uint8_t* tile, int kchunks, int k0, int id, float inv) {
-    const int lane = threadIdx.x & 31, warp = (threadIdx.x & (kRows - 1)) >> 5;
-    const int r = lane & 7, q = lane >> 3;
-    float own = 1.f;
+  // as E4M3 codes under each row's own scale (the owner lane gets it)
+  __device__ __forceinline__ float put_e4m3(uint8_t* tile) const {
+    const int lane = threadIdx.x & 31, half = lane >> 4, piece = lane & 15;
+    const int warp = (threadIdx.x & (kRows - 1)) >> 5;
+    float m = 0.f;  // lane (half, piece): the maximum of row 2 piece + half
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const int row = __shfl_sync(0xffffffffu, id, 8 * g + r);
-      float iv;
-      if constexpr (OWN) {
-        float m = 0.f;
+    for (int i = 0; i < 16; ++i) {
+      uint32_t q = max_abs_bf16x2(max_abs_bf16x2(v[i].x, v[i].y), max_abs_bf16x2(v[i].z, v[i].w));
 #pragma unroll
-        for (int j = 0; j < PER; ++j) m = fmaxf(m, fmaxf(amax_bf16(v[g][j].a), amax_bf16(v[g][j].b)));
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-        iv = m > 0.f ? 448.f / m : 1.f;
-        const float mine = __shfl_sync(0xffffffffu, m, lane & 7);
-        if (q == g) own = mine > 0.f ? mine / 448.f : 1.f;
-      } else {
-        iv = __shfl_sync(0xffffffffu, inv, 8 * g + r);
-      }
-#pragma unroll
-      for (int j = 0; j < PER; ++j)
-        *reinterpret_cast<uint4*>(tile + tile_off(32 * warp + 8 * g + r, (k0 >> 4) + q + 4 * j, kchunks)) =
-            row >= 0 ? e4m3_of_bf16(v[g][j], iv) : make_uint4(0, 0, 0, 0);
+      for (int d = 8; d > 0; d >>= 1) q = max_abs_bf16x2(q, __shfl_xor_sync(0xffffffffu, q, d));
+      if (piece == i) m = fmaxf(bf16_lo(q), bf16_hi(q));
     }
-    return own;
+    const float iv = m > 0.f ? 448.f / m : 1.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float f = __shfl_sync(0xffffffffu, iv, 16 * half + i);
+      const int row = 32 * warp + 2 * i + half;
+      uint2 o;
+      o.x = e4m3x4_of_bf16(v[i].x, v[i].y, f);
+      o.y = e4m3x4_of_bf16(v[i].z, v[i].w, f);
+      *reinterpret_cast<uint2*>(tile + row * 128 + (((piece >> 1) ^ (row & 7)) << 4) + (piece & 1) * 8) = o;
+    }
+    return __shfl_sync(0xffffffffu, m > 0.f ? m / 448.f : 1.f, (lane & 1) * 16 + (lane >> 1));
   }
 };
 
@@ -541,11 +510,10 @@ __device__ __forceinline__ void issue_blocks_bf16(uint32_t tmem, const uint8_t* 
 
 // One pass of a three-pass FP8 layer 1 (K = 3H, H = 128): the one-segment A tile
 // (E4M3, 128 bytes per row, 128-byte swizzle) times K chunk `pass` of the weight
-// image (E4M3, 3H per row); pass 0 starts its accumulator, pass 1 starts the
-// other, pass 2 adds to it.
+// image (E4M3, 3H per row), starting its accumulator or adding to it.
 template <int H>
 __device__ __forceinline__ void issue_pass_e4m3(uint32_t tmem, const uint8_t* A, const uint8_t* W,
-                                                int pass) {
+                                                int pass, bool add) {
   static_assert(H == 128, "a row of one segment is one 128-byte swizzle row");
   constexpr uint32_t IDESC = idesc_e4m3(kRows, H);
   constexpr uint32_t SBO_W = uint32_t(3 * H / 16) * 128;
@@ -553,24 +521,23 @@ __device__ __forceinline__ void issue_pass_e4m3(uint32_t tmem, const uint8_t* A,
 #pragma unroll
   for (int k = 0; k < H; k += 32)
     mma_e4m3(tmem, smem_desc_sw128(a0 + uint32_t(k)), smem_desc(w0 + uint32_t(k / 16) * 128, 128, SBO_W), IDESC,
-             (pass == 2 || k > 0) ? 1u : 0u);
+             (add || k > 0) ? 1u : 0u);
 }
 
 // One pass of the split edge encoder's layer 1 at hidden 128 (K = 2H): the
-// one-segment BF16 A tile times K half pass % 2 of the weight image; pass 0
+// one-segment BF16 A tile (two blocks of 64 columns, 128-byte swizzle) times K half pass % 2 of the weight image; pass 0
 // starts the accumulator, the others add to it.
 template <int H>
 __device__ __forceinline__ void issue_pass_bf16(uint32_t tmem, const uint8_t* A, const uint8_t* W,
                                                 int pass) {
   constexpr uint32_t IDESC = idesc_bf16(kRows, H);
-  constexpr uint32_t SBO_A = uint32_t(H * 2 / 16) * 128;
   constexpr uint32_t SBO_W = uint32_t(2 * H * 2 / 16) * 128;
   const uint32_t a0 = smem_u32(A), w0 = smem_u32(W) + uint32_t((pass & 1) * (H * 2 / 16)) * 128;
 #pragma unroll
   for (int k = 0; k < H; k += 16) {
     const uint32_t byte_k = uint32_t(k * 2 / 16) * 128;
-    mma_bf16(tmem, smem_desc(a0 + byte_k, 128, SBO_A), smem_desc(w0 + byte_k, 128, SBO_W), IDESC,
-             (pass > 0 || k > 0) ? 1u : 0u);
+    mma_bf16(tmem, smem_desc_sw128(a0 + uint32_t((k / 64) * HalfRows::kBlock + (k % 64) * 2)),
+             smem_desc(w0 + byte_k, 128, SBO_W), IDESC, (pass > 0 || k > 0) ? 1u : 0u);
   }
 }
 
@@ -840,7 +807,6 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
   const int n_tiles = (hi - lo + kRows - 1) / kRows;
   constexpr int K1 = L::K1;
   constexpr int KCH1 = K1 * L::ESZ / 16;  // 16-byte chunks per A row, layer 1
-  constexpr int KCHA = L::P3 || L::SPLIT2 ? H * L::ESZ / 16 : KCH1;  // per row of the A tile
   constexpr int KCHH = H * L::ESZ / 16;   // 16-byte chunks per A row, K = H
   constexpr int KCH2 = L::K2 * L::ESZ / 16;  // 16-byte chunks per A row, layer 2
 
@@ -861,8 +827,8 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
   };
 
   const int t_first = int(blockIdx.x) * G + wg;
-  CoopRows<L::SPLIT2 || L::NODE8 ? H : 64> pre;
-  CoopRows<L::NODE8 ? H : 64> pre_m;  // NODE8: the 2H message codes of a hit
+  HalfRows pre, pre_m;  // (pre_m: the 2H message codes of a hit)
+  (void)pre;
   float n_scale[2] = {1.f, 1.f};
   (void)pre_m;
   (void)n_scale;
@@ -878,7 +844,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
     const int r = lo + t * kRows + tid;
     const bool in = t < n_tiles && r < hi;
     pre.load(w.hstate16, in ? r : -1);
-    pre_m.load(reinterpret_cast<const __nv_bfloat16*>(msg_codes<H>(w, 0)), in ? r : -1);
+    pre_m.load(msg_codes<H>(w, 0), in ? r : -1);
     const float2 sc = *reinterpret_cast<const float2*>(msg_scales<H>(w, in ? r : 0));
     n_scale[0] = in ? sc.x : 1.f;
     n_scale[1] = in ? sc.y : 1.f;
@@ -978,8 +944,8 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       // h under its own scale, the messages as the message kernel left them
       sa[1] = n_scale[0];
       sa[2] = n_scale[1];
-      sa[0] = pre.template put_e4m3<true>(sA, KCH1, 0, valid ? r : -1, 1.f);
-      pre_m.put(sA, KCH1, H / 16, valid ? r : -1);
+      sa[0] = pre.put_e4m3(sA);
+      pre_m.put(sA + HalfRows::kBlock);
     } else if constexpr (MODE == M_NODE_UPD) {
       // (FP8, hidden 32 and 64)
       if (valid) {
@@ -1002,7 +968,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       id_s = nid_s;
       id_d = nid_d;
       next_ids(t + int(gridDim.x) * G);
-      pre.put(sA, KCHA, 0, id_s);
+      pre.put(sA);
     } else {
       // (FP8) edge rows: [e], [h_src, h_dst], [e, h_src, h_dst]
       if (valid) {
@@ -1042,10 +1008,13 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
             const int use = p3_uses + (p3_slot + pass) / L::P3_SLOTS;
             filled = mbar_wait_bounded(&full[sl], uint32_t(use) & 1u, kWaitCycles);
             if (!filled) break;
-            issue_pass_e4m3<H>(tmem_base + uint32_t(pass > 0 ? H : 0), sA + sl * (kRows * H), sW1, pass);
+            issue_pass_e4m3<H>(tmem_base + uint32_t(pass > 0 ? H : 0), sA + sl * (kRows * H), sW1, pass, pass == 2);
             mma_commit(&full[L::P3_SLOTS + sl]);
           }
           late = !filled;
+        } else if constexpr (L::NODE8) {
+          issue_pass_e4m3<H>(tmem_base, sA, sW1, 0, false);
+          issue_pass_e4m3<H>(tmem_base + uint32_t(H), sA + HalfRows::kBlock, sW1, 1, false);
         } else if constexpr (L::SPLIT2)
           issue_pass_bf16<H>(tmem_base, sA, sW1, 0);
         else if constexpr (L::SWZ)
@@ -1071,7 +1040,7 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       if constexpr (L::SPLIT2) {
         // hi(h_dst), lo(h_src), lo(h_dst) into the same tile, accumulated
         for (int pass = 1; pass <= 3 && !aborted; ++pass) {
-          pre.put(sA, KCHA, 0, id_s);  // (id_s: whether the row exists)
+          pre.put(sA);
           fence_proxy_async();
           tc_fence_before();
           group_sync<G>(wg);
@@ -1118,8 +1087,37 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       // the three passes over it waited on tcgen05.ld each time: FP8 edge step on
       // 5.2 M rows 2.22 -> 1.95 ms, node step on 0.87 M rows 0.52 -> 0.42 ms)
       float xc[H / 32][32];
+      if constexpr (L::NODE8) {
+        auto add_block = [&](int block, float f, bool first) {
 #pragma unroll
-      for (int c = 0; c < H / 32; ++c) xval_ld(c, xc[c]);
+          for (int c = 0; c < H / 32; ++c) {
+            float u[32];
+            tmem_ld32(tmem_lane + uint32_t(block * H + c * 32), u);
+            tmem_wait_ld();
+#pragma unroll
+            for (int j = 0; j < 32; ++j) xc[c][j] = first ? u[j] * f : fmaf(u[j], f, xc[c][j]);
+          }
+        };
+        add_block(0, sa[0], true);
+        tc_fence_before();
+        group_sync<G>(wg);
+        if (tid == 0) {
+          tc_fence_after();
+          issue_pass_e4m3<H>(tmem_base, sA + 2 * HalfRows::kBlock, sW1, 2, false);
+          mma_commit(mma_bar);
+        }
+        add_block(1, sa[1], false);
+        if (!wait_mma()) {
+          aborted = true;
+          break;
+        }
+        add_block(0, sa[2], false);
+#pragma unroll
+        for (int c = 0; c < H / 32; ++c) add_par<FP8>(xc[c], q.b1, q.s1, c);
+      } else {
+#pragma unroll
+        for (int c = 0; c < H / 32; ++c) xval_ld(c, xc[c]);
+      }
       auto xval = [&](int c, float (&x)[32]) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) x[j] = xc[c][j];
