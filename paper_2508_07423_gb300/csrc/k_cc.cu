@@ -128,10 +128,11 @@ __global__ void k_na_label(const int32_t* scratch, int n, int32_t* labels) {
 // same hooking rule. An event with more than kCcSmemHits hits runs the same
 // steps on its slice of the global parent array.
 // ---------------------------------------------------------------------------
-constexpr int kCcThreads = 512;
 constexpr int kCcSmemHits = 6144;
 
-__global__ void __launch_bounds__(kCcThreads) k_cc_event(Batch b, Ws w) {
+template <int NT>
+__global__ void __launch_bounds__(NT) k_cc_event(Batch b, Ws w) {
+  constexpr int U = 4;
   extern __shared__ int32_t sm_cc[];
   int32_t* sP = sm_cc;                // [kCcSmemHits] parents (event-local input index)
   int32_t* sL = sm_cc + kCcSmemHits;  // [kCcSmemHits] local input index of sorted position
@@ -145,20 +146,32 @@ __global__ void __launch_bounds__(kCcThreads) k_cc_event(Batch b, Ws w) {
     const int e0 = min(w.row_ptr[v0], E), e1 = min(w.row_ptr[v1], E);
     const bool small = n <= kCcSmemHits;
     int32_t* P = small ? sP : w.parent + v0;  // local index -> parent
-    for (int i = threadIdx.x; i < n; i += kCcThreads) {
+    for (int i = threadIdx.x; i < n; i += NT) {
       P[i] = i;
       if (small) sL[i] = w.perm[v0 + i] - v0;
     }
     __syncthreads();
-    for (int e = e0 + threadIdx.x; e < e1; e += kCcThreads) {
-      if (!w.keep[e]) continue;
-      ++kept;
-      const int a = w.src[e] - v0, c = w.col[e] - v0;
-      uf_union(P, small ? sL[a] : w.perm[v0 + a] - v0, small ? sL[c] : w.perm[v0 + c] - v0,
-               w.counters);
+    for (int base = e0 + threadIdx.x; base < e1; base += U * NT) {
+      // (U edges' loads in flight together)
+      bool k[U];
+      int s[U], t[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = min(base + u * NT, e1 - 1);
+        k[u] = w.keep[e];
+        s[u] = w.src[e] - v0;
+        t[u] = w.col[e] - v0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (base + u * NT >= e1 || !k[u]) continue;
+        ++kept;
+        uf_union(P, small ? sL[s[u]] : w.perm[v0 + s[u]] - v0, small ? sL[t[u]] : w.perm[v0 + t[u]] - v0,
+                 w.counters);
+      }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += kCcThreads) {
+    for (int i = threadIdx.x; i < n; i += NT) {
       const int li = small ? sL[i] : w.perm[v0 + i] - v0;
       b.labels[v0 + li] = uf_find(P, li);
     }
@@ -198,20 +211,32 @@ static cudaError_t noalloc_scratch(cudaStream_t s, int32_t** out) {
   return cudaSuccess;
 }
 
+namespace {
+template <int NT>
+void cc_event(const Batch& b, const Ws& w, cudaStream_t s) {
+  // set once per process (thread-safe initialisation of a local static)
+  static const bool attr_set = [] {
+    cudaFuncSetAttribute(k_cc_event<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         2 * kCcSmemHits * int(sizeof(int32_t)));
+    return true;
+  }();
+  (void)attr_set;
+  launch_pdl(true, k_cc_event<NT>, std::min(b.n_events, device_sms() * 16), NT,
+             2 * kCcSmemHits * sizeof(int32_t), s, 1, b, w);
+}
+}  // namespace
+
 void launch_cc(const Batch& b, const Ws& w, cudaStream_t s) {
   if (b.n_events <= 0 || b.n_hits <= 0) {
     launch_pdl(true, k_cc_union, device_sms() * 8, 256, 0, s, 1, w);
     return;
   }
-  // set once per process (thread-safe initialisation of a local static)
-  static const bool attr_set = [] {
-    cudaFuncSetAttribute(k_cc_event, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         2 * kCcSmemHits * int(sizeof(int32_t)));
-    return true;
-  }();
-  (void)attr_set;
-  launch_pdl(true, k_cc_event, std::min(b.n_events, device_sms() * 16), kCcThreads,
-             2 * kCcSmemHits * sizeof(int32_t), s, 1, b, w);
+  // blocks twice as wide while all events still have one at once (an event of 16.7 k
+  // edges, alone: 77 us with 512 threads and one edge in flight per thread, 62 now)
+  if (b.n_events <= 2 * device_sms())
+    cc_event<1024>(b, w, s);
+  else
+    cc_event<512>(b, w, s);
 }
 
 }  // namespace gnntrk

@@ -80,8 +80,6 @@ __device__ __forceinline__ void rs_step_edge(const EvLevels& L, int ke, int a, i
 // counts up to and including it), so a block only waits for blocks that took
 // their tickets before it. Counts the band edges into counters[C_BAND] and the
 // events holding one into counters[C_RERUN].
-constexpr int kRsEvThreads = 512;
-constexpr int kRsEvWarps = kRsEvThreads / 32;
 constexpr int kRsLists = 2 * (kMaxIters + 1);
 constexpr int kRsLookbackSpins = 1 << 22;  // x >= 100 ns sleeps: about half a second
 constexpr int kRsSmemBytes = 96 * 1024;  // endpoints and levels: about 19 k edges per event
@@ -99,18 +97,20 @@ __device__ __forceinline__ int ld_vol(const int32_t* p) { return *(volatile cons
 // barrier inside their loops: warp q counts its segment's rows per list,
 // a block scan over the warps gives each warp its offset in every list, and
 // the warp then places its rows in order (ballot ranks).
+template <int NW>
 __device__ __forceinline__ void rs_segment(int r0, int r1, int warp, int& a, int& z) {
-  const int len = (((r1 - r0) + kRsEvWarps - 1) / kRsEvWarps + 31) / 32 * 32;
+  const int len = (((r1 - r0) + NW - 1) / NW + 31) / 32 * 32;
   a = min(r1, r0 + warp * len);
   z = min(r1, a + len);
 }
 
 // counts of this warp's rows per list t (t = 0 .. K) into wcnt[t][warp]
-__device__ void rs_count_warp(const int8_t* lev, int r0, int r1, int K, int (*wcnt)[kRsEvWarps]) {
+template <int NW>
+__device__ void rs_count_warp(const int8_t* lev, int r0, int r1, int K, int (*wcnt)[NW]) {
   // lev[r - r0]: the level of row r
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int a, z;
-  rs_segment(r0, r1, warp, a, z);
+  rs_segment<NW>(r0, r1, warp, a, z);
   int mine = 0;  // lane t holds the count of list t
   for (int c0 = a; c0 < z; c0 += 32) {
     const int r = c0 + lane;
@@ -124,12 +124,13 @@ __device__ void rs_count_warp(const int8_t* lev, int r0, int r1, int K, int (*wc
 }
 
 // this warp's rows into list t at run[t][warp] (t = 0 .. K), in index order
+template <int NW>
 __device__ void rs_place_warp(const int8_t* lev, int r0, int r1, int K, int32_t* list,
-                              int64_t stride, int (*run)[kRsEvWarps]) {
+                              int64_t stride, int (*run)[NW]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   int a, z;
-  rs_segment(r0, r1, warp, a, z);
+  rs_segment<NW>(r0, r1, warp, a, z);
   int mine = lane <= K ? run[lane][warp] : 0;  // lane t: next position in list t
   for (int c0 = a; c0 < z; c0 += 32) {
     const int r = c0 + lane;
@@ -194,13 +195,15 @@ __device__ void rs_lookback(const RsDesc& d, int ev, int nv, const int* cnt, int
   }
 }
 
-__global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc d, float lo,
+template <int NT>
+__global__ void __launch_bounds__(NT) k_rs_event(Batch b, Ws w, RsDesc d, float lo,
                                                           float hi, int K) {
+  constexpr int NW = NT / 32, U = 4;
   extern __shared__ __align__(16) int8_t sm_lev[];  // endpoints and levels of the event
   pdl_begin();
   if (input_bad(w.counters)) return;
-  __shared__ int wsum[kRsEvWarps];
-  __shared__ int wcnt[kRsLists][kRsEvWarps];  // per list and warp: rows, then offsets
+  __shared__ int wsum[NW];
+  __shared__ int wcnt[kRsLists][NW];  // per list and warp: rows, then offsets
   __shared__ int cnt_s[kRsLists];
   __shared__ int base_s[kRsLists];
   __shared__ int ticket_s;
@@ -226,19 +229,33 @@ __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc
     uint32_t* ep = reinterpret_cast<uint32_t*>(sm_lev);
     int8_t* lev0 = eps ? sm_lev + 4 * ne : sm_lev;
     const EvLevels L{staged ? lev0 + nh : w.rs_elev + e0, staged ? lev0 : w.rs_nlev + v0, e0, v0};
-    for (int i = tid; i < nh; i += kRsEvThreads) L.nl[i] = 0;
-    for (int e = tid; e < ne; e += kRsEvThreads) L.el[e] = 0;
+    for (int i = tid; i < nh; i += NT) L.nl[i] = 0;
+    for (int e = tid; e < ne; e += NT) L.el[e] = 0;
     __syncthreads();
     int n = 0;
-    for (int k = tid; k < ne; k += kRsEvThreads) {
-      const int a = w.src[e0 + k] - v0, c = w.col[e0 + k] - v0;
-      if (eps) ep[k] = uint32_t(a) | (uint32_t(c) << 16);
-      n += rs_init_edge(L, k, a, c, w.logit[e0 + k], lo, hi, top);
+    for (int k0 = tid; k0 < ne; k0 += U * NT) {
+      // (U edges' loads in flight together)
+      int a[U], c[U];
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = e0 + min(k0 + u * NT, ne - 1);
+        a[u] = w.src[e] - v0;
+        c[u] = w.col[e] - v0;
+        x[u] = w.logit[e];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int k = k0 + u * NT;
+        if (k >= ne) break;
+        if (eps) ep[k] = uint32_t(a[u]) | (uint32_t(c[u]) << 16);
+        n += rs_init_edge(L, k, a[u], c[u], x[u], lo, hi, top);
+      }
     }
     __syncthreads();
     for (int kk = K - 1; kk >= 0; --kk) {
       const int8_t ge_k = int8_t(kk + 2), km1 = int8_t(kk + 1);
-      for (int k = tid; k < ne; k += kRsEvThreads) {
+      for (int k = tid; k < ne; k += NT) {
         int a, c;
         if (eps) {
           const uint32_t u = ep[k];
@@ -257,17 +274,17 @@ __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc
     __syncthreads();
     if (tid == 0) {
       int t = 0;
-      for (int q = 0; q < kRsEvWarps; ++q) t += wsum[q];
+      for (int q = 0; q < NW; ++q) t += wsum[q];
       band_total += t;
       band_events += t > 0;
     }
     // the event's rows per list, their offsets, then placement
-    rs_count_warp(L.el, e0, e1, K, wcnt);
-    rs_count_warp(L.nl, v0, v1, K, wcnt + K + 1);
+    rs_count_warp<NW>(L.el, e0, e1, K, wcnt);
+    rs_count_warp<NW>(L.nl, v0, v1, K, wcnt + K + 1);
     __syncthreads();
     if (tid < nv) {  // exclusive scan over the warps, the event's count per list
       int run = 0;
-      for (int q = 0; q < kRsEvWarps; ++q) {
+      for (int q = 0; q < NW; ++q) {
         const int c = wcnt[tid][q];
         wcnt[tid][q] = run;
         run += c;
@@ -278,10 +295,10 @@ __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc
     if (warp == 0) rs_lookback(d, ev, nv, cnt_s, base_s, w.counters);
     __syncthreads();
     if (tid < nv)
-      for (int q = 0; q < kRsEvWarps; ++q) wcnt[tid][q] += base_s[tid];
+      for (int q = 0; q < NW; ++q) wcnt[tid][q] += base_s[tid];
     __syncthreads();
-    rs_place_warp(L.el, e0, e1, K, w.rs_elist, w.e_cap, wcnt);
-    rs_place_warp(L.nl, v0, v1, K, w.rs_nlist, w.h_cap, wcnt + K + 1);
+    rs_place_warp<NW>(L.el, e0, e1, K, w.rs_elist, w.e_cap, wcnt);
+    rs_place_warp<NW>(L.nl, v0, v1, K, w.rs_nlist, w.h_cap, wcnt + K + 1);
     if (ev == b.n_events - 1 && tid <= K) {
       // the totals of every list
       w.rs_counts[2 * NL + tid] = base_s[tid] + cnt_s[tid];
@@ -299,6 +316,18 @@ __global__ void __launch_bounds__(kRsEvThreads) k_rs_event(Batch b, Ws w, RsDesc
   }
 }
 
+template <int NT>
+void rs_event(const Batch& b, const Ws& w, const RsDesc& d, float lo, float hi, int K, cudaStream_t s) {
+  // set once per process (thread-safe initialisation of a local static)
+  static const bool attr = [] {
+    cudaFuncSetAttribute(k_rs_event<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemBytes);
+    return true;
+  }();
+  (void)attr;
+  launch_pdl(true, k_rs_event<NT>, std::min(b.n_events, device_sms() * 2), NT, kRsSmemBytes, s, 1, b, w, d, lo,
+             hi, K);
+}
+
 }  // namespace
 
 int launch_rescore_sets(const Batch& b, const Ws& w, float band_lo, float band_hi, int K,
@@ -306,14 +335,12 @@ int launch_rescore_sets(const Batch& b, const Ws& w, float band_lo, float band_h
   if (b.n_events <= 0) return 0;  // (k_sort clears the counts and the look-back flags)
   const int nv = 2 * (K + 1);
   const RsDesc d{w.rs_desc, w.rs_desc + b.n_events, w.rs_desc + b.n_events + size_t(b.n_events) * nv};
-  // set once per process (thread-safe initialisation of a local static)
-  static const bool attr = [] {
-    cudaFuncSetAttribute(k_rs_event, cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemBytes);
-    return true;
-  }();
-  (void)attr;
-  launch_pdl(true, k_rs_event, std::min(b.n_events, device_sms() * 2), kRsEvThreads, kRsSmemBytes, s, 1, b,
-             w, d, band_lo, band_hi, K);
+  // one event per SM at most: blocks twice as wide (an event of 16.7 k edges, alone:
+  // 92 us with 512 threads and one edge's loads in flight each, 72 now)
+  if (b.n_events <= device_sms())
+    rs_event<1024>(b, w, d, band_lo, band_hi, K, s);
+  else
+    rs_event<512>(b, w, d, band_lo, band_hi, K, s);
   return 1;
 }
 

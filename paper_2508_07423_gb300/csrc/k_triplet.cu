@@ -38,7 +38,6 @@ int device_sms();
 
 namespace {
 
-constexpr int kTbThreads = 256;
 constexpr int kUnionRetries = 1 << 20;
 constexpr int kPairSort = 1024;  // pairs sorted in shared memory (else in place, O(n^2))
 
@@ -72,10 +71,11 @@ __device__ __forceinline__ void tb_union(volatile int32_t* P, int a, int b, int3
   set_status(counters, ST_TIMEOUT);
 }
 
-// Inclusive scan of one int per thread over a kTbThreads block (warp shuffles,
-// then the warp totals); `sw` holds kTbThreads / 32 ints of shared scratch.
+// Inclusive scan of one int per thread over a block of NT threads (warp shuffles,
+// then the warp totals); `sw` holds NT / 32 ints of shared scratch.
 // Returns the thread's inclusive sum, the block total in `total`. Every thread
 // must call it (two barriers inside).
+template <int NT>
 __device__ __forceinline__ int block_scan(int v, int* sw, int& total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -87,7 +87,7 @@ __device__ __forceinline__ int block_scan(int v, int* sw, int& total) {
   __syncthreads();
   int off = 0, tot = 0;
 #pragma unroll
-  for (int k = 0; k < kTbThreads / 32; ++k) {
+  for (int k = 0; k < NT / 32; ++k) {
     const int t = sw[k];
     off += k < wid ? t : 0;
     tot += t;
@@ -190,11 +190,12 @@ __device__ __forceinline__ void for_hit_components(const Ws& w, const int32_t* C
 // ---- 4. track building, per event ------------------------------------------------
 // Phase 1: groups, links, components, component hit lists, pair list; counts
 // of tracks and track hits per event.
-__global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_tb_event(Batch b, Ws w) {
   __shared__ int s_np, s_nuniq, s_tracks, s_hits;
   __shared__ unsigned long long s_last;
   __shared__ unsigned long long s_pairs[kPairSort];
-  __shared__ int s_w[kTbThreads / 32];
+  __shared__ int s_w[NT / 32];
   pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
   const int tid = threadIdx.x;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
       s_tracks = 0;
       s_hits = 0;
     }
-    for (int e = E0 + tid; e < E1; e += kTbThreads) {
+    for (int e = E0 + tid; e < E1; e += NT) {
       P[e] = e;
       P2[e] = e;
       w.tb_out[e] = -1;
@@ -220,21 +221,21 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     }
     __syncthreads();
     // 1. kept elbows join their two edges
-    for (int t = L0 + tid; t < L1; t += kTbThreads)
+    for (int t = L0 + tid; t < L1; t += NT)
       if (w.trip_ekeep[t]) tb_union(P, w.trip_e1[t], w.trip_e2[t], w.counters);
     __syncthreads();
     // compress in two passes: a find's path halving may still move a pointer
     // that another thread has just set to its root, so the roots are found
     // first (into tb_cur) and stored after every find has finished
-    for (int e = E0 + tid; e < E1; e += kTbThreads)
+    for (int e = E0 + tid; e < E1; e += NT)
       if (w.keep[e]) w.tb_cur[e] = tb_find(P, e);
     __syncthreads();
-    for (int e = E0 + tid; e < E1; e += kTbThreads)
+    for (int e = E0 + tid; e < E1; e += NT)
       if (w.keep[e]) P[e] = w.tb_cur[e];
     __syncthreads();
     // 2. articulation links: first partner per group and direction; a second,
     //    different partner marks the group (bit 0 onwards, bit 1 backwards)
-    for (int t = A0 + tid; t < A1; t += kTbThreads) {
+    for (int t = A0 + tid; t < A1; t += NT) {
       if (!w.trip_akeep[t]) continue;
       const int ga = P[w.trip_a1[t]], gb = P[w.trip_a2[t]];
       if (ga == gb) continue;
@@ -244,7 +245,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
       if (i != -1 && i != ga) atomicOr(&w.tb_flag[gb], 2);
     }
     __syncthreads();
-    for (int t = A0 + tid; t < A1; t += kTbThreads) {
+    for (int t = A0 + tid; t < A1; t += NT) {
       if (!w.trip_akeep[t]) continue;
       const int ga = P[w.trip_a1[t]], gb = P[w.trip_a2[t]];
       if (ga == gb) continue;
@@ -252,14 +253,14 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     }
     __syncthreads();
     // component of every group root (two passes, as above)
-    for (int e = E0 + tid; e < E1; e += kTbThreads)
+    for (int e = E0 + tid; e < E1; e += NT)
       if (w.keep[e] && P[e] == e) w.tb_off[e] = tb_find(P2, e);
     __syncthreads();
-    for (int e = E0 + tid; e < E1; e += kTbThreads)
+    for (int e = E0 + tid; e < E1; e += NT)
       if (w.keep[e] && P[e] == e) P2[e] = w.tb_off[e];
     __syncthreads();
     // 3. shared links -> component pairs (X << 32 | Y), X != Y
-    for (int t = A0 + tid; t < A1; t += kTbThreads) {
+    for (int t = A0 + tid; t < A1; t += NT) {
       if (!w.trip_akeep[t]) continue;
       const int ga = P[w.trip_a1[t]], gb = P[w.trip_a2[t]];
       if (ga == gb || (!(w.tb_flag[ga] & 1) && !(w.tb_flag[gb] & 2))) continue;
@@ -277,11 +278,11 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
       // bitonic sort in shared memory (padded with the maximum key)
       int m = 1;
       while (m < np) m <<= 1;
-      for (int i = tid; i < m; i += kTbThreads) s_pairs[i] = i < np ? pairs[i] : ~0ull;
+      for (int i = tid; i < m; i += NT) s_pairs[i] = i < np ? pairs[i] : ~0ull;
       __syncthreads();
       for (int k = 2; k <= m; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-          for (int i = tid; i < m; i += kTbThreads) {
+          for (int i = tid; i < m; i += NT) {
             const int l = i ^ j;
             if (l > i) {
               const unsigned long long a = s_pairs[i], c = s_pairs[l];
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
           }
           __syncthreads();
         }
-      for (int i = tid; i < np; i += kTbThreads) pairs[i] = s_pairs[i];
+      for (int i = tid; i < np; i += NT) pairs[i] = s_pairs[i];
       __syncthreads();
     } else if (tid == 0) {
       // rare: more shared links than the shared-memory sort holds
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     // compact the distinct pairs to the front (block scan of first-occurrence flags)
     {
       int nu = 0;
-      for (int base = 0; base < np; base += kTbThreads) {
+      for (int base = 0; base < np; base += NT) {
         const int i = base + tid;
         const unsigned long long v = i < np ? pairs[i] : 0ull;
         // the previous entry as it was before this pass compacted anything:
@@ -321,8 +322,8 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
             tid > 0 ? (i < np ? pairs[i - 1] : 0ull) : (base > 0 ? s_last : ~v);
         const bool f = i < np && (i == 0 || v != prev);
         int tot;
-        const int inc = block_scan(f ? 1 : 0, s_w, tot);
-        if (tid == kTbThreads - 1 || i == np - 1) s_last = v;
+        const int inc = block_scan<NT>(f ? 1 : 0, s_w, tot);
+        if (tid == NT - 1 || i == np - 1) s_last = v;
         // every thread read its entries before the scan's barriers; a write
         // goes to slot nu + inc - 1 <= i
         if (f) pairs[nu + inc - 1] = v;
@@ -337,20 +338,20 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     //    edge first (-1 if not kept; tb_in is free again), so a hit reads
     //    one value per incident edge.
     int32_t* CE = w.tb_in;
-    for (int e = E0 + tid; e < E1; e += kTbThreads) CE[e] = w.keep[e] ? P2[P[e]] : -1;
+    for (int e = E0 + tid; e < E1; e += NT) CE[e] = w.keep[e] ? P2[P[e]] : -1;
     __syncthreads();
-    for (int v = h0 + tid; v < h1; v += kTbThreads)
+    for (int v = h0 + tid; v < h1; v += NT)
       for_hit_components(w, CE, v, [&](int X) { atomicAdd(&w.tb_cnt[X], 1); });
     __syncthreads();
     // offsets of the component hit lists (block scan over the event's edges),
     // and counts of the plain tracks
     {
       int run = 0;
-      for (int base = E0; base < E1; base += kTbThreads) {
+      for (int base = E0; base < E1; base += NT) {
         const int e = base + tid;
         const int c = (e < E1 && w.keep[e] && P[e] == e && P2[e] == e) ? w.tb_cnt[e] : 0;
         int tot;
-        const int inc = block_scan(c, s_w, tot);
+        const int inc = block_scan<NT>(c, s_w, tot);
         if (c > 0) {
           w.tb_off[e] = 2 * E0 + run + inc - c;
           w.tb_cur[e] = 0;
@@ -364,12 +365,12 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     }
     __syncthreads();
     // place the hits (sorted positions), then sort each list
-    for (int v = h0 + tid; v < h1; v += kTbThreads)
+    for (int v = h0 + tid; v < h1; v += NT)
       for_hit_components(w, CE, v, [&](int X) {
         w.tb_hits[w.tb_off[X] + atomicAdd(&w.tb_cur[X], 1)] = v;
       });
     __syncthreads();
-    for (int e = E0 + tid; e < E1; e += kTbThreads) {
+    for (int e = E0 + tid; e < E1; e += NT) {
       if (!(w.keep[e] && P[e] == e && P2[e] == e)) continue;
       int32_t* L = w.tb_hits + w.tb_off[e];
       const int n = w.tb_cnt[e];
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
     }
     __syncthreads();
     // pair tracks: size of the union of the two sorted lists
-    for (int k = tid; k < s_nuniq; k += kTbThreads) {
+    for (int k = tid; k < s_nuniq; k += NT) {
       const int X = int(pairs[k] >> 32), Y = int(pairs[k] & 0xffffffffu);
       const int32_t *a = w.tb_hits + w.tb_off[X], *c = w.tb_hits + w.tb_off[Y];
       const int na = w.tb_cnt[X], nc = w.tb_cnt[Y];
@@ -410,10 +411,11 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_event(Batch b, Ws w) {
 }
 
 // Phase 2: write the tracks at the scanned offsets (capacity-checked).
-__global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const int32_t* ev_tracks,
+template <int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_tb_write(Batch b, Ws w, const int32_t* ev_tracks,
                                                           int64_t* track_off, int32_t* track_hits,
                                                           int64_t max_tracks, int64_t max_hits) {
-  __shared__ int s_w[kTbThreads / 32];
+  __shared__ int s_w[NT / 32];
   __shared__ int s_t, s_h;
   pdl_begin();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & (ST_INPUT | ST_CAPACITY)) return;
@@ -439,13 +441,13 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
     }
     __syncthreads();
     // plain components in ascending root order: ranks by a block scan
-    for (int base = E0; base < E1; base += kTbThreads) {
+    for (int base = E0; base < E1; base += NT) {
       const int e = base + tid;
       const bool f = e < E1 && w.keep[e] && P[e] == e && P2[e] == e && !(w.tb_flag[e] & 4);
       const int c = f ? w.tb_cnt[e] : 0;
       int last, last2;
-      const int inc = block_scan(f ? 1 : 0, s_w, last);
-      const int inc2 = block_scan(c, s_w, last2);
+      const int inc = block_scan<NT>(f ? 1 : 0, s_w, last);
+      const int inc2 = block_scan<NT>(c, s_w, last2);
       if (f) {
         const int t = s_t + inc - 1;
         const int64_t o = s_h + inc2 - c;
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
     }
     // component pairs: sizes again (union of two sorted lists), then a scan
     const int nu = w.tb_ev_pairs[ev];
-    for (int base = 0; base < nu; base += kTbThreads) {
+    for (int base = 0; base < nu; base += NT) {
       const int k = base + tid;
       int u = 0, X = 0, Y = 0;
       if (k < nu) {
@@ -479,7 +481,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
         }
       }
       int last;
-      const int inc = block_scan(u, s_w, last);
+      const int inc = block_scan<NT>(u, s_w, last);
       if (k < nu) {
         const int t = s_t + k - base;
         const int64_t o = s_h + inc - u;
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(kTbThreads) k_tb_write(Batch b, Ws w, const in
       }
       __syncthreads();
       if (tid == 0) {
-        s_t += min(kTbThreads, nu - base);
+        s_t += min(NT, nu - base);
         s_h += last;
       }
       __syncthreads();
@@ -536,16 +538,34 @@ void launch_triplet_kept(const Ws& w, cudaStream_t s) {
              w.trip_ekeep, w.counters + C_TRIP_E, w.counters);
 }
 
-void launch_track_build(const Batch& b, const Ws& w, const TrackOut& out, cudaStream_t s) {
-  if (b.n_events <= 0) return;
-  const int grid = std::min(b.n_events, device_sms() * 8);
-  launch_pdl(false, k_tb_event, grid, kTbThreads, 0, s, 1, b, w);
+namespace {
+template <int NT>
+void track_build(const Batch& b, const Ws& w, const TrackOut& out, cudaStream_t s) {
+  const int grid = std::min(b.n_events, device_sms() * (2048 / NT));
+  launch_pdl(false, k_tb_event<NT>, grid, NT, 0, s, 1, b, w);
   launch_scan(w.tb_ev_tracks, out.ev_tracks, b.n_events, 1 << 30, w.counters, C_TRACKS,
               int64_t(1) << 40, w.scan_blocks, s);
   launch_scan(w.tb_ev_hits, w.tb_ev_hit_off, b.n_events, 1 << 30, w.counters, C_TRACK_HITS,
               int64_t(1) << 40, w.scan_blocks, s);
-  launch_pdl(false, k_tb_write, grid, kTbThreads, 0, s, 1, b, w, out.ev_tracks, out.track_off,
+  launch_pdl(false, k_tb_write<NT>, grid, NT, 0, s, 1, b, w, out.ev_tracks, out.track_off,
              out.track_hits, out.max_tracks, out.max_hits);
+}
+}  // namespace
+
+void launch_track_build(const Batch& b, const Ws& w, const TrackOut& out, cudaStream_t s) {
+  if (b.n_events <= 0) return;
+  // A block walks its event in some twenty passes of loads that depend on one
+  // another, so the wider the block the fewer rounds each pass takes, as long as
+  // every event has a block at once. us for 8 / 60 / 140 / 300 / 500 / 900 events of
+  // 1.8 k hits: 256 threads 344 / 353 / 372 / 454 / 495 / 610, 512 threads 232 / 248
+  // / 265 / 328 / 364 / 659, 1024 threads 191 / 209 / 235 / 309 / 524 / 799.
+  const int64_t fit = int64_t(device_sms()) * 2048 / b.n_events;
+  if (fit >= 1024)
+    track_build<1024>(b, w, out, s);
+  else if (fit >= 512)
+    track_build<512>(b, w, out, s);
+  else
+    track_build<256>(b, w, out, s);
 }
 
 }  // namespace gnntrk

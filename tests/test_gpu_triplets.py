@@ -236,3 +236,31 @@ def test_triplet_workspace_capacity_latches_and_recovers(cfg6):
     # a call that fits works afterwards
     small = synth.gen_batch(1, 5, {"kind": "fixed", "n": 3}, 0.0)
     pkg.run_batch_triplets(tr, small)
+
+
+@pytest.mark.parametrize("per_sm,extra", [(1, 0), (1, 1), (2, 0), (2, 1), (4, 0), (4, 1)])
+def test_event_blocks_at_their_widths(cfg6, per_sm, extra):
+    """The components, receptive-field and track kernels take wider blocks the
+    fewer events there are (the widths change after 1, 2 and 4 events per SM):
+    at each change, sampled events get the graph, labels, triplets and tracks
+    that they get alone, to the bit."""
+    wl, _ = cfg6
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    b = synth.concat([synth.gen_batch(1, 40, {"kind": "fixed", "n": (i * 7) % 11 + (60 if i == 3 else 0)},
+                                      0.05, first_event=i) for i in range(n)])
+    tr = pkg.tracker_for_workload(wl, max_hits=b.n_hits, max_events=n)
+    assert tr.cfg.rescore_band > 0
+    sample = (0, 3, n // 2, n - 1)
+
+    def one(batch, events):
+        labels, tracks = pkg.run_batch_triplets(tr, batch)
+        return [(labels[batch.offsets[e]:batch.offsets[e + 1]], [t.tolist() for t in tracks[e]],
+                 tr.get_graph(e), tr.get_triplets(e)) for e in events]
+
+    for e, got in zip(sample, one(b, sample)):
+        (want,) = one(b.event(e), (0,))
+        assert np.array_equal(got[0], want[0]) and got[1] == want[1], e
+        for k in (2, 3):
+            for key in want[k]:
+                assert np.array_equal(got[k][key], want[k][key]), (e, key)
+    tr.close()
