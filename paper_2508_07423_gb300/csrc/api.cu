@@ -1005,7 +1005,7 @@ gnntrk_status gnntrk_autotune(gnntrk_handle* h, int32_t n_events, int64_t n_hits
       tc_set_ctas(prec, hd, f, best_n[f]);
       if (choice) choice[f] = best_n[f];
     }
-    // BF16 edge step at hidden 32: per-thread row copies or TMA (choice[7])
+    // BF16 edge step at hidden 32: cp.async row copies or TMA (choice[7])
     if (!st && prec == GNNTRK_BF16 && h->tc.maps) {
       double best = 1e30;
       int best_form = 0;

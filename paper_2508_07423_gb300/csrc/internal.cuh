@@ -93,9 +93,12 @@ struct Ws {
   int32_t* in_cnt;      // [H] CSR offsets, then in-degrees (large events)
   int32_t* in_ptr;      // [H + 1]
   int32_t* in_edge;     // [Ecap] edge ids grouped by target, ascending
-  float* hstate;        // [H][h]   FP32 node state (FP32 path and re-score)
+  float* hstate;        // [H][h]   FP32 node state (FP32 path and re-score); until the
+                        //          re-score, the encoders' BF16 lo parts
   float* estate;        // [Ecap][h] FP32 edge state
-  float* pstate;        // [H][2h]  FP32 node projections for the next edge layer
+  float* pstate;        // [H][2h]  FP32 node projections for the next edge layer; before
+                        //          them the node step's messages (FP32, BF16, or E4M3
+                        //          codes followed by their scales)
   __nv_bfloat16* hstate16;  // [H][h]   BF16 node state (tensor-core paths)
   __nv_bfloat16* estate16;  // [Ecap][h] BF16 edge state
   float* hamax;         // [H] largest |BF16 node state| per hit (FP8 handles at h = 128)

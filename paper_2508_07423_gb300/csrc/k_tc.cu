@@ -25,8 +25,9 @@
 // its own per-row scale amax/448 and accumulated in its own TMEM block, so the
 // epilogue can apply the scales (the edge steps at hidden 128: h_src and h_dst
 // under one scale in one block, layer 1 in three passes, see Layout::P3);
-// weights carry per-output-channel scales amax/448. Hidden rows are quantised per row as well. The K = 3 first layer of
-// the node encoder and the 1-unit last layer of the classifier stay FP32.
+// weights carry per-output-channel scales amax/448. Hidden rows are quantised per
+// row as well. The K = 3 first layer of the node encoder and the 1-unit last layer
+// of the classifier stay FP32.
 #include <cuda_fp8.h>
 #include <cudaTypedefs.h>
 
@@ -2194,7 +2195,7 @@ constexpr int family_of(int mode) {
 static_assert(family_of(M_TRIP) == 3, "triplet classifier tunes with the edge family");
 constexpr int hidx(int h) { return h == 32 ? 0 : (h == 64 ? 1 : 2); }
 
-// BF16 edge step at hidden 32: 0 per-thread copies, 1 TMA-staged tiles, 2
+// BF16 edge step at hidden 32: 0 cp.async row copies, 1 TMA-staged tiles, 2
 // warp-specialised with TMA-staged tiles
 std::atomic<int> g_edge_form{0};
 
@@ -2437,7 +2438,7 @@ int tc_upload(TcModel& m, const HostLayer* L, int n_layers, int n_embed, int h, 
   m.enc16 = fp8;
   if (m.enc16) {
     items.push_back({c + 1, &m.node_enc16.l2, true, true});
-    items.push_back({c + 2, &m.edge_enc16.l1, h <= 64, true});  // h 128: two passes, plain image
+    items.push_back({c + 2, &m.edge_enc16.l1, h <= 64, true});  // h 128: four passes, plain image
     items.push_back({c + 3, &m.edge_enc16.l2, false, true});
   }
   c += 4;

@@ -16,7 +16,7 @@ struct TcModel {
   Mlp2TC node_enc{}, edge_enc{}, cls{}, node[kMaxIters]{}, edge[kMaxIters]{};
   // FP8: BF16 split-operand encoders (node_enc16.l2, edge_enc16.l1 and .l2
   // hold BF16 images; edge_enc16.l1 repeated along K up to hidden 64, plain at
-  // 128 where the edge encoder runs its layer 1 in two passes)
+  // 128 where the edge encoder runs its layer 1 in four passes)
   Mlp2TC node_enc16{}, edge_enc16{};
   bool enc16 = false;
   // first layers of the triplet classifiers (BF16 images in every precision)
@@ -30,12 +30,13 @@ struct TcModel {
 };
 
 // Encode the tensor maps of a BF16 handle's workspace (hidden 32); on failure
-// the TMA edge step stays unavailable and the per-thread copies run.
+// the TMA edge step stays unavailable and form 0 runs.
 void tc_make_maps(TcModel& m, const Ws& w, int h);
 
-// BF16 edge-step form at hidden 32, process wide: 0 per-thread row copies, 1
+// BF16 edge-step form at hidden 32, process wide: 0 cp.async row copies (k_tc), 1
 // TMA tile load and row gathers, 2 the same loads in a ring with producer,
-// MMA and epilogue warps (1 and 2 only where the handle has tensor maps).
+// MMA and epilogue warps (1 and 2 only where the handle has tensor maps). Form 0 is
+// the fastest: 1.25 ms per pass of 4 x 10.1 M rows against 2.27 and 3.02.
 void tc_set_edge_form(int form);
 int tc_get_edge_form();
 
@@ -63,8 +64,9 @@ void tc_node_prep(const Batch& b, const Ws& w, const TcModel& m, const LayerF32*
                   int n_embed, int D, int h, const GraphParams& g, const LayerF32& ne1_f32,
                   cudaStream_t s, bool do_embed = true);
 
-// Messages of a node step from the BF16 edge states (FP32 sums, stored
-// rounded to BF16 for BF16 handles and in FP32 for FP8 handles), for every hit.
+// Messages of a node step from the BF16 edge states (FP32 sums, stored rounded to
+// BF16 for BF16 handles and as E4M3 codes with their scales for FP8 handles), for
+// every hit.
 void tc_messages(const Batch& b, const Ws& w, int h, bool fp8, cudaStream_t s);
 
 // Edge encoder, K message-passing steps and the classifier with the cut;
