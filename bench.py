@@ -164,32 +164,29 @@ def stage_work(stage: str, precision: str, N: int, E: int, h: int, K: int, D: in
             # W_e e (h x h) and the second layer (h x h); the h_src / h_dst
             # products come precomputed per hit from the node step
             return "alu", E * 2.0 * (h * h + h * h), "flop"
-        # read e, h_src, h_dst rows; write e
-        return "hbm", E * (4 * h * sb + 8), "byte"
+        # read e; write e; indices; the node rows once (their repeated gathers
+        # hit L2)
+        return "hbm", E * (2 * h * sb + 8) + N * h * sb, "byte"
     if stage == "node_messages":
         # every edge row read twice (its source's out sum, its target's in
         # sum), the in-edge ids, the list bounds; the message row written
-        # (BF16 path: rounded to BF16; FP8 path and FP32: FP32)
-        mb = 2 if precision == "bf16" else 4
+        # (BF16 path: rounded to BF16; FP8 path: E4M3 codes; FP32: FP32)
+        mb = {"bf16": 2, "fp8": 1}.get(precision, 4)
         return "hbm", 2 * E * h * sb + 4 * E + N * (16 + 2 * h * mb), "byte"
     if stage == "node_update":
         if precision == "fp32":
             # node network (3h x h, h x h) and the two projections (2 x h x h)
             return "alu", N * 2.0 * (3 * h * h + h * h + 2 * h * h), "flop"
         # read h and the message row, write h
-        mb = 2 if precision == "bf16" else 4
+        mb = 2 if precision == "bf16" else 1
         return "hbm", N * (2 * h * sb + 2 * h * mb), "byte"
     if stage == "edge_encoder":
         if precision == "fp32":
-            # 2 h^2 flop per edge against 3 rows of 4h bytes: memory-bound;
-            # read the two projection halves P[src], P[dst], write e, indices
-            return "hbm", E * (3 * h * 4 + 8), "byte"
-        if precision == "bf16":
-            # read the FP32 encodings h_src, h_dst (split into hi + lo BF16
-            # operands on chip); write e (BF16); indices
-            return "hbm", E * (2 * h * 4 + h * sb + 8), "byte"
-        # read h_src, h_dst rows; write e; indices
-        return "hbm", E * (3 * h * sb + 8), "byte"
+            # 2 h^2 flop per edge against 4h bytes written: memory-bound; the two
+            # projection halves of every hit once, write e, indices
+            return "hbm", E * (h * 4 + 8) + N * 2 * h * 4, "byte"
+        # the node encodings' hi and lo BF16 parts once; write e (BF16); indices
+        return "hbm", E * (h * sb + 8) + N * 2 * h * 2, "byte"
     if stage == "node_prep":
         # embedding MLP (FP32 in every precision), plus the FP32 node encoder
         # (3 x h, h x h) and its two projections (2 x h x h) on the FP32 path
@@ -206,28 +203,26 @@ def stage_work(stage: str, precision: str, N: int, E: int, h: int, K: int, D: in
     return "hbm", N * 16, "byte"
 
 
-# DRAM bytes (read + write) per row of the dominant kernels, from ncu
-# captures of 300 events of the same workload (the re-score edge step:
-# profiles/k_gnn_f32_rescore_edge_weights_in_smem_300ev.md, variant 2, steps 0
-# and 1; the others: profiles/dram_traffic_edge_steps_300ev.md), averaged over
+# DRAM bytes (read + write) per row of the dominant kernels, from ncu captures of
+# 300 events of the same workload (profiles/step_kernels_300ev.md), averaged over
 # the captured launches; scaled to this run's rows.
 TRAFFIC_PER_ROW = {
-    ("rescore_edge_update", "bf16"): 280.3,
-    ("edge_update", "bf16"): 116.9,
-    ("edge_update", "fp32"): 257.6,
+    ("rescore_edge_update", "bf16"): 280.2,
+    ("edge_update", "bf16"): 127.3,
+    ("edge_update", "fp32"): 283.9,
 }
 
 
-# What the counters of the dominant kernels show (ncu --set full, same
-# 300-event captures as the traffic above): the roof their work is counted
-# against is not what limits them.
+# What the counters of the dominant kernels show (ncu, same 300-event captures as
+# the traffic above): the roof their work is counted against is not what limits
+# them.
 COUNTERS = {
     ("rescore_edge_update", "bf16"): {
-        "limiter": "latency: FMA pipe 50 % active, DRAM 28 % of peak, warps active 22.6 % of 64 "
-                   "(16 resident: registers and shared memory), stalls spread over shared-memory "
-                   "operand loads, fixed-latency dependencies and the FMA pipe",
-        "fma_pipe_active_pct": 50.1, "dram_pct_of_peak": 28.0, "warps_active_pct": 22.6,
-        "source": "profiles/k_gnn_f32_rescore_edge_weights_in_smem_300ev.md"},
+        "limiter": "shared-memory pipe 81 % of its cycles (operand and weight loads of the FP32 "
+                   "products), FMA pipe 59 %, DRAM 33 %, warps active 30 % of 64 (20 per SM: "
+                   "registers)",
+        "fma_pipe_active_pct": 59.1, "dram_pct_of_peak": 33.4, "warps_active_pct": 30.3,
+        "source": "profiles/step_kernels_300ev.md"},
 }
 
 
