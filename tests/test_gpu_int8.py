@@ -132,3 +132,27 @@ def test_int8_wide_embedding_graph():
     assert n_edges > 1000
     assert n_diff <= 0.01 * n_edges, (n_diff, n_edges)
     assert n_same >= 0.99 * (n_edges - n_diff), (n_same, n_edges - n_diff)
+
+
+@pytest.mark.parametrize("tracks", [1, 77])
+def test_int8_many_hits_equal_few(trained, tracks):
+    """Large batches take two hits per thread: a batch past that line, whose last
+    event ends inside a thread's pair, gives its first, middle and last events the
+    graphs they get alone (one hit per thread), to the bit."""
+    wl, layers = trained
+    n = 2 * 8 * torch.cuda.get_device_properties(0).multi_processor_count * 128
+    unit = synth.workload_batch(wl, 20)
+    reps = n // unit.n_hits + 1
+    b = synth.concat([unit] * reps + [synth.gen_batch(1, 9, {"kind": "fixed", "n": tracks}, 0.05)])
+    assert b.n_hits > n
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=b.n_hits, max_events=b.n_events,
+                                  embed_int8=True, edges_per_hit=8)
+    tr.set_embed_scales(tr.embed_amax(torch.from_numpy(unit.xyz_soa()).cuda()))
+    pkg.run_batch(tr, b)
+    sample = (0, b.n_events // 2, b.n_events - 2, b.n_events - 1)
+    graphs = [tr.get_graph(e) for e in sample]
+    for e, g in zip(sample, graphs):
+        pkg.run_batch(tr, b.event(e))
+        alone = tr.get_graph(0)
+        for k in g:
+            assert np.array_equal(g[k], alone[k]), (e, k)
