@@ -184,7 +184,7 @@ struct Layout {
   static constexpr bool OUT_STAGE = !FP8 && H <= 64 && MODE != M_CLS && MODE != M_TRIP && MODE != M_EDGE_UPD_CLS;
   static_assert(THREADS <= 512 && !(SWZ && (NODE8 || P3)) && !(OUT_STAGE && COOP), "one way in, one way out");
   // P3: full and empty barriers of the rings, and the rows' two scales (of two
-  // tiles, by turns)
+  // tiles, by turns; written after the wait for the tile's first slot, see p3_loader)
   static constexpr int RING = BAR + 64;
   static constexpr int SCALES = RING + (P3 ? 128 : 0);
   static constexpr int STAGE = SCALES + (P3 ? G * 2 * kRows * 8 : 0);
@@ -663,7 +663,6 @@ __device__ __forceinline__ void p3_loader(const TcArgs& p, uint8_t* smem, int wg
     const int nid_s = w.src[row_of(tn)], nid_d = w.col[row_of(tn)];
     const float h_scale = amax > 0.f ? amax / 448.f : 1.f;
     const float hinv = 1.f / h_scale;
-    scales[turn * kRows + tid].y = h_scale;
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
       const int seg = k / 4, g = k % 4, n = k + 1;
@@ -677,6 +676,10 @@ __device__ __forceinline__ void p3_loader(const TcArgs& p, uint8_t* smem, int wg
       if (g == 0) {  // (the slot's last MMA has read it)
         const bool free = uses == 0 || mbar_wait_bounded(&empty[slot], uint32_t(uses - 1) & 1u, kWaitCycles);
         if (!__all_sync(0xffffffffu, free)) return;
+        // (the tile's first slot was last read by an MMA of the tile before, which the
+        // warpgroup issues once all its threads have the scales of the tile before
+        // that one: this tile's place)
+        if (k == 0) scales[turn * kRows + tid].y = h_scale;
       }
       uint4 (&u)[4] = v[k % 2];
       float iv = hinv;

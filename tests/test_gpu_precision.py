@@ -538,3 +538,23 @@ def test_tensor_core_tiles_at_ragged_sizes(name, prec, tol, tracks):
     if both:
         assert np.mean([abs(t[k] - t32[k]) for k in both]) < tol
     assert tracks < 13 or (len(g["src"]) > 20 and len(both) > 20)
+
+
+def test_fp8_edge_step_repeats_to_the_bit():
+    """FP8 at hidden 128 with several tiles per warpgroup (the edge kernels' rings of
+    tiles and scales go round many times): twelve calls on the same hits give the
+    same logits of every edge."""
+    wl = synth.workload("cfg4_batched_fp8")
+    b = synth.workload_batch(wl, 24)
+    tr = pkg.tracker_for_workload(wl, precision="fp8", rescore_band=0.0, max_hits=b.n_hits,
+                                  max_events=b.n_events, edges_per_hit=16)
+    ref = None
+    for _ in range(12):
+        pkg.run_batch(tr, b)
+        logits = np.concatenate([tr.get_graph(e)["logit"] for e in range(b.n_events)])
+        if ref is None:
+            ref = logits
+            sms = torch.cuda.get_device_properties(0).multi_processor_count
+            assert ref.size > 3 * 2 * sms * 128 and np.isfinite(ref).all()
+        assert np.array_equal(logits, ref)
+    tr.close()

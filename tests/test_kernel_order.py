@@ -1,0 +1,37 @@
+"""Orderings inside the kernels that no result shows: a write that must follow a
+wait, a barrier that must come before an access. Breaking one gives a race whose
+window is a few instructions wide, so the sources are read instead (comments
+taken out, the text of one function at a time)."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2508_07423_gb300", "csrc")
+
+
+def body(path, name):
+    """Text of the function `name` of csrc/<path>, from its parameters to its
+    closing brace, without comments and with single spaces."""
+    with open(os.path.join(CSRC, path)) as f:
+        text = f.read()
+    text = re.sub(r"//[^\n]*|/\*.*?\*/", "", text, flags=re.S)
+    m = re.search(r"(__global__|__device__)[^;{}]*\b%s\(" % name, text)
+    assert m, name
+    i = text.index("{", m.end())
+    depth, j = 1, i + 1
+    while depth:
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        j += 1
+    return " ".join(text[m.end():j].split())
+
+
+def test_fp8_loader_stores_scales_after_the_slot_wait():
+    """FP8 edge step at hidden 128: a tile's scales take the place of those of two
+    tiles before. Only the wait for the tile's first ring slot says that every
+    thread has read them (the slot's last MMA is issued behind a barrier that
+    follows those reads), so no store of a scale may come before it."""
+    b = body("k_tc.cu", "p3_loader")
+    wait = b.index("mbar_wait_bounded(&empty[slot]")
+    stores = [m.start() for m in re.finditer(r"scales\[[^;]*\]\.[xy] = ", b)]
+    assert len(stores) == 2
+    assert all(s > wait for s in stores)
