@@ -778,10 +778,13 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
   __shared__ int wsum[kGraphWarps];
   __shared__ int ticket_s;
   __shared__ long long base_s;
+  const cg::cluster_group cluster = cg::this_cluster();
+  // (no access to another block's shared memory before every block runs; in the time of
+  // the kernel before)
+  if constexpr (CLUSTER) cluster.sync();
   pdl_begin();
   if (input_bad(w)) return;  // (written by an earlier kernel: uniform over the grid)
   constexpr int NT = kGraphThreads;
-  const cg::cluster_group cluster = cg::this_cluster();
   const int rank = CLUSTER ? int(cluster.block_rank()) : 0;
   const int ranks = CLUSTER ? int(cluster.num_blocks()) : 1;
   const int P = g.n_planes;

@@ -35,3 +35,12 @@ def test_fp8_loader_stores_scales_after_the_slot_wait():
     stores = [m.start() for m in re.finditer(r"scales\[[^;]*\]\.[xy] = ", b)]
     assert len(stores) == 2
     assert all(s > wait for s in stores)
+
+
+def test_graph_clusters_meet_before_the_first_remote_write():
+    """Graph kernel, several blocks per event: the first block writes the others'
+    shared memory, which exists only once they run. A cluster barrier that every
+    block reaches comes before the ticket loop."""
+    b = body("k_graph.cu", "k_graph_event")
+    sync = b.index("if constexpr (CLUSTER) cluster.sync();")
+    assert sync < b.index("return;") and sync < b.index("map_shared_rank") and sync < b.index("for (;;)")
