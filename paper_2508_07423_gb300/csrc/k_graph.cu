@@ -841,14 +841,14 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
     // 1. degrees (uncapped); with masks, a hit over k_max keeps only its
     //    k_max selected candidates in its mask (the masks then hold exactly
     //    the edges)
-    if (masks) {
-      if constexpr (CLUSTER) {
-        graph_masks<D>(cst, pl, P, r2, masks_s ? cluster.map_shared_rank(mask, 0) : mask, rank, ranks);
-        cluster.sync();
-      } else {
-        graph_masks<D>(cst, pl, P, r2, mask, 0, 1);
-        __syncthreads();
-      }
+    if constexpr (CLUSTER) {
+      if (masks) graph_masks<D>(cst, pl, P, r2, masks_s ? cluster.map_shared_rank(mask, 0) : mask, rank, ranks);
+      // (without masks too: every block has read its ticket, so the first may write the
+      // next one)
+      cluster.sync();
+    } else if (masks) {
+      graph_masks<D>(cst, pl, P, r2, mask, 0, 1);
+      __syncthreads();
     }
     if (rank > 0) continue;  // (the next ticket comes when the first block is done)
     if (masks) {

@@ -151,3 +151,31 @@ def test_graph_kernel_branches_match_float64(n_events, dim):
             assert not rep.bad_pairs, (tracks, e, rep.bad_pairs[:3])
             assert rep.max_score_err <= 1e-4, (tracks, e, rep.max_score_err)
         tr.close()
+
+
+@pytest.mark.parametrize("line", [12, 5, 2])
+@pytest.mark.parametrize("over", [0, 1])
+def test_graph_of_large_events_in_every_cluster_width(line, over):
+    """Events whose masks lie in global memory, and events without staged rows or
+    masks, in the first and the last place of batches on both sides of each change
+    of the cluster's width (1/12, 1/5 and 1/2 of the SMs): the graphs, logits and
+    labels they get alone, to the bit."""
+    n = torch.cuda.get_device_properties(0).multi_processor_count // line + over
+    wl = synth.workload("cfg1_plain_fp32")
+    for tracks, k_max, r2 in ((520, 64, 0.002), (900, 5, 0.004)):
+        w = dict(wl, k_max=k_max, radius2=r2)
+        big = [synth.gen_batch(1, 61 + i + tracks, {"kind": "fixed", "n": tracks}, 0.02) for i in range(2)]
+        small = [synth.gen_batch(1, 7000 + i, {"kind": "fixed", "n": 3}, 0.1) for i in range(n - 2)]
+        b = synth.concat([big[0]] + small + [big[1]])
+        tr = pkg.tracker_for_workload(w, precision="fp32", max_hits=b.n_hits, max_events=n,
+                                      edges_per_hit=64)
+        labels = pkg.run_batch(tr, b)
+        got = [(tr.get_graph(e), labels[b.offsets[e]:b.offsets[e + 1]]) for e in (0, n - 1)]
+        for (g, lab), ev in zip(got, big):
+            want_lab = pkg.run_batch(tr, ev)
+            want = tr.get_graph(0)
+            assert want["src"].size > 1000
+            for k in want:
+                assert np.array_equal(g[k], want[k]), (tracks, k)
+            assert np.array_equal(lab, want_lab), tracks
+        tr.close()

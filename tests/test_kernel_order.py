@@ -44,3 +44,24 @@ def test_graph_clusters_meet_before_the_first_remote_write():
     b = body("k_graph.cu", "k_graph_event")
     sync = b.index("if constexpr (CLUSTER) cluster.sync();")
     assert sync < b.index("return;") and sync < b.index("map_shared_rank") and sync < b.index("for (;;)")
+
+
+def test_graph_clusters_read_every_ticket_before_the_next_is_written():
+    """Graph kernel, several blocks per event: between a block's read of its ticket
+    and the first block's next write of it lies a cluster barrier that does not
+    depend on the event (whether it has masks, say): within the ticket loop only
+    `if constexpr (CLUSTER)` encloses it."""
+    b = body("k_graph.cu", "k_graph_event")
+    loop = b[b.index("for (;;)"):]
+    read, leave = loop.index("const int ev = ticket_s;"), loop.index("if (rank > 0) continue;")
+    assert loop.count("atomicAdd(&w.counters[C_GRAPH_TICKET]") == 1
+    opened, depths = [], []  # texts before the open braces, those of each barrier
+    for m in re.finditer(r"cluster\.sync\(\)|[{}]", loop[:leave]):
+        if m.group() == "{":
+            opened.append(re.split(r"[{};] ", loop[:m.start()])[-1].strip())
+        elif m.group() == "}":
+            opened.pop()
+        elif m.start() > read:
+            before = re.split(r"[{};] ", loop[:m.start()])[-1].strip()
+            depths.append([o for o in opened[1:] + [before] if o])
+    assert ["if constexpr (CLUSTER)"] in depths, depths
