@@ -1520,7 +1520,7 @@ __global__ void __launch_bounds__(kRows, 5)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Ws& w = p.w;
-  pdl_begin();
+  pdl_wait();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
 
   if (tid == 0) {
@@ -1542,6 +1542,7 @@ __global__ void __launch_bounds__(kRows, 5)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tslot;
+  pdl_trigger();  // (not before this block has its tensor memory)
   const uint32_t tmem_lane = tmem_base + (uint32_t(warp * 32) << 16);
 
   if (tid == 0) {
@@ -1866,7 +1867,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Ws& w = p.w;
-  pdl_begin();
+  pdl_wait();
   if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_INPUT) return;
 
   if (tid == 0) {
@@ -1900,6 +1901,7 @@ __global__ void __launch_bounds__(kWsThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tslot;
+  pdl_trigger();  // (not before this block has its tensor memory)
 
   // the weights come with the first tile: their bytes are counted on the
   // first full barrier, which the MMA warp waits for before its first MMA

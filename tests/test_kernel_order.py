@@ -5,6 +5,8 @@ taken out, the text of one function at a time)."""
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_2508_07423_gb300", "csrc")
 
@@ -65,3 +67,14 @@ def test_graph_clusters_read_every_ticket_before_the_next_is_written():
             before = re.split(r"[{};] ", loop[:m.start()])[-1].strip()
             depths.append([o for o in opened[1:] + [before] if o])
     assert ["if constexpr (CLUSTER)"] in depths, depths
+
+
+@pytest.mark.parametrize("kernel", ["k_tc", "k_tc_edge_tma", "k_tc_edge_ws"])
+def test_tensor_memory_before_the_next_kernel_may_start(kernel):
+    """The next kernel's blocks take tensor memory and keep it while they wait for
+    this kernel. So a block lets them in only after its own allocation; else its
+    allocation could wait for columns that are held by blocks waiting for it."""
+    b = body("k_tc.cu", kernel)
+    trigger = min(b.index(t) for t in ("pdl_begin();", "pdl_trigger();") if t in b)
+    alloc = b.index("tmem_alloc(")
+    assert alloc < b.index("__syncthreads();", alloc) < trigger
