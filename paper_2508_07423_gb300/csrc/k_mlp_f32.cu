@@ -451,10 +451,13 @@ struct GnnShape {
 };
 
 // The ring of weight chunks of one block: chunk g (g = 0, 1, ...) is rows
-// [(g % CPL) KC, + KC) of matrix (g / CPL) % RMATS and lies in stage g % NST;
+// [(g % CPL) KC, + KC) of matrix (g / CPL) % MATS and lies in stage g % NST;
 // a stage's barrier completes when its bytes have landed, and the last of the
 // `users` warps that have a tile to finish a chunk refills the stage with chunk
-// g + NST. A wait that runs out latches ST_TIMEOUT; the warp then waits no more.
+// g + NST. A wait that runs out (of chunk `late`) latches ST_TIMEOUT; the warp then
+// waits no more and no longer counts as done with a chunk, so that no stage whose
+// copy may still be in flight is refilled: of the chunks that it has not seen land,
+// only late .. late + NST - 1 can have been asked for.
 constexpr long long kRingWaitCycles = 4000000000LL;  // about 2 s
 
 template <class X>
@@ -466,7 +469,7 @@ struct WeightRing {
   uint64_t* full;
   int* done;
   int g = 0, total = 0, users = 0;
-  bool dead = false;
+  int late = -1;
 
   __device__ __forceinline__ void load(const typename X::Args& p, int c) {
     const int m = (c / CPL) % W::MATS, k = (c % CPL) * W::KC;
@@ -499,14 +502,14 @@ struct WeightRing {
 #pragma unroll 1
     for (int c = 0; c < CPL; ++c) {
       const int st = g % W::NST;
-      if (!dead && !tc::mbar_wait_bounded(full + st, (g / W::NST) & 1, kRingWaitCycles)) {
-        dead = true;
+      if (late < 0 && !tc::mbar_wait_bounded(full + st, (g / W::NST) & 1, kRingWaitCycles)) {
+        late = g;
         set_status(p.w.counters, ST_TIMEOUT);
       }
       warp_product<T, W::KC, W::KC, T::LDH, true>(A + c * W::KC, buf + st * STAGE, X::H, rg, cg,
                                                   acc);
       __syncwarp();  // every lane is done with the chunk
-      if ((threadIdx.x & 31) == 0 && g + W::NST < total) {
+      if ((threadIdx.x & 31) == 0 && late < 0 && g + W::NST < total) {
         __threadfence_block();
         if (atomicAdd(done + st, 1) == users - 1) {
           done[st] = 0;
@@ -516,6 +519,12 @@ struct WeightRing {
       }
       ++g;
     }
+  }
+  // before the warp ends, after a wait that ran out: the copies that may be in flight
+  __device__ __forceinline__ void drain() {
+    if (late < 0 || (threadIdx.x & 31) != 0) return;
+    for (int c = late; c < late + W::NST && c < total; ++c)
+      tc::mbar_wait_bounded(full + c % W::NST, (c / W::NST) & 1, kRingWaitCycles / W::NST);
   }
 };
 
@@ -562,10 +571,7 @@ struct LayerWeights {
   }
   // before a block ends (after a timeout: no copy may land after it is gone)
   __device__ __forceinline__ void finish() {
-    if constexpr (W::RING) {
-      if (ring.dead && (threadIdx.x & 31) == 0)
-        for (int st = 0; st < W::NST; ++st) tc::mbar_wait_bounded(ring.full + st, 0, kRingWaitCycles);
-    }
+    if constexpr (W::RING) ring.drain();
   }
 };
 

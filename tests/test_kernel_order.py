@@ -78,3 +78,16 @@ def test_tensor_memory_before_the_next_kernel_may_start(kernel):
     trigger = min(b.index(t) for t in ("pdl_begin();", "pdl_trigger();") if t in b)
     alloc = b.index("tmem_alloc(")
     assert alloc < b.index("__syncthreads();", alloc) < trigger
+
+
+def test_weight_ring_after_a_wait_that_ran_out():
+    """FP32 kernels at hidden 128: a warp whose wait for a chunk ran out neither
+    counts as done with a chunk nor refills a stage (its copy may be in flight), and
+    before it ends waits for each chunk that may be, by that chunk's own parity."""
+    b = body("k_mlp_f32.cu", "product")
+    refill = b[b.index("__syncwarp();"):]
+    assert "late < 0" in refill[:refill.index("atomicAdd")]
+    d = body("k_mlp_f32.cu", "drain")
+    assert "c < late + W::NST && c < total" in d
+    assert "mbar_wait_bounded(full + c % W::NST, (c / W::NST) & 1" in d
+    assert "ring.drain()" in body("k_mlp_f32.cu", "finish")
