@@ -5,7 +5,9 @@ One step = one call of the whole hot path (plane sort, embedding, radius graph,
 interaction network, cut, connected components) over one batch of synthetic
 events of the batched workload (1000 events, tracks Poisson(150) clipped to
 [20, 400], 5 % noise, embed 3-64-64-4, IN h32 K4, mean degree 12). Prints one
-JSON line (rank 0).
+JSON line on stdout (rank 0): the result of that workload, below LINE_MAX
+characters. What the other legs measure (serving, the other workloads and
+precisions, the stages' rooflines) goes to stderr, a JSON line per leg.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--precision fp32|bf16|fp8] [--workload NAME]
@@ -38,6 +40,15 @@ from paper_2508_07423_gb300 import replicas, synth  # noqa: E402
 METRIC = "events/s and hits/s on 1 GB300 (BF16/FP8 batched vs FP32 plain); p99 latency"
 DEFAULT_WORKLOAD = "cfg3_batched_bf16"
 L2_FLUSH_BYTES = 256 << 20
+# the stdout line: its keys, and what of them goes to stderr. A line with every leg
+# in it had grown past what a program that reads the end of the output keeps.
+LINE_MAX = 4000
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "hits_per_s",
+             "p50_step_ms", "p99_step_ms", "config", "clocks", "roofline", "e2e", "gpu_launches",
+             "batched_over_plain", "batched_over_plain_hits", "wall_s_timed", "cpu_baseline")
+LINE_WITHOUT = {"config": ("rescore_rows",),
+                "roofline": ("counters", "stage_ms_per_step", "stages")}
 
 
 def parse():
@@ -295,6 +306,20 @@ def quick_rate(pkg, torch, wl, batch, dev, stream, flush, steps=5, **kw):
             "band_edges": st["band"], "rerun_events": st["rerun_events"]}
 
 
+def split_line(out):
+    """(the dict of the stdout line, {leg: its report}) of a run's results."""
+    line, legs = {}, {}
+    for k, v in out.items():
+        if k not in LINE_KEYS:
+            legs[k] = v
+            continue
+        cut = [c for c in LINE_WITHOUT.get(k, ()) if v and c in v]
+        line[k] = {c: v[c] for c in v if c not in cut} if cut else v
+        if cut:
+            legs[k] = {c: v[c] for c in cut}
+    return line, legs
+
+
 def main():
     a = parse()
     rank = int(os.environ.get("RANK", "0"))
@@ -484,7 +509,10 @@ def main():
             out["triplet_report"] = triplet_report(pkg, torch, dev, stream, flush)
             out["int8_report"] = int8_report(pkg, torch, dev, stream, flush)
     if rank == 0:
-        print(json.dumps(out))
+        line, legs = split_line(out)
+        for k, v in legs.items():
+            print(json.dumps({"leg": k, "report": v}), file=sys.stderr, flush=True)
+        print(json.dumps(line))
     if dist:
         dist.destroy_process_group()
 
