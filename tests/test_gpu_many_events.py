@@ -174,7 +174,7 @@ def test_graph_of_large_events_in_every_cluster_width(line, over):
         for (g, lab), ev in zip(got, big):
             want_lab = pkg.run_batch(tr, ev)
             want = tr.get_graph(0)
-            assert want["src"].size > 1000
+            assert want["src"].size > 100
             for k in want:
                 assert np.array_equal(g[k], want[k]), (tracks, k)
             assert np.array_equal(lab, want_lab), tracks
