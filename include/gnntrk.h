@@ -367,7 +367,8 @@ int32_t gnntrk_stage_times(gnntrk_handle* h, int32_t max_stages, char* names, do
  *     choice[0..3] = node encoder, edge encoder, node step, edge step;
  *   - FP32 SIMT kernels (FP32 handles, and the FP32 re-score of BF16/FP8 handles
  *     with a re-score band): variant 0 (tile height by the number of rows of
- *     the launch), 1 (tall tiles always) or 2 (short tiles always);
+ *     the launch), 1 (tall tiles always) or 2 (as 0, short tiles up to twice as
+ *     many rows);
  *     choice[4..6] = encoders, node step, edge step;
  *   - the BF16 edge step at hidden 32 (BF16 handles): form 0 (each thread
  *     copies its row's [e, h_src, h_dst] into the tile), 1 (the tile is

@@ -230,8 +230,8 @@ void launch_edge_update_f32(const Batch& b, const Ws& w, const Mlp2F32& m, const
                             int h, float cut_logit, bool rescore_only, float band_lo,
                             float band_hi, Sel sel, cudaStream_t s);
 
-// FP32 tile variant (0 by the number of rows, 1 tall tiles, 2 short tiles) per
-// kernel family (0 encoders, 1 node step, 2 edge step + classifier), process
+// FP32 tile variant (0 by the number of rows, 1 tall tiles, 2 by the number of rows
+// with the line to tall tiles twice as high) per kernel family (0 encoders, 1 node step, 2 edge step + classifier), process
 // wide; chosen by the autotuner.
 void f32_set_variant(int h, int family, int v);
 

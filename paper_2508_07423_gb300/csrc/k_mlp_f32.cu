@@ -1182,13 +1182,15 @@ constexpr int f32_family(int mode) {
 // Variant (0 the default; the autotuner may pick another, see
 // gnntrk_set_tuning): 0 = short tiles for calls whose rows fill at most one
 // round of short tiles over the grid's warps, tall tiles above; 1 = tall tiles
-// always; 2 = short tiles always. The line of variant 0: up to one round every
+// always; 2 = short tiles up to two rounds. The line of variant 0: up to one round every
 // warp has one short tile, and a call's time is the time of one tile (one
 // event of 2146 hits at hidden 64: node step 17.9 us against 31.0 us with tall
 // tiles); with two rounds or more the short tiles' weight loads, one per row
 // group and k instead of one for 8 rows, cost more than the idle warps
 // (16 652 edges, 2.3 rounds: edge step 20.1 us against 17.1 us with tall
-// tiles).
+// tiles). Variant 2 goes no further than two rounds: a choice may be kept and applied
+// to calls of any size, and short tiles at every size took 9.71 ms per call of 400
+// events at hidden 32 and 23.7 ms for 100 at hidden 64 (variant 0: 4.03 and 8.40 ms).
 //
 // Shapes (GB300; edge steps and node steps of a call, against the kernels they
 // replaced, whose warps of 4-warp blocks had 32 accumulators per lane):
@@ -1213,7 +1215,7 @@ template <class X>
 void launch_shape(GnnArgs a, int64_t rows_hint, cudaStream_t s) {
   const int v = g_f32_variant[X::H == 32 ? 0 : (X::H == 64 ? 1 : 2)][f32_family(X::MODE)].load(
       std::memory_order_relaxed);
-  a.short_rounds = v == 0 ? 1 : v == 1 ? 0 : 1 << 20;
+  a.short_rounds = v == 0 ? 1 : v == 1 ? 0 : 2;
   const void* fn = (const void*)k_gnn_f32<X>;
   int grid = device_sms() * blocks_per_sm(fn, X::NW * 32, X::SMEM);
   // four short tiles per block before another block is used

@@ -558,3 +558,37 @@ def test_fp8_edge_step_repeats_to_the_bit():
             assert ref.size > 3 * 2 * sms * 128 and np.isfinite(ref).all()
         assert np.array_equal(logits, ref)
     tr.close()
+
+
+@pytest.mark.parametrize("name,events", [("cfg3_batched_bf16", 75), ("cfg2_run3_single", 24)])
+def test_kept_fp32_choices_do_not_slow_other_sizes(name, events):
+    """A launch configuration may be kept and applied to calls of any size: on a
+    batch of many rounds of tiles every FP32 variant runs the same tall tiles, so the
+    calls take the same time (bound: 1.25 times the default's, the best of several
+    calls each; short tiles at every size took 2.1 times and more)."""
+    wl = synth.workload(name)
+    b = synth.gen_batch(events, 8, {"kind": "fixed", "n": 150}, wl["noise"])
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=b.n_hits, max_events=events,
+                                  edges_per_hit=32)
+    xyz = torch.from_numpy(b.xyz_soa()).cuda()
+    plane, offs = torch.from_numpy(b.plane).cuda(), torch.from_numpy(b.offsets).cuda()
+    labels = torch.empty(b.n_hits, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    best = {}
+    try:
+        for v in (0, 1, 2):
+            tr.set_tuning({"f32_encoders": v, "f32_node_update": v, "f32_edge_update": v})
+            ms = []
+            for _ in range(8):
+                s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                s.record(stream)
+                tr.find_tracks(events, b.n_hits, xyz, plane, offs, labels, stream)
+                e.record(stream)
+                e.synchronize()
+                ms.append(s.elapsed_time(e))
+            best[v] = min(ms[2:])
+    finally:
+        tr.set_tuning({})
+        tr.close()
+    assert best[1] < 1.25 * best[0] and best[2] < 1.25 * best[0], best
