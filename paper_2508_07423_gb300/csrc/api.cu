@@ -389,7 +389,9 @@ void enqueue_pipeline(gnntrk_handle* h, const Batch& b, const int64_t* offsets, 
     else
       tc_node_prep(b, w, h->tc, h->embed, h->n_embed, h->D, h->h, g, h->node_enc.l1, s, !i8);
   });
-  stage(h, "graph", s, 1, [&] { launch_graph(b, w, g, h->D, s); });
+  int gk = 0;
+  stage(h, "graph", s, 0, [&] { gk = launch_graph(b, w, g, h->D, s); });
+  h->last_launches += gk;
   if (!tc) {
     stage(h, "edge_encoder", s, 1, [&] { launch_edge_enc_f32(b, w, h->edge_enc, h->h, all, s); });
     for (int k = 0; k < h->K; ++k) {

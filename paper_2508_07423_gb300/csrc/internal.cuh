@@ -40,7 +40,8 @@ enum Counter : int {
   C_TRIP_KEPT = 13,   // triplets above the triplet cut
   C_GRAPH_TICKET = 14,  // next event of the graph kernel
   C_RS_TICKET = 15,     // next event of the re-score receptive-field kernel
-  C_COUNT = 16
+  C_LARGE_EVENT = 16,   // an event is too large for the graph kernel's smaller blocks
+  C_COUNT = 17
 };
 
 // A layer as parsed from the weight blob (host memory).
@@ -205,8 +206,9 @@ void launch_node_prep_f32(const Batch& b, const Ws& w, const LayerF32* embed, in
                           const GraphParams& g, bool do_embed, bool do_node_enc, Sel sel,
                           cudaStream_t s);
 // rough graph (CSR: row_ptr, col, src, d2; counters[C_EDGES]) and the in-edge
-// index (in_ptr, in_edge), one kernel
-void launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s);
+// index (in_ptr, in_edge), one kernel (two launches, of which one works, for
+// thousands of small events); returns the number of launches
+int launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s);
 // exclusive scan of n entries of `in` (each clamped to clamp_max) into out[0..n],
 // out[n] = total; the total also goes to counters[total_slot] and is checked
 // against `cap` (ST_CAPACITY when above).

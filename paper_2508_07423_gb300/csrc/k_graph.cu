@@ -26,6 +26,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kSortThreads = 256;
 constexpr int kScanThreads = 512;
+constexpr int kMidHits = 1280;  // see GraphShape
 constexpr int kScanPer = 8;
 constexpr int kScanChunk = kScanThreads * kScanPer;
 
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort(Batch b, Ws w, const int6
     if (ev == b.n_events - 1) w.ev_off[ev + 1] = o1;
     w.graph_desc[ev] = 0;
     if (w.rs_desc != nullptr) w.rs_desc[ev] = 0;
+    if (o1 - o0 > kMidHits) w.counters[C_LARGE_EVENT] = 1;
     int f = 0;
     if (o0 < 0 || o1 < o0 || o1 > b.n_hits) f = 1;
     if (ev == 0 && o0 != 0) f = 1;
@@ -370,9 +372,27 @@ __device__ void select_capped(const Cand& cd, const float (&qe)[D], int c0, int 
 // lists were built in shared memory): 1000 events of 1685 hits 433 us (568;
 // 626), 400 events of 2185 hits and 13 k edges 248 us (648; 622), one event of
 // 2146 hits in 8 dimensions 116 us (299; 287).
-constexpr int kGraphThreads = 1024;
-constexpr int kGraphWarps = kGraphThreads / 32;
-constexpr int kGraphInts = 224 * 1024 / 4;
+//
+// Batches of thousands of small events spend those blocks' time at barriers. Such a
+// call takes two blocks of 512 threads per SM if no event has more than kMidHits hits,
+// which the sort finds out. Graph kernel in us with one / two blocks per SM (and with
+// the two blocks of before): 40 000 events of 11 hits 2366 / 1030 (1357), 5000 of 56
+// hits 316 / 164 (218), 1000 of 450 hits 93 / 65 (85). The line is where half the shared
+// memory no longer holds an event in 8 dimensions: 1000 events of 1340 hits 351 / 349
+// (402); two events of 4400 hits among 600 of 32: 205 / 768 (476).
+template <int NT_, int PER_SM_, int KB>
+struct GraphShape {
+  static constexpr int NT = NT_, WARPS = NT_ / 32, PER_SM = PER_SM_;
+  static constexpr int INTS = KB * 1024 / 4;  // shared memory of an event's arrays
+};
+using GraphWide = GraphShape<1024, 1, 224>;
+using GraphMid = GraphShape<512, 2, 110>;
+// calls whose largest event decides (a launch more: of the two one ends at once, about
+// 2 us): a few thousand events at least, of half that size on average
+inline bool by_largest_event(int n_events, int n_hits, int sms) {
+  return n_events >= 16 * sms && n_hits <= int64_t(n_events) * (kMidHits / 2);
+}
+enum GraphWhen : int { G_ALWAYS = 0, G_ALL_SMALL = 1, G_SOME_LARGE = 2 };
 constexpr unsigned long long kDescAgg = 1ull << 62;  // the event's own edge count
 constexpr unsigned long long kDescInc = 2ull << 62;  // edges up to and including the event
 constexpr unsigned long long kDescVal = (1ull << 62) - 1;
@@ -422,9 +442,10 @@ __device__ long long graph_wait(unsigned long long* desc, int ev, long long agg,
 
 // exclusive scan of min(in[i], clamp) over i < n into out (both may be
 // shared or global memory); every thread gets the total
+template <class S>
 __device__ int block_scan(const int32_t* in, int32_t* out, int n, int clamp, int* wsum) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int per = (n + kGraphThreads - 1) / kGraphThreads;
+  const int per = (n + S::NT - 1) / S::NT;
   const int a = min(n, tid * per), z = min(n, a + per);
   int sum = 0;
   for (int i = a; i < z; ++i) sum += min(in[i], clamp);
@@ -438,7 +459,7 @@ __device__ int block_scan(const int32_t* in, int32_t* out, int n, int clamp, int
   __syncthreads();
   int before = 0, total = 0;
 #pragma unroll
-  for (int k = 0; k < kGraphWarps; ++k) {
+  for (int k = 0; k < S::WARPS; ++k) {
     const int t = wsum[k];
     if (k < warp) before += t;
     total += t;
@@ -527,12 +548,12 @@ __device__ __forceinline__ int mask_word(const GraphPlanes& g, int p, int q) {
 
 // 1. mask words: bit b of word k of a hit is candidate mask_first + 32 k + b; this
 // block's share of the items, rank of `ranks` blocks
-template <int D>
+template <class S, int D>
 __device__ void graph_masks(const CandNegT<D>& cd, const GraphPlanes& g, int P, float r2,
                             uint32_t* mask, int rank, int ranks) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n_items = g.items[P - 1];
-  for (int t = warp * ranks + rank; t < n_items; t += kGraphWarps * ranks) {
+  for (int t = warp * ranks + rank; t < n_items; t += S::WARPS * ranks) {
     const int p = plane_of(g.items, P, t);
     const int nw = g.nw[p], chunk = (t - g.items[p]) / nw, k = t - g.items[p] - chunk * nw;
     const int q = g.po[p] + 32 * chunk + lane, c0 = g.po[p + 1], c1 = g.po[min(p + 3, P)];
@@ -554,10 +575,10 @@ __device__ void graph_masks(const CandNegT<D>& cd, const GraphPlanes& g, int P, 
 }
 
 // 1. degrees (uncapped) of the event's query hits, without masks
-template <int D, class Cand>
+template <class S, int D, class Cand>
 __device__ void graph_degrees(const Cand& cd, const GraphPlanes& g, int P, float r2, int32_t* deg) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+  for (int t = warp; t < g.chunk[P - 1]; t += S::WARPS) {
     const GraphItem it = graph_item(g, P, t);
     const int q = it.q0 + lane;
     const bool valid = q < it.q1;
@@ -573,11 +594,11 @@ __device__ void graph_degrees(const Cand& cd, const GraphPlanes& g, int P, float
 // capped hits reduced to their selection): one lane per query hit walks the
 // set bits of its mask in ascending order, recomputes d^2 there from the
 // staged rows and writes its edges at base + off[q].
-template <int D>
+template <class S, int D>
 __device__ void graph_fill_masks(const Ws& w, const CandNegT<D>& cd, const GraphPlanes& g, int P,
                                  const int32_t* off, const uint32_t* mask, long long base, int v0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+  for (int t = warp; t < g.chunk[P - 1]; t += S::WARPS) {
     const int p = plane_of(g.chunk, P, t);
     const int q = g.po[p] + (t - g.chunk[p]) * 32 + lane;
     if (q >= g.po[p + 1]) continue;
@@ -604,12 +625,12 @@ __device__ void graph_fill_masks(const Ws& w, const CandNegT<D>& cd, const Graph
 // 3. fill without masks: one lane per query hit tests its candidates again in
 // ascending order and writes its edges at base + off[q]; a hit over k_max is
 // filled by its warp (fill_capped).
-template <int D, class Cand>
+template <class S, int D, class Cand>
 __device__ void graph_fill(const Ws& w, const Cand& cd, const GraphPlanes& g, int P, float r2,
                            int k_max, const int32_t* deg, const int32_t* off, long long base,
                            int v0) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int t = warp; t < g.chunk[P - 1]; t += kGraphWarps) {
+  for (int t = warp; t < g.chunk[P - 1]; t += S::WARPS) {
     const GraphItem it = graph_item(g, P, t);
     const int q = it.q0 + lane;
     const bool valid = q < it.q1;
@@ -648,30 +669,31 @@ __device__ void graph_fill(const Ws& w, const Cand& cd, const GraphPlanes& g, in
 // in_edge (an entry's place is the number of smaller entries in its list);
 // else the lists are placed in the event's slice of in_edge and sorted there
 // (counts in in_cnt for events of more hits than fit).
+template <class S>
 __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, int32_t* sm_i,
                             int* wsum) {
   const int tid = threadIdx.x;
   const int ne = e1 - e0;
-  const bool full = 2 * int64_t(n) + 2 * int64_t(ne) <= kGraphInts;
-  const bool c_smem = n <= kGraphInts;
+  const bool full = 2 * int64_t(n) + 2 * int64_t(ne) <= S::INTS;
+  const bool c_smem = n <= S::INTS;
   int32_t* C = c_smem ? sm_i : w.in_cnt + v0;
   int32_t* St = sm_i + n;               // (full only) list starts, event-local
   int32_t* L = full ? sm_i + 2 * n : w.in_edge + e0;
   int32_t* Tg = sm_i + 2 * n + ne;      // (full only) target of each list entry
-  for (int i = tid; i < n; i += kGraphThreads) C[i] = 0;
+  for (int i = tid; i < n; i += S::NT) C[i] = 0;
   __syncthreads();
-  for (int e = e0 + tid; e < e1; e += kGraphThreads) atomicAdd(&C[w.col[e] - v0], 1);
+  for (int e = e0 + tid; e < e1; e += S::NT) atomicAdd(&C[w.col[e] - v0], 1);
   __syncthreads();
   if (full) {
-    block_scan(C, St, n, 0x7fffffff, wsum);
-    for (int i = tid; i < n; i += kGraphThreads) {
+    block_scan<S>(C, St, n, 0x7fffffff, wsum);
+    for (int i = tid; i < n; i += S::NT) {
       C[i] = St[i];  // cursor
       w.in_ptr[v0 + i] = e0 + St[i];
     }
   } else {
     // in place: C becomes the cursors, in_ptr the starts
     const int lane = tid & 31, warp = tid >> 5;
-    const int per = (n + kGraphThreads - 1) / kGraphThreads;
+    const int per = (n + S::NT - 1) / S::NT;
     const int a = min(n, tid * per), z = min(n, a + per);
     int sum = 0;
     for (int i = a; i < z; ++i) sum += C[i];
@@ -695,7 +717,7 @@ __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, 
   }
   if (tid == 0) w.in_ptr[v1] = e1;  // the next event writes the same value
   __syncthreads();
-  for (int e = e0 + tid; e < e1; e += kGraphThreads) {
+  for (int e = e0 + tid; e < e1; e += S::NT) {
     const int t = w.col[e] - v0;
     const int k = atomicAdd(&C[t], 1);
     L[k] = e;
@@ -704,7 +726,7 @@ __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, 
   __syncthreads();
   // C[i] is now the end of target i's list (event-local position)
   if (full) {
-    for (int k = tid; k < ne; k += kGraphThreads) {
+    for (int k = tid; k < ne; k += S::NT) {
       const int e = L[k], t = Tg[k];
       const int lo = St[t], hi = C[t];
       int rank = 0;
@@ -712,7 +734,7 @@ __device__ void csc_general(const Ws& w, int n, int v0, int v1, int e0, int e1, 
       w.in_edge[e0 + lo + rank] = e;
     }
   } else {
-    for (int i = tid; i < n; i += kGraphThreads) {
+    for (int i = tid; i < n; i += S::NT) {
       const int lo = w.in_ptr[v0 + i] - e0, hi = C[i];
       for (int j = lo + 1; j < hi; ++j) {
         const int key = L[j];
@@ -756,7 +778,7 @@ struct GraphPlan {
   __device__ __forceinline__ void place_rows(bool masks) {
     rows = (mask + (masks ? words : 0) + 3) & ~3;
   }
-  template <int D>
+  template <class S, int D>
   __device__ __forceinline__ void edges(int ne_) {
     ne = ne_;
     const int half = (ne + 1) / 2;
@@ -764,18 +786,18 @@ struct GraphPlan {
     lists = half <= words ? mask : targets + half;
     sources = half <= words ? targets + half : lists + half;
     ints_all = sources;
-    with_sources = int64_t(sources) + half <= kGraphInts;
+    with_sources = int64_t(sources) + half <= S::INTS;
   }
 };
 
 // CLUSTER: the blocks of a cluster share an event's mask items (the bulk of its
 // arithmetic) and write their words into the first block's shared memory, which
 // alone does the rest.
-template <int D, bool CLUSTER>
-__global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w, GraphParams g) {
+template <class S, int D, bool CLUSTER>
+__global__ void __launch_bounds__(S::NT, S::PER_SM) k_graph_event(Batch b, Ws w, GraphParams g, GraphWhen when) {
   extern __shared__ __align__(16) float sm_graph[];
   __shared__ GraphPlanes pl;
-  __shared__ int wsum[kGraphWarps];
+  __shared__ int wsum[S::WARPS];
   __shared__ int ticket_s;
   __shared__ long long base_s;
   const cg::cluster_group cluster = cg::this_cluster();
@@ -783,8 +805,10 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
   // the kernel before)
   if constexpr (CLUSTER) cluster.sync();
   pdl_begin();
-  if (input_bad(w)) return;  // (written by an earlier kernel: uniform over the grid)
-  constexpr int NT = kGraphThreads;
+  // (both written by an earlier kernel: uniform over the grid)
+  if (input_bad(w)) return;
+  if (when != G_ALWAYS && (w.counters[C_LARGE_EVENT] != 0) != (when == G_SOME_LARGE)) return;
+  constexpr int NT = S::NT;
   const int rank = CLUSTER ? int(cluster.block_rank()) : 0;
   const int ranks = CLUSTER ? int(cluster.num_blocks()) : 1;
   const int P = g.n_planes;
@@ -814,12 +838,12 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
     __syncthreads();  // the layout below depends on the planes
     GraphPlan L{};
     L.rows_and_masks<D>(n, pl.words[P - 1]);
-    const bool staged = L.ints_rows <= kGraphInts;
+    const bool staged = L.ints_rows <= S::INTS;
     // The masks, where the shared memory has no room for them, lie in the event's
     // part of the edge states, which the encoder writes later (32 words per hit at
     // least). Testing every candidate again in the fill instead took 446 / 856
     // us for one event of 3.4 k / 4.6 k hits, against 249 / 564.
-    const bool masks_s = staged && L.ints_masks <= kGraphInts;
+    const bool masks_s = staged && L.ints_masks <= S::INTS;
     const bool masks = masks_s || (staged && L.words <= 32 * int64_t(n) && w.e_cap >= w.h_cap);
     if (!masks_s) L.words = 0;
     L.place_rows<D>(masks_s);
@@ -842,17 +866,17 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
     //    k_max selected candidates in its mask (the masks then hold exactly
     //    the edges)
     if constexpr (CLUSTER) {
-      if (masks) graph_masks<D>(cst, pl, P, r2, masks_s ? cluster.map_shared_rank(mask, 0) : mask, rank, ranks);
+      if (masks) graph_masks<S, D>(cst, pl, P, r2, masks_s ? cluster.map_shared_rank(mask, 0) : mask, rank, ranks);
       // (without masks too: every block has read its ticket, so the first may write the
       // next one)
       cluster.sync();
     } else if (masks) {
-      graph_masks<D>(cst, pl, P, r2, mask, 0, 1);
+      graph_masks<S, D>(cst, pl, P, r2, mask, 0, 1);
       __syncthreads();
     }
     if (rank > 0) continue;  // (the next ticket comes when the first block is done)
     if (masks) {
-      for (int t = warp; t < pl.chunk[P - 1]; t += kGraphWarps) {
+      for (int t = warp; t < pl.chunk[P - 1]; t += S::WARPS) {
         const int p = plane_of(pl.chunk, P, t);
         const int q0 = pl.po[p] + (t - pl.chunk[p]) * 32, q = q0 + lane;
         const int c0 = pl.po[p + 1], c1 = pl.po[min(p + 3, P)];
@@ -871,19 +895,19 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
         }
       }
     } else if (staged) {
-      graph_degrees<D>(cst, pl, P, r2, deg);
+      graph_degrees<S, D>(cst, pl, P, r2, deg);
     } else {
-      graph_degrees<D>(cgl, pl, P, r2, deg);
+      graph_degrees<S, D>(cgl, pl, P, r2, deg);
     }
     for (int q = pl.po[P - 1] + tid; q < n; q += NT) deg[q] = 0;  // no candidates
     __syncthreads();
 
     // 2. offsets: event-local exclusive scan of min(deg, k_max), the event's
     //    count published
-    const int total = block_scan(deg, off, n, k_max, wsum);
+    const int total = block_scan<S>(deg, off, n, k_max, wsum);
     if (tid == 0) graph_publish(w.graph_desc, ev, total);
-    L.edges<D>(total);
-    const bool lists = masks && L.ints_all <= kGraphInts && n <= 65535 && total <= 65535;
+    L.edges<S, D>(total);
+    const bool lists = masks && L.ints_all <= S::INTS && n <= 65535 && total <= 65535;
     uint16_t* tgt = reinterpret_cast<uint16_t*>(sm_i + L.targets);
     uint16_t* list = reinterpret_cast<uint16_t*>(sm_i + L.lists);
     uint16_t* srcs = reinterpret_cast<uint16_t*>(sm_i + L.sources);
@@ -893,7 +917,7 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
       if (tid == 0) off[n] = total;
       for (int i = tid; i < n; i += NT) deg[i] = 0;
       __syncthreads();
-      for (int t = warp; t < pl.chunk[P - 1]; t += kGraphWarps) {
+      for (int t = warp; t < pl.chunk[P - 1]; t += S::WARPS) {
         const int p = plane_of(pl.chunk, P, t);
         const int q = pl.po[p] + (t - pl.chunk[p]) * 32 + lane;
         if (q >= pl.po[p + 1]) continue;
@@ -913,7 +937,7 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
       }
       __syncthreads();
       // 4. in-edge lists
-      block_scan(deg, start, n, 0x7fffffff, wsum);
+      block_scan<S>(deg, start, n, 0x7fffffff, wsum);
       for (int i = tid; i < n; i += NT) deg[i] = start[i];
       __syncthreads();
       for (int k = tid; k < total; k += NT) list[atomicAdd(&deg[tgt[k]], 1)] = uint16_t(k);
@@ -961,11 +985,11 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
         w.d2[base + k] = cst.d2(qe, c);
       }
     } else if (masks) {
-      graph_fill_masks<D>(w, cst, pl, P, off, mask, base, v0);
+      graph_fill_masks<S, D>(w, cst, pl, P, off, mask, base, v0);
     } else if (staged) {
-      graph_fill<D>(w, cst, pl, P, r2, k_max, deg, off, base, v0);
+      graph_fill<S, D>(w, cst, pl, P, r2, k_max, deg, off, base, v0);
     } else {
-      graph_fill<D>(w, cgl, pl, P, r2, k_max, deg, off, base, v0);
+      graph_fill<S, D>(w, cgl, pl, P, r2, k_max, deg, off, base, v0);
     }
     if (lists && fits) {
       for (int i = tid; i < total; i += NT) {
@@ -979,7 +1003,7 @@ __global__ void __launch_bounds__(kGraphThreads, 1) k_graph_event(Batch b, Ws w,
       if (tid == 0) w.in_ptr[v1] = e1;  // the next event writes the same value
     } else {  // (an event that overflows the workspace: its lists end there)
       __syncthreads();  // edges written; shared memory free
-      csc_general(w, n, v0, v1, e0, e1, sm_i, wsum);
+      csc_general<S>(w, n, v0, v1, e0, e1, sm_i, wsum);
     }
     __syncthreads();  // shared memory and ticket_s are reused by the next event
   }
@@ -1001,21 +1025,31 @@ int num_sms() {
 // 215 thousand cycles in one block; 75 events of 1671 hits: 44 of 83 thousand).
 // A block takes a whole SM, and clusters are placed within groups of SMs, so
 // the lines leave room: 8 blocks up to 12 events, 4 up to 30, 2 up to 76.
-template <int D>
-void graph_d(const Batch& b, const Ws& w, const GraphParams& g, cudaStream_t s) {
+template <class S, int D, bool CLUSTER>
+void graph_shape(const Batch& b, const Ws& w, const GraphParams& g, int ranks, GraphWhen when, cudaStream_t s) {
   // set once per instantiation (thread-safe initialisation of a local static)
   static const bool attr = [] {
-    cudaFuncSetAttribute(k_graph_event<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kGraphInts * 4);
-    cudaFuncSetAttribute(k_graph_event<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kGraphInts * 4);
+    cudaFuncSetAttribute(k_graph_event<S, D, CLUSTER>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         S::INTS * 4);
     return true;
   }();
   (void)attr;
+  launch_pdl(true, k_graph_event<S, D, CLUSTER>, std::min(b.n_events, num_sms() * S::PER_SM) * ranks, S::NT,
+             S::INTS * 4, s, ranks, b, w, g, when);
+}
+
+template <int D>
+int graph_d(const Batch& b, const Ws& w, const GraphParams& g, cudaStream_t s) {
   const int sms = num_sms(), n = b.n_events;
   const int ranks = 12 * n <= sms ? 8 : 5 * n <= sms ? 4 : 2 * n <= sms ? 2 : 1;
-  launch_pdl(true, ranks > 1 ? k_graph_event<D, true> : k_graph_event<D, false>,
-             std::min(n, sms) * ranks, kGraphThreads, kGraphInts * 4, s, ranks, b, w, g);
+  if (ranks > 1) {
+    graph_shape<GraphWide, D, true>(b, w, g, ranks, G_ALWAYS, s);
+    return 1;
+  }
+  const bool by_largest = by_largest_event(n, b.n_hits, sms);
+  if (by_largest) graph_shape<GraphMid, D, false>(b, w, g, 1, G_ALL_SMALL, s);
+  graph_shape<GraphWide, D, false>(b, w, g, 1, by_largest ? G_SOME_LARGE : G_ALWAYS, s);
+  return by_largest ? 2 : 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -1135,19 +1169,19 @@ void launch_scan(const int32_t* in, int32_t* out, int n, int clamp_max, int32_t*
              total_slot);
 }
 
-void launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s) {
-  if (b.n_events <= 0) return;
+int launch_graph(const Batch& b, const Ws& w, const GraphParams& g, int D, cudaStream_t s) {
+  if (b.n_events <= 0) return 0;
   switch (D) {
-    case 1: graph_d<1>(b, w, g, s); break;
-    case 2: graph_d<2>(b, w, g, s); break;
-    case 3: graph_d<3>(b, w, g, s); break;
-    case 4: graph_d<4>(b, w, g, s); break;
-    case 5: graph_d<5>(b, w, g, s); break;
-    case 6: graph_d<6>(b, w, g, s); break;
-    case 7: graph_d<7>(b, w, g, s); break;
-    case 8: graph_d<8>(b, w, g, s); break;
-    case 16: graph_d<16>(b, w, g, s); break;
-    default: break;
+    case 1: return graph_d<1>(b, w, g, s);
+    case 2: return graph_d<2>(b, w, g, s);
+    case 3: return graph_d<3>(b, w, g, s);
+    case 4: return graph_d<4>(b, w, g, s);
+    case 5: return graph_d<5>(b, w, g, s);
+    case 6: return graph_d<6>(b, w, g, s);
+    case 7: return graph_d<7>(b, w, g, s);
+    case 8: return graph_d<8>(b, w, g, s);
+    case 16: return graph_d<16>(b, w, g, s);
+    default: return 0;
   }
 }
 

@@ -179,3 +179,65 @@ def test_graph_of_large_events_in_every_cluster_width(line, over):
                 assert np.array_equal(g[k], want[k]), (tracks, k)
             assert np.array_equal(lab, want_lab), tracks
         tr.close()
+
+
+def _cut(ev, n):
+    return synth.Batch(ev.x[:n], ev.y[:n], ev.z[:n], ev.plane[:n], ev.pid[:n], np.array([0, n]))
+
+
+@pytest.mark.parametrize("largest", [140, 1280, 1281])
+@pytest.mark.parametrize("dim,k_max", [(4, 64), (8, 3), (16, 64)])
+def test_thousands_of_small_events(largest, dim, k_max):
+    """Batches of thousands of small events take smaller blocks in the graph kernel
+    unless one event is large (the line lies at 1280 hits): sampled events, empty ones
+    and the largest among them, get the graphs and labels they get alone, to the bit."""
+    n = 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    wl = dict(synth.workload("cfg1_plain_fp32"), k_max=k_max, radius2=0.05)
+    wl["model"] = {"embed": [3, 8, dim], "hidden": 32, "iters": 1}
+    kinds = [synth.gen_batch(1, 40 + t, {"kind": "fixed", "n": t}, 0.05) for t in range(9)]
+    parts = [kinds[(i * 7) % 9] for i in range(n)]
+    parts[n // 3] = _cut(synth.gen_batch(1, 77, {"kind": "fixed", "n": 130}, 0.05), largest)
+    b = synth.concat(parts)
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=b.n_hits, max_events=n,
+                                  edges_per_hit=64)
+    labels = pkg.run_batch(tr, b)
+    sample = [0, 1, 2, n // 3 - 1, n // 3, n // 3 + 1, n - 2, n - 1]
+    got = [(tr.get_graph(e), labels[b.offsets[e]:b.offsets[e + 1]]) for e in sample]
+    assert sum(g["src"].size for g, _ in got) > 20
+    for e, (g, lab) in zip(sample, got):
+        want_lab = pkg.run_batch(tr, parts[e])
+        want = tr.get_graph(0)
+        for k in want:
+            assert np.array_equal(g[k], want[k]), (e, k)
+        assert np.array_equal(lab, want_lab), e
+    tr.close()
+
+
+def test_small_events_do_not_wait_for_a_whole_sm_each():
+    """The graph kernel's time for 20000 events of one track, alone and with one event
+    of 300 hits more: below two thirds of the time with one event of 1300 hits more, which
+    sends the batch to the blocks that take an SM each (1.2 ms, the time that every such
+    batch took with those blocks alone; 0.7 ms before they were introduced)."""
+    wl = synth.workload("cfg3_trained_bf16")
+    small = synth.gen_batch(20000, 5, {"kind": "fixed", "n": 1}, wl["noise"])
+    big = synth.gen_batch(1, 6, {"kind": "fixed", "n": 150}, wl["noise"])
+
+    def plus(n):
+        return synth.Batch(*(np.concatenate([getattr(small, k), getattr(big, k)[:n]])
+                             for k in ("x", "y", "z", "plane", "pid")),
+                           np.concatenate([small.offsets, [small.n_hits + n]]))
+
+    tr = pkg.tracker_for_workload(wl, precision="fp32", max_hits=small.n_hits + 1300,
+                                  max_events=20001, edges_per_hit=16)
+    ms = []
+    for b in (small, plus(300), plus(1300)):
+        pkg.run_batch(tr, b)
+        best = 1e9
+        for _ in range(5):
+            tr.set_profiling(True)
+            pkg.run_batch(tr, b)
+            best = min(best, tr.stage_times()["graph"][0])
+            tr.set_profiling(False)
+        ms.append(best)
+    tr.close()
+    assert max(ms[:2]) < ms[2] * 2 / 3, ms
