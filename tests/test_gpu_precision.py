@@ -592,3 +592,28 @@ def test_kept_fp32_choices_do_not_slow_other_sizes(name, events):
         tr.set_tuning({})
         tr.close()
     assert best[1] < 1.25 * best[0] and best[2] < 1.25 * best[0], best
+
+
+@pytest.mark.parametrize("name,prec", [("cfg3_batched_bf16", "bf16"), ("cfg2_run3_single", "bf16"),
+                                       ("cfg3_batched_bf16", "fp8"), ("cfg2_run3_single", "fp8"),
+                                       ("cfg4_batched_fp8", "fp8")])
+def test_every_tensor_core_row_against_emulated_formats(name, prec):
+    """Every edge's logit against a host emulation of the format's roundings, row by
+    row, the event behind two others. Both round the same values; they differ where
+    sums taken in another order round to a neighbouring code, so by no more than the
+    largest error that all the roundings together make (emulated against exact: 0.02 to
+    0.03 in BF16, 0.2 to 0.3 in FP8, where the logits spread by 0.3 to 0.5 and a row
+    that took another's data or scale is off by about as much)."""
+    from quant_net import edge_logits
+    wl = synth.workload(name)
+    sh = synth.shape_of(wl)
+    ev = [synth.gen_batch(1, 300 + i, {"kind": "fixed", "n": n}, wl["noise"])
+          for i, n in enumerate((37, 5, 100))]
+    b, last = synth.concat(ev), ev[-1]
+    g = run(wl, b, prec)[1][2]
+    layers = synth.weight_arrays(synth.workload_weights(wl))[len(sh.embed) - 1:]
+    exact, emulated = (edge_logits(layers, sh.hidden, sh.iters, last.x, last.y, last.z, g["src"],
+                                   g["dst"], fmt) for fmt in ("exact", prec))
+    assert g["src"].size > 1000
+    err, bound = np.abs(g["logit"] - emulated).max(), np.abs(emulated - exact).max()
+    assert err <= bound, (err, bound)
