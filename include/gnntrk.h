@@ -370,8 +370,9 @@ int32_t gnntrk_stage_times(gnntrk_handle* h, int32_t max_stages, char* names, do
  *     the launch), 1 (tall tiles always) or 2 (as 0, short tiles up to twice as
  *     many rows);
  *     choice[4..6] = encoders, node step, edge step;
- *   - the BF16 edge step at hidden 32 (BF16 handles): form 0 (each thread
- *     copies its row's [e, h_src, h_dst] into the tile), 1 (the tile is
+ *   - the BF16 edge step at hidden 32 (BF16 handles): form 0 (the rows
+ *     [e, h_src, h_dst] copied into the tile by cp.async, four lanes per row, a
+ *     tile ahead), 1 (the tile is
  *     loaded by TMA: one box of 128 e rows and row gathers of h_src, h_dst)
  *     or 2 (TMA-loaded tiles in a ring, with a producer warp, an MMA warp and
  *     two epilogue warpgroups keeping several tiles in flight); choice[7]

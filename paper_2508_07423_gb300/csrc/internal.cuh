@@ -308,12 +308,16 @@ __device__ __forceinline__ int clamp_edges(const int32_t* counters, int64_t cap)
 // trained events (33 kernels) 516 -> 473 us.
 //
 // `early` (launch_pdl) says whether a kernel's blocks may come in before the
-// kernel ahead of it is done. Not the message kernels: their blocks, which need
-// no shared memory, then share SMs with a kernel that holds most of it, and
-// with what L1 is left the sums run slower (400 events in FP32 4.04 -> 4.46 ms per
-// call). Not the triplet kernels (500 events 2.96 -> 3.10 ms), and the
-// tensor-core kernels only up to kEarlyTcHits hits, where the launches count
-// (one event of 2146 hits in BF16 1.11 -> 1.07 ms; 1000 events 9.67 -> 9.78 ms).
+// kernel ahead of it is done: always for the sort, the per-event kernels of graph,
+// components and receptive field, the embedding and the FP32 network kernels
+// (triplet classifiers among them). Never for the message kernels: their blocks,
+// which need no shared memory, then share SMs with a kernel that holds most of it,
+// and with what L1 is left the sums run slower (measured on 400 events in FP32 only,
+// 4.04 -> 4.46 ms per call, and applied to every size). Never for the kernels that
+// list triplets and build tracks (measured on 500 events only, 2.96 -> 3.10 ms), nor
+// for the FP8 kernels. The BF16 tensor-core kernels (triplet classifiers and the FP8
+// path's encoders among them) up to kEarlyTcHits hits, a line between two measured
+// points: one event of 2146 hits 1.11 -> 1.07 ms, 1000 events 9.67 -> 9.78 ms.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

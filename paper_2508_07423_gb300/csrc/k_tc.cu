@@ -1209,7 +1209,8 @@ __global__ void __launch_bounds__((Layout<H, FP8, MODE>::THREADS), min_ctas(H, F
       hid_scale = sa[0];
     }
 
-    // hidden 128, BF16: the warp's state rows through its staging block
+    // the warp's state rows on their way out (and in, the residual, at hidden 128) through
+    // its staging block: the forms of Layout::OUT_STAGE and COOP
     constexpr bool NODE_ROWS = MODE == M_NODE_ENC || MODE == M_NODE_UPD;
     const int row0 = r - (tid & 31);
     RowStage<H, L::OUT_STAGE ? 64 : L::STAGE_ROW> st{
