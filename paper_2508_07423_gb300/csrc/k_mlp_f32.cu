@@ -410,8 +410,8 @@ struct WeightSource {
   static constexpr bool COPIES = WEIGHTS == W_BLOCK, RING = WEIGHTS == W_RING;
   // ring: KC rows of a matrix per chunk, NST chunks
   static constexpr int KC = 16, NST = 4;
-  // copies, or chunks with their barriers and counts
-  static constexpr int FLOATS = COPIES ? MATS * H * H : NST * KC * H + 4 * NST;
+  // copies with their barrier, or chunks with their barriers and counts
+  static constexpr int FLOATS = COPIES ? MATS * H * H + 4 : NST * KC * H + 4 * NST;
 };
 
 // Shape of one kernel: a tall and a short warp tile, warps per block (one block
@@ -530,25 +530,48 @@ struct WeightRing {
 
 // The weights a kernel multiplies by: matrix m of its layer sequence from the
 // copies in shared memory, or from the ring (which serves the matrices of every
-// tile in their order).
+// tile in their order). One thread asks for the copies in bulk, and they land while
+// the block waits for the kernel before it: copied by the block's threads they took
+// longer than that wait in kernels of a few microseconds, which hold an SM each (one
+// run-3 event, 18 such kernels: 417 -> 403 us per call alone, 253 -> 218 with eight
+// handles on eight streams).
 template <class X>
 struct LayerWeights {
   using W = typename X::W;
   const typename X::Args& p;
   WeightRing<X> ring;
   const float* copies = nullptr;
+  uint64_t* bar = nullptr;  // of the copies
 
   // block-wide, before pdl_wait (the weights are constant); smem: W::FLOATS floats
   __device__ __forceinline__ LayerWeights(const typename X::Args& a, float* smem) : p(a) {
     if constexpr (W::RING) ring.init(smem);
     if constexpr (W::COPIES) {
-      constexpr int N = X::H * X::H / 4;
-      for (int i = threadIdx.x; i < W::MATS * N; i += X::NW * 32)
-        reinterpret_cast<float4*>(smem)[i] =
-            __ldg(reinterpret_cast<const float4*>(X::mat(p, i / N)) + i % N);
+      constexpr int N = X::H * X::H;
       copies = smem;
+      bar = reinterpret_cast<uint64_t*>(smem + W::MATS * N);
+      if (threadIdx.x == 0) {
+        tc::mbar_init(bar, 1);
+        tc::fence_mbar_init();
+        tc::mbar_expect_tx(bar, W::MATS * N * 4);
+        for (int m = 0; m < W::MATS; ++m) tc::bulk_g2s(smem + m * N, X::mat(p, m), N * 4, bar);
+      }
     }
     __syncthreads();
+  }
+  // block-wide, before the first use of the copies and before any return (no copy may
+  // land after the block is gone); false: the wait ran out
+  __device__ __forceinline__ bool landed() {
+    if constexpr (W::COPIES) {
+      if (__syncthreads_or(!tc::mbar_wait_bounded(bar, 0, kRingWaitCycles))) {
+        if (threadIdx.x == 0) {
+          set_status(p.w.counters, ST_TIMEOUT);
+          tc::mbar_wait_bounded(bar, 0, kRingWaitCycles);
+        }
+        return false;
+      }
+    }
+    return true;
   }
   // the block walks tiles of `step` rows (per block) from block0 on
   __device__ __forceinline__ void start(int block0, int step, int hi) {
@@ -821,7 +844,7 @@ __global__ void __launch_bounds__(X::NW * 32, 1) k_gnn_f32(const GnnArgs p) {
   const Ws& w = p.w;
   LayerWeights<X> weights(p, sm + X::NW * X::WARP_FLOATS);
   pdl_begin();
-  if (input_bad(w)) return;
+  if (!weights.landed() || input_bad(w)) return;
   int lo, hi;
   if constexpr (X::MODE == G_TRIP) {
     if (*(volatile int32_t*)&w.counters[C_STATUS] & ST_CAPACITY) return;
@@ -1140,7 +1163,7 @@ __global__ void __launch_bounds__(X::NW * 32, 1) k_embed_tiles(const EmbedArgs p
     sm[X::NW * X::WARP_FLOATS + X::W::FLOATS + i] = lo.WT[i];
   LayerWeights<X> weights(p, sm + X::NW * X::WARP_FLOATS);  // (ends with a block barrier)
   pdl_begin();
-  if (input_bad(p.w)) return;
+  if (!weights.landed() || input_bad(p.w)) return;
   // short tiles while they fill at most one round of the grid's warps, as the
   // interaction-network kernels
   if (p.b.n_hits <= int64_t(gridDim.x) * X::NW * X::Short::WR)

@@ -91,3 +91,13 @@ def test_weight_ring_after_a_wait_that_ran_out():
     assert "c < late + W::NST && c < total" in d
     assert "mbar_wait_bounded(full + c % W::NST, (c / W::NST) & 1" in d
     assert "ring.drain()" in body("k_mlp_f32.cu", "finish")
+
+
+@pytest.mark.parametrize("kernel", ["k_gnn_f32", "k_embed_tiles"])
+def test_weight_copies_land_before_a_block_can_end(kernel):
+    """FP32 kernels: the bulk copies of the weights are waited for before the first
+    return, else a copy could land after the block is gone."""
+    b = body("k_mlp_f32.cu", kernel)
+    assert b.index("pdl_begin();") < b.index("weights.landed()") < b.index("return;")
+    w = body("k_mlp_f32.cu", "landed")
+    assert w.count("mbar_wait_bounded(bar, 0, kRingWaitCycles)") == 2  # once more on a timeout
